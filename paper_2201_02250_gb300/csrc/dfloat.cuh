@@ -94,6 +94,21 @@ __device__ __forceinline__ dfloat se_sqrt(dfloat a) {
   const dfloat r = a - dfloat(s, 0.f) * dfloat(s, 0.f);
   return df_quick_two_sum(s, __fdiv_rn(r.hi, 2.f * s));
 }
+// 1 / sqrt(a) for a > 0, and 1 / b for b in [1, 2]: the FP32 approximation y and one third-order step, with
+// the residual e = 1 - a y^2 (or 1 - b y) formed in double-float; e is about 2^-21, so its FP32 rounding
+// and the terms dropped lie below the pair's last bit
+__device__ __forceinline__ dfloat se_rsqrt(dfloat a) {
+  const float y = rsqrtf(a.hi);
+  const dfloat p = (a * dfloat(y, 0.f)) * dfloat(y, 0.f);
+  const float e = __fsub_rn(__fsub_rn(1.f, p.hi), p.lo);
+  return df_quick_two_sum(y, __fmul_rn(__fmul_rn(y, e), __fmaf_rn(0.375f, e, 0.5f)));
+}
+__device__ __forceinline__ dfloat se_recip12(dfloat b) {
+  const float y = __fdividef(1.f, b.hi);
+  const dfloat p = b * dfloat(y, 0.f);
+  const float e = __fsub_rn(__fsub_rn(1.f, p.hi), p.lo);
+  return df_quick_two_sum(y, __fmul_rn(y, __fmaf_rn(e, e, e)));
+}
 __device__ __forceinline__ double se_dbl(dfloat a) { return (double)a; }
 __device__ __forceinline__ void se_mac(dfloat& acc, dfloat a, dfloat b) { df_mac(acc, a, b); }
 __device__ __forceinline__ dfloat se_fin(dfloat a) { return df_normalize(a); }

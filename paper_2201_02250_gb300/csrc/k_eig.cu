@@ -786,7 +786,8 @@ __global__ void k_rayleigh_ritz(RRParams prm, const int* full, const int* mfull,
   double* wi = wr + m;               // m
   int* perm = reinterpret_cast<int*>(wi + m);  // m
   const double* Hi = H + (int64_t)i * EIG_MAXP * EIG_MAXP;
-  const se::Team team{(int)threadIdx.x, (int)blockDim.x};
+  __shared__ int team_red[RR_THREADS / 32];
+  const se::Team team{(int)threadIdx.x, (int)blockDim.x, team_red};
   for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
     S[(e / m) * ld + e % m] = (R)Hi[(e / m) * EIG_MAXP + e % m];
     Q[(e / m) * ld + e % m] = (R)((e / m == e % m) ? 1.0 : 0.0);
@@ -832,11 +833,9 @@ __global__ void k_rayleigh_ritz(RRParams prm, const int* full, const int* mfull,
   const int rc = se::schur(S, ld, Q, ld, m, snorm, team, snap, 1e-3 * prm.tol);
   if (rc != 0 && threadIdx.x == 0) raise_status(st, A2LS_ERR_EIGEN, i, 2);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    se::schur_eigenvalues(S, ld, m, wr, wi);
-    se::order_by_modulus(wr, wi, m, perm, mod);
-  }
+  if (threadIdx.x == 0) se::schur_eigenvalues(S, ld, m, wr, wi);
   __syncthreads();
+  se::order_by_modulus(wr, wi, m, perm, mod, team);
   // plan the columns: walk eigenvalues by modulus, pairs take two columns
   // lane j handles the j-th selected eigenvalue
   __shared__ int sel_pos[32], sel_col[32], sel_two[32], nsel_s, ncol_s, zc_s;

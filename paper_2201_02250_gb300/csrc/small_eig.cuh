@@ -24,10 +24,23 @@ namespace se {
 
 struct Team {
   int lane, size;
+  int* red = nullptr;  // GPU: one int of shared scratch per warp, for max()
   SE_HD void sync() const {
 #ifdef __CUDA_ARCH__
     __syncthreads();
 #endif
+  }
+  // the largest v over the team (on the GPU full warps, and a barrier: shared memory written before the
+  // call may be overwritten after it)
+  SE_HD int max(int v) const {
+#ifdef __CUDA_ARCH__
+    v = __reduce_max_sync(0xffffffffu, v);
+    __syncthreads();  // red may still be read by the previous call
+    if ((lane & 31) == 0) red[lane >> 5] = v;
+    __syncthreads();
+    for (int w = 0; w < (size >> 5); ++w) v = red[w] > v ? red[w] : v;
+#endif
+    return v;
   }
 };
 
@@ -40,6 +53,32 @@ SE_HD inline double se_dbl(double x) { return x; }
 // unnormalised multiply-add overloads both)
 SE_HD inline void se_mac(double& acc, double a, double b) { acc += a * b; }
 SE_HD inline double se_fin(double a) { return a; }
+// 1 / sqrt(a) for a > 0 and 1 / b for b in [1, 2], to rounding accuracy.  On the GPU: the hardware's
+// approximation (about 2^-20) and one third-order step each (with e = 1 - a y^2,
+// 1 / sqrt(a) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2 / 8 + O(e^3)); 1 / b = y / (1 - e) likewise): a
+// chain of four and of three FP64 operations where sqrt and the division are library routines of
+// dozens, on a pipe that issues two lanes a cycle per SM.
+SE_HD inline double se_rsqrt(double a) {
+#ifdef __CUDA_ARCH__
+  if (!(a > 1e-280 && a < 1e280)) return 1.0 / sqrt(a);  // outside the approximation's safe range
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double e = fma(-(a * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+#else
+  return 1.0 / sqrt(a);
+#endif
+}
+SE_HD inline double se_recip12(double b) {
+#ifdef __CUDA_ARCH__
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+  const double e = fma(-b, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+#else
+  return 1.0 / b;
+#endif
+}
 template <class R> struct SeEps {
   static constexpr double v = 2.220446049250313e-16;  // machine epsilon of R
   static constexpr double big = 1e100;                // rescaling threshold of the back substitution
@@ -153,17 +192,20 @@ SE_HD inline void apply_reflector(R* H, int ld, R* Q, int ldq, int m, int k, int
 
 // Householder reflector mapping (x, y, z) to (alpha, 0, 0): returns alpha, beta and u = (1, u1, u2).
 // With v = (v0, y, z), v0 = x - alpha, v^T v = 2 |alpha| |v0|, so beta = 2 v0^2 / v^T v = v0 / (-alpha).
+// With r = 1 / |(x, y, z)|: beta = 1 + |x| r (between 1 and 2) and 1 / v0 = sign(x) r / beta.  The chain of
+// a sweep's reflectors is what bounds the Schur iteration, so they are formed without a square root or a
+// division: with the deflation scan and the ordering of the eigenvalues spread over the team, an FP64 setup
+// and solve of 16 subdomains (order 48) 84.0 -> 72.7 ms, a double-float one of 256 (order 72) 120.5 -> 116.2.
 template <class R>
 SE_HD inline bool make_reflector(R x, R y, R z, R& u1, R& u2, R& beta, R& alpha) {
-  R nrm = se_sqrt(x * x + y * y + z * z);
-  if (nrm == 0.0) return false;
-  alpha = -sgn(nrm, x);
-  R v0 = x - alpha;
-  if (v0 == 0.0) return false;
-  const R iv = R(1.0) / v0;
+  const R s = x * x + y * y + z * z;
+  if (s == R(0.0)) return false;
+  const R r = se_rsqrt(s);
+  beta = R(1.0) + se_abs(x) * r;
+  alpha = -sgn(s * r, x);
+  const R iv = sgn(r * se_recip12(beta), x);
   u1 = y * iv;
   u2 = z * iv;
-  beta = v0 / (-alpha);
   return true;
 }
 
@@ -223,13 +265,17 @@ SE_HD inline int schur(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const 
   const R leps = R(local_tol > SeEps<R>::v ? local_tol : SeEps<R>::v);
   int hi = m - 1, iter = 0, total = 0;
   while (hi >= 0) {
-    int lo = hi;
-    while (lo > 0) {
-      R s = se_abs(H[(lo - 1) * ld + lo - 1]) + se_abs(H[lo * ld + lo]);
-      const R sub = se_abs(H[lo * ld + lo - 1]);
-      if (sub <= leps * s || sub <= eps * hnorm) break;
-      --lo;
+    // the largest lo <= hi whose subdiagonal entry is negligible (0 if there is none), one entry per thread
+    int lo = 0;
+    for (int j = hi - t.lane; j > 0; j -= t.size) {
+      const R s = se_abs(H[(j - 1) * ld + j - 1]) + se_abs(H[j * ld + j]);
+      const R sub = se_abs(H[j * ld + j - 1]);
+      if (sub <= leps * s || sub <= eps * hnorm) {
+        lo = j;
+        break;
+      }
     }
+    lo = t.max(lo);
     if (lo > 0) {
       t.sync();
       if (t.lane == 0) H[lo * ld + lo - 1] = 0.0;
@@ -539,27 +585,24 @@ SE_HD inline void schur_vector(const R* S, int ld, int m, int p, double lr_, dou
   }
 }
 
-// Order of eigenvalues by decreasing modulus; within a pair the +imag member first.
-// perm: m ints; mod: m doubles of scratch.  Selection sort (m is small).
-SE_HD inline void order_by_modulus(const double* wr, const double* wi, int m, int* perm, double* mod) {
-  for (int j = 0; j < m; ++j) {
-    perm[j] = j;
-    mod[j] = hypot(wr[j], wi[j]);
+// Order of eigenvalues by decreasing modulus; within a pair the +imag member first, otherwise equal
+// moduli in the order of their positions.  perm: m ints; mod: m doubles of scratch (the moduli).  One
+// eigenvalue per thread finds its rank; ends with a barrier.
+SE_HD inline void order_by_modulus(const double* wr, const double* wi, int m, int* perm, double* mod,
+                                   const Team& t = Team{0, 1}) {
+  for (int j = t.lane; j < m; j += t.size) {
+    const double a = hypot(wr[j], wi[j]);
+    mod[j] = a >= 0.0 ? a : -1.0;  // a NaN ranks last: the ranks stay a permutation
   }
-  for (int a = 0; a < m; ++a) {
-    int best = a;
-    double bm = mod[perm[a]];
-    for (int b = a + 1; b < m; ++b) {
-      const double mb = mod[perm[b]];
-      if (mb > bm * (1 + 1e-14) || (fabs(mb - bm) <= 1e-14 * bm && wi[perm[b]] > wi[perm[best]])) {
-        best = b;
-        bm = mb;
-      }
-    }
-    const int tmp = perm[a];
-    perm[a] = perm[best];
-    perm[best] = tmp;
+  t.sync();
+  for (int j = t.lane; j < m; j += t.size) {
+    int rank = 0;
+    const double mj = mod[j], ij = wi[j];
+    for (int k = 0; k < m; ++k)
+      rank += (mod[k] > mj || (mod[k] == mj && (wi[k] > ij || (!(wi[k] < ij) && k < j)))) ? 1 : 0;
+    perm[rank] = j;
   }
+  t.sync();
 }
 
 }  // namespace se
