@@ -359,6 +359,71 @@ __global__ void __launch_bounds__(256) k_propagate(const int* off, const int64_t
   }
 }
 
+// The same steps with the iterates in shared memory.  The columns of p are independent, so a CTA takes
+// one subdomain and PROP_COLS of the 16 columns (blockIdx.y), keeps both iterates and the third array
+// (p_0, or the adjoint's accumulator) there, and only the edge lists come from L1 / L2 each step.  What
+// bounds the kernel above is the dependent chain row pointer -> column -> iterate through L2 in each of
+// the 32 steps on N of the 152 SMs; here the last link is shared memory, a thread moves four columns
+// with one access, and four times as many CTAs run.  A loss and gradient over 64 subdomains of 1024 to
+// 1284 rows (two propagations): 6.64 -> 2.35 ms, the propagations 2.2 ms each before.
+constexpr int PROP_COLS = 4, PROP_THREADS = 512;
+constexpr size_t PROP_ROW_BYTES = 3 * PROP_COLS * sizeof(float);
+constexpr size_t PROP_SMEM_MAX = 220 * 1024;   // subdomains of up to 4693 rows; larger ones above
+
+template <bool ADJ>
+__global__ void __launch_bounds__(PROP_THREADS) k_propagate_smem(const int* off, const int64_t* __restrict__ rp,
+                                                                 const int* __restrict__ col,
+                                                                 const float* __restrict__ s,
+                                                                 const float* __restrict__ in, float* out) {
+  extern __shared__ __align__(16) float4 prop_smem[];
+  const int i = blockIdx.x, o = off[i], n = off[i + 1] - o;
+  const int c0 = blockIdx.y * PROP_COLS;
+  float4 *src = prop_smem, *dst = src + n, *third = dst + n;
+  // a row is always touched by the same thread, but for the iterates that its neighbours read
+  for (int l = threadIdx.x; l < n; l += PROP_THREADS) {
+    const float4 v = *reinterpret_cast<const float4*>(in + (int64_t)(o + l) * OUT + c0);
+    src[l] = v;
+    third[l] = ADJ ? make_float4(0.f, 0.f, 0.f, 0.f) : v;
+  }
+  __syncthreads();
+  for (int k = 0; k < K_PROP; ++k) {
+    for (int l = threadIdx.x; l < n; l += PROP_THREADS) {
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+      const int64_t e1 = rp[o + l + 1];
+#pragma unroll 4
+      for (int64_t e = rp[o + l]; e < e1; ++e) {
+        const int q = col[e];
+        if (q >= 0) {
+          const float w = s[e];
+          const float4 v = src[q - o];
+          a.x = fmaf(w, v.x, a.x);
+          a.y = fmaf(w, v.y, a.y);
+          a.z = fmaf(w, v.z, a.z);
+          a.w = fmaf(w, v.w, a.w);
+        }
+      }
+      const float4 t = third[l];
+      float4 r;
+      if (!ADJ) {
+        r = make_float4((1.f - ALPHA) * a.x + ALPHA * t.x, (1.f - ALPHA) * a.y + ALPHA * t.y,
+                        (1.f - ALPHA) * a.z + ALPHA * t.z, (1.f - ALPHA) * a.w + ALPHA * t.w);
+      } else {
+        const float4 g = src[l];
+        const float4 av = make_float4(t.x + ALPHA * g.x, t.y + ALPHA * g.y, t.z + ALPHA * g.z, t.w + ALPHA * g.w);
+        r = make_float4((1.f - ALPHA) * a.x, (1.f - ALPHA) * a.y, (1.f - ALPHA) * a.z, (1.f - ALPHA) * a.w);
+        if (k == K_PROP - 1) r = make_float4(r.x + av.x, r.y + av.y, r.z + av.z, r.w + av.w);
+        third[l] = av;
+      }
+      if (k == K_PROP - 1) *reinterpret_cast<float4*>(out + (int64_t)(o + l) * OUT + c0) = r;
+      else dst[l] = r;
+    }
+    __syncthreads();
+    float4* tmp = src;
+    src = dst;
+    dst = tmp;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // loss: one CTA per subdomain
 // ---------------------------------------------------------------------------
@@ -767,6 +832,8 @@ static void set_smem_limits() {
   A2LS_CUDA(cudaFuncSetAttribute(k_layer_fwd<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FWD_SMEM));
   A2LS_CUDA(cudaFuncSetAttribute(k_layer_bwd<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BWD1_SMEM));
   A2LS_CUDA(cudaFuncSetAttribute(k_layer_bwd<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BWD_SMEM));
+  A2LS_CUDA(cudaFuncSetAttribute(k_propagate_smem<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PROP_SMEM_MAX));
+  A2LS_CUDA(cudaFuncSetAttribute(k_propagate_smem<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PROP_SMEM_MAX));
   done = true;
 }
 
@@ -779,6 +846,7 @@ struct Graph {
   const float* w;
   const float* s;
   const float* X;
+  int max_n;  // rows of the largest subdomain
 };
 
 // activations of one forward pass; h[0..3] and m[1..3] are kept only when training
@@ -797,6 +865,19 @@ static void build_graph(cudaStream_t st, int64_t* cnt, int N, const int* off, co
   double* dscr = galloc<double>(tmp, S, st);
   double* gscr = galloc<double>(tmp, S, st);
   k_graph_features<<<N, 256, 0, st>>>(off, nI, lrow, lcol, lval, lump, col, w, s, X, dscr, gscr);
+  GNN_LAUNCH(cnt);
+}
+
+// in, out: rows x 16; bufA, bufB, acc: scratch of the same shape, used only by subdomains too large for
+// the shared-memory form
+template <bool ADJ>
+static void propagate(cudaStream_t st, int64_t* cnt, const Graph& g, const float* in, float* bufA, float* bufB,
+                      float* acc, float* out) {
+  const size_t smem = PROP_ROW_BYTES * (size_t)g.max_n;
+  if (smem <= PROP_SMEM_MAX)
+    k_propagate_smem<ADJ><<<dim3(g.N, OUT / PROP_COLS), PROP_THREADS, smem, st>>>(g.off, g.rp, g.col, g.s, in, out);
+  else
+    k_propagate<ADJ><<<g.N, 256, 0, st>>>(g.off, g.rp, g.col, g.s, in, bufA, bufB, acc, out);
   GNN_LAUNCH(cnt);
 }
 
@@ -826,8 +907,7 @@ static void forward(cudaStream_t st, int64_t* cnt, const Graph& g, const __nv_bf
     }
     GNN_LAUNCH(cnt);
   }
-  k_propagate<false><<<g.N, 256, 0, st>>>(g.off, g.rp, g.col, g.s, a.p0, a.pa, a.pb, nullptr, a.Y);
-  GNN_LAUNCH(cnt);
+  propagate<false>(st, cnt, g, a.p0, a.pa, a.pb, nullptr, a.Y);
 }
 
 static void alloc_acts(std::vector<void*>& tmp, cudaStream_t st, int S, bool train, Acts& a) {
@@ -842,7 +922,11 @@ static void alloc_acts(std::vector<void*>& tmp, cudaStream_t st, int S, bool tra
   a.pb = galloc<float>(tmp, ps, st);
 }
 
-static Graph sample_graph(const a2ls_gnn_sample* s) { return Graph{s->N, s->S, s->off, s->rp, s->col, s->w, s->s, s->X}; }
+static Graph sample_graph(const a2ls_gnn_sample* s) {
+  int max_n = 0;
+  for (int i = 0; i < s->N; ++i) max_n = std::max(max_n, s->h_off[i + 1] - s->h_off[i]);
+  return Graph{s->N, s->S, s->off, s->rp, s->col, s->w, s->s, s->X, max_n};
+}
 
 }  // namespace gnn
 
@@ -863,7 +947,7 @@ void gnn_infer(a2ls_handle* h, const a2ls_gnn* model, float* Y) {
     float* X = galloc<float>(tmp, (size_t)S * FX, st);
     build_graph(st, &h->launches, h->N, h->d_off, h->d_nI, h->d_lrow, h->d_lcol, h->d_lval, h->d_lump, S, col, w,
                 sv, X, tmp);
-    Graph g{h->N, S, h->d_off, h->d_lrow, col, w, sv, X};
+    Graph g{h->N, S, h->d_off, h->d_lrow, col, w, sv, X, h->max_n};
     Acts a;
     alloc_acts(tmp, st, S, false, a);
     forward(st, &h->launches, g, model->w16, model->theta, false, a);
@@ -1182,8 +1266,7 @@ int a2ls_gnn_loss_grad(a2ls_gnn* g, a2ls_gnn_sample* s, double* loss) {
       k_loss<<<N, 256, 0, st>>>(s->off, s->zm, s->zoff, s->Z, a.Y, 1.f / (float)s->ntarget, d_loss, dY);
       GNN_LAUNCH(&g->launches);
       // dp_0 into a.p0 (p_0 itself is no longer needed), scratch a.pa / a.pb / a.Y
-      k_propagate<true><<<N, 256, 0, st>>>(s->off, s->rp, s->col, s->s, dY, a.pa, a.pb, a.Y, a.p0);
-      GNN_LAUNCH(&g->launches);
+      propagate<true>(st, &g->launches, gr, dY, a.pa, a.pb, a.Y, a.p0);
       const int tiles = (S + TILE - 1) / TILE;
       const int G = std::max(1, std::min(tiles, 2 * 152));
       float* part = galloc<float>(tmp, (size_t)G * NP, st);
