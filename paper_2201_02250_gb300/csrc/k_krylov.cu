@@ -16,27 +16,53 @@
 namespace a2ls {
 
 // ---------------------------------------------------------------------------
-// CSR SpMV: y = A x, or y = bm - A x when bm != nullptr; one warp per 32 rows,
-// 4 lanes per row for short rows
+// CSR SpMV: y = A x, or y = bm - A x when bm != nullptr.  A CTA takes ROWS consecutive rows: their entries
+// are one contiguous piece of colind and val, which the threads read coalesced (SPMV_UNROLL entries each
+// in flight) into products in shared memory, and one thread per row sums its own in order; rows whose
+// entries do not fit the products' space are summed piece by piece.  Bound by memory: 12 bytes an entry.
+// Against 4 lanes per row, whose loads leave one gather in flight at a time: 41.7 -> 32.8 us on
+// the 96^3 seven-point operator (91 MB).
+// ROWS: 256, or 64 where 256 would leave SMs idle (fewer rows than two CTAs per SM).
 // ---------------------------------------------------------------------------
-__global__ void k_spmv(int n, const int* __restrict__ rowptr, const int* __restrict__ colind,
-                       const double* __restrict__ val, const double* __restrict__ x, double* __restrict__ y,
-                       const double* __restrict__ bm) {
-  const int sub = threadIdx.x & 3;
-  for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 2; r < n; r += (gridDim.x * blockDim.x) >> 2) {
-    double s = 0.0;
-    const int a = rowptr[r], b = rowptr[r + 1];
-    for (int q = a + sub; q < b; q += 4) s += val[q] * __ldg(x + colind[q]);
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    if (sub == 0) y[r] = bm ? bm[r] - s : s;
+constexpr int SPMV_UNROLL = 8;
+template <int ROWS>
+__global__ void __launch_bounds__(ROWS) k_spmv(int n, const int* __restrict__ rowptr, const int* __restrict__ colind,
+                                               const double* __restrict__ val, const double* __restrict__ x,
+                                               double* __restrict__ y, const double* __restrict__ bm) {
+  constexpr int CAP = ROWS * SPMV_UNROLL;
+  __shared__ double prod[CAP];
+  const int tid = threadIdx.x, r0 = blockIdx.x * ROWS, r = r0 + tid;
+  const int e0 = rowptr[r0], e1 = rowptr[min(r0 + ROWS, n)];
+  const int a = r < n ? rowptr[r] : e1, b = r < n ? rowptr[r + 1] : e1;
+  double s = 0.0;
+  for (int base = e0; base < e1; base += CAP) {
+    const int cnt = min(CAP, e1 - base);
+    int c[SPMV_UNROLL];
+    double v[SPMV_UNROLL];
+#pragma unroll
+    for (int u = 0; u < SPMV_UNROLL; ++u) {
+      const int e = tid + u * ROWS;
+      c[u] = e < cnt ? colind[base + e] : 0;
+      v[u] = e < cnt ? val[base + e] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < SPMV_UNROLL; ++u) {
+      const int e = tid + u * ROWS;
+      if (e < cnt) prod[e] = v[u] * __ldg(x + c[u]);
+    }
+    __syncthreads();
+    const int q1 = min(b - base, cnt);
+    for (int q = max(a - base, 0); q < q1; ++q) s += prod[q];
+    __syncthreads();
   }
+  if (r < n) y[r] = bm ? bm[r] - s : s;
 }
 
 void spmv(a2ls_handle* h, const double* x, double* y, const double* b_minus, cudaStream_t st) {
-  const int threads = 256;
-  const int blocks = std::min(152 * 8, ceil_div((int64_t)h->n * 4, threads));
-  k_spmv<<<blocks, threads, 0, st>>>(h->n, h->rowptr, h->colind, h->val, x, y, b_minus);
+  if (h->n >= 2 * 152 * 256)
+    k_spmv<256><<<ceil_div(h->n, 256), 256, 0, st>>>(h->n, h->rowptr, h->colind, h->val, x, y, b_minus);
+  else
+    k_spmv<64><<<ceil_div(h->n, 64), 64, 0, st>>>(h->n, h->rowptr, h->colind, h->val, x, y, b_minus);
   A2LS_LAUNCH();
 }
 
