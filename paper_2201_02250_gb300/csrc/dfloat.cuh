@@ -94,27 +94,57 @@ __device__ __forceinline__ dfloat se_sqrt(dfloat a) {
   const dfloat r = a - dfloat(s, 0.f) * dfloat(s, 0.f);
   return df_quick_two_sum(s, __fdiv_rn(r.hi, 2.f * s));
 }
-// 1 / sqrt(a) for a > 0, and 1 / b for b in [1, 2]: the FP32 approximation y and one third-order step, with
-// the residual e = 1 - a y^2 (or 1 - b y) formed in double-float; e is about 2^-21, so its FP32 rounding
-// and the terms dropped lie below the pair's last bit
+// 1 / sqrt(a) for a > 0, and 1 / b for b in [1, 2]: the FP32 approximation y and one third-order step with
+// the residual e = 1 - a y^2 (or 1 - b y), which is about 2^-21.  e is kept as a pair and its product with
+// y exactly, so that the result is good to the pair's 48 bits, as the library-division forms above are.
+__device__ __forceinline__ dfloat df_one_minus(dfloat p) { return df_two_sum(__fsub_rn(1.f, p.hi), -p.lo); }
 __device__ __forceinline__ dfloat se_rsqrt(dfloat a) {
   const float y = rsqrtf(a.hi);
-  const dfloat p = (a * dfloat(y, 0.f)) * dfloat(y, 0.f);
-  const float e = __fsub_rn(__fsub_rn(1.f, p.hi), p.lo);
-  return df_quick_two_sum(y, __fmul_rn(__fmul_rn(y, e), __fmaf_rn(0.375f, e, 0.5f)));
+  const dfloat e = df_one_minus((a * dfloat(y, 0.f)) * dfloat(y, 0.f));
+  const float g = __fmul_rn(0.5f, e.hi), p = __fmul_rn(y, g), err = __fmaf_rn(y, g, -p);
+  const float tail = __fmul_rn(y, __fmaf_rn(__fmul_rn(0.375f, e.hi), e.hi, __fmul_rn(0.5f, e.lo)));
+  const dfloat s = df_quick_two_sum(y, p);
+  return df_quick_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(err, tail)));
 }
 __device__ __forceinline__ dfloat se_recip12(dfloat b) {
   const float y = __fdividef(1.f, b.hi);
-  const dfloat p = b * dfloat(y, 0.f);
-  const float e = __fsub_rn(__fsub_rn(1.f, p.hi), p.lo);
-  return df_quick_two_sum(y, __fmul_rn(y, __fmaf_rn(e, e, e)));
+  const dfloat e = df_one_minus(b * dfloat(y, 0.f));
+  const float p = __fmul_rn(y, e.hi), err = __fmaf_rn(y, e.hi, -p);
+  const float tail = __fmul_rn(y, __fmaf_rn(e.hi, e.hi, e.lo));
+  const dfloat s = df_quick_two_sum(y, p);
+  return df_quick_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(err, tail)));
 }
+__device__ __forceinline__ dfloat se_scale_to_one(dfloat a) {
+  return dfloat(a.hi > 1e-30f && a.hi < 1e30f ? __fdividef(1.f, a.hi) : 1.f, 0.f);
+}
+// the power of two of a's exponent (1 outside 2^-120 .. 2^120) and the inverse of such a power
+__device__ __forceinline__ dfloat se_pow2(dfloat a) {
+  const unsigned e = __float_as_uint(a.hi) & 0x7f800000u;
+  return dfloat(e - (7u << 23) <= (240u << 23) ? __uint_as_float(e) : 1.f, 0.f);
+}
+__device__ __forceinline__ dfloat se_pow2_inv(dfloat p) {
+  return dfloat(__uint_as_float((254u << 23) - __float_as_uint(p.hi)), 0.f);
+}
+__device__ __forceinline__ dfloat se_warp_maxabs(dfloat a) {
+  float v = a.hi;
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return dfloat(v, 0.f);
+}
+__device__ __forceinline__ constexpr bool se_range_limited(dfloat) { return true; }
+__device__ __forceinline__ bool se_is_zero(dfloat a) { return a.hi == 0.f; }
 __device__ __forceinline__ double se_dbl(dfloat a) { return (double)a; }
 __device__ __forceinline__ void se_mac(dfloat& acc, dfloat a, dfloat b) { df_mac(acc, a, b); }
 __device__ __forceinline__ dfloat se_fin(dfloat a) { return df_normalize(a); }
 
 __device__ __forceinline__ dfloat shfl_xor(dfloat v, int lane_mask) {
   return dfloat(__shfl_xor_sync(0xffffffffu, v.hi, lane_mask), __shfl_xor_sync(0xffffffffu, v.lo, lane_mask));
+}
+__device__ __forceinline__ dfloat se_warp_sum(dfloat v) {
+  for (int o = 16; o > 0; o >>= 1) v += shfl_xor(v, o);
+  return v;
+}
+__device__ __forceinline__ dfloat se_warp_get(dfloat v, int lane) {
+  return dfloat(__shfl_sync(0xffffffffu, v.hi, lane), __shfl_sync(0xffffffffu, v.lo, lane));
 }
 #endif
 

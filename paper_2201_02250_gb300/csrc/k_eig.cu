@@ -38,7 +38,6 @@ template <> struct SeEps<dfloat> {
   static constexpr double v = 1.4210854715202004e-14;  // 2^-46
   static constexpr double big = 1e30;                  // within FP32's exponent range
 };
-template <> struct SeEarlyReflector<dfloat> { static constexpr bool value = false; };
 }  // namespace se
 
 template <class T> struct EAcc;
@@ -737,13 +736,14 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
 // Rayleigh-Ritz on H (one CTA per subdomain): Ritz values, the real basis Y of
 // the leading Ritz vectors (bcols columns), residual norms and convergence.
 // ---------------------------------------------------------------------------
-// Threads per subdomain of the Rayleigh-Ritz kernel (measured on the 512x512 high-contrast problem:
-// 32 and 256 threads were both slower than 128)
-constexpr int RR_THREADS = 128;
-
 // arithmetic of the Rayleigh-Ritz step: FP64, or double-float when the eigensolve runs in double-float
 template <class T> struct RRType { using type = double; };
 template <> struct RRType<dfloat> { using type = dfloat; };
+
+// Threads per subdomain of the Rayleigh-Ritz kernel: the FP64 updates fill the FP64 pipe with one warp per
+// SM quarter, the double-float ones take two.
+template <class R> struct RRThreads { static constexpr int v = 128; };
+template <> struct RRThreads<dfloat> { static constexpr int v = 256; };
 
 struct RRParams {
   int sb_krylov;   // s*b in Krylov mode
@@ -756,7 +756,7 @@ struct RRParams {
 };
 
 template <class R>
-__global__ void k_rayleigh_ritz(RRParams prm, const int* full, const int* mfull, const int* nf,
+__global__ void __launch_bounds__(RRThreads<R>::v) k_rayleigh_ritz(RRParams prm, const int* full, const int* mfull, const int* nf,
                                 const int* active, const double* H, double* Y, int* ycols, int* zcols,
                                 double* eigout, int* conv, double* worst, int* illcond, int* thick, int* st) {
   extern __shared__ double sm[];
@@ -786,7 +786,7 @@ __global__ void k_rayleigh_ritz(RRParams prm, const int* full, const int* mfull,
   double* wi = wr + m;               // m
   int* perm = reinterpret_cast<int*>(wi + m);  // m
   const double* Hi = H + (int64_t)i * EIG_MAXP * EIG_MAXP;
-  __shared__ int team_red[RR_THREADS / 32];
+  __shared__ int team_red[RRThreads<R>::v / 32];
   const se::Team team{(int)threadIdx.x, (int)blockDim.x, team_red};
   for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
     S[(e / m) * ld + e % m] = (R)Hi[(e / m) * EIG_MAXP + e % m];
@@ -794,8 +794,8 @@ __global__ void k_rayleigh_ritz(RRParams prm, const int* full, const int* mfull,
   }
   __syncthreads();
   // largest |H| entry and finiteness, reduced over the CTA
-  __shared__ double red_norm[RR_THREADS / 32];
-  __shared__ int red_fin[RR_THREADS / 32];
+  __shared__ double red_norm[RRThreads<R>::v / 32];
+  __shared__ int red_fin[RRThreads<R>::v / 32];
   double snorm = 0.0;
   int fin = 1;
   for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
@@ -827,7 +827,7 @@ __global__ void k_rayleigh_ritz(RRParams prm, const int* full, const int* mfull,
     return;
   }
   se::hessenberg(S, ld, Q, ld, m, vtmp, team);
-  __shared__ R snap[14];
+  __shared__ R snap[se::SE_SNAP];
   // the Ritz pairs are wanted to a relative residual of prm.tol: a subdiagonal entry below 1e-3 tol of
   // its diagonal neighbours is already far below what the residual test resolves
   const int rc = se::schur(S, ld, Q, ld, m, snorm, team, snap, 1e-3 * prm.tol);
@@ -881,61 +881,63 @@ __global__ void k_rayleigh_ritz(RRParams prm, const int* full, const int* mfull,
     se::schur_vector(S, ld, m, pidx, wr[pidx], wi[pidx] > 0 ? wi[pidx] : 0.0, xs + j * m, ys + j * m, snorm);
   }
   __syncthreads();
-  // coefficients in the V basis, Q x and Q y: one (row, vector) pair per thread; each row's sum starts
-  // at its own column so that the threads of a warp read different shared-memory banks
-  for (int e = threadIdx.x; e < nsel * m; e += blockDim.x) {
-    const int j = e / m, a = e % m;
+  // one warp per selected vector: its coefficients in the V basis, Q x (and Q y of a pair), one row per
+  // lane, normalised, and the residual ||H_{s,s-1} y_last|| of the pair (zero in the full space)
+  const int lane = threadIdx.x & 31;
+  constexpr int RPL = EIG_MAXP / 32;  // rows per lane
+  for (int j = threadIdx.x >> 5; j < nsel; j += (int)blockDim.x >> 5) {
     const R* x = xs + j * m;
     const R* y = ys + j * m;
-    const R* Qa = Q + a * ld;
-    R qx = 0.0, qy = 0.0;
-    for (int c = 0, cc = a; c < m; ++c, cc = (cc + 1 == m) ? 0 : cc + 1) {
-      mac(qx, Qa[cc], x[cc]);
-      mac(qy, Qa[cc], y[cc]);
+    const int two = sel_two[j], col = sel_col[j], pidx = sel_pos[j];
+    double qx[RPL], qy[RPL], nrm2 = 0.0;
+#pragma unroll
+    for (int u = 0; u < RPL; ++u) {
+      const int a = lane + 32 * u;
+      R sx = 0.0, sy = 0.0;
+      if (a < m) {
+        const R* Qa = Q + a * ld;  // an odd row stride: the lanes read different banks
+#pragma unroll 4
+        for (int c = 0; c < m; ++c) mac(sx, Qa[c], x[c]);
+        if (two == 1)
+#pragma unroll 4
+          for (int c = 0; c < m; ++c) mac(sy, Qa[c], y[c]);
+      }
+      qx[u] = (double)finish(sx);
+      qy[u] = (double)finish(sy);
+      nrm2 += qx[u] * qx[u];
+      if (two == 1) nrm2 += qy[u] * qy[u];
     }
-    Yi[a * EIG_MAXP + sel_col[j]] = (double)finish(qx);
-    if (sel_two[j] == 1) Yi[a * EIG_MAXP + sel_col[j] + 1] = (double)finish(qy);
-  }
-  __syncthreads();
-  if ((int)threadIdx.x < nsel) {
-    const int j = threadIdx.x;
-    const int pidx = sel_pos[j];
-    const int two = sel_two[j];
-    // norms
-    double nx = 0.0, ny = 0.0;
-    for (int a = 0; a < m; ++a) {
-      const double qx = Yi[a * EIG_MAXP + sel_col[j]];
-      nx += qx * qx;
-      if (two == 1) {
-        const double qy = Yi[a * EIG_MAXP + sel_col[j] + 1];
-        ny += qy * qy;
+    for (int o = 16; o > 0; o >>= 1) nrm2 += __shfl_xor_sync(0xffffffffu, nrm2, o);
+    const double inv = 1.0 / sqrt(nrm2);
+#pragma unroll
+    for (int u = 0; u < RPL; ++u) {
+      const int a = lane + 32 * u;
+      if (a < m) {
+        Yi[a * EIG_MAXP + col] = qx[u] * inv;
+        if (two == 1) Yi[a * EIG_MAXP + col + 1] = qy[u] * inv;
       }
     }
-    const double nrm = sqrt(nx + (two ? ny : 0.0));
-    for (int a = 0; a < m; ++a) {
-      Yi[a * EIG_MAXP + sel_col[j]] /= (two == 2 ? sqrt(nx) : nrm);
-      if (two == 1) Yi[a * EIG_MAXP + sel_col[j] + 1] /= nrm;
-    }
-    // residual ||H_{s,s-1} y_last|| (Krylov mode); zero in the full space
+    __syncwarp();
     double res = 0.0;
     if (!full[i]) {
       const int b = prm.b, r0 = prm.sb_krylov, c0 = prm.sb_krylov - b;
-      double rr = 0.0;
-      for (int a = 0; a < b; ++a) {
+      if (lane < b) {  // b <= 32
         double ux = 0.0, uy = 0.0;
+#pragma unroll 8
         for (int c = 0; c < b; ++c) {
-          const double hv = Hi[(r0 + a) * EIG_MAXP + c0 + c];
-          ux += hv * Yi[(c0 + c) * EIG_MAXP + sel_col[j]];
-          if (two == 1) uy += hv * Yi[(c0 + c) * EIG_MAXP + sel_col[j] + 1];
+          const double hv = Hi[(r0 + lane) * EIG_MAXP + c0 + c];
+          ux += hv * Yi[(c0 + c) * EIG_MAXP + col];
+          if (two == 1) uy += hv * Yi[(c0 + c) * EIG_MAXP + col + 1];
         }
-        rr += ux * ux + uy * uy;
+        res = ux * ux + uy * uy;
       }
-      res = sqrt(rr);
+      for (int o = 16; o > 0; o >>= 1) res += __shfl_xor_sync(0xffffffffu, res, o);
+      res = sqrt(res);
     }
-    const double lam = hypot(wr[pidx], wi[pidx]);
-    const bool wanted = sel_col[j] < zc_s;
+    const double lam = mod[pidx];
+    const bool wanted = col < zc_s;
     if (wanted && !(res <= prm.tol * lam)) conv_all = 0;
-    if (wanted) {
+    if (wanted && lane == 0) {
       const double ratio = res / lam;
       // non-negative doubles order like their bit patterns; a NaN or infinite ratio counts as huge
       atomicMax(&worst_bits, (unsigned long long)__double_as_longlong(ratio < 1e300 ? ratio : 1e300));
@@ -1597,7 +1599,7 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
         rr_flops += 25.0 * m * m * m + 2.0 * b * m * m;
       }
       KTime kt(h, KT_EIG_RR, rr_flops);
-      k_rayleigh_ritz<RT><<<N, RR_THREADS, rr_smem, st>>>(prm, d_full, d_mfull, d_nf, G.d_act, H, Y, d_ycols, d_zcols,
+      k_rayleigh_ritz<RT><<<N, RRThreads<RT>::v, rr_smem, st>>>(prm, d_full, d_mfull, d_nf, G.d_act, H, Y, d_ycols, d_zcols,
                                               eigout, d_conv, d_worst, d_illcond, d_thick, h->d_status);
       A2LS_LAUNCH();
     }

@@ -55,12 +55,14 @@ SE_HD inline void se_mac(double& acc, double a, double b) { acc += a * b; }
 SE_HD inline double se_fin(double a) { return a; }
 // 1 / sqrt(a) for a > 0 and 1 / b for b in [1, 2], to rounding accuracy.  On the GPU: the hardware's
 // approximation (about 2^-20) and one third-order step each (with e = 1 - a y^2,
-// 1 / sqrt(a) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2 / 8 + O(e^3)); 1 / b = y / (1 - e) likewise): a
-// chain of four and of three FP64 operations where sqrt and the division are library routines of
-// dozens, on a pipe that issues two lanes a cycle per SM.
+// 1 / sqrt(a) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2 / 8 + O(e^3)); 1 / b = y / (1 - e) likewise).  GB300's
+// FP64 pipe takes about 64 cycles for every warp instruction of an SM quarter, however few lanes are
+// active, so a chain's length in FP64 instructions (comparisons among them) is its time: five and three
+// here, dozens in the library's square root and division.
 SE_HD inline double se_rsqrt(double a) {
 #ifdef __CUDA_ARCH__
-  if (!(a > 1e-280 && a < 1e280)) return 1.0 / sqrt(a);  // outside the approximation's safe range
+  const unsigned ex = (unsigned)__double2hiint(a) >> 20;  // sign and exponent
+  if (ex - 0x60u > 0x740u) return 1.0 / sqrt(a);          // outside the approximation's safe range
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
   const double e = fma(-(a * y), y, 1.0);
@@ -79,19 +81,80 @@ SE_HD inline double se_recip12(double b) {
   return 1.0 / b;
 #endif
 }
+// a positive factor near 1 / a (a > 0) that brings numbers of a's size to about 1
+SE_HD inline double se_scale_to_one(double a) {
+#ifdef __CUDA_ARCH__
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const unsigned ex = (unsigned)__double2hiint(a) >> 20;
+  return ex - 0x10u > 0x7d0u ? 1.0 : y;
+#else
+  return 1.0 / a;
+#endif
+}
+// The largest of some magnitudes as a power of two, and its inverse, where the arithmetic's exponent range
+// is short of squares (one in FP64).
+SE_HD inline double se_pow2(double) { return 1.0; }
+SE_HD inline double se_pow2_inv(double p) { return p; }
+SE_HD inline double se_warp_maxabs(double) { return 1.0; }
+SE_HD inline bool se_range_limited(double) { return false; }
+SE_HD inline bool se_is_zero(double a) {
+#ifdef __CUDA_ARCH__
+  return (__double_as_longlong(a) << 1) == 0;
+#else
+  return a == 0.0;
+#endif
+}
+// the sum of v over a warp (every lane receives it); a one-thread team has v itself
+SE_HD inline double se_warp_sum(double v) {
+#ifdef __CUDA_ARCH__
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+#endif
+  return v;
+}
+SE_HD inline double se_warp_get(double v, int lane) {
+#ifdef __CUDA_ARCH__
+  return __shfl_sync(0xffffffffu, v, lane);
+#else
+  (void)lane;
+  return v;
+#endif
+}
 template <class R> struct SeEps {
   static constexpr double v = 2.220446049250313e-16;  // machine epsilon of R
   static constexpr double big = 1e100;                // rescaling threshold of the back substitution
 };
 
-// Whether the Francis iteration forms the next bulge reflector during the right update (one thread,
-// from a snapshot) rather than with every thread after it.  Measured on GB300: faster in FP64
-// (Rayleigh-Ritz 178 -> 147 ms per 512x512 setup), slower in double-float (28.7 -> 30.3 ms), whose
-// longer reflector arithmetic on one thread outlasts the right update.
-template <class R> struct SeEarlyReflector { static constexpr bool value = true; };
-
 template <class R>
 SE_HD inline R sgn(R a, R b) { return b >= R(0.0) ? se_abs(a) : -se_abs(a); }
+SE_HD inline double sgn(double a, double b) { return copysign(a, b); }
+
+// x_r -= d v_r for r = 0 .. n-1 (x with stride st), four elements loaded ahead of their stores: x and v may
+// be the same kind of memory, so the compiler may not move a load over a store by itself
+template <class R>
+SE_HD inline void subtract_multiple(R* x, int st, const R* v, int n, R d) {
+  int r = 0;
+  for (; r + 4 <= n; r += 4) {
+    R a[4], b[4];
+    for (int u = 0; u < 4; ++u) {
+      a[u] = x[(r + u) * st];
+      b[u] = v[r + u];
+    }
+    for (int u = 0; u < 4; ++u) x[(r + u) * st] = a[u] - d * b[u];
+  }
+  for (; r < n; ++r) x[r * st] -= d * v[r];
+}
+
+// sum of x_r v_r for r = 0 .. n-1
+template <class R>
+SE_HD inline R strided_dot(const R* x, int st, const R* v, int n) {
+  R d = 0.0;
+#ifdef __CUDACC__
+#pragma unroll 4
+#endif
+  for (int r = 0; r < n; ++r) se_mac(d, v[r], x[r * st]);
+  return se_fin(d);
+}
 
 // Reduce H (m x m) to upper Hessenberg form, accumulating the orthogonal factor in Q (Q <- Q P).
 // v: scratch of m values.  Each reflector takes two phases of the team: the left update (one column
@@ -101,112 +164,89 @@ SE_HD inline R sgn(R a, R b) { return b >= R(0.0) ? se_abs(a) : -se_abs(a); }
 template <class R>
 SE_HD inline void hessenberg(R* H, int ld, R* Q, int ldq, int m, R* v, const Team& t) {
   for (int k = 0; k + 2 < m; ++k) {
-    // Householder vector for x = H[k+1.., k]
+    // Householder vector for x = H[k+1.., k]; every warp sums |x|^2 for itself, in the same order (x scaled)
+#ifdef __CUDA_ARCH__
+    const int l0 = t.lane & 31, ls = 32;
+#else
+    const int l0 = 0, ls = 1;
+#endif
+    R xm = 0.0;
+    for (int r = k + 1 + l0; r < m; r += ls) {
+      const R a = se_abs(H[r * ld + k]);
+      if (se_range_limited(a) && a > xm) xm = a;
+    }
+    const R up = se_pow2(se_warp_maxabs(xm)), dn = se_pow2_inv(up);
     R nrm2 = 0.0;
-    for (int r = k + 1; r < m; ++r) se_mac(nrm2, H[r * ld + k], H[r * ld + k]);
-    nrm2 = se_fin(nrm2);
-    R nrm = se_sqrt(nrm2);
-    if (nrm == 0.0) continue;
-    R x0 = H[(k + 1) * ld + k];
-    R alpha = -sgn(nrm, x0);
-    // v = x - alpha e1, scaled so that P = I - 2 v v^T / (v^T v); v^T v = 2 nrm |x0 - alpha|
-    R vtv = nrm2 - x0 * x0 + (x0 - alpha) * (x0 - alpha);
-    if (vtv == 0.0) continue;
+    for (int r = k + 1 + l0; r < m; r += ls) {
+      const R a = H[r * ld + k] * dn;
+      se_mac(nrm2, a, a);
+    }
+    nrm2 = se_warp_sum(se_fin(nrm2));
+    if (se_is_zero(nrm2)) continue;
+    const R rn = se_rsqrt(nrm2);
+    const R x0 = H[(k + 1) * ld + k] * dn;
+    const R alpha = -sgn(nrm2 * rn, x0);
+    // v = x - alpha e1; P = I - beta v v^T with beta = 2 / v^T v, v^T v = 2 |x| (|x| + |x0|)
+    const R beta = rn * rn * se_recip12(R(1.0) + se_abs(x0) * rn);
     t.sync();
-    for (int r = k + 1 + t.lane; r < m; r += t.size) v[r] = (r == k + 1) ? (x0 - alpha) : H[r * ld + k];
+    for (int r = k + 1 + t.lane; r < m; r += t.size) v[r] = (r == k + 1) ? (x0 - alpha) : H[r * ld + k] * dn;
     t.sync();
-    const R beta = 2.0 / vtv;
+    const int len = m - k - 1;
     const int ncol = m - k;                                  // left update: columns k..m-1
     const int qa = (t.size > ncol) ? ((t.size - ncol < m) ? t.size - ncol : m) : 0;  // Q rows in phase 1
     for (int idx = t.lane; idx < ncol + qa; idx += t.size) {
-      if (idx < ncol) {
-        const int c = k + idx;
-        R d = 0.0;
-        for (int r = k + 1; r < m; ++r) se_mac(d, v[r], H[r * ld + c]);
-        d = se_fin(d) * beta;
-        for (int r = k + 1; r < m; ++r) H[r * ld + c] -= d * v[r];
-      } else {
-        const int r = idx - ncol;
-        R e = 0.0;
-        for (int c = k + 1; c < m; ++c) se_mac(e, Q[r * ldq + c], v[c]);
-        e = se_fin(e) * beta;
-        for (int c = k + 1; c < m; ++c) Q[r * ldq + c] -= e * v[c];
-      }
+      R* x = idx < ncol ? H + (k + 1) * ld + k + idx : Q + (idx - ncol) * ldq + k + 1;
+      const int st = idx < ncol ? ld : 1;
+      const R d = strided_dot(x, st, v + k + 1, len) * beta;
+      subtract_multiple(x, st, v + k + 1, len, d);
     }
     t.sync();
     // right: all rows of H, columns k+1..; the remaining rows of Q
     for (int idx = t.lane; idx < m + (m - qa); idx += t.size) {
-      if (idx < m) {
-        const int r = idx;
-        R d = 0.0;
-        for (int c = k + 1; c < m; ++c) se_mac(d, H[r * ld + c], v[c]);
-        d = se_fin(d) * beta;
-        for (int c = k + 1; c < m; ++c) H[r * ld + c] -= d * v[c];
-      } else {
-        const int r = qa + idx - m;
-        R e = 0.0;
-        for (int c = k + 1; c < m; ++c) se_mac(e, Q[r * ldq + c], v[c]);
-        e = se_fin(e) * beta;
-        for (int c = k + 1; c < m; ++c) Q[r * ldq + c] -= e * v[c];
-      }
+      R* x = idx < m ? H + idx * ld + k + 1 : Q + (qa + idx - m) * ldq + k + 1;
+      const R d = strided_dot(x, 1, v + k + 1, len) * beta;
+      subtract_multiple(x, 1, v + k + 1, len, d);
     }
     t.sync();
-    if (t.lane == 0) {
-      H[(k + 1) * ld + k] = alpha;
-      for (int r = k + 2; r < m; ++r) H[r * ld + k] = 0.0;
-    }
+    for (int r = k + 1 + t.lane; r < m; r += t.size) H[r * ld + k] = r == k + 1 ? alpha * up : R(0.0);
     t.sync();
   }
-}
-
-// Apply a 3-element (or 2-element when nv == 2) reflector I - beta u u^T with u = (1, u1, u2)
-// to rows k..k+nv-1 of H from the left (columns c0..m-1) and to columns k..k+nv-1 from the
-// right (rows 0..r1) and to Q's columns.
-template <class R>
-SE_HD inline void apply_reflector(R* H, int ld, R* Q, int ldq, int m, int k, int nv, R u1, R u2, R beta,
-                                  int c0, int r1, const Team& t) {
-  for (int c = c0 + t.lane; c < m; c += t.size) {
-    R d = H[k * ld + c] + u1 * H[(k + 1) * ld + c] + (nv == 3 ? u2 * H[(k + 2) * ld + c] : 0.0);
-    d *= beta;
-    H[k * ld + c] -= d;
-    H[(k + 1) * ld + c] -= d * u1;
-    if (nv == 3) H[(k + 2) * ld + c] -= d * u2;
-  }
-  t.sync();
-  for (int r = t.lane; r <= r1; r += t.size) {
-    R d = H[r * ld + k] + u1 * H[r * ld + k + 1] + (nv == 3 ? u2 * H[r * ld + k + 2] : 0.0);
-    d *= beta;
-    H[r * ld + k] -= d;
-    H[r * ld + k + 1] -= d * u1;
-    if (nv == 3) H[r * ld + k + 2] -= d * u2;
-  }
-  for (int r = t.lane; r < m; r += t.size) {
-    R d = Q[r * ldq + k] + u1 * Q[r * ldq + k + 1] + (nv == 3 ? u2 * Q[r * ldq + k + 2] : 0.0);
-    d *= beta;
-    Q[r * ldq + k] -= d;
-    Q[r * ldq + k + 1] -= d * u1;
-    if (nv == 3) Q[r * ldq + k + 2] -= d * u2;
-  }
-  t.sync();
 }
 
 // Householder reflector mapping (x, y, z) to (alpha, 0, 0): returns alpha, beta and u = (1, u1, u2).
 // With v = (v0, y, z), v0 = x - alpha, v^T v = 2 |alpha| |v0|, so beta = 2 v0^2 / v^T v = v0 / (-alpha).
 // With r = 1 / |(x, y, z)|: beta = 1 + |x| r (between 1 and 2) and 1 / v0 = sign(x) r / beta.  The chain of
 // a sweep's reflectors is what bounds the Schur iteration, so they are formed without a square root or a
-// division: with the deflation scan and the ordering of the eigenvalues spread over the team, an FP64 setup
-// and solve of 16 subdomains (order 48) 84.0 -> 72.7 ms, a double-float one of 256 (order 72) 120.5 -> 116.2.
+// division (an FP64 setup and solve of 16 subdomains, order 48: 84.0 -> 72.7 ms).
+// (0, 0, 0) gives beta = 0 and alpha = x: no reflection.  An arithmetic of short exponent range scales the
+// three first: entries of 1e-16 and less, as a converging block has them, would lose the low parts of
+// their squares, and the reflector its orthogonality.
 template <class R>
-SE_HD inline bool make_reflector(R x, R y, R z, R& u1, R& u2, R& beta, R& alpha) {
+SE_HD inline void make_reflector(R x, R y, R z, R& u1, R& u2, R& beta, R& alpha) {
+  R up = R(1.0);
+  if (se_range_limited(x)) {
+    R xm = se_abs(x);
+    if (se_abs(y) > xm) xm = se_abs(y);
+    if (se_abs(z) > xm) xm = se_abs(z);
+    up = se_pow2(xm);
+    const R dn = se_pow2_inv(up);
+    x *= dn;
+    y *= dn;
+    z *= dn;
+  }
   const R s = x * x + y * y + z * z;
-  if (s == R(0.0)) return false;
+  if (se_is_zero(s)) {
+    u1 = u2 = beta = R(0.0);
+    alpha = x;
+    return;
+  }
   const R r = se_rsqrt(s);
   beta = R(1.0) + se_abs(x) * r;
   alpha = -sgn(s * r, x);
+  if (se_range_limited(x)) alpha *= up;
   const R iv = sgn(r * se_recip12(beta), x);
   u1 = y * iv;
   u2 = z * iv;
-  return true;
 }
 
 // Make a 2x2 diagonal block with real eigenvalues upper triangular by a rotation (rows/cols p, p+1).
@@ -217,14 +257,20 @@ SE_HD inline void split_2x2(R* H, int ld, R* Q, int ldq, int m, int p, const Tea
   R hm = 0.5 * (a - d);
   R disc = hm * hm + b * c;
   if (disc < 0.0 || c == 0.0) return;
-  // eigenvalue closest to d: lambda = d + (hm +- se_sqrt(disc)) ... pick the one of larger magnitude shift
-  R sq = se_sqrt(disc);
+  // eigenvalue closest to d: lambda = d + (hm +- sqrt(disc)) ... pick the one of larger magnitude shift
+  R sq = se_is_zero(disc) ? R(0.0) : disc * se_rsqrt(disc);
   R lam = 0.5 * (a + d) + (hm >= 0 ? sq : -sq);
   // eigenvector (lam - d, c) of the block; rotation taking it to e1
   R x = lam - d, y = c;
-  R r = se_sqrt(x * x + y * y);
-  if (r == 0.0) return;
-  R cs = x / r, sn = y / r;
+  if (se_range_limited(x)) {
+    const R dn = se_pow2_inv(se_pow2(se_abs(x) > se_abs(y) ? se_abs(x) : se_abs(y)));
+    x *= dn;
+    y *= dn;
+  }
+  const R r2 = x * x + y * y;
+  if (se_is_zero(r2)) return;
+  const R ri = se_rsqrt(r2);
+  R cs = x * ri, sn = y * ri;
   // rows p, p+1: G^T H
   for (int col = p + t.lane; col < m; col += t.size) {
     R h1 = H[p * ld + col], h2 = H[(p + 1) * ld + col];
@@ -247,19 +293,56 @@ SE_HD inline void split_2x2(R* H, int ld, R* Q, int ldq, int m, int p, const Tea
   t.sync();
 }
 
-// Francis R-shift QR on an upper Hessenberg H, full Schur form, Q accumulated.
+// Most bulges chased together, their distance in rows, and the scratch schur() wants: per bulge the nine
+// entries of the next reflector's snapshot, the four shift values and two sets of u1, u2, beta, alpha.
+constexpr int SE_BULGES = 3;
+constexpr int SE_BULGE_GAP = 4;
+constexpr int SE_SLOT = 21;
+constexpr int SE_W2 = 10, SE_W3 = 24;  // active block sizes from which a second and a third bulge are chased
+constexpr int SE_SNAP = SE_BULGES * SE_SLOT;
+enum { SE_SHIFTS = 9, SE_REFL = 13 };
+
+// The shift pair (s1r, s2r, s1i, s2i) of the 2 x 2 block a, b; c, d: a real pair is replaced by its member
+// closer to d, used twice.
+template <class R>
+SE_HD inline void shift_pair(R a, R b, R c, R d, R* s) {
+  const R hm = 0.5 * (a - d);
+  const R disc = hm * hm + b * c;
+  const R mean = 0.5 * (a + d);
+  if (disc >= 0.0) {
+    const R sq = se_is_zero(disc) ? R(0.0) : disc * se_rsqrt(disc);
+    const R r1 = mean + sq, r2 = mean - sq;
+    s[0] = s[1] = (se_abs(r1 - d) <= se_abs(r2 - d)) ? r1 : r2;
+    s[2] = s[3] = 0.0;
+  } else {
+    s[0] = s[1] = mean;
+    s[2] = -disc * se_rsqrt(-disc);
+    s[3] = -s[2];
+  }
+}
+
+// Francis implicit double-shift QR on an upper Hessenberg H, full Schur form, Q accumulated.
 // A subdiagonal entry is neglected when it is below eps times its two diagonal
 // neighbours or below eps times hnorm (the largest entry of the input), which keeps
 // clusters of eigenvalues near zero from stalling the iteration; the result is
 // backward stable relative to hnorm.  Returns 0 on success, -1 on no convergence.
-// snap: 14 values of scratch shared by the team (may be null for a one-thread team).
+// snap: SE_SNAP values of scratch shared by the team (may be null for a one-thread team).
 // local_tol (>= the machine epsilon of R; 0 selects it): the neighbour-relative test may use a looser
 // threshold when the caller needs the Schur form only to that relative accuracy; the test against
 // hnorm always uses the machine epsilon.
+//
+// A sweep's time is the chain of its reflectors, each formed from what the one before it leaves, and not
+// the updates.  A sweep therefore chases up to SE_BULGES bulges, each with the shifts of its own 2 x 2
+// block (the trailing one, the one before it, ...), SE_BULGE_GAP rows apart and in step with one another
+// (the small-bulge multishift iteration of Braman, Byers and Mathias, SIAM J. Matrix Anal. Appl. 23,
+// 2002, with the neighbouring diagonal blocks' shifts): the bulges' rows and columns are disjoint, so that
+// one step updates for all of them and one warp forms their next reflectors side by side, in its lanes.
+// Against one bulge a sweep (order 48 FP64, 72 double-float, random spectra of six decades): FP64 4.76 ->
+// 2.30 million cycles, double-float 8.19 -> 3.34 million; the same FP64 setup and solve 72.7 -> 56.5 ms.
 template <class R>
 SE_HD inline int schur(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const Team& t, R* snap = nullptr,
                        double local_tol = 0.0) {
-  R snap_local[14];
+  R snap_local[SE_SNAP];
   if (!snap) snap = snap_local;
   const R eps = R(SeEps<R>::v), hnorm = R(hnorm_);
   const R leps = R(local_tol > SeEps<R>::v ? local_tol : SeEps<R>::v);
@@ -294,161 +377,171 @@ SE_HD inline int schur(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const 
     }
     ++iter;
     if (++total > 60 * m) return -1;
-    // Shifts: the eigenvalues of the trailing 2x2 block (a real pair is replaced by its member
-    // closer to the last diagonal entry, used twice), or an exceptional pair every 11th step.
-    R s1r, s1i, s2r, s2i;
-    {
-      R a, b, c, d;
-      if (iter % 11 == 10) {
-        const R w = se_abs(H[hi * ld + hi - 1]) + se_abs(H[(hi - 1) * ld + hi - 2]);
-        a = 0.75 * w + H[hi * ld + hi];
-        b = -0.4375 * w;
-        c = w;
-        d = a;
-      } else {
-        a = H[(hi - 1) * ld + hi - 1];
-        b = H[(hi - 1) * ld + hi];
-        c = H[hi * ld + hi - 1];
-        d = H[hi * ld + hi];
-      }
-      const R hm = 0.5 * (a - d);
-      const R disc = hm * hm + b * c;
-      const R mean = 0.5 * (a + d);
-      if (disc >= 0.0) {
-        const R sq = se_sqrt(disc);
-        const R r1 = mean + sq, r2 = mean - sq;
-        const R sh = (se_abs(r1 - d) <= se_abs(r2 - d)) ? r1 : r2;
-        s1r = s2r = sh;
-        s1i = s2i = 0.0;
-      } else {
-        s1r = s2r = mean;
-        s1i = se_sqrt(-disc);
-        s2i = -s1i;
-      }
-    }
-    // first column of (H - s1)(H - s2), formed from differences to avoid cancellation
-    R x, y, z;
-    {
+    const int w = hi - lo + 1;
+    const int nb = w >= SE_W3 ? 3 : (w >= SE_W2 ? 2 : 1);
+    // On the GPU the last warp forms the reflectors, lanes 3 q .. 3 q + 2 for bulge q (lane 3 q keeps it); the
+    // right updates and Q are left to the other warps.
+#ifdef __CUDA_ARCH__
+    const int nwork = t.size - 32, rl = t.lane - nwork;
+    const int mq0 = rl >= 0 ? (rl < 3 * nb ? rl / 3 : nb - 1) : nb, mq1 = mq0 < nb ? mq0 + 1 : nb;
+    const bool keeps = rl == 3 * mq0;
+#else
+    const int nwork = t.size, mq0 = 0, mq1 = nb;
+    const bool keeps = true;
+#endif
+    // the reflector that starts bulge q: the first column of (H - s1)(H - s2), formed from differences to
+    // avoid cancellation, times a factor that keeps it in range (only its direction matters)
+    auto start = [&](int q) {
+      const R* s = snap + q * SE_SLOT + SE_SHIFTS;
+      const R s1r = s[0], s2r = s[1], s1i = s[2], s2i = s[3];
       const R h00 = H[lo * ld + lo], h01 = H[lo * ld + lo + 1], h10 = H[(lo + 1) * ld + lo];
       const R h11 = H[(lo + 1) * ld + lo + 1], h21 = H[(lo + 2) * ld + lo + 1];
       const R sc = se_abs(h00 - s2r) + se_abs(s2i) + se_abs(h10);
-      const R g = (sc > 0.0) ? h10 / sc : 0.0;
-      x = g * h01 + (h00 - s1r) * ((h00 - s2r) / (sc > 0.0 ? sc : 1.0)) - s1i * (s2i / (sc > 0.0 ? sc : 1.0));
-      y = g * (h00 + h11 - s1r - s2r);
-      z = g * h21;
+      const R f = se_is_zero(sc) ? R(1.0) : se_scale_to_one(sc);
+      const R g = h10 * f;
+      R r[4];
+      make_reflector<R>(g * h01 + (h00 - s1r) * ((h00 - s2r) * f) - s1i * (s2i * f), g * (h00 + h11 - s1r - s2r),
+                        g * h21, r[0], r[1], r[2], r[3]);
+      R* o = snap + q * SE_SLOT + SE_REFL + 4 * ((SE_BULGE_GAP * q) & 1);
+      if (keeps)
+        for (int u = 0; u < 4; ++u) o[u] = r[u];
+    };
+    for (int q = mq0; q < mq1; ++q) {
+      const int p = hi - 1 - 2 * q;
+      R a, b, c, d;
+      if (iter % 11 == 10) {  // an exceptional pair every 11th sweep
+        const R e = se_abs(H[(p + 1) * ld + p]) + se_abs(H[p * ld + p - 1]);
+        a = 0.75 * e + H[(p + 1) * ld + p + 1];
+        b = -0.4375 * e;
+        c = e;
+        d = a;
+      } else {
+        a = H[p * ld + p];
+        b = H[p * ld + p + 1];
+        c = H[(p + 1) * ld + p];
+        d = H[(p + 1) * ld + p + 1];
+      }
+      R s[4];
+      shift_pair(a, b, c, d, s);
+      if (keeps)
+        for (int u = 0; u < 4; ++u) snap[q * SE_SLOT + SE_SHIFTS + u] = s[u];
     }
-    // Bulge chase.  For k > lo the reflector is built from column k-1 (rows k..k+2), which it maps to
-    // (alpha, 0, 0) exactly; that column is therefore not part of the left update but written
-    // directly, after the barrier that separates every thread's read of (x, y, z) from the writes,
-    // which keeps each step at two barriers.  The next step's reflector comes from column k after
-    // this step's right update; one thread recomputes its three entries from a snapshot of rows
-    // k+1..k+3 (columns k..k+2) taken in the left phase and forms the reflector while the others run
-    // the right update, instead of every thread forming it after that update (the entries are the
-    // values the right update writes).
-    t.sync();  // the shift and deflation reads above precede the first update
-    const bool early = SeEarlyReflector<R>::value;
-    R u1, u2, beta, alpha;
-    bool have = make_reflector(x, y, z, u1, u2, beta, alpha);
-    for (int k = lo; k <= hi - 2; ++k) {
-      const bool more = k + 1 <= hi - 2;  // a next step exists (then k + 3 <= hi)
-      R nu1 = R(0.0), nu2 = R(0.0), nbeta = R(0.0), nalpha = R(0.0);
-      bool nhave = false;
-      if (have) {
-        const int c0 = k > lo ? k : lo;
-        const int r1 = (k + 3 <= hi) ? k + 3 : hi;
-        // phase 1: rows k..k+2 from the left (columns c0..m-1) and the first qa rows of Q; phase 2:
-        // columns k..k+2 from the right (rows 0..r1) and the remaining rows of Q (Q's update depends
-        // on the reflector only, so it fills the threads that the H updates leave idle)
-        const int ncol = m - c0;
-        const int qa = (t.size > ncol) ? ((t.size - ncol < m) ? t.size - ncol : m) : 0;
-        for (int idx = t.lane; idx < ncol + qa; idx += t.size) {
-          R* a;
-          int st;
-          if (idx < ncol) {
-            a = H + k * ld + c0 + idx;
-            st = ld;
-          } else {
-            a = Q + (idx - ncol) * ldq + k;
-            st = 1;
+#ifdef __CUDA_ARCH__
+    __syncwarp();
+#endif
+    if (mq0 == 0) start(0);
+    t.sync();  // the reads of H above precede the first update
+    // Bulge q is at row k = lo + step - SE_BULGE_GAP q.  For k > lo its reflector was built from column
+    // k - 1 (rows k .. k + 2), which it maps to (alpha, 0, 0) exactly; that column is therefore not part of
+    // the left update but written directly, after the barrier that separates the reads of it from the
+    // writes.  At k = hi - 1 the reflector has two rows.  The next reflector comes from column k after this
+    // step's right update; its three entries are recomputed from a snapshot of rows k + 1 .. k + 3
+    // (columns k .. k + 2) taken in the left phase, and the reflector is formed while the others run the
+    // right update (the entries are the values the right update writes).
+    const int steps = hi - lo + SE_BULGE_GAP * (nb - 1);
+    for (int step = 0; step < steps; ++step) {
+      // the active bulges q0 <= q < q1 (those between the start and the end of the block)
+      const int q0 = step - (hi - 1 - lo) > 0 ? (step - (hi - 1 - lo) + SE_BULGE_GAP - 1) / SE_BULGE_GAP : 0;
+      const int q1 = step / SE_BULGE_GAP + 1 < nb ? step / SE_BULGE_GAP + 1 : nb;
+      const R* refl = snap + SE_REFL + 4 * (step & 1);
+      auto reflect = [&](R* a, int st, const R* r, bool three) {
+        const R u1 = r[0], u2 = r[1], beta = r[2];
+        const R a0 = a[0], a1 = a[st], a2 = three ? a[2 * st] : R(0.0);
+        R d = a0;
+        se_mac(d, u1, a1);
+        if (three) se_mac(d, u2, a2);
+        d = se_fin(d) * beta;
+        a[0] = a0 - d;
+        a[st] = a1 - d * u1;
+        if (three) a[2 * st] = a2 - d * u2;
+      };
+      // phase 1: rows k .. k + 2 from the left (columns k .. m - 1), one column per item, the active bulges'
+      // items one after another
+      const int k1 = lo + step;  // bulge 0's row
+      // (the item's bulge is found with selections and the update done once: a branch per bulge would issue
+      // the update once for every bulge that meets in a warp)
+      {
+        int total = 0;
+        for (int q = q0; q < q1; ++q) total += m - (k1 - SE_BULGE_GAP * q);
+        for (int at = t.lane; at < total; at += t.size) {
+          int idx = at, q = q0, k = k1 - SE_BULGE_GAP * q0;
+          for (int u = 1; u < SE_BULGES; ++u) {
+            const bool next = idx >= m - k;
+            idx -= next ? m - k : 0;
+            q += next ? 1 : 0;
+            k -= next ? SE_BULGE_GAP : 0;
           }
-          R d = a[0];
-          se_mac(d, u1, a[st]);
-          se_mac(d, u2, a[2 * st]);
-          d = se_fin(d) * beta;
-          a[0] -= d;
-          a[st] -= d * u1;
-          a[2 * st] -= d * u2;
-          if (early && more && idx < 3) {  // column c0 + idx = k + idx
-            snap[idx] = a[st];
-            snap[3 + idx] = a[2 * st];
-            snap[6 + idx] = H[(k + 3) * ld + k + idx];
+          const bool three = k <= hi - 2;
+          R* a = H + k * ld + k + idx;
+          reflect(a, ld, refl + q * SE_SLOT, three);
+          if (idx < 3 && three) {  // column k + idx
+            R* v = snap + q * SE_SLOT + idx;
+            v[0] = a[ld];
+            v[3] = a[2 * ld];
+            v[6] = k + 3 <= hi ? a[3 * ld] : R(0.0);
           }
         }
-        t.sync();
-        if (k > lo && t.lane == 0) {
-          H[k * ld + k - 1] = alpha;
+      }
+      t.sync();
+      // phase 2: columns k .. k + 2 from the right (rows 0 .. k + 3) and Q, one row per item; the next
+      // reflectors
+      for (int q = mq0; q < mq1; ++q) {
+        const int k = k1 - SE_BULGE_GAP * q;
+        R* slot = snap + q * SE_SLOT;
+        const R* r = refl + q * SE_SLOT;
+        R v[3] = {R(0.0), R(0.0), R(0.0)};
+        const R u1 = r[0], u2 = r[1], beta = r[2];
+        auto entry = [&](int rr) {
+          const R a0 = slot[3 * rr], a1 = slot[3 * rr + 1], a2 = slot[3 * rr + 2];
+          R d = a0;
+          se_mac(d, u1, a1);
+          se_mac(d, u2, a2);
+          d = se_fin(d) * beta;
+          return a0 - d;
+        };
+#ifdef __CUDA_ARCH__
+        // one lane per entry (a bulge outside the block computes on what its slot happens to hold, and the
+        // result is not used)
+        const R e = entry(rl < 3 * nb ? rl - 3 * mq0 : 2);
+        v[0] = se_warp_get(e, 3 * mq0);
+        v[1] = se_warp_get(e, 3 * mq0 + 1);
+        v[2] = se_warp_get(e, 3 * mq0 + 2);
+#else
+        for (int rr = 0; rr < 3; ++rr) v[rr] = entry(rr);
+#endif
+        if (k == lo - 1) {
+          start(q);
+        } else if (k >= lo && k <= hi - 2) {
+          R n[4];
+          make_reflector<R>(v[0], v[1], v[2], n[0], n[1], n[2], n[3]);
+          R* o = slot + SE_REFL + 4 * ((step + 1) & 1);
+          if (keeps)
+            for (int u = 0; u < 4; ++u) o[u] = n[u];
+        }
+        if (keeps && k > lo && k <= hi - 1) {
+          H[k * ld + k - 1] = r[3];
           H[(k + 1) * ld + k - 1] = 0.0;
-          H[(k + 2) * ld + k - 1] = 0.0;
+          if (k <= hi - 2) H[(k + 2) * ld + k - 1] = 0.0;
         }
-        if (early && more && t.lane == t.size - 1) {  // the last thread, usually idle in the right update
-          R v[3];
-          for (int rr = 0; rr < 3; ++rr) {
-            const R a0 = snap[3 * rr], a1 = snap[3 * rr + 1], a2 = snap[3 * rr + 2];
-            R d = a0;
-            se_mac(d, u1, a1);
-            se_mac(d, u2, a2);
-            d = se_fin(d) * beta;
-            v[rr] = a0 - d;
+      }
+      if (t.lane < nwork) {
+        auto rows_of = [&](int k) { return (k + 3 <= hi ? k + 3 : hi) + 1; };
+        int total = 0;
+        for (int q = q0; q < q1; ++q) total += rows_of(k1 - SE_BULGE_GAP * q) + m;
+        for (int at = t.lane; at < total; at += nwork) {
+          int idx = at, q = q0, k = k1 - SE_BULGE_GAP * q0;
+          for (int u = 1; u < SE_BULGES; ++u) {
+            const int cnt = rows_of(k) + m;
+            const bool next = idx >= cnt;
+            idx -= next ? cnt : 0;
+            q += next ? 1 : 0;
+            k -= next ? SE_BULGE_GAP : 0;
           }
-          const bool ok = make_reflector(v[0], v[1], v[2], nu1, nu2, nbeta, nalpha);
-          snap[9] = nu1;
-          snap[10] = nu2;
-          snap[11] = nbeta;
-          snap[12] = nalpha;
-          snap[13] = ok ? R(1.0) : R(0.0);
+          const int rows = rows_of(k);
+          reflect(idx < rows ? H + idx * ld + k : Q + (idx - rows) * ldq + k, 1, refl + q * SE_SLOT, k <= hi - 2);
         }
-        for (int idx = t.lane; idx < (r1 + 1) + (m - qa); idx += t.size) {
-          R* a = (idx <= r1) ? H + idx * ld + k : Q + (qa + idx - (r1 + 1)) * ldq + k;
-          R d = a[0];
-          se_mac(d, u1, a[1]);
-          se_mac(d, u2, a[2]);
-          d = se_fin(d) * beta;
-          a[0] -= d;
-          a[1] -= d * u1;
-          a[2] -= d * u2;
-        }
-        t.sync();
-        if (more && early) {
-          nu1 = snap[9];
-          nu2 = snap[10];
-          nbeta = snap[11];
-          nalpha = snap[12];
-          nhave = snap[13] != R(0.0);
-        } else if (more) {
-          nhave = make_reflector(H[(k + 1) * ld + k], H[(k + 2) * ld + k], H[(k + 3) * ld + k], nu1, nu2, nbeta,
-                                 nalpha);
-        }
-      } else if (more) {
-        nhave = make_reflector(H[(k + 1) * ld + k], H[(k + 2) * ld + k], H[(k + 3) * ld + k], nu1, nu2, nbeta,
-                               nalpha);
       }
-      u1 = nu1;
-      u2 = nu2;
-      beta = nbeta;
-      alpha = nalpha;
-      have = nhave;
-    }
-    x = H[(hi - 1) * ld + hi - 2];
-    y = H[hi * ld + hi - 2];
-    // final 2-element reflector on rows hi-1, hi
-    {
-      R u1, u2, beta, alpha;
-      if (make_reflector<R>(x, y, R(0.0), u1, u2, beta, alpha)) {
-        t.sync();
-        apply_reflector<R>(H, ld, Q, ldq, m, hi - 1, 2, u1, R(0.0), beta, hi - 2, hi, t);
-        if (t.lane == 0) H[hi * ld + hi - 2] = 0.0;
-        t.sync();
-      }
+      t.sync();
     }
   }
   return 0;
