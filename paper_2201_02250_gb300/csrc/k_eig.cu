@@ -562,11 +562,61 @@ __device__ int warp_cholesky_inverse(double* G, int p, double* Ri, double* dsc, 
   return ok;
 }
 
-// Orthogonalisation: block CGS2 of W against V[:, 0:jb], then Cholesky QR three times (the first
-// shifted).  Writes the Gram coefficients into H[0:jb, hc:hc+p] and R into H[hr:hr+p, hc:hc+p] and
+// Thread-block clusters: the CTA's rank and count, the barrier over all threads of the cluster, and a
+// double of another CTA's shared memory.
+__device__ __forceinline__ int cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ int cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ double cluster_ld(const double* p, int rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
+  return v;
+}
+
+// G <- the sum of the cluster's G (count doubles of shared memory at the same place in every CTA), added in
+// the order of the ranks, so that every CTA holds the same values.  tmp: count doubles of scratch in shared
+// memory that no other CTA reads.  All threads of the cluster; G complete in every CTA (the barrier orders
+// it), ends with a CTA barrier.
+__device__ __forceinline__ void cluster_sum(double* G, int count, double* tmp) {
+  const int C = cluster_size();
+  if (C == 1) return;
+  cluster_sync();
+  for (int e = threadIdx.x; e < count; e += ORTH_THREADS) {
+    double s = cluster_ld(G + e, 0);
+    for (int r = 1; r < C; ++r) s += cluster_ld(G + e, r);
+    tmp[e] = s;
+  }
+  cluster_sync();  // every CTA has read this one's G
+  for (int e = threadIdx.x; e < count; e += ORTH_THREADS) G[e] = tmp[e];
+  __syncthreads();
+}
+
+// Orthogonalisation: block CGS2 of W against V[:, 0:jb], then Cholesky QR twice or three times (see
+// below).  Writes the Gram coefficients into H[0:jb, hc:hc+p] and R into H[hr:hr+p, hc:hc+p] and
 // the orthonormal block into V[:, vout:vout+p].  full != 0: only H[0:jb, hc:hc+p].  illcond (if given):
 // set to 1 for a subdomain whose block needed the shifted factorisation (an ill-conditioned block).
 // Shared memory: G and Ri (gcap doubles each), trow, two staging chunks of orc x EIG_MAXP.
+//
+// The work of a subdomain is bound by the arithmetic of the SM that does it, so with fewer subdomains than
+// SMs a cluster of CTAs takes each: a CTA holds a slice of the rows, forms its part of every Gram product
+// and applies the updates to its rows; the parts are summed through distributed shared memory and every CTA
+// factors the same small Gram matrix.  The launch picks the largest cluster (at most 8) with which the
+// active subdomains still fit the SMs; clusters only where the Gram matrices of full-space subdomains are
+// not in play (their shared memory leaves no room, and they have at most 96 rows).  Setup and solve, one
+// CTA each against clusters (and k_vy's chunks spread likewise): 16 subdomains in FP64 56.5 -> 47.0 ms, 64 in
+// double-float 48.2 -> 43.1 ms, 64 in FP64 (about 1950 rows each) 1311 -> 1195 ms; 256 subdomains unchanged.
 template <class T, class TW>
 __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int64_t* xoff, int ldx,
                                                         const int* pvec, const int* active, int jb_blocks,
@@ -575,35 +625,42 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
                                                         int orc, int* illcond, int* status) {
   using Acc = typename EAcc<T>::type;
   extern __shared__ __align__(16) double sm[];
-  const int i = blockIdx.x;
+  const int C = cluster_size(), rank = cluster_rank();
+  const int i = blockIdx.x / C;
   if (active && !active[i]) return;
   const int full = fullv ? fullv[i] : 0;
   if (full && jb_blocks != 1) return;
-  const int n = ni[i], p = pvec[i];
+  const int p = pvec[i];
   const int jb = full ? p : jb_blocks * bcols;  // basis columns to orthogonalise against
   if (p * p > gcap || jb * p > gcap) {          // the Gram matrices would not fit the launch's space
-    if (threadIdx.x == 0) raise_status(status, A2LS_ERR_EIGEN, i, 3);
+    if (threadIdx.x == 0 && rank == 0) raise_status(status, A2LS_ERR_EIGEN, i, 3);
     return;
   }
-  T* Vi = V + xoff[i];
-  TW* Wi = W + xoff[i];
+  // this CTA's rows
+  const int per = (ni[i] + C - 1) / C, row0 = min(ni[i], rank * per), n = min(per, ni[i] - row0);
+  T* Vi = V + xoff[i] + (int64_t)row0 * ldx;
+  TW* Wi = W + xoff[i] + (int64_t)row0 * ldx;
   double* Hi = H + (int64_t)i * EIG_MAXP * EIG_MAXP;
+  const int h0 = rank == 0 ? 0 : EIG_MAXP * EIG_MAXP;  // H is written by rank 0 only: first entry of the loops
   double* G = sm;                               // gcap: Gram, then R in place
   double* Ri = G + gcap;                        // gcap
   double* trow = Ri + gcap;                     // EIG_MAXP: column scales of the Cholesky
   Acc* sv = reinterpret_cast<Acc*>(trow + EIG_MAXP);           // orc * SROW
   Acc* sw = sv + orc * SROW;                                   // orc * SROW
+  // scratch of the cluster sums: both staging chunks (a Gram matrix of a clustered launch fits them)
+  double* ctmp = reinterpret_cast<double*>(sv);
   __shared__ int rank_ok;
   const int tid = threadIdx.x;
   // the updates W -= V G and W <- W inv(R): each thread forms one row of a group of 3 columns (with
   // 64-row chunks and p = 24 that is exactly one item per thread); coefficients padded to pp columns
   const int ncg = (p + 2) / 3, pp = 3 * ncg;
   const int npass = jb > 0 ? 2 : 0;
-  for (int e = tid; e < jb * p; e += ORTH_THREADS) Hi[(e / p) * EIG_MAXP + hc + e % p] = 0.0;
+  for (int e = tid + h0; e < jb * p; e += ORTH_THREADS) Hi[(e / p) * EIG_MAXP + hc + e % p] = 0.0;
   for (int pass = 0; pass < npass; ++pass) {
     // G = V[:, 0:jb]^T W[:, 0:p]
     gram_product<Acc>(Vi, Wi, (int64_t)ldx, n, jb, p, false, sv, sw, G, sv, orc);
-    for (int e = tid; e < jb * p; e += ORTH_THREADS) Hi[(e / p) * EIG_MAXP + hc + e % p] += G[e];
+    cluster_sum(G, jb * p, ctmp);
+    for (int e = tid + h0; e < jb * p; e += ORTH_THREADS) Hi[(e / p) * EIG_MAXP + hc + e % p] += G[e];
     if (full) return;  // Rayleigh quotient only
     // W -= V G; G converted once to the working arithmetic (in Ri's space, padded to pp columns)
     Acc* Ga = reinterpret_cast<Acc*>(Ri);
@@ -646,18 +703,20 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
   int passes = 2;
   for (int pass = 0; pass < passes; ++pass) {
     gram_product<Acc>(Wi, Wi, (int64_t)ldx, n, p, p, true, sw, sw, G, sv, orc);
+    cluster_sum(G, p * p, ctmp);
     if (tid < 32) {
       // shifted pass: Gs + 11 (n p + p (p + 1)) u tr(Gs) I
       const double shift_u =
-          (pass == 0 && shifted) ? 11.0 * ((double)n * p + (double)p * (p + 1)) * Unit<Acc>::u : 0.0;
+          (pass == 0 && shifted) ? 11.0 * ((double)ni[i] * p + (double)p * (p + 1)) * Unit<Acc>::u : 0.0;
       double ratio = 0.0;
       const int ok = warp_cholesky_inverse(G, p, Ri, trow, Tiny<Acc>::v, fmax(1e-28, Unit<Acc>::u * Unit<Acc>::u),
                                            shift_u, &ratio);
       if (tid == 0) {
+        const bool first = rank == 0;  // the CTA that reports
         retry_shifted = (pass == 0 && !shifted && !(ok && ratio > plain_ratio)) ? 1 : 0;
         rank_ok = ok;
-        if (!ok && !retry_shifted && rank_flag) atomicAdd(rank_flag + i, 1);
-        if (retry_shifted && illcond) illcond[i] = 1;
+        if (!ok && !retry_shifted && rank_flag && first) atomicAdd(rank_flag + i, 1);
+        if (retry_shifted && illcond && first) illcond[i] = 1;
       }
     }
     __syncthreads();
@@ -667,7 +726,9 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
       pass = -1;
       continue;
     }
-    if (pass == 0) {
+    if (rank != 0) {
+      // (H below is rank 0's)
+    } else if (pass == 0) {
       for (int e = tid; e < p * p; e += ORTH_THREADS) {
         const int a = e / p, c = e % p;
         Hi[(hr + a) * EIG_MAXP + hc + c] = (c >= a) ? G[a * p + c] : 0.0;
@@ -963,7 +1024,9 @@ __global__ void __launch_bounds__(RRThreads<R>::v) k_rayleigh_ritz(RRParams prm,
   }
 }
 
-// X[:, 0:q] = V[:, 0:m] Y[0:m, 0:q] (q = qvec[i]); rows staged through shared memory
+// X[:, 0:q] = V[:, 0:m] Y[0:m, 0:q] (q = qvec[i]); rows staged through shared memory.  The chunks of
+// VY_RC rows are independent (X may be V: a chunk is staged before its rows are written), so the
+// gridDim.y CTAs of a subdomain take every gridDim.y-th.
 template <class T, class TX>
 __global__ void __launch_bounds__(EIG_THREADS) k_vy(const int* ni, const int64_t* xoff, int ldx, const int* mvec,
                                                      const int* qvec, const int* active, const T* V,
@@ -983,7 +1046,7 @@ __global__ void __launch_bounds__(EIG_THREADS) k_vy(const int* ni, const int64_t
   }
   const T* Vi = V + xoff[i];
   TX* Xi = X + xoff[i];
-  for (int l0 = 0; l0 < n; l0 += VY_RC) {
+  for (int l0 = blockIdx.y * VY_RC; l0 < n; l0 += gridDim.y * VY_RC) {
     const int rows = min(VY_RC, n - l0);
     __syncthreads();
     for (int e = threadIdx.x; e < rows * m; e += EIG_THREADS)
@@ -1362,7 +1425,10 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
   auto orth_smem_for = [&](int gcap) {
     return sizeof(double) * (2 * (size_t)gcap + EIG_MAXP) + sizeof(Acc) * 2 * (size_t)orc_for(gcap) * SROW;
   };
-  const size_t orth_smem = orth_smem_for(gcap_f);
+  const size_t orth_smem = std::max(orth_smem_for(gcap_f), orth_smem_for(gcap_k));
+  int dev = 0, sms = 152;
+  A2LS_CUDA(cudaGetDevice(&dev));
+  A2LS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   using RT = typename RRType<T>::type;
   int m_max = s * b;
   for (int i = 0; i < N; ++i)
@@ -1449,17 +1515,40 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
     k_project_k<T><<<N, EIG_THREADS, 0, st>>>(h->d_ni, h->d_off, d_vo, P, 0, d_pv, actv, d_kd, kvB, W);
     A2LS_LAUNCH();
   };
+  // k_orth over the subdomains actv (nact of them active in the launches that may run at the same time);
+  // with_full: the block may be one of a full-space subdomain
+  int nact = N;
+  // two CTAs of k_vy fit an SM
+  auto vy_grid = [&]() { return dim3(N, std::max(1, std::min(16, 2 * sms / std::max(nact, 1)))); };
+  auto launch_orth = [&](const int* actv, bool with_full, int jb_blocks, double* Hout, int hr, int hc, int vout,
+                         const int* fullv, int* illc) {
+    const int gcap = with_full ? gcap_f : gcap_k;
+    int C = 1;
+    if (gcap == gcap_k)
+      while (C < 8 && 2 * C * std::max(nact, 1) <= sms) C *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(N * C);
+    cfg.blockDim = dim3(ORTH_THREADS);
+    cfg.dynamicSmemBytes = orth_smem_for(gcap);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    A2LS_CUDA(cudaLaunchKernelEx(&cfg, k_orth<TV, T>, (const int*)h->d_ni, (const int64_t*)d_vo, P, (const int*)d_pv,
+                                 actv, jb_blocks, b, V, W, Hout, hr, hc, vout, fullv, d_rank, gcap, orc_for(gcap),
+                                 illc, h->d_status));
+    A2LS_LAUNCH();
+  };
   // full = the subdomains in the launch may include full-space ones, whose block has up to EIG_MAXP
   // columns (their Gram matrices need gcap_f)
   auto orthonormalize_W_into_V0 = [&](const int* actv, bool with_full) {
     k_project_k<T><<<N, EIG_THREADS, 0, st>>>(h->d_ni, h->d_off, d_vo, P, 0, d_pv, actv, d_kd, kvB, W);
     A2LS_LAUNCH();
     // no previous basis: jb = 0; R written into H's last rows (discarded)
-    const int gcap = with_full ? gcap_f : gcap_k;
-    k_orth<TV, T><<<N, ORTH_THREADS, orth_smem_for(gcap), st>>>(h->d_ni, d_vo, P, d_pv, actv, 0, b, V, W, Rscr, 0,
-                                                                0, 0, nullptr, d_rank, gcap, orc_for(gcap), nullptr,
-                                                                h->d_status);
-    A2LS_LAUNCH();
+    launch_orth(actv, with_full, 0, Rscr, 0, 0, 0, nullptr, nullptr);
   };
 
   // initial block: random or the warm-start network's proposal, then orthogonal to k, orthonormal
@@ -1571,16 +1660,16 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
       // full-space subdomains (j == 0 only): H = V0^T (T V0)
       {
         KTime kt(h, KT_EIG_ORTH, orth_flops);
-        const int gcap = (j == 0) ? gcap_f : gcap_k;
-        k_orth<TV, T><<<N, ORTH_THREADS, orth_smem_for(gcap), st>>>(h->d_ni, d_vo, P, d_pv, actv, j + 1, b, V, W, H,
-                                                      (j + 1) * b, j * b, (j + 1) * b, d_full, d_rank, gcap,
-                                                      orc_for(gcap), d_illcond, h->d_status);
-        A2LS_LAUNCH();
+        launch_orth(actv, j == 0, j + 1, H, (j + 1) * b, j * b, (j + 1) * b, d_full, d_illcond);
       }
   };
   auto queue_cycle = [&](int g, int j0) {
     Group& G = grp[g];
     use_stream(G.s);
+    nact = 0;  // both groups' subdomains share the SMs
+    for (int q = 0; q < ngroups; ++q)
+      if (!grp[q].finished)
+        for (int i = q; i < N; i += ngroups) nact += grp[q].act[i];
     for (int i = 0; i < N; ++i) G.actk[i] = G.act[i] && !full[i];
     A2LS_CUDA(cudaMemcpyAsync(G.d_actk, G.actk.data(), sizeof(int) * N, cudaMemcpyHostToDevice, st));
     for (int j = j0; j < s; ++j) {
@@ -1661,14 +1750,14 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
         A2LS_CUDA(cudaMemcpyAsync(G.d_thk, G.thk.data(), sizeof(int) * N, cudaMemcpyHostToDevice, st));
         k_thick_restart<RT><<<N, TR_THREADS, tr_smem, st>>>(G.d_thk, s * b, b, Y, H, Rscr, h->d_status);
         A2LS_LAUNCH();
-        k_vy<TV, TV><<<N, EIG_THREADS, vy_smem, st>>>(h->d_ni, d_vo, P, d_mb, d_b2, G.d_thk, V, Rscr, V);
+        k_vy<TV, TV><<<vy_grid(), EIG_THREADS, vy_smem, st>>>(h->d_ni, d_vo, P, d_mb, d_b2, G.d_thk, V, Rscr, V);
         A2LS_LAUNCH();
       }
       if (nexl) {
         // explicit restart block: W = V[:, 0:sb] Y[:, 0:b], orthonormalised into V_0; with thick
         // restarts elsewhere in the group, block step 0 of these subdomains runs here
         A2LS_CUDA(cudaMemcpyAsync(G.d_exl, G.exl.data(), sizeof(int) * N, cudaMemcpyHostToDevice, st));
-        k_vy<TV, T><<<N, EIG_THREADS, vy_smem, st>>>(h->d_ni, d_vo, P, d_msb, d_pv, G.d_exl, V, Y, W);
+        k_vy<TV, T><<<vy_grid(), EIG_THREADS, vy_smem, st>>>(h->d_ni, d_vo, P, d_msb, d_pv, G.d_exl, V, Y, W);
         A2LS_LAUNCH();
         orthonormalize_W_into_V0(G.d_exl, false);  // restarted subdomains are Krylov ones
         if (thick) block_step(0, G.d_exl, G.exl);
@@ -1710,7 +1799,7 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
   std::vector<int> zc(N), yc(N);
   A2LS_CUDA(cudaMemcpyAsync(zc.data(), d_zcols, sizeof(int) * N, cudaMemcpyDeviceToHost, st));
   A2LS_CUDA(cudaStreamSynchronize(st));
-  k_vy<TV, T><<<N, EIG_THREADS, vy_smem, st>>>(h->d_ni, d_vo, P, d_msb, d_zcols, d_active, V, Y, W);
+  k_vy<TV, T><<<vy_grid(), EIG_THREADS, vy_smem, st>>>(h->d_ni, d_vo, P, d_msb, d_zcols, d_active, V, Y, W);
   A2LS_LAUNCH();
   const int zld = nev + 2;
   std::vector<int64_t> hzo(N + 1, 0);
