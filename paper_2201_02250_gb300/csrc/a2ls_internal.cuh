@@ -240,7 +240,9 @@ template <class T> void block_solve(a2ls_handle* h, const T* fac, T* X, const in
 struct TcSolve {
   bool ready = false;
   int64_t ntiles = 0;
-  int64_t *d_ftoff = nullptr, *d_ftab = nullptr, *d_xdoff = nullptr;
+  int64_t* d_xdoff = nullptr;
+  int64_t* d_ioff[2] = {nullptr, nullptr};   // [0] the backward, [1] the forward sweep: products of each subdomain
+  int2* d_items[2] = {nullptr, nullptr};
   unsigned char *d_fdig = nullptr, *d_xdig = nullptr;
 };
 void tc_solve_prepare(a2ls_handle* h, const dfloat* fac, TcSolve& ts);   // digits of the factor tiles

@@ -38,27 +38,62 @@ constexpr size_t SMEM_BYTES = (size_t)NDIG * (A_DIGIT_BYTES + B_DIGIT_BYTES);   
 constexpr uint32_t TMEM_COLS = 512;
 constexpr long WAIT_LIMIT = 1L << 26;        // polls of the completion barrier before giving up
 
-// the NDIG digits of y = x / 2^e (|y| <= 1), as BF16 values t_s 2^(-8 s)
-__device__ __forceinline__ void df_digits(dfloat x, int e, __nv_bfloat16 (&d)[NDIG]) {
-  float yh = ldexpf(x.hi, -e), yl = ldexpf(x.lo, -e);
+// 2^k as a float for k in [-126, 127]
+__device__ __forceinline__ float pow2f(int k) { return __uint_as_float((uint32_t)(k + 127) << 23); }
+
+// x 2^k for any k a sum of two scale exponents can be: two exact multiplications by powers of two (ldexpf
+// takes a score of instructions, and the digit kernels need it for every value)
+__device__ __forceinline__ dfloat df_scale(dfloat x, int k) {
+  const int k1 = min(max(k, -126), 127), k2 = min(max(k - k1, -126), 127);
+  const float f1 = pow2f(k1), f2 = pow2f(k2);
+  return dfloat(__fmul_rn(__fmul_rn(x.hi, f1), f2), __fmul_rn(__fmul_rn(x.lo, f1), f2));
+}
+
+// The NDIG digits of y = x / 2^e (|y| <= 1), as the values t_s 2^(-8 s), exact in BF16.  y 2^56 as a 64-bit
+// integer (the pair's two parts convert separately) plus 128 at every digit but the first has the digits
+// plus 128 as its bytes, the first signed above them; a byte becomes a float by way of 2^23's mantissa.
+// About 40 instructions where rounding digit by digit in double-float takes 90, and the split of an
+// operand is on the critical chain of every block of the triangular solves (k_tcsolve.cu).
+__device__ __forceinline__ void df_digits(dfloat x, int e, float (&d)[NDIG]) {
+  const dfloat y = df_scale(x, 56 - e);
+  const long long v = __float2ll_rn(y.hi) + __float2ll_rn(y.lo) + 0x0000808080808080ll;
+  const uint32_t lo = (uint32_t)v, mid = (uint32_t)((unsigned long long)v >> 32);
+  d[0] = (float)(int)(v >> 48);
 #pragma unroll
-  for (int s = 0; s < NDIG; ++s) {
-    const float t = rintf(__fmul_rn(yh, 256.f));
-    d[s] = __float2bfloat16_rn(ldexpf(t, -8 * s));
-    // y <- 256 y - t: exact (256 y is exact and t is within one half of it)
-    yh = __fsub_rn(__fmul_rn(yh, 256.f), t);
-    yl = __fmul_rn(yl, 256.f);
-    const dfloat r = df_two_sum(yh, yl);
-    yh = r.hi;
-    yl = r.lo;
+  for (int s = 1; s < NDIG; ++s) {
+    const uint32_t byte = s < 3 ? (mid >> (8 * (2 - s))) & 0xffu : (lo >> (8 * (6 - s))) & 0xffu;
+    d[s] = __fmul_rn(__fsub_rn(__uint_as_float(0x4b000000u | byte), 8388736.f), 1.f / (float)(1ull << (8 * s)));
   }
 }
 
-// exponent e with |v| < 2^e (0 for v = 0)
+// digit s of eight consecutive values as 16 bytes of BF16
+__device__ __forceinline__ uint4 pack_digits(const float (&d)[8][NDIG], int s) {
+  __nv_bfloat162 p0 = __floats2bfloat162_rn(d[0][s], d[1][s]), p1 = __floats2bfloat162_rn(d[2][s], d[3][s]),
+                 p2 = __floats2bfloat162_rn(d[4][s], d[5][s]), p3 = __floats2bfloat162_rn(d[6][s], d[7][s]);
+  uint4 w;
+  w.x = *reinterpret_cast<uint32_t*>(&p0);
+  w.y = *reinterpret_cast<uint32_t*>(&p1);
+  w.z = *reinterpret_cast<uint32_t*>(&p2);
+  w.w = *reinterpret_cast<uint32_t*>(&p3);
+  return w;
+}
+
+// exponent e with |v| < 2^e (0 for v = 0), at least -100: smaller values keep the digits above 2^-156
 __device__ __forceinline__ int scale_exponent(float maxabs) {
   int e = 0;
   if (maxabs > 0.f) frexpf(maxabs, &e);
-  return e;
+  return max(e, -100);
+}
+
+// The sum of the seven accumulator blocks: a_d is an integer of at most 9 x 2^20 times 2^(-8 d).  a_0 plus
+// a_1 rounded to an integer is exact, so is what a_1 leaves plus a_2 (multiples of 2^-16 below 2^8); a_3
+// joins with its rounding error, and the last three, in FP32, weigh 2^-32 of the first and less.  The pair
+// is not normalised (|lo| may exceed ulp(hi) / 2).
+__device__ __forceinline__ dfloat sum_blocks(float a0, float a1, float a2, float a3, float a4, float a5, float a6) {
+  const float t1 = rintf(a1);
+  const dfloat q = df_two_sum(__fadd_rn(__fsub_rn(a1, t1), a2), a3);
+  const dfloat v = df_two_sum(__fadd_rn(a0, t1), q.hi);
+  return dfloat(v.hi, __fadd_rn(v.lo, __fadd_rn(q.lo, __fadd_rn(a4, __fadd_rn(a5, a6)))));
 }
 
 struct Ctx {
@@ -86,21 +121,12 @@ __device__ __forceinline__ void split_a(Ctx& c, FA fa) {
   if (h == 0) c.eA[r] = e;
 #pragma unroll
   for (int q8 = 0; q8 < 4; ++q8) {
-    __nv_bfloat16 dg[8][NDIG];
+    float dg[8][NDIG];
 #pragma unroll
     for (int q = 0; q < 8; ++q) df_digits(v[q8 * 8 + q], e, dg[q]);
     const uint32_t off = tc::operand_offset(r, h * 32 + q8 * 8, TK);
 #pragma unroll
-    for (int s = 0; s < NDIG; ++s) {
-      __nv_bfloat162 p0 = __halves2bfloat162(dg[0][s], dg[1][s]), p1 = __halves2bfloat162(dg[2][s], dg[3][s]),
-                     p2 = __halves2bfloat162(dg[4][s], dg[5][s]), p3 = __halves2bfloat162(dg[6][s], dg[7][s]);
-      uint4 w;
-      w.x = *reinterpret_cast<uint32_t*>(&p0);
-      w.y = *reinterpret_cast<uint32_t*>(&p1);
-      w.z = *reinterpret_cast<uint32_t*>(&p2);
-      w.w = *reinterpret_cast<uint32_t*>(&p3);
-      *reinterpret_cast<uint4*>(c.smem + s * A_DIGIT_BYTES + off) = w;
-    }
+    for (int s = 0; s < NDIG; ++s) *reinterpret_cast<uint4*>(c.smem + s * A_DIGIT_BYTES + off) = pack_digits(dg, s);
   }
 }
 
@@ -123,21 +149,12 @@ __device__ __forceinline__ void split_b(Ctx& c, FB fb, float* red) {
   if (qk == 0) c.eB[n] = e;
 #pragma unroll
   for (int q8 = 0; q8 < 2; ++q8) {
-    __nv_bfloat16 dg[8][NDIG];
+    float dg[8][NDIG];
 #pragma unroll
     for (int q = 0; q < 8; ++q) df_digits(v[q8 * 8 + q], e, dg[q]);
     const uint32_t off = tc::operand_offset(n, qk * 16 + q8 * 8, TK);
 #pragma unroll
-    for (int s = 0; s < NDIG; ++s) {
-      __nv_bfloat162 p0 = __halves2bfloat162(dg[0][s], dg[1][s]), p1 = __halves2bfloat162(dg[2][s], dg[3][s]),
-                     p2 = __halves2bfloat162(dg[4][s], dg[5][s]), p3 = __halves2bfloat162(dg[6][s], dg[7][s]);
-      uint4 w;
-      w.x = *reinterpret_cast<uint32_t*>(&p0);
-      w.y = *reinterpret_cast<uint32_t*>(&p1);
-      w.z = *reinterpret_cast<uint32_t*>(&p2);
-      w.w = *reinterpret_cast<uint32_t*>(&p3);
-      *reinterpret_cast<uint4*>(c.smem + NDIG * A_DIGIT_BYTES + s * B_DIGIT_BYTES + off) = w;
-    }
+    for (int s = 0; s < NDIG; ++s) *reinterpret_cast<uint4*>(c.smem + NDIG * A_DIGIT_BYTES + s * B_DIGIT_BYTES + off) = pack_digits(dg, s);
   }
 }
 
@@ -221,12 +238,10 @@ __device__ __forceinline__ void epilogue_subtract(Ctx& c, dfloat* C, int64_t ldc
       tc::tmem_wait_ld();
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        dfloat sum = df_two_sum(acc[0][q], acc[1][q]);
-#pragma unroll
-        for (int g = 2; g < NBLK; ++g) sum = sum + dfloat(acc[g][q], 0.f);
+        const dfloat sum = sum_blocks(acc[0][q], acc[1][q], acc[2][q], acc[3][q], acc[4][q], acc[5][q], acc[6][q]);
         const int e = em + c.eB[cbase + nq + cb + q] - 16;
         dfloat& o = S[m * SUB_LD + nq + cb + q];
-        o = o - dfloat(ldexpf(sum.hi, e), ldexpf(sum.lo, e));
+        o = o - df_scale(sum, e);
       }
     }
     __syncthreads();
