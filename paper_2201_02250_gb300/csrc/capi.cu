@@ -525,6 +525,7 @@ int a2ls_setup(const a2ls_csr* A, const int32_t* partition, int32_t overlap, int
     // the factors repacked for the streaming local solves
     if (o.precision == A2LS_BF16) stream_prepare<__nv_bfloat16>(h, static_cast<const __nv_bfloat16*>(h->d_fac));
     else if (o.precision == A2LS_FP32) stream_prepare<float>(h, static_cast<const float*>(h->d_fac));
+    else if (o.local_solve_kernel == 0) stream_prepare<double>(h, static_cast<const double*>(h->d_fac));
     // apply workspace
     h->d_q = dalloc<double>(h, h->n);
     h->d_t = dalloc<double>(h, h->n);

@@ -950,11 +950,8 @@ static void launch_local_solve_width(a2ls_handle* h, int width, const T* fac, co
     case LS_STREAM:
     case LS_STREAM2:
     case LS_STREAM3:
-      if constexpr (!std::is_same<T, double>::value) {
-        launch_local_solve_stream<T>(h, width, t, q, z, mode);
-        break;
-      }
-      [[fallthrough]];
+      launch_local_solve_stream<T>(h, width, t, q, z, mode);
+      break;
     default: launch_local_solve<T, 512>(h, fac, t, q, z, mode); break;
   }
 }
@@ -978,7 +975,7 @@ void local_solves(a2ls_handle* h, const T* fac, const double* t, const double* q
 template <class T>
 void autotune_local_solves(a2ls_handle* h, const T* fac, const double* t, double* scratch, int mode) {
   char key[128];
-  snprintf(key, sizeof(key), "local_solve3_%s_N%d_max%d_mode%d",
+  snprintf(key, sizeof(key), "local_solve4_%s_N%d_max%d_mode%d",
            sizeof(T) == 8 ? "fp64" : (sizeof(T) == 4 ? "fp32" : "bf16"), h->N, h->max_n, mode);
   int cached = autotune_lookup(key);
   if (cached > 0 && (cached != LS_STREAM || h->ss.shape[0].ready) && (cached != LS_STREAM2 || h->ss.shape[1].ready) &&
@@ -987,11 +984,9 @@ void autotune_local_solves(a2ls_handle* h, const T* fac, const double* t, double
     return;
   }
   std::vector<int> widths = {256, 512, 1024, 1256, 1512, 2256};
-  if (!std::is_same<T, double>::value) {
-    if (h->ss.shape[0].ready) widths.push_back(LS_STREAM);
-    if (h->ss.shape[1].ready) widths.push_back(LS_STREAM2);
-    if (h->ss.shape[2].ready) widths.push_back(LS_STREAM3);
-  }
+  if (h->ss.shape[0].ready) widths.push_back(LS_STREAM);
+  if (h->ss.shape[1].ready) widths.push_back(LS_STREAM2);
+  if (h->ss.shape[2].ready) widths.push_back(LS_STREAM3);
   float best_ms = 1e30f;
   int best = 512;
   cudaEvent_t e0, e1;

@@ -67,9 +67,17 @@ template <int W> __host__ __device__ __forceinline__ int ud_off(int rr, int tb) 
   return rr * tri_up<W>(tb) - tri_sumlo<W>(rr);
 }
 
-template <class T> struct V16;                   // elements per 16 bytes
-template <> struct V16<float> { static constexpr int W = 4; };
-template <> struct V16<__nv_bfloat16> { static constexpr int W = 8; };
+template <class T> struct V16;                   // elements per 16 bytes; the solves' arithmetic
+template <> struct V16<float> { static constexpr int W = 4; using Acc = float; };
+template <> struct V16<__nv_bfloat16> { static constexpr int W = 8; using Acc = float; };
+template <> struct V16<double> { static constexpr int W = 2; using Acc = double; };
+
+// The diagonal triangles of FP64 factors are stored as dense 64 x 64 tiles, column-major like a panel of L (the
+// other triangle zero), and applied like one.  By rows a row's 32 lanes end in five shuffled FP64 additions
+// a row, each of which holds GB300's FP64 pipe as long as 32 useful multiply-adds; a thread per two rows
+// adds its columns up alone and the warps' sums meet in shared memory.  FP64 applies against the pipelined
+// kernel: 16 subdomains of 300 rows 132 -> 52 us, 125 of 2600 rows 3.81 -> 2.6 ms.
+template <class T> constexpr bool dense_diag() { return V16<T>::W == 2; }
 
 // the W values of the 16 bytes at d (shared memory)
 __device__ __forceinline__ void unpack16(const float* d, float (&v)[4]) {
@@ -87,6 +95,12 @@ __device__ __forceinline__ void unpack16(const __nv_bfloat16* d, float (&v)[8]) 
     v[2 * k] = __uint_as_float(w[k] << 16);
     v[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
   }
+}
+
+__device__ __forceinline__ void unpack16(const double* d, double (&v)[2]) {
+  const double2 a = *reinterpret_cast<const double2*>(d);
+  v[0] = a.x;
+  v[1] = a.y;
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -135,16 +149,18 @@ __global__ void __launch_bounds__(32 * CW + 32, CTAS_PER_SM) k_local_solve_strea
     const int* __restrict__ nI, const int* __restrict__ ni, const int* __restrict__ idx, const double* __restrict__ D,
     const double* __restrict__ t, const double* __restrict__ q, double* __restrict__ out, int mode, int* st) {
   constexpr int W = V16<T>::W;
+  using Acc = typename V16<T>::Acc;
+  constexpr bool DENSE = dense_diag<T>();
   constexpr int CONSUMER_WARPS = CW, CONSUMERS = 32 * CW;
   // diagonal blocks: LPR lanes a row (one 16-byte vector each), RPI rows a warp step, RPW rows a warp,
   // IT steps
-  constexpr int LPR = 64 / W, RPI = 32 / LPR, RPW = 64 / CW, IT = RPW / RPI;
+  [[maybe_unused]] constexpr int LPR = 64 / W, RPI = 32 / LPR, RPW = 64 / CW, IT = RPW / RPI;
   extern __shared__ __align__(128) unsigned char sm[];
   unsigned char* stages = sm;                                                  // nstages x STAGE_BYTES
-  float* rhs = reinterpret_cast<float*>(sm + (size_t)nstages * STAGE_BYTES);  // xcap: R_i r, then the solution
-  float* x = rhs + xcap;                                                       // xcap: y, then the backward work
-  float* part = x + xcap;                                                      // CW x 64: each warp's panel sums
-  float* s64 = part + CW * 64;                                                 // 64: the block's s = rhs - L y
+  Acc* rhs = reinterpret_cast<Acc*>(sm + (size_t)nstages * STAGE_BYTES);       // xcap: R_i r, then the solution
+  Acc* x = rhs + xcap;                                                         // xcap: y, then the backward work
+  Acc* part = x + xcap;                                                        // CW x 64: each warp's panel sums
+  Acc* s64 = part + CW * 64;                                                   // 64: the block's s = rhs - L y
   __shared__ __align__(8) uint64_t full[MAX_STAGES], empty[MAX_STAGES];
   __shared__ int stage_sub[MAX_STAGES];
   __shared__ volatile int abort_flag;
@@ -244,10 +260,10 @@ __global__ void __launch_bounds__(32 * CW + 32, CTAS_PER_SM) k_local_solve_strea
     if (i < 0) break;  // the same stage for every warp: uniform
     const int n = ni[i], o = off[i];
     for (int l = tid; l < xcap; l += CONSUMERS) {
-      rhs[l] = l < n ? (float)t[idx[o + l]] : 0.f;
-      x[l] = 0.f;
+      rhs[l] = l < n ? (Acc)t[idx[o + l]] : (Acc)0;
+      x[l] = 0;
     }
-    for (int e = tid; e < CW * 64; e += CONSUMERS) part[e] = 0.f;
+    for (int e = tid; e < CW * 64; e += CONSUMERS) part[e] = 0;
     if (consumer_sync_or<CONSUMERS>(aborted)) {
       aborted = 1;
       break;
@@ -275,11 +291,11 @@ __global__ void __launch_bounds__(32 * CW + 32, CTAS_PER_SM) k_local_solve_strea
       if (kind == LD) {
         // s = (R_i r)_b - L_b y from the warps' panel sums, which are then cleared for the next block
         if (tid < 64) {
-          float sum = 0.f;
+          Acc sum = 0;
 #pragma unroll
           for (int w = 0; w < CW; ++w) {
             sum += part[w * 64 + tid];
-            part[w * 64 + tid] = 0.f;
+            part[w * 64 + tid] = 0;
           }
           s64[tid] = rhs[r0 + tid] - sum;
         }
@@ -290,21 +306,22 @@ __global__ void __launch_bounds__(32 * CW + 32, CTAS_PER_SM) k_local_solve_strea
       }
       if (have) {
         const T* data = reinterpret_cast<const T*>(sp + STAGE_META);
-        if (kind == LP) {
+        if (kind == LP || (DENSE && diag)) {
+          // (dense diagonal tiles: the product with s or with the block's y, summed over the warps below)
           // part[warp][r] += sum over the chunk's columns c of L[r0 + r][c] y[c]: the chunk is column-major
           // (64 rows a column); a thread takes W rows (row group g) and the columns sub, sub + NSUB, ...
           constexpr int G = 64 / W, NSUB = CONSUMERS / G;
           const int g = tid % G, sub = tid / G;
           const int c0 = hd.x, ncols = hd.z / 64;
-          const float* yc = x + c0;
-          float acc[W];
+          const Acc* yc = kind == LP ? x + c0 : (kind == LD ? s64 : x + r0);
+          Acc acc[W];
 #pragma unroll
-          for (int v = 0; v < W; ++v) acc[v] = 0.f;
+          for (int v = 0; v < W; ++v) acc[v] = 0;
 #pragma unroll 4
           for (int c = sub; c < ncols; c += NSUB) {
-            float e[W];
+            Acc e[W];
             unpack16(data + c * 64 + g * W, e);
-            const float yv = yc[c];
+            const Acc yv = yc[c];
 #pragma unroll
             for (int v = 0; v < W; ++v) acc[v] += e[v] * yv;
           }
@@ -317,6 +334,7 @@ __global__ void __launch_bounds__(32 * CW + 32, CTAS_PER_SM) k_local_solve_strea
 #pragma unroll
             for (int v = 0; v < W; ++v) part[warp * 64 + g * W + v] += acc[v];
         } else if (kind == LD) {
+          if constexpr (!DENSE) {
           // y[r0 + rr] = s[rr] + sum_{c < rr} inv(L_bb)[rr][c] s[c]: LPR lanes a row, one 16-byte vector
           // each; a warp's rows RPI at a time, their reductions interleaved at the end
           const int q = lane % LPR, sl = lane / LPR;
@@ -346,7 +364,9 @@ __global__ void __launch_bounds__(32 * CW + 32, CTAS_PER_SM) k_local_solve_strea
             const int rr = warp * RPW + it * RPI + sl;
             if (rr < tb && q == 0) x[r0 + rr] = s64[rr] + acc[it];
           }
+          }
         } else if (kind == UD) {
+          if constexpr (!DENSE) {
           // solution rows: rhs[r0 + rr] = sum_{c >= rr} inv(U_bb)[rr][c] y[r0 + c], mapped as above
           const int q = lane % LPR, sl = lane / LPR;
           float yv[W], e[W], acc[IT];
@@ -376,6 +396,7 @@ __global__ void __launch_bounds__(32 * CW + 32, CTAS_PER_SM) k_local_solve_strea
             const int rr = warp * RPW + it * RPI + sl;
             if (rr < tb && q == 0) rhs[r0 + rr] = acc[it];
           }
+          }
         } else {
           // right-looking update of the rows above the block: y[r] -= sum_{cc < 64} U[r][r0 + cc] x[r0 + cc]
           // for the chunk's rows r = ra .. ra + R.  The chunk is column-major, R rows a column (R x the
@@ -385,15 +406,15 @@ __global__ void __launch_bounds__(32 * CW + 32, CTAS_PER_SM) k_local_solve_strea
           const int sub = lane >> 2;
           for (int gb = warp * 4; gb < ng; gb += 4 * CW) {
             const int gq = gb + (lane & 3);
-            float acc[W];
+            Acc acc[W];
 #pragma unroll
-            for (int v = 0; v < W; ++v) acc[v] = 0.f;
+            for (int v = 0; v < W; ++v) acc[v] = 0;
             if (gq < ng) {
 #pragma unroll 4
               for (int cc = sub; cc < 64; cc += 8) {
-                float e[W];
+                Acc e[W];
                 unpack16(data + cc * R + gq * W, e);
-                const float xv = rhs[r0 + cc];
+                const Acc xv = rhs[r0 + cc];
 #pragma unroll
                 for (int v = 0; v < W; ++v) acc[v] += e[v] * xv;
               }
@@ -413,6 +434,24 @@ __global__ void __launch_bounds__(32 * CW + 32, CTAS_PER_SM) k_local_solve_strea
       if (diag && consumer_sync_or<CONSUMERS>(aborted)) {
         aborted = 1;
         break;
+      }
+      if constexpr (DENSE) {
+        if (diag) {
+          if (tid < 64) {
+            Acc sum = 0;
+#pragma unroll
+            for (int w = 0; w < CW; ++w) {
+              sum += part[w * 64 + tid];
+              part[w * 64 + tid] = 0;
+            }
+            if (kind == LD) x[r0 + tid] = tid < tb ? s64[tid] + sum : (Acc)0;
+            else rhs[r0 + tid] = sum;
+          }
+          if (consumer_sync_or<CONSUMERS>(aborted)) {
+            aborted = 1;
+            break;
+          }
+        }
       }
     }
     if (aborted) break;
@@ -458,15 +497,18 @@ __global__ void __launch_bounds__(256) k_pack_stream(int nchunks, int N, const i
     const int4 hd = meta[c];
     T* dst = stream + soff[i] + hd.w;
     const int kind = hd.y & 3, r0 = (hd.y >> 2) * 64, tb = min(64, n - r0);
-    if (kind == LP) {
-      // column-major: (c0 + cl, rr) at cl * 64 + rr = L[r0 + rr][c0 + cl], in groups of 64 columns
-      const int c0 = hd.x, ncols = hd.z / 64;
+    const bool dense = dense_diag<T>() && (kind == LD || kind == UD);
+    if (kind == LP || dense) {
+      // column-major: (c0 + cl, rr) at cl * 64 + rr = L[r0 + rr][c0 + cl], in groups of 64 columns; a dense
+      // diagonal tile keeps its own triangle
+      const int c0 = dense ? r0 : hd.x, ncols = hd.z / 64;
       for (int g = 0; g < ncols; g += 64) {
         const int gc = min(64, ncols - g);
         __syncthreads();
         for (int e = tid; e < 64 * 64; e += 256) {
           const int rr = e >> 6, cl = e & 63;
-          if (cl < gc) tile[rr * 65 + cl] = rr < tb ? F[(int64_t)(r0 + rr) * L + c0 + g + cl] : T(0.f);
+          const bool in = rr < tb && (!dense || (cl < tb && (kind == LD ? cl < rr : cl >= rr)));
+          if (cl < gc) tile[rr * 65 + cl] = in ? F[(int64_t)(r0 + rr) * L + c0 + g + cl] : T(0.f);
         }
         __syncthreads();
         for (int e = tid; e < gc * 64; e += 256) {
@@ -550,11 +592,11 @@ void stream_prepare(a2ls_handle* h, const T* fac) {
       int cmin = r0;
       for (int r = r0; r < r0 + tb; ++r) cmin = std::min(cmin, lo(pf[o + r]));
       for (int c = cmin; c < r0; c += lp_cols) chunk(LP, b, c, 64 * std::min(lp_cols, r0 - c));
-      chunk(LD, b, 0, ld_elems<W>(tb));
+      chunk(LD, b, 0, dense_diag<T>() ? 64 * 64 : ld_elems<W>(tb));
     }
     for (int b = nb - 1; b >= 0; --b) {
       const int r0 = b * TB, tb = std::min(TB, n - r0);
-      chunk(UD, b, 0, ud_elems<W>(tb));
+      chunk(UD, b, 0, dense_diag<T>() ? 64 * 64 : ud_elems<W>(tb));
       // U panel of the block: rows from the first envelope row of its columns up to r0, all 64 columns
       int rmin = r0;
       for (int c = r0; c < r0 + tb; ++c) rmin = std::min(rmin, lo(pg[o + c]));
@@ -571,7 +613,13 @@ void stream_prepare(a2ls_handle* h, const T* fac) {
   S.elem_bytes = (int)sizeof(T);
   S.nchunks = (int)meta.size();
   S.stream_elems = soff[N];
-  S.d_stream = dalloc<T>(h, (size_t)soff[N] + W);
+  try {
+    S.d_stream = dalloc<T>(h, (size_t)soff[N] + W);
+  } catch (const Error& e) {
+    // FP64 handles hold the largest factors: without room for the second copy they keep to the other kernels
+    if (sizeof(T) != 8 || e.code != A2LS_ERR_OOM) throw;
+    return;
+  }
   S.d_meta = dalloc<int4>(h, meta.size());
   S.d_choff = dalloc<int>(h, N + 1);
   S.d_soff = dalloc<int64_t>(h, N + 1);
@@ -589,7 +637,7 @@ void stream_prepare(a2ls_handle* h, const T* fac) {
   A2LS_LAUNCH();
   S.xcap = (int)round_up(h->max_n, TB);
   // the two vectors, the warps' panel sums (8 warps at most) and the block's s
-  const size_t fixed = sizeof(float) * (2 * (size_t)S.xcap + 8 * 64 + 64);
+  const size_t fixed = sizeof(typename V16<T>::Acc) * (2 * (size_t)S.xcap + 8 * 64 + 64);
   // the kernel shapes: 8 consumer warps, one CTA per SM; 4 consumer warps, two CTAs per SM; 8 consumer
   // warps, two CTAs per SM
   for (int v = 0; v < 3; ++v) {
@@ -601,17 +649,19 @@ void stream_prepare(a2ls_handle* h, const T* fac) {
     sh.smem = (size_t)sh.nstages * STAGE_BYTES + fixed;
     if (sh.nstages < 2) continue;
     int occ = 0;
+    // the limit belongs to the kernel, not to this handle: the most any handle can ask for, so that a later
+    // handle with a smaller need does not take it from this one
     if (v == 0) {
       A2LS_CUDA(cudaFuncSetAttribute(k_local_solve_stream<T, 8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)sh.smem));
+                                     (int)budget));
       A2LS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local_solve_stream<T, 8, 1>, 288, sh.smem));
     } else if (v == 1) {
       A2LS_CUDA(cudaFuncSetAttribute(k_local_solve_stream<T, 4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)sh.smem));
+                                     (int)budget));
       A2LS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local_solve_stream<T, 4, 2>, 160, sh.smem));
     } else {
       A2LS_CUDA(cudaFuncSetAttribute(k_local_solve_stream<T, 8, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)sh.smem));
+                                     (int)budget));
       A2LS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local_solve_stream<T, 8, 2>, 288, sh.smem));
     }
     if (occ < ctas) continue;
@@ -653,6 +703,8 @@ void launch_local_solve_stream(a2ls_handle* h, int config, const double* t, cons
   A2LS_LAUNCH();
 }
 
+template void stream_prepare<double>(a2ls_handle*, const double*);
+template void launch_local_solve_stream<double>(a2ls_handle*, int, const double*, const double*, double*, int);
 template void stream_prepare<float>(a2ls_handle*, const float*);
 template void stream_prepare<__nv_bfloat16>(a2ls_handle*, const __nv_bfloat16*);
 template void launch_local_solve_stream<float>(a2ls_handle*, int, const double*, const double*, double*, int);
