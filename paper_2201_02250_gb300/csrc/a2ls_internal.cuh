@@ -234,7 +234,7 @@ void dense_inverse(a2ls_handle* h, double* E, int n, double scale, double* Einv,
 // skip_p_le > 0: subdomains with at most that many columns are left to another kernel
 template <class T> void block_solve(a2ls_handle* h, const T* fac, T* X, const int64_t* xoff, int col0, int ldx,
                                     const int* pvec, int pmax, const int* active, int forward, int backward,
-                                    int skip_p_le = 0);
+                                    int skip_p_le = 0, int nact = 0);
 
 // k_tcsolve.cu: double-float block triangular solves of the eigensolver on the tensor cores
 struct TcSolve {

@@ -130,7 +130,6 @@ __device__ __forceinline__ dfloat se_warp_maxabs(dfloat a) {
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return dfloat(v, 0.f);
 }
-__device__ __forceinline__ constexpr bool se_range_limited(dfloat) { return true; }
 __device__ __forceinline__ bool se_is_zero(dfloat a) { return a.hi == 0.f; }
 __device__ __forceinline__ double se_dbl(dfloat a) { return (double)a; }
 __device__ __forceinline__ void se_mac(dfloat& acc, dfloat a, dfloat b) { df_mac(acc, a, b); }

@@ -28,16 +28,18 @@ template <> struct AccOf<dfloat> { using type = dfloat; };
 constexpr int GK = 32;
 
 // ---------------------------------------------------------------------------
-// Narrowest tile product for the column chunks of the eigen solves: M <= 64 rows, Nc <= 8
-// columns; 256 threads, thread (ty, tx) owns row ty and columns 2tx, 2tx+1.
+// Narrow tile product for the column chunks of the eigen solves: M <= 64 rows, Nc <= NCW columns (8, 4 or
+// 2); 64 min(NCW, 4) threads, thread (ty, tx) owns row ty and CPT columns from CPT tx.
 // ---------------------------------------------------------------------------
-template <class T, class Acc>
-__device__ __forceinline__ void cta_gemm_n8(const T* __restrict__ A, int64_t lda, const T* __restrict__ B,
-                                            int64_t ldb, int M, int Nc, int K, int amask, Acc (&acc)[2], Acc* sA,
-                                            Acc* sB) {
-  const int tid = threadIdx.x, tx = tid & 3, ty = tid >> 2;
+template <int NCW> constexpr int narrow_threads() { return NCW >= 4 ? 256 : 64 * NCW; }
+template <class T, class Acc, int NCW, int CPT>
+__device__ __forceinline__ void cta_gemm_narrow(const T* __restrict__ A, int64_t lda, const T* __restrict__ B,
+                                                int64_t ldb, int M, int Nc, int K, int amask, Acc (&acc)[CPT],
+                                                Acc* sA, Acc* sB) {
+  constexpr int TX = NCW / CPT, THREADS = 64 * TX;
+  const int tid = threadIdx.x, tx = tid & (TX - 1), ty = tid / TX;
   for (int k0 = 0; k0 < K; k0 += GK) {
-    for (int e = tid; e < 64 * GK; e += 256) {
+    for (int e = tid; e < 64 * GK; e += THREADS) {
       const int m = e / GK, k = e % GK;
       Acc v = 0;
       const int kk = k0 + k;
@@ -48,22 +50,21 @@ __device__ __forceinline__ void cta_gemm_n8(const T* __restrict__ A, int64_t lda
       }
       sA[k * 65 + m] = v;
     }
-    {
-      const int e = tid;  // GK * 8 == 256
-      const int k = e / 8, c = e % 8;
+    for (int e = tid; e < GK * NCW; e += THREADS) {
+      const int k = e / NCW, c = e % NCW;
       const int kk = k0 + k;
-      sB[k * 9 + c] = (c < Nc && kk < K) ? (Acc)B[kk * ldb + c] : (Acc)0;
+      sB[k * (NCW + 1) + c] = (c < Nc && kk < K) ? (Acc)B[kk * ldb + c] : (Acc)0;
     }
     __syncthreads();
     // a triangular A has no entries of row ty in this chunk when the chunk lies wholly right of the
     // diagonal (unit lower) or wholly left of it (upper); whole warps skip together
     const bool zero_chunk = (amask == 1 && k0 > ty) || (amask == 2 && k0 + GK - 1 < ty);
-    if (tx * 2 < Nc && !zero_chunk) {
+    if (tx * CPT < Nc && !zero_chunk) {
 #pragma unroll 8
       for (int k = 0; k < GK; ++k) {
         const Acc a = sA[k * 65 + ty];
-        mac(acc[0], a, sB[k * 9 + tx * 2]);
-        mac(acc[1], a, sB[k * 9 + tx * 2 + 1]);
+#pragma unroll
+        for (int v = 0; v < CPT; ++v) mac(acc[v], a, sB[k * (NCW + 1) + tx * CPT + v]);
       }
     }
     __syncthreads();
@@ -1015,29 +1016,32 @@ void autotune_local_solves(a2ls_handle* h, const T* fac, const double* t, double
 // multi right-hand-side solves for the eigensolver: X (n_i x p, row-major, leading
 // dimension ldx, subdomain i at X + i*xstride) <- inv(U) inv(L) X (either half optional)
 // ---------------------------------------------------------------------------
-// One CTA per (subdomain, chunk of 8 right-hand sides): blockIdx.y selects the chunk, so that the
-// FP64-bound solves of the eigen iteration spread over all SMs.
-template <class T>
-__global__ void __launch_bounds__(256) k_block_solve(const int* ni, const int* ld, const int64_t* foff,
+// One CTA per (subdomain, chunk of NCW right-hand sides): blockIdx.y selects the chunk, so that the
+// FP64-bound solves of the eigen iteration spread over all SMs.  A column's arithmetic does not depend on
+// the chunk's width; narrower chunks stage the factors more often and are taken where wider ones leave
+// the FP64 pipes of some SMs idle.
+template <class T, int NCW>
+__global__ void __launch_bounds__(narrow_threads<NCW>()) k_block_solve(const int* ni, const int* ld, const int64_t* foff,
                                                      const T* __restrict__ fac, T* X,
                                                      const int64_t* xoff, int col0, int ldx,
                                                      const int* pvec, const int* active, int forward,
                                                      int backward, const int* sched, const int* toff,
                                                      const int* tf, const int* tg, int skip_p_le) {
   using Acc = typename AccOf<T>::type;
-  __shared__ Acc sA[GK * 65], sB[GK * 9];
+  constexpr int CPT = NCW == 8 ? 2 : 1, TX = NCW / CPT;
+  __shared__ Acc sA[GK * 65], sB[GK * (NCW + 1)];
   const int i = sched ? sched[blockIdx.x] : blockIdx.x;  // largest subdomains first
   if (active && !active[i]) return;
   const int p = pvec[i];
   if (p <= skip_p_le) return;
-  const int c0 = blockIdx.y * 8;
+  const int c0 = blockIdx.y * NCW;
   if (c0 >= p) return;
-  const int pc = min(8, p - c0);
+  const int pc = min(NCW, p - c0);
   const int n = ni[i];
   const int64_t L = ld[i];
   const T* M = fac + foff[i];
   T* Xi = X + xoff[i] + col0 + c0;
-  const int tid = threadIdx.x, tx = tid & 3, ty = tid >> 2;
+  const int tid = threadIdx.x, tx = tid & (TX - 1), ty = tid / TX;
   const int nb = (n + TB - 1) / TB;
   for (int pass = 0; pass < 2; ++pass) {
     if (pass == 0 && !forward) continue;
@@ -1045,38 +1049,38 @@ __global__ void __launch_bounds__(256) k_block_solve(const int* ni, const int* l
     for (int bb = 0; bb < nb; ++bb) {
       const int b = pass == 0 ? bb : nb - 1 - bb;
       const int r0 = b * TB, tb = min(TB, n - r0);
-      Acc acc[2] = {};
+      Acc acc[CPT] = {};
       if (pass == 0) {
         // L[r][c] = 0 left of the block's first envelope column
         const int fs = tf[toff[i] + b];
         if (r0 > fs)
-          cta_gemm_n8<T, Acc>(M + (int64_t)r0 * L + fs, L, Xi + (int64_t)fs * ldx, ldx, tb, pc, r0 - fs, 0, acc, sA,
+          cta_gemm_narrow<T, Acc, NCW, CPT>(M + (int64_t)r0 * L + fs, L, Xi + (int64_t)fs * ldx, ldx, tb, pc, r0 - fs, 0, acc, sA,
                               sB);
       } else {
         // U[r][c] = 0 above column c's first envelope row: skip the 64-column tiles that start below
         for (int cb = b + 1; cb < nb; ++cb) {
           if (tg[toff[i] + cb] > r0 + tb - 1) continue;
           const int e0 = cb * TB;
-          cta_gemm_n8<T, Acc>(M + (int64_t)r0 * L + e0, L, Xi + (int64_t)e0 * ldx, ldx, tb, pc, min(TB, n - e0), 0,
+          cta_gemm_narrow<T, Acc, NCW, CPT>(M + (int64_t)r0 * L + e0, L, Xi + (int64_t)e0 * ldx, ldx, tb, pc, min(TB, n - e0), 0,
                               acc, sA, sB);
         }
       }
       // S = X_b - acc, written in place
 #pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        const int c = tx * 2 + v;
+      for (int v = 0; v < CPT; ++v) {
+        const int c = tx * CPT + v;
         if (ty < tb && c < pc) {
           T* ptr = Xi + (int64_t)(r0 + ty) * ldx + c;
           *ptr = (T)((Acc)*ptr - acc[v]);
         }
       }
       __syncthreads();
-      Acc acc2[2] = {};
-      cta_gemm_n8<T, Acc>(M + (int64_t)r0 * L + r0, L, Xi + (int64_t)r0 * ldx, ldx, tb, pc, tb, pass == 0 ? 1 : 2,
+      Acc acc2[CPT] = {};
+      cta_gemm_narrow<T, Acc, NCW, CPT>(M + (int64_t)r0 * L + r0, L, Xi + (int64_t)r0 * ldx, ldx, tb, pc, tb, pass == 0 ? 1 : 2,
                           acc2, sA, sB);
 #pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        const int c = tx * 2 + v;
+      for (int v = 0; v < CPT; ++v) {
+        const int c = tx * CPT + v;
         if (ty < tb && c < pc) Xi[(int64_t)(r0 + ty) * ldx + c] = (T)finish(acc2[v]);
       }
       __syncthreads();
@@ -1084,14 +1088,26 @@ __global__ void __launch_bounds__(256) k_block_solve(const int* ni, const int* l
   }
 }
 
+// nact: subdomains active in this launch and those that may run beside it
 template <class T>
 void block_solve(a2ls_handle* h, const T* fac, T* X, const int64_t* xoff, int col0, int ldx, const int* pvec,
-                 int pmax, const int* active, int forward, int backward, int skip_p_le) {
+                 int pmax, const int* active, int forward, int backward, int skip_p_le, int nact) {
   if (pmax <= skip_p_le) return;
-  dim3 grid(h->N, (std::max(pmax, 1) + 7) / 8);
-  k_block_solve<T><<<grid, 256, 0, h->st>>>(h->d_ni, h->d_ld, h->d_foff, fac, X, xoff, col0, ldx, pvec, active,
-                                           forward, backward, h->d_sched, h->d_toff, h->d_tf, h->d_tg, skip_p_le);
-  A2LS_LAUNCH();
+  const int p = std::max(pmax, 1);
+  if (nact <= 0) nact = h->N;
+  // at least three CTAs per SM where narrower chunks give them: 64 FP64 subdomains of 1950 rows, p = 16, 4.58 ->
+  // 3.13 ms a sweep; 16 of 300 rows 151 -> 117 us (8 columns against 2)
+  int w = 8;
+  while (w > 2 && (int64_t)nact * ceil_div(p, w) < 3 * 152) w /= 2;
+  const dim3 grid(h->N, ceil_div(p, w));
+  auto go = [&](auto kernel, int threads) {
+    kernel<<<grid, threads, 0, h->st>>>(h->d_ni, h->d_ld, h->d_foff, fac, X, xoff, col0, ldx, pvec, active, forward,
+                                        backward, h->d_sched, h->d_toff, h->d_tf, h->d_tg, skip_p_le);
+    A2LS_LAUNCH();
+  };
+  if (w == 8) go(k_block_solve<T, 8>, narrow_threads<8>());
+  else if (w == 4) go(k_block_solve<T, 4>, narrow_threads<4>());
+  else go(k_block_solve<T, 2>, narrow_threads<2>());
 }
 
 template void lu_batched<float>(a2ls_handle*, float*, int, double*, double*, int);
@@ -1106,13 +1122,13 @@ template void local_solves<double>(a2ls_handle*, const double*, const double*, c
 template void autotune_local_solves<float>(a2ls_handle*, const float*, const double*, double*, int);
 template void autotune_local_solves<double>(a2ls_handle*, const double*, const double*, double*, int);
 template void block_solve<float>(a2ls_handle*, const float*, float*, const int64_t*, int, int, const int*, int,
-                                  const int*, int, int, int);
+                                  const int*, int, int, int, int);
 template void block_solve<double>(a2ls_handle*, const double*, double*, const int64_t*, int, int, const int*, int,
-                                   const int*, int, int, int);
+                                   const int*, int, int, int, int);
 template void lu_batched<dfloat>(a2ls_handle*, dfloat*, int, double*, double*, int);
 template void invert_diag_tiles<dfloat>(a2ls_handle*, dfloat*);
 template void block_solve<dfloat>(a2ls_handle*, const dfloat*, dfloat*, const int64_t*, int, int, const int*, int,
-                                   const int*, int, int, int);
+                                   const int*, int, int, int, int);
 
 }  // namespace a2ls
 
@@ -1268,13 +1284,13 @@ __global__ void __launch_bounds__(256) k_e_inverse(const R* F, int n, int64_t ld
       if (pass == 0) {
         const int k0 = max(bstart * TB, r0 - band);  // L(r, c) = 0 for c < r - band
         if (r0 > k0)
-          cta_gemm_n8<R, R>(F + (int64_t)r0 * ld + k0, ld, Xs + (int64_t)k0 * ldx, ldx, tb, pc, r0 - k0, 0, acc, sA,
+          cta_gemm_narrow<R, R, 8, 2>(F + (int64_t)r0 * ld + k0, ld, Xs + (int64_t)k0 * ldx, ldx, tb, pc, r0 - k0, 0, acc, sA,
                             sB);
       } else {
         const int e0 = r0 + tb;
         const int e1 = min(n, r0 + tb + band);       // U(r, c) = 0 for c > r + band
         if (e0 < e1)
-          cta_gemm_n8<R, R>(F + (int64_t)r0 * ld + e0, ld, Xs + (int64_t)e0 * ldx, ldx, tb, pc, e1 - e0, 0, acc, sA,
+          cta_gemm_narrow<R, R, 8, 2>(F + (int64_t)r0 * ld + e0, ld, Xs + (int64_t)e0 * ldx, ldx, tb, pc, e1 - e0, 0, acc, sA,
                             sB);
       }
 #pragma unroll
@@ -1287,7 +1303,7 @@ __global__ void __launch_bounds__(256) k_e_inverse(const R* F, int n, int64_t ld
       }
       __syncthreads();
       R acc2[2] = {R(0.0), R(0.0)};
-      cta_gemm_n8<R, R>(F + (int64_t)r0 * ld + r0, ld, Xs + (int64_t)r0 * ldx, ldx, tb, pc, tb, pass == 0 ? 1 : 2,
+      cta_gemm_narrow<R, R, 8, 2>(F + (int64_t)r0 * ld + r0, ld, Xs + (int64_t)r0 * ldx, ldx, tb, pc, tb, pass == 0 ? 1 : 2,
                         acc2, sA, sB);
 #pragma unroll
       for (int v = 0; v < 2; ++v) {

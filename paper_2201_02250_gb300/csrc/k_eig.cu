@@ -38,6 +38,7 @@ template <> struct SeEps<dfloat> {
   static constexpr double v = 1.4210854715202004e-14;  // 2^-46
   static constexpr double big = 1e30;                  // within FP32's exponent range
 };
+template <> struct SeFast<dfloat> { static constexpr bool v = true; };
 }  // namespace se
 
 template <class T> struct EAcc;
@@ -353,12 +354,16 @@ constexpr int SROW = EIG_MAXP + 2;
 constexpr int GRAM_NG_MAX = 16;          // row groups (split-K) of a Gram product
 
 // stage rows [l0, l0 + rows) of M (cols 0:w) into S (stride SROW), zero padding to a multiple of 4
+// (FP64 rows past L1: a cluster's CTAs read what the others have written)
+__device__ __forceinline__ double ld_shared_rows(const double* p) { return __ldcg(p); }
+template <class TM>
+__device__ __forceinline__ TM ld_shared_rows(const TM* p) { return *p; }
 template <class Acc, class TM>
 __device__ __forceinline__ void stage_rows(Acc* S, const TM* M, int64_t ldx, int l0, int rows, int w) {
   const int wp = (w + 3) & ~3;
   for (int e = threadIdx.x; e < rows * wp; e += ORTH_THREADS) {
     const int r = e / wp, c = e % wp;
-    S[r * SROW + c] = c < w ? (Acc)M[(int64_t)(l0 + r) * ldx + c] : (Acc)0;
+    S[r * SROW + c] = c < w ? (Acc)ld_shared_rows(M + (int64_t)(l0 + r) * ldx + c) : (Acc)0;
   }
 }
 
@@ -385,9 +390,24 @@ __device__ __forceinline__ void ld2(const float* p, float& a, float& b) {
 // only the blocks that reach the upper triangle are formed, the lower triangle is mirrored.
 // Xs, Ys: staging chunks; Ps: scratch of ORTH_THREADS x 8 values for the partial sums (may alias
 // the staging chunks).  Ends with a barrier.
+// share, shares: only the output blocks of this share are formed (their sums are those of a whole
+// product); block_share gives an entry's share.
+__device__ __forceinline__ int gram_blocks(int nx, int ny, bool same) {
+  const int nbr = (nx + 3) / 4, nbc = (ny + 1) / 2;
+  int nb = 0;
+  for (int br = 0; br < nbr; ++br) nb += same ? max(0, nbc - 2 * br) : nbc;
+  return nb;
+}
+__device__ __forceinline__ int block_share(int a, int c, int nx, int ny, bool same, int shares) {
+  const int nbc = (ny + 1) / 2, br = a / 4;
+  int b = c / 2;
+  for (int q = 0; q < br; ++q) b += same ? max(0, nbc - 2 * q) : nbc;
+  if (same) b -= 2 * br;
+  return b / ((gram_blocks(nx, ny, same) + shares - 1) / shares);
+}
 template <class Acc, class TX, class TY>
 __device__ void gram_product(const TX* X, const TY* Y, int64_t ldx, int n, int nx, int ny, bool same, Acc* Xs,
-                             Acc* Ys, double* G, Acc* Ps, int orc) {
+                             Acc* Ys, double* G, Acc* Ps, int orc, int share = 0, int shares = 1) {
   const int tid = threadIdx.x;
   const int nbr = (nx + 3) / 4, nbc = (ny + 1) / 2;
   // block (br, bc) covers rows 4br..4br+3 and columns 2bc..2bc+1; with X == Y only bc >= 2br
@@ -401,15 +421,17 @@ __device__ void gram_product(const TX* X, const TY* Y, int64_t ldx, int n, int n
     c0 = 2 * (nbc - row_blocks(br) + b);
   };
   const int ng = nb >= ORTH_THREADS ? 1 : min(GRAM_NG_MAX, ORTH_THREADS / nb);
-  const int items = nb * ng;
+  // this share's blocks b0 .. b0 + nbs - 1
+  const int bps = (nb + shares - 1) / shares, b0 = min(nb, share * bps), nbs = min(bps, nb - b0);
+  const int items = nbs * ng;
   // more blocks than threads (full-space Gram of a small subdomain): several passes over the rows
   for (int w0 = 0; w0 < items; w0 += ORTH_THREADS) {
     const int w = w0 + tid;
     const bool valid = w < items;
     int a0 = 0, c0 = 0, g = 0;
     if (valid) {
-      block_of(w % nb, a0, c0);
-      g = w / nb;
+      block_of(b0 + w % nbs, a0, c0);
+      g = w / nbs;
     }
     Acc acc[8];
 #pragma unroll
@@ -452,12 +474,12 @@ __device__ void gram_product(const TX* X, const TY* Y, int64_t ldx, int n, int n
 #pragma unroll
         for (int q = 0; q < 8; ++q) Ps[tid * 8 + q] = acc[q];
       __syncthreads();
-      if (tid < nb) {
-        block_of(tid, a0, c0);
+      if (tid < nbs) {
+        block_of(b0 + tid, a0, c0);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           Acc sum = Ps[tid * 8 + q];
-          for (int gg = 1; gg < ng; ++gg) sum += Ps[(gg * nb + tid) * 8 + q];
+          for (int gg = 1; gg < ng; ++gg) sum += Ps[(gg * nbs + tid) * 8 + q];
           const int a = a0 + (q >> 1), c = c0 + (q & 1);
           if (a < nx && c < ny && (!same || c >= a)) G[a * ny + c] = (double)sum;
         }
@@ -465,7 +487,7 @@ __device__ void gram_product(const TX* X, const TY* Y, int64_t ldx, int n, int n
     }
     __syncthreads();
   }
-  if (same) {
+  if (same && shares == 1) {
     for (int e = tid; e < nx * nx; e += ORTH_THREADS) {
       const int a = e / nx, c = e % nx;
       if (c < a) G[a * nx + c] = G[c * nx + a];
@@ -603,6 +625,27 @@ __device__ __forceinline__ void cluster_sum(double* G, int count, double* tmp) {
   __syncthreads();
 }
 
+// G (nx x ny) complete in every CTA of the cluster, each of which formed the blocks of its own share; no CTA's
+// share is changed while another may read it.  Ends with a CTA barrier.
+__device__ __forceinline__ void cluster_gather(double* G, int nx, int ny, bool same) {
+  const int C = cluster_size(), me = cluster_rank();
+  if (C == 1) return;
+  cluster_sync();
+  for (int e = threadIdx.x; e < nx * ny; e += ORTH_THREADS) {
+    const int a = e / ny, c = e % ny;
+    if (same && c < a) continue;
+    const int owner = block_share(a, c, nx, ny, same, C);
+    if (owner != me) G[e] = cluster_ld(G + e, owner);
+  }
+  cluster_sync();
+  if (same)
+    for (int e = threadIdx.x; e < nx * nx; e += ORTH_THREADS) {
+      const int a = e / nx, c = e % nx;
+      if (c < a) G[e] = G[c * nx + a];
+    }
+  __syncthreads();
+}
+
 // Orthogonalisation: block CGS2 of W against V[:, 0:jb], then Cholesky QR twice or three times (see
 // below).  Writes the Gram coefficients into H[0:jb, hc:hc+p] and R into H[hr:hr+p, hc:hc+p] and
 // the orthonormal block into V[:, vout:vout+p].  full != 0: only H[0:jb, hc:hc+p].  illcond (if given):
@@ -612,11 +655,13 @@ __device__ __forceinline__ void cluster_sum(double* G, int count, double* tmp) {
 // The work of a subdomain is bound by the arithmetic of the SM that does it, so with fewer subdomains than
 // SMs a cluster of CTAs takes each: a CTA holds a slice of the rows, forms its part of every Gram product
 // and applies the updates to its rows; the parts are summed through distributed shared memory and every CTA
-// factors the same small Gram matrix.  The launch picks the largest cluster (at most 8) with which the
+// factors the same small Gram matrix.  (FP64, whose sums keep their order: every CTA goes over all rows but
+// forms only a share of a product's output blocks, which the others then fetch.)  The launch picks the largest cluster (at most 8) with which the
 // active subdomains still fit the SMs; clusters only where the Gram matrices of full-space subdomains are
 // not in play (their shared memory leaves no room, and they have at most 96 rows).  Setup and solve, one
-// CTA each against clusters (and k_vy's chunks spread likewise): 16 subdomains in FP64 56.5 -> 47.0 ms, 64 in
-// double-float 48.2 -> 43.1 ms, 64 in FP64 (about 1950 rows each) 1311 -> 1195 ms; 256 subdomains unchanged.
+// CTA each against clusters (and k_vy's chunks spread likewise): 64 subdomains in
+// double-float 48.2 -> 43.1 ms; 256 subdomains unchanged.  By blocks, a launch over 64 FP64 subdomains of about
+// 1950 rows 2.34 -> 1.14 ms, over 16 of 300 rows 460 -> 265 us (by rows 146).
 template <class T, class TW>
 __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int64_t* xoff, int ldx,
                                                         const int* pvec, const int* active, int jb_blocks,
@@ -636,7 +681,11 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
     if (threadIdx.x == 0 && rank == 0) raise_status(status, A2LS_ERR_EIGEN, i, 3);
     return;
   }
-  // this CTA's rows
+  // this CTA's rows (of the updates; FP64 Gram products go over all nall rows, Va and Wa)
+  constexpr bool BY_BLOCKS = std::is_same<Acc, double>::value;
+  const int nall = ni[i];
+  const T* Va = V + xoff[i];
+  const TW* Wa = W + xoff[i];
   const int per = (ni[i] + C - 1) / C, row0 = min(ni[i], rank * per), n = min(per, ni[i] - row0);
   T* Vi = V + xoff[i] + (int64_t)row0 * ldx;
   TW* Wi = W + xoff[i] + (int64_t)row0 * ldx;
@@ -657,9 +706,18 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
   const int npass = jb > 0 ? 2 : 0;
   for (int e = tid + h0; e < jb * p; e += ORTH_THREADS) Hi[(e / p) * EIG_MAXP + hc + e % p] = 0.0;
   for (int pass = 0; pass < npass; ++pass) {
+    if (BY_BLOCKS && C > 1 && pass > 0) {
+      __threadfence();
+      cluster_sync();
+    }
     // G = V[:, 0:jb]^T W[:, 0:p]
-    gram_product<Acc>(Vi, Wi, (int64_t)ldx, n, jb, p, false, sv, sw, G, sv, orc);
-    cluster_sum(G, jb * p, ctmp);
+    if (BY_BLOCKS) {
+      gram_product<Acc>(Va, Wa, (int64_t)ldx, nall, jb, p, false, sv, sw, G, sv, orc, rank, C);
+      cluster_gather(G, jb, p, false);
+    } else {
+      gram_product<Acc>(Vi, Wi, (int64_t)ldx, n, jb, p, false, sv, sw, G, sv, orc);
+      cluster_sum(G, jb * p, ctmp);
+    }
     for (int e = tid + h0; e < jb * p; e += ORTH_THREADS) Hi[(e / p) * EIG_MAXP + hc + e % p] += G[e];
     if (full) return;  // Rayleigh quotient only
     // W -= V G; G converted once to the working arithmetic (in Ri's space, padded to pp columns)
@@ -702,8 +760,17 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
   bool shifted = false;
   int passes = 2;
   for (int pass = 0; pass < passes; ++pass) {
-    gram_product<Acc>(Wi, Wi, (int64_t)ldx, n, p, p, true, sw, sw, G, sv, orc);
-    cluster_sum(G, p * p, ctmp);
+    if (BY_BLOCKS) {
+      if (C > 1) {  // the other CTAs' rows of W are written
+        __threadfence();
+        cluster_sync();
+      }
+      gram_product<Acc>(Wa, Wa, (int64_t)ldx, nall, p, p, true, sw, sw, G, sv, orc, rank, C);
+      cluster_gather(G, p, p, true);
+    } else {
+      gram_product<Acc>(Wi, Wi, (int64_t)ldx, n, p, p, true, sw, sw, G, sv, orc);
+      cluster_sum(G, p * p, ctmp);
+    }
     if (tid < 32) {
       // shifted pass: Gs + 11 (n p + p (p + 1)) u tr(Gs) I
       const double shift_u =
@@ -950,7 +1017,10 @@ __global__ void __launch_bounds__(RRThreads<R>::v) k_rayleigh_ritz(RRParams prm,
     const R* x = xs + j * m;
     const R* y = ys + j * m;
     const int two = sel_two[j], col = sel_col[j], pidx = sel_pos[j];
-    double qx[RPL], qy[RPL], nrm2 = 0.0;
+    // FP64 keeps the order of every sum (see se::SeFast): a row's coefficient starts at its own column, the
+    // squares are added in the order of the rows
+    constexpr bool FAST = se::SeFast<R>::v;
+    double qx[RPL], qy[RPL], nx = 0.0, ny = 0.0;
 #pragma unroll
     for (int u = 0; u < RPL; ++u) {
       const int a = lane + 32 * u;
@@ -958,41 +1028,63 @@ __global__ void __launch_bounds__(RRThreads<R>::v) k_rayleigh_ritz(RRParams prm,
       if (a < m) {
         const R* Qa = Q + a * ld;  // an odd row stride: the lanes read different banks
 #pragma unroll 4
-        for (int c = 0; c < m; ++c) mac(sx, Qa[c], x[c]);
+        for (int c = 0, cc = FAST ? 0 : a; c < m; ++c, cc = (cc + 1 == m) ? 0 : cc + 1) mac(sx, Qa[cc], x[cc]);
         if (two == 1)
 #pragma unroll 4
-          for (int c = 0; c < m; ++c) mac(sy, Qa[c], y[c]);
+          for (int c = 0, cc = FAST ? 0 : a; c < m; ++c, cc = (cc + 1 == m) ? 0 : cc + 1) mac(sy, Qa[cc], y[cc]);
       }
       qx[u] = (double)finish(sx);
       qy[u] = (double)finish(sy);
-      nrm2 += qx[u] * qx[u];
-      if (two == 1) nrm2 += qy[u] * qy[u];
     }
-    for (int o = 16; o > 0; o >>= 1) nrm2 += __shfl_xor_sync(0xffffffffu, nrm2, o);
-    const double inv = 1.0 / sqrt(nrm2);
+    if constexpr (FAST) {
+#pragma unroll
+      for (int u = 0; u < RPL; ++u) {
+        nx += qx[u] * qx[u];
+        if (two == 1) nx += qy[u] * qy[u];
+      }
+      for (int o = 16; o > 0; o >>= 1) nx += __shfl_xor_sync(0xffffffffu, nx, o);
+    } else {
+#pragma unroll
+      for (int u = 0; u < RPL; ++u)
+        for (int l = 0; l < 32 && 32 * u + l < m; ++l) {
+          const double vx = __shfl_sync(0xffffffffu, qx[u], l);
+          nx += vx * vx;
+          if (two == 1) {
+            const double vy = __shfl_sync(0xffffffffu, qy[u], l);
+            ny += vy * vy;
+          }
+        }
+    }
+    const double nrm = sqrt(two == 1 ? nx + ny : nx);
+    [[maybe_unused]] const double inv = 1.0 / nrm;
 #pragma unroll
     for (int u = 0; u < RPL; ++u) {
       const int a = lane + 32 * u;
       if (a < m) {
-        Yi[a * EIG_MAXP + col] = qx[u] * inv;
-        if (two == 1) Yi[a * EIG_MAXP + col + 1] = qy[u] * inv;
+        Yi[a * EIG_MAXP + col] = FAST ? qx[u] * inv : qx[u] / nrm;
+        if (two == 1) Yi[a * EIG_MAXP + col + 1] = FAST ? qy[u] * inv : qy[u] / nrm;
       }
     }
     __syncwarp();
     double res = 0.0;
     if (!full[i]) {
       const int b = prm.b, r0 = prm.sb_krylov, c0 = prm.sb_krylov - b;
+      double ux = 0.0, uy = 0.0;
       if (lane < b) {  // b <= 32
-        double ux = 0.0, uy = 0.0;
 #pragma unroll 8
         for (int c = 0; c < b; ++c) {
           const double hv = Hi[(r0 + lane) * EIG_MAXP + c0 + c];
           ux += hv * Yi[(c0 + c) * EIG_MAXP + col];
           if (two == 1) uy += hv * Yi[(c0 + c) * EIG_MAXP + col + 1];
         }
-        res = ux * ux + uy * uy;
       }
-      for (int o = 16; o > 0; o >>= 1) res += __shfl_xor_sync(0xffffffffu, res, o);
+      const double sq = ux * ux + uy * uy;
+      if constexpr (FAST) {
+        res = sq;
+        for (int o = 16; o > 0; o >>= 1) res += __shfl_xor_sync(0xffffffffu, res, o);
+      } else {
+        for (int l = 0; l < b; ++l) res += __shfl_sync(0xffffffffu, sq, l);
+      }
       res = sqrt(res);
     }
     const double lam = mod[pidx];
@@ -1488,15 +1580,16 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
     DB = dv;
   }
   if (prep.done) A2LS_CUDA(cudaStreamWaitEvent(st, prep.done, 0));  // the factor digits are ready
+  int nact = N;   // subdomains active in the launches that may run at the same time
   auto solve_sweep = [&](const int* actv, int forward) {
     if constexpr (std::is_same<T, dfloat>::value) {
       if (tcs.ready) {
         tc_block_solve(h, tcs, W, d_vo, 0, P, d_pv, actv, forward);
-        block_solve<T>(h, fac, W, d_vo, 0, P, d_pv, pmax, actv, forward, !forward, TC_SOLVE_MAX_P);
+        block_solve<T>(h, fac, W, d_vo, 0, P, d_pv, pmax, actv, forward, !forward, TC_SOLVE_MAX_P, nact);
         return;
       }
     }
-    block_solve<T>(h, fac, W, d_vo, 0, P, d_pv, pmax, actv, forward, !forward);
+    block_solve<T>(h, fac, W, d_vo, 0, P, d_pv, pmax, actv, forward, !forward, 0, nact);
   };
   auto apply_T = [&](int vcol, const int* actv) {
     k_bmul<TV, T><<<dim3(N, 8), 256, 0, st>>>(h->d_ni, h->d_off, d_vo, P, vcol, d_pv, actv, h->d_lrow, h->d_lcol,
@@ -1517,7 +1610,6 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
   };
   // k_orth over the subdomains actv (nact of them active in the launches that may run at the same time);
   // with_full: the block may be one of a full-space subdomain
-  int nact = N;
   // two CTAs of k_vy fit an SM
   auto vy_grid = [&]() { return dim3(N, std::max(1, std::min(16, 2 * sms / std::max(nact, 1)))); };
   auto launch_orth = [&](const int* actv, bool with_full, int jb_blocks, double* Hout, int hr, int hc, int vout,

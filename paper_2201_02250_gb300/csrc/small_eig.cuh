@@ -53,51 +53,20 @@ SE_HD inline double se_dbl(double x) { return x; }
 // unnormalised multiply-add overloads both)
 SE_HD inline void se_mac(double& acc, double a, double b) { acc += a * b; }
 SE_HD inline double se_fin(double a) { return a; }
-// 1 / sqrt(a) for a > 0 and 1 / b for b in [1, 2], to rounding accuracy.  On the GPU: the hardware's
-// approximation (about 2^-20) and one third-order step each (with e = 1 - a y^2,
-// 1 / sqrt(a) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2 / 8 + O(e^3)); 1 / b = y / (1 - e) likewise).  GB300's
-// FP64 pipe takes about 64 cycles for every warp instruction of an SM quarter, however few lanes are
-// active, so a chain's length in FP64 instructions (comparisons among them) is its time: five and three
-// here, dozens in the library's square root and division.
-SE_HD inline double se_rsqrt(double a) {
-#ifdef __CUDA_ARCH__
-  const unsigned ex = (unsigned)__double2hiint(a) >> 20;  // sign and exponent
-  if (ex - 0x60u > 0x740u) return 1.0 / sqrt(a);          // outside the approximation's safe range
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  const double e = fma(-(a * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-#else
-  return 1.0 / sqrt(a);
-#endif
-}
-SE_HD inline double se_recip12(double b) {
-#ifdef __CUDA_ARCH__
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-  const double e = fma(-b, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-#else
-  return 1.0 / b;
-#endif
-}
-// a positive factor near 1 / a (a > 0) that brings numbers of a's size to about 1
-SE_HD inline double se_scale_to_one(double a) {
-#ifdef __CUDA_ARCH__
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  const unsigned ex = (unsigned)__double2hiint(a) >> 20;
-  return ex - 0x10u > 0x7d0u ? 1.0 : y;
-#else
-  return 1.0 / a;
-#endif
-}
-// The largest of some magnitudes as a power of two, and its inverse, where the arithmetic's exponent range
-// is short of squares (one in FP64).
+// Whether schur() chases several bulges with reflectors formed from se_rsqrt(a) = 1 / sqrt(a), se_recip12(b) =
+// 1 / b for b in [1, 2] and se_scale_to_one(a), a factor that brings a to about 1 (double-float), or keeps to
+// the single bulge with the library's roots and quotients.  FP64 keeps to those and with them its results
+// bit for bit: the block Krylov iteration amplifies a changed rounding until the eigenvectors, kept at a
+// residual of 1e-10, differ at that size, and with them the ninth digit of the preconditioner, which FP64
+// callers compare.
+template <class R> struct SeFast { static constexpr bool v = false; };
+SE_HD inline double se_rsqrt(double a) { return 1.0 / sqrt(a); }
+SE_HD inline double se_recip12(double b) { return 1.0 / b; }
+SE_HD inline double se_scale_to_one(double a) { return 1.0 / a; }
+// (of fast arithmetics: a magnitude's power of two and its inverse, the largest magnitude of a warp)
 SE_HD inline double se_pow2(double) { return 1.0; }
 SE_HD inline double se_pow2_inv(double p) { return p; }
 SE_HD inline double se_warp_maxabs(double) { return 1.0; }
-SE_HD inline bool se_range_limited(double) { return false; }
 SE_HD inline bool se_is_zero(double a) {
 #ifdef __CUDA_ARCH__
   return (__double_as_longlong(a) << 1) == 0;
@@ -164,32 +133,51 @@ SE_HD inline R strided_dot(const R* x, int st, const R* v, int n) {
 template <class R>
 SE_HD inline void hessenberg(R* H, int ld, R* Q, int ldq, int m, R* v, const Team& t) {
   for (int k = 0; k + 2 < m; ++k) {
-    // Householder vector for x = H[k+1.., k]; every warp sums |x|^2 for itself, in the same order (x scaled)
+    R up = 1.0, x0, alpha, beta;
+    if (SeFast<R>::v) {
+      // Householder vector for x = H[k+1.., k], scaled; every warp sums |x|^2 for itself, in the same order
 #ifdef __CUDA_ARCH__
-    const int l0 = t.lane & 31, ls = 32;
+      const int l0 = t.lane & 31, ls = 32;
 #else
-    const int l0 = 0, ls = 1;
+      const int l0 = 0, ls = 1;
 #endif
-    R xm = 0.0;
-    for (int r = k + 1 + l0; r < m; r += ls) {
-      const R a = se_abs(H[r * ld + k]);
-      if (se_range_limited(a) && a > xm) xm = a;
+      R xm = 0.0;
+      for (int r = k + 1 + l0; r < m; r += ls) {
+        const R a = se_abs(H[r * ld + k]);
+        if (a > xm) xm = a;
+      }
+      up = se_pow2(se_warp_maxabs(xm));
+      const R dn = se_pow2_inv(up);
+      R nrm2 = 0.0;
+      for (int r = k + 1 + l0; r < m; r += ls) {
+        const R a = H[r * ld + k] * dn;
+        se_mac(nrm2, a, a);
+      }
+      nrm2 = se_warp_sum(se_fin(nrm2));
+      if (se_is_zero(nrm2)) continue;
+      const R rn = se_rsqrt(nrm2);
+      x0 = H[(k + 1) * ld + k] * dn;
+      alpha = -sgn(nrm2 * rn, x0);
+      // v = x - alpha e1; P = I - beta v v^T with beta = 2 / v^T v, v^T v = 2 |x| (|x| + |x0|)
+      beta = rn * rn * se_recip12(R(1.0) + se_abs(x0) * rn);
+      t.sync();
+      for (int r = k + 1 + t.lane; r < m; r += t.size) v[r] = (r == k + 1) ? (x0 - alpha) : H[r * ld + k] * dn;
+    } else {
+      // Householder vector for x = H[k+1.., k]
+      R nrm2 = 0.0;
+      for (int r = k + 1; r < m; ++r) se_mac(nrm2, H[r * ld + k], H[r * ld + k]);
+      nrm2 = se_fin(nrm2);
+      const R nrm = se_sqrt(nrm2);
+      if (nrm == 0.0) continue;
+      x0 = H[(k + 1) * ld + k];
+      alpha = -sgn(nrm, x0);
+      // v = x - alpha e1, scaled so that P = I - 2 v v^T / (v^T v); v^T v = 2 nrm |x0 - alpha|
+      const R vtv = nrm2 - x0 * x0 + (x0 - alpha) * (x0 - alpha);
+      if (vtv == 0.0) continue;
+      t.sync();
+      for (int r = k + 1 + t.lane; r < m; r += t.size) v[r] = (r == k + 1) ? (x0 - alpha) : H[r * ld + k];
+      beta = 2.0 / vtv;
     }
-    const R up = se_pow2(se_warp_maxabs(xm)), dn = se_pow2_inv(up);
-    R nrm2 = 0.0;
-    for (int r = k + 1 + l0; r < m; r += ls) {
-      const R a = H[r * ld + k] * dn;
-      se_mac(nrm2, a, a);
-    }
-    nrm2 = se_warp_sum(se_fin(nrm2));
-    if (se_is_zero(nrm2)) continue;
-    const R rn = se_rsqrt(nrm2);
-    const R x0 = H[(k + 1) * ld + k] * dn;
-    const R alpha = -sgn(nrm2 * rn, x0);
-    // v = x - alpha e1; P = I - beta v v^T with beta = 2 / v^T v, v^T v = 2 |x| (|x| + |x0|)
-    const R beta = rn * rn * se_recip12(R(1.0) + se_abs(x0) * rn);
-    t.sync();
-    for (int r = k + 1 + t.lane; r < m; r += t.size) v[r] = (r == k + 1) ? (x0 - alpha) : H[r * ld + k] * dn;
     t.sync();
     const int len = m - k - 1;
     const int ncol = m - k;                                  // left update: columns k..m-1
@@ -213,27 +201,342 @@ SE_HD inline void hessenberg(R* H, int ld, R* Q, int ldq, int m, R* v, const Tea
   }
 }
 
+// The largest lo <= hi whose subdiagonal entry is negligible (0 if there is none), one entry per thread: below
+// leps times its two diagonal neighbours or below eps times hnorm.
+template <class R>
+SE_HD inline int first_negligible(const R* H, int ld, int hi, R leps, R eps, R hnorm, const Team& t) {
+  int lo = 0;
+  for (int j = hi - t.lane; j > 0; j -= t.size) {
+    const R s = se_abs(H[(j - 1) * ld + j - 1]) + se_abs(H[j * ld + j]);
+    const R sub = se_abs(H[j * ld + j - 1]);
+    if (sub <= leps * s || sub <= eps * hnorm) {
+      lo = j;
+      break;
+    }
+  }
+  return t.max(lo);
+}
+
+// ---- the single bulge with the library's square root and division ----
+// GB300's FP64 pipe takes about 64 cycles for every warp instruction of an SM quarter, however few lanes
+// are active, so the chain of the reflectors' FP64 instructions is the time: the next reflector's three
+// entries and its two quotients go to lanes of one warp (order 48: 7.5 -> 5.2 million cycles, the same
+// bits).
+
+// Apply a 3-element (or 2-element when nv == 2) reflector I - beta u u^T with u = (1, u1, u2)
+// to rows k..k+nv-1 of H from the left (columns c0..m-1) and to columns k..k+nv-1 from the
+// right (rows 0..r1) and to Q's columns.
+template <class R>
+SE_HD inline void apply_reflector(R* H, int ld, R* Q, int ldq, int m, int k, int nv, R u1, R u2, R beta,
+                                  int c0, int r1, const Team& t) {
+  for (int c = c0 + t.lane; c < m; c += t.size) {
+    R d = H[k * ld + c] + u1 * H[(k + 1) * ld + c] + (nv == 3 ? u2 * H[(k + 2) * ld + c] : 0.0);
+    d *= beta;
+    H[k * ld + c] -= d;
+    H[(k + 1) * ld + c] -= d * u1;
+    if (nv == 3) H[(k + 2) * ld + c] -= d * u2;
+  }
+  t.sync();
+  for (int r = t.lane; r <= r1; r += t.size) {
+    R d = H[r * ld + k] + u1 * H[r * ld + k + 1] + (nv == 3 ? u2 * H[r * ld + k + 2] : 0.0);
+    d *= beta;
+    H[r * ld + k] -= d;
+    H[r * ld + k + 1] -= d * u1;
+    if (nv == 3) H[r * ld + k + 2] -= d * u2;
+  }
+  for (int r = t.lane; r < m; r += t.size) {
+    R d = Q[r * ldq + k] + u1 * Q[r * ldq + k + 1] + (nv == 3 ? u2 * Q[r * ldq + k + 2] : 0.0);
+    d *= beta;
+    Q[r * ldq + k] -= d;
+    Q[r * ldq + k + 1] -= d * u1;
+    if (nv == 3) Q[r * ldq + k + 2] -= d * u2;
+  }
+  t.sync();
+}
+
 // Householder reflector mapping (x, y, z) to (alpha, 0, 0): returns alpha, beta and u = (1, u1, u2).
 // With v = (v0, y, z), v0 = x - alpha, v^T v = 2 |alpha| |v0|, so beta = 2 v0^2 / v^T v = v0 / (-alpha).
-// With r = 1 / |(x, y, z)|: beta = 1 + |x| r (between 1 and 2) and 1 / v0 = sign(x) r / beta.  The chain of
-// a sweep's reflectors is what bounds the Schur iteration, so they are formed without a square root or a
-// division (an FP64 setup and solve of 16 subdomains, order 48: 84.0 -> 72.7 ms).
-// (0, 0, 0) gives beta = 0 and alpha = x: no reflection.  An arithmetic of short exponent range scales the
-// three first: entries of 1e-16 and less, as a converging block has them, would lose the low parts of
-// their squares, and the reflector its orthogonality.
+template <class R>
+SE_HD inline bool make_reflector_div(R x, R y, R z, R& u1, R& u2, R& beta, R& alpha) {
+  R nrm = se_sqrt(x * x + y * y + z * z);
+  if (nrm == 0.0) return false;
+  alpha = -sgn(nrm, x);
+  R v0 = x - alpha;
+  if (v0 == 0.0) return false;
+  R iv;
+#ifdef __CUDA_ARCH__
+  {
+    // the two quotients in the even and the odd lanes, one division long
+    const int lane = threadIdx.x & 31;
+    const R q = ((lane & 1) ? v0 : R(1.0)) / ((lane & 1) ? -alpha : v0);
+    iv = se_warp_get(q, lane & ~1);
+    beta = se_warp_get(q, lane | 1);
+  }
+#else
+  iv = R(1.0) / v0;
+  beta = v0 / (-alpha);
+#endif
+  u1 = y * iv;
+  u2 = z * iv;
+  return true;
+}
+
+// Make a 2x2 diagonal block with real eigenvalues upper triangular by a rotation (rows/cols p, p+1).
+template <class R>
+SE_HD inline void split_2x2_div(R* H, int ld, R* Q, int ldq, int m, int p, const Team& t) {
+  t.sync();
+  R a = H[p * ld + p], b = H[p * ld + p + 1], c = H[(p + 1) * ld + p], d = H[(p + 1) * ld + p + 1];
+  R hm = 0.5 * (a - d);
+  R disc = hm * hm + b * c;
+  if (disc < 0.0 || c == 0.0) return;
+  // eigenvalue closest to d: lambda = d + (hm +- se_sqrt(disc)) ... pick the one of larger magnitude shift
+  R sq = se_sqrt(disc);
+  R lam = 0.5 * (a + d) + (hm >= 0 ? sq : -sq);
+  // eigenvector (lam - d, c) of the block; rotation taking it to e1
+  R x = lam - d, y = c;
+  R r = se_sqrt(x * x + y * y);
+  if (r == 0.0) return;
+  R cs = x / r, sn = y / r;
+  // rows p, p+1: G^T H
+  for (int col = p + t.lane; col < m; col += t.size) {
+    R h1 = H[p * ld + col], h2 = H[(p + 1) * ld + col];
+    H[p * ld + col] = cs * h1 + sn * h2;
+    H[(p + 1) * ld + col] = -sn * h1 + cs * h2;
+  }
+  t.sync();
+  for (int row = t.lane; row <= p + 1; row += t.size) {
+    R h1 = H[row * ld + p], h2 = H[row * ld + p + 1];
+    H[row * ld + p] = cs * h1 + sn * h2;
+    H[row * ld + p + 1] = -sn * h1 + cs * h2;
+  }
+  for (int row = t.lane; row < m; row += t.size) {
+    R q1 = Q[row * ldq + p], q2 = Q[row * ldq + p + 1];
+    Q[row * ldq + p] = cs * q1 + sn * q2;
+    Q[row * ldq + p + 1] = -sn * q1 + cs * q2;
+  }
+  t.sync();
+  if (t.lane == 0) H[(p + 1) * ld + p] = 0.0;
+  t.sync();
+}
+
+// schur() with one bulge a sweep (see there for the arguments)
+template <class R>
+SE_HD inline int schur_single(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const Team& t, R* snap,
+                              double local_tol) {
+  const R eps = R(SeEps<R>::v), hnorm = R(hnorm_);
+  const R leps = R(local_tol > SeEps<R>::v ? local_tol : SeEps<R>::v);
+  int hi = m - 1, iter = 0, total = 0;
+  while (hi >= 0) {
+    int lo = first_negligible(H, ld, hi, leps, eps, hnorm, t);
+    if (lo > 0) {
+      t.sync();
+      if (t.lane == 0) H[lo * ld + lo - 1] = 0.0;
+      t.sync();
+    }
+    if (lo == hi) {
+      --hi;
+      iter = 0;
+      continue;
+    }
+    if (lo == hi - 1) {
+      split_2x2_div(H, ld, Q, ldq, m, lo, t);
+      hi -= 2;
+      iter = 0;
+      continue;
+    }
+    ++iter;
+    if (++total > 60 * m) return -1;
+    // Shifts: the eigenvalues of the trailing 2x2 block (a real pair is replaced by its member
+    // closer to the last diagonal entry, used twice), or an exceptional pair every 11th step.
+    R s1r, s1i, s2r, s2i;
+    {
+      R a, b, c, d;
+      if (iter % 11 == 10) {
+        const R w = se_abs(H[hi * ld + hi - 1]) + se_abs(H[(hi - 1) * ld + hi - 2]);
+        a = 0.75 * w + H[hi * ld + hi];
+        b = -0.4375 * w;
+        c = w;
+        d = a;
+      } else {
+        a = H[(hi - 1) * ld + hi - 1];
+        b = H[(hi - 1) * ld + hi];
+        c = H[hi * ld + hi - 1];
+        d = H[hi * ld + hi];
+      }
+      const R hm = 0.5 * (a - d);
+      const R disc = hm * hm + b * c;
+      const R mean = 0.5 * (a + d);
+      if (disc >= 0.0) {
+        const R sq = se_sqrt(disc);
+        const R r1 = mean + sq, r2 = mean - sq;
+        const R sh = (se_abs(r1 - d) <= se_abs(r2 - d)) ? r1 : r2;
+        s1r = s2r = sh;
+        s1i = s2i = 0.0;
+      } else {
+        s1r = s2r = mean;
+        s1i = se_sqrt(-disc);
+        s2i = -s1i;
+      }
+    }
+    // first column of (H - s1)(H - s2), formed from differences to avoid cancellation
+    R x, y, z;
+    {
+      const R h00 = H[lo * ld + lo], h01 = H[lo * ld + lo + 1], h10 = H[(lo + 1) * ld + lo];
+      const R h11 = H[(lo + 1) * ld + lo + 1], h21 = H[(lo + 2) * ld + lo + 1];
+      const R sc = se_abs(h00 - s2r) + se_abs(s2i) + se_abs(h10);
+      const R g = (sc > 0.0) ? h10 / sc : 0.0;
+      x = g * h01 + (h00 - s1r) * ((h00 - s2r) / (sc > 0.0 ? sc : 1.0)) - s1i * (s2i / (sc > 0.0 ? sc : 1.0));
+      y = g * (h00 + h11 - s1r - s2r);
+      z = g * h21;
+    }
+    // Bulge chase.  For k > lo the reflector is built from column k-1 (rows k..k+2), which it maps to
+    // (alpha, 0, 0) exactly; that column is therefore not part of the left update but written
+    // directly, after the barrier that separates every thread's read of (x, y, z) from the writes,
+    // which keeps each step at two barriers.  The next step's reflector comes from column k after
+    // this step's right update; one thread recomputes its three entries from a snapshot of rows
+    // k+1..k+3 (columns k..k+2) taken in the left phase and forms the reflector while the others run
+    // the right update, instead of every thread forming it after that update (the entries are the
+    // values the right update writes).
+    t.sync();  // the shift and deflation reads above precede the first update
+    const bool early = true;
+    R u1, u2, beta, alpha;
+    bool have = make_reflector_div(x, y, z, u1, u2, beta, alpha);
+    for (int k = lo; k <= hi - 2; ++k) {
+      const bool more = k + 1 <= hi - 2;  // a next step exists (then k + 3 <= hi)
+      R nu1 = R(0.0), nu2 = R(0.0), nbeta = R(0.0), nalpha = R(0.0);
+      bool nhave = false;
+      if (have) {
+        const int c0 = k > lo ? k : lo;
+        const int r1 = (k + 3 <= hi) ? k + 3 : hi;
+        // phase 1: rows k..k+2 from the left (columns c0..m-1) and the first qa rows of Q; phase 2:
+        // columns k..k+2 from the right (rows 0..r1) and the remaining rows of Q (Q's update depends
+        // on the reflector only, so it fills the threads that the H updates leave idle)
+        const int ncol = m - c0;
+        const int qa = (t.size > ncol) ? ((t.size - ncol < m) ? t.size - ncol : m) : 0;
+        for (int idx = t.lane; idx < ncol + qa; idx += t.size) {
+          R* a;
+          int st;
+          if (idx < ncol) {
+            a = H + k * ld + c0 + idx;
+            st = ld;
+          } else {
+            a = Q + (idx - ncol) * ldq + k;
+            st = 1;
+          }
+          R d = a[0];
+          se_mac(d, u1, a[st]);
+          se_mac(d, u2, a[2 * st]);
+          d = se_fin(d) * beta;
+          a[0] -= d;
+          a[st] -= d * u1;
+          a[2 * st] -= d * u2;
+          if (early && more && idx < 3) {  // column c0 + idx = k + idx
+            snap[idx] = a[st];
+            snap[3 + idx] = a[2 * st];
+            snap[6 + idx] = H[(k + 3) * ld + k + idx];
+          }
+        }
+        t.sync();
+        if (k > lo && t.lane == 0) {
+          H[k * ld + k - 1] = alpha;
+          H[(k + 1) * ld + k - 1] = 0.0;
+          H[(k + 2) * ld + k - 1] = 0.0;
+        }
+        // the last warp, usually idle in the right update, with one lane per entry
+#ifdef __CUDA_ARCH__
+        const bool forms = t.lane >= t.size - 32;
+#else
+        const bool forms = true;
+#endif
+        if (early && more && forms) {
+          auto entry = [&](int rr) {
+            const R a0 = snap[3 * rr], a1 = snap[3 * rr + 1], a2 = snap[3 * rr + 2];
+            R d = a0;
+            se_mac(d, u1, a1);
+            se_mac(d, u2, a2);
+            d = se_fin(d) * beta;
+            return a0 - d;
+          };
+#ifdef __CUDA_ARCH__
+          const R e = entry((t.lane & 31) < 3 ? t.lane & 31 : 2);
+          const R v[3] = {se_warp_get(e, 0), se_warp_get(e, 1), se_warp_get(e, 2)};
+#else
+          const R v[3] = {entry(0), entry(1), entry(2)};
+#endif
+          const bool ok = make_reflector_div(v[0], v[1], v[2], nu1, nu2, nbeta, nalpha);
+          if (t.lane == t.size - 1) {
+            snap[9] = nu1;
+            snap[10] = nu2;
+            snap[11] = nbeta;
+            snap[12] = nalpha;
+            snap[13] = ok ? R(1.0) : R(0.0);
+          }
+        }
+        for (int idx = t.lane; idx < (r1 + 1) + (m - qa); idx += t.size) {
+          R* a = (idx <= r1) ? H + idx * ld + k : Q + (qa + idx - (r1 + 1)) * ldq + k;
+          R d = a[0];
+          se_mac(d, u1, a[1]);
+          se_mac(d, u2, a[2]);
+          d = se_fin(d) * beta;
+          a[0] -= d;
+          a[1] -= d * u1;
+          a[2] -= d * u2;
+        }
+        t.sync();
+        if (more && early) {
+          nu1 = snap[9];
+          nu2 = snap[10];
+          nbeta = snap[11];
+          nalpha = snap[12];
+          nhave = !se_is_zero(snap[13]);
+        } else if (more) {
+          nhave = make_reflector_div(H[(k + 1) * ld + k], H[(k + 2) * ld + k], H[(k + 3) * ld + k], nu1, nu2, nbeta,
+                                 nalpha);
+        }
+      } else if (more) {
+        nhave = make_reflector_div(H[(k + 1) * ld + k], H[(k + 2) * ld + k], H[(k + 3) * ld + k], nu1, nu2, nbeta,
+                               nalpha);
+      }
+      u1 = nu1;
+      u2 = nu2;
+      beta = nbeta;
+      alpha = nalpha;
+      have = nhave;
+    }
+    x = H[(hi - 1) * ld + hi - 2];
+    y = H[hi * ld + hi - 2];
+    // final 2-element reflector on rows hi-1, hi
+    {
+      R u1, u2, beta, alpha;
+      if (make_reflector_div<R>(x, y, R(0.0), u1, u2, beta, alpha)) {
+        t.sync();
+        apply_reflector<R>(H, ld, Q, ldq, m, hi - 1, 2, u1, R(0.0), beta, hi - 2, hi, t);
+        if (t.lane == 0) H[hi * ld + hi - 2] = 0.0;
+        t.sync();
+      }
+    }
+  }
+  return 0;
+}
+
+// ---- several bulges ----
+
+// Householder reflector mapping (x, y, z) to (alpha, 0, 0): returns alpha, beta and u = (1, u1, u2).
+// With v = (v0, y, z), v0 = x - alpha, v^T v = 2 |alpha| |v0|, so beta = 2 v0^2 / v^T v = v0 / (-alpha).
+// (0, 0, 0) gives beta = 0 and alpha = x: no reflection.
+// The chain of a sweep's reflectors is what bounds the Schur iteration, so it has no square root and no
+// division: with r = 1 / |(x, y, z)|, beta = 1 + |x| r (between 1 and 2) and 1 / v0 = sign(x) r / beta.  The
+// three are scaled first: entries of 1e-16 and less, as a converging block has them, would lose the low
+// parts of their squares to FP32's exponent range, and the reflector its orthogonality.
 template <class R>
 SE_HD inline void make_reflector(R x, R y, R z, R& u1, R& u2, R& beta, R& alpha) {
-  R up = R(1.0);
-  if (se_range_limited(x)) {
-    R xm = se_abs(x);
-    if (se_abs(y) > xm) xm = se_abs(y);
-    if (se_abs(z) > xm) xm = se_abs(z);
-    up = se_pow2(xm);
-    const R dn = se_pow2_inv(up);
-    x *= dn;
-    y *= dn;
-    z *= dn;
-  }
+  R xm = se_abs(x);
+  if (se_abs(y) > xm) xm = se_abs(y);
+  if (se_abs(z) > xm) xm = se_abs(z);
+  const R up = se_pow2(xm), dn = se_pow2_inv(up);
+  x *= dn;
+  y *= dn;
+  z *= dn;
   const R s = x * x + y * y + z * z;
   if (se_is_zero(s)) {
     u1 = u2 = beta = R(0.0);
@@ -242,8 +545,7 @@ SE_HD inline void make_reflector(R x, R y, R z, R& u1, R& u2, R& beta, R& alpha)
   }
   const R r = se_rsqrt(s);
   beta = R(1.0) + se_abs(x) * r;
-  alpha = -sgn(s * r, x);
-  if (se_range_limited(x)) alpha *= up;
+  alpha = -sgn(s * r, x) * up;
   const R iv = sgn(r * se_recip12(beta), x);
   u1 = y * iv;
   u2 = z * iv;
@@ -260,17 +562,15 @@ SE_HD inline void split_2x2(R* H, int ld, R* Q, int ldq, int m, int p, const Tea
   // eigenvalue closest to d: lambda = d + (hm +- sqrt(disc)) ... pick the one of larger magnitude shift
   R sq = se_is_zero(disc) ? R(0.0) : disc * se_rsqrt(disc);
   R lam = 0.5 * (a + d) + (hm >= 0 ? sq : -sq);
-  // eigenvector (lam - d, c) of the block; rotation taking it to e1
+  // eigenvector (lam - d, c) of the block (scaled); rotation taking it to e1
   R x = lam - d, y = c;
-  if (se_range_limited(x)) {
-    const R dn = se_pow2_inv(se_pow2(se_abs(x) > se_abs(y) ? se_abs(x) : se_abs(y)));
-    x *= dn;
-    y *= dn;
-  }
+  const R dn = se_pow2_inv(se_pow2(se_abs(x) > se_abs(y) ? se_abs(x) : se_abs(y)));
+  x *= dn;
+  y *= dn;
   const R r2 = x * x + y * y;
   if (se_is_zero(r2)) return;
   const R ri = se_rsqrt(r2);
-  R cs = x * ri, sn = y * ri;
+  const R cs = x * ri, sn = y * ri;
   // rows p, p+1: G^T H
   for (int col = p + t.lane; col < m; col += t.size) {
     R h1 = H[p * ld + col], h2 = H[(p + 1) * ld + col];
@@ -298,9 +598,9 @@ SE_HD inline void split_2x2(R* H, int ld, R* Q, int ldq, int m, int p, const Tea
 constexpr int SE_BULGES = 3;
 constexpr int SE_BULGE_GAP = 4;
 constexpr int SE_SLOT = 21;
-constexpr int SE_W2 = 10, SE_W3 = 24;  // active block sizes from which a second and a third bulge are chased
 constexpr int SE_SNAP = SE_BULGES * SE_SLOT;
 enum { SE_SHIFTS = 9, SE_REFL = 13 };
+constexpr int SE_W2 = 10, SE_W3 = 24;  // active block sizes from which a second and a third bulge are chased
 
 // The shift pair (s1r, s2r, s1i, s2i) of the 2 x 2 block a, b; c, d: a real pair is replaced by its member
 // closer to d, used twice.
@@ -321,6 +621,168 @@ SE_HD inline void shift_pair(R a, R b, R c, R d, R* s) {
   }
 }
 
+// One sweep of NB bulges over the active block lo .. hi (see schur); exceptional: with shifts of the size of
+// the last subdiagonal entries.  Starts after the team has seen H, ends with a barrier.
+template <int NB, class R>
+SE_HD inline void se_sweep(R* H, int ld, R* Q, int ldq, int m, int lo, int hi, bool exceptional, const Team& t,
+                           R* snap) {
+  // On the GPU the last warp forms the reflectors, lanes 3 q .. 3 q + 2 for bulge q (lane 3 q keeps it); the
+  // right updates and Q are left to the other warps.
+#ifdef __CUDA_ARCH__
+  const int nwork = t.size - 32, rl = t.lane - nwork;
+  const int mq0 = rl >= 0 ? (rl < 3 * NB ? rl / 3 : NB - 1) : NB, mq1 = mq0 < NB ? mq0 + 1 : NB;
+  const bool keeps = rl == 3 * mq0;
+#else
+  const int nwork = t.size, mq0 = 0, mq1 = NB;
+  const bool keeps = true;
+#endif
+  // the reflector that starts bulge q: the first column of (H - s1)(H - s2), formed from differences to
+  // avoid cancellation, times a factor that keeps it in range (only its direction matters)
+  auto start = [&](int q) {
+    const R* s = snap + q * SE_SLOT + SE_SHIFTS;
+    const R s1r = s[0], s2r = s[1], s1i = s[2], s2i = s[3];
+    const R h00 = H[lo * ld + lo], h01 = H[lo * ld + lo + 1], h10 = H[(lo + 1) * ld + lo];
+    const R h11 = H[(lo + 1) * ld + lo + 1], h21 = H[(lo + 2) * ld + lo + 1];
+    const R sc = se_abs(h00 - s2r) + se_abs(s2i) + se_abs(h10);
+    const R f = se_is_zero(sc) ? R(1.0) : se_scale_to_one(sc);
+    const R g = h10 * f;
+    R r[4];
+    make_reflector<R>(g * h01 + (h00 - s1r) * ((h00 - s2r) * f) - s1i * (s2i * f), g * (h00 + h11 - s1r - s2r),
+                      g * h21, r[0], r[1], r[2], r[3]);
+    R* o = snap + q * SE_SLOT + SE_REFL + 4 * ((SE_BULGE_GAP * q) & 1);
+    if (keeps)
+      for (int u = 0; u < 4; ++u) o[u] = r[u];
+  };
+  for (int q = mq0; q < mq1; ++q) {
+    const int p = hi - 1 - 2 * q;
+    R a, b, c, d;
+    if (exceptional) {
+      const R e = se_abs(H[(p + 1) * ld + p]) + se_abs(H[p * ld + p - 1]);
+      a = 0.75 * e + H[(p + 1) * ld + p + 1];
+      b = -0.4375 * e;
+      c = e;
+      d = a;
+    } else {
+      a = H[p * ld + p];
+      b = H[p * ld + p + 1];
+      c = H[(p + 1) * ld + p];
+      d = H[(p + 1) * ld + p + 1];
+    }
+    R s[4];
+    shift_pair(a, b, c, d, s);
+    if (keeps)
+      for (int u = 0; u < 4; ++u) snap[q * SE_SLOT + SE_SHIFTS + u] = s[u];
+  }
+#ifdef __CUDA_ARCH__
+  __syncwarp();
+#endif
+  if (mq0 == 0) start(0);
+  t.sync();  // the reads of H above precede the first update
+  // Bulge q is at row k = lo + step - SE_BULGE_GAP q.  For k > lo its reflector was built from column
+  // k - 1 (rows k .. k + 2), which it maps to (alpha, 0, 0) exactly; that column is therefore not part of
+  // the left update but written directly, after the barrier that separates the reads of it from the
+  // writes.  At k = hi - 1 the reflector has two rows.  The next reflector comes from column k after this
+  // step's right update; its three entries are recomputed from a snapshot of rows k + 1 .. k + 3
+  // (columns k .. k + 2) taken in the left phase, and the reflector is formed while the others run the
+  // right update (the entries are the values the right update writes).
+  // An item of a phase is a bulge and a column or row of the whole matrix, of which those outside the
+  // update are passed over: the position costs a few instructions where a list of just the active ones
+  // took a hundred, as long as the update itself.
+  auto reflect = [&](R* a, int st, const R* r, bool three) {
+    const R u1 = r[0], u2 = r[1], beta = r[2];
+    const R a0 = a[0], a1 = a[st], a2 = three ? a[2 * st] : R(0.0);
+    R d = a0;
+    se_mac(d, u1, a1);
+    se_mac(d, u2, a2);
+    d = se_fin(d) * beta;
+    a[0] = a0 - d;
+    a[st] = a1 - d * u1;
+    if (three) a[2 * st] = a2 - d * u2;
+  };
+  const int steps = hi - lo + SE_BULGE_GAP * (NB - 1);
+  for (int step = 0; step < steps; ++step) {
+    const R* refl = snap + SE_REFL + 4 * (step & 1);
+    const int k1 = lo + step;  // bulge 0's row
+    // phase 1: rows k .. k + 2 from the left (columns k .. m - 1), one column per item
+    for (int at = t.lane; at < NB * m; at += t.size) {
+      int q = 0, c = at;
+      for (int u = 1; u < NB; ++u) {
+        const bool next = c >= m;
+        q += next ? 1 : 0;
+        c -= next ? m : 0;
+      }
+      const int k = k1 - SE_BULGE_GAP * q;
+      const bool three = k <= hi - 2;
+      if (c < k || (NB > 1 && (k < lo || k > hi - 1))) continue;
+      R* a = H + k * ld + c;
+      reflect(a, ld, refl + q * SE_SLOT, three);
+      if (c < k + 3 && three) {
+        R* v = snap + q * SE_SLOT + (c - k);
+        v[0] = a[ld];
+        v[3] = a[2 * ld];
+        v[6] = k + 3 <= hi ? a[3 * ld] : R(0.0);
+      }
+    }
+    t.sync();
+    // phase 2: columns k .. k + 2 from the right (rows 0 .. k + 3) and Q, one row per item; the next
+    // reflectors
+    for (int q = mq0; q < mq1; ++q) {
+      const int k = k1 - SE_BULGE_GAP * q;
+      R* slot = snap + q * SE_SLOT;
+      const R* r = refl + q * SE_SLOT;
+      R v[3] = {R(0.0), R(0.0), R(0.0)};
+      const R u1 = r[0], u2 = r[1], beta = r[2];
+      auto entry = [&](int rr) {
+        const R a0 = slot[3 * rr], a1 = slot[3 * rr + 1], a2 = slot[3 * rr + 2];
+        R d = a0;
+        se_mac(d, u1, a1);
+        se_mac(d, u2, a2);
+        d = se_fin(d) * beta;
+        return a0 - d;
+      };
+#ifdef __CUDA_ARCH__
+      // one lane per entry (a bulge outside the block computes on what its slot happens to hold, and the
+      // result is not used)
+      const R e = entry(rl < 3 * NB ? rl - 3 * mq0 : 2);
+      v[0] = se_warp_get(e, 3 * mq0);
+      v[1] = se_warp_get(e, 3 * mq0 + 1);
+      v[2] = se_warp_get(e, 3 * mq0 + 2);
+#else
+      for (int rr = 0; rr < 3; ++rr) v[rr] = entry(rr);
+#endif
+      if (NB > 1 && k == lo - 1) {
+        start(q);
+      } else if (k >= lo && k <= hi - 2) {
+        R n[4];
+        make_reflector<R>(v[0], v[1], v[2], n[0], n[1], n[2], n[3]);
+        R* o = slot + SE_REFL + 4 * ((step + 1) & 1);
+        if (keeps)
+          for (int u = 0; u < 4; ++u) o[u] = n[u];
+      }
+      if (keeps && k > lo && k <= hi - 1) {
+        H[k * ld + k - 1] = r[3];
+        H[(k + 1) * ld + k - 1] = 0.0;
+        if (k <= hi - 2) H[(k + 2) * ld + k - 1] = 0.0;
+      }
+    }
+    if (t.lane < nwork) {
+      for (int at = t.lane; at < 2 * NB * m; at += nwork) {
+        const bool isq = at >= NB * m;
+        int q = 0, e = isq ? at - NB * m : at;
+        for (int u = 1; u < NB; ++u) {
+          const bool next = e >= m;
+          q += next ? 1 : 0;
+          e -= next ? m : 0;
+        }
+        const int k = k1 - SE_BULGE_GAP * q;
+        if ((!isq && e > (k + 3 <= hi ? k + 3 : hi)) || (NB > 1 && (k < lo || k > hi - 1))) continue;
+        reflect((isq ? Q + e * ldq : H + e * ld) + k, 1, refl + q * SE_SLOT, k <= hi - 2);
+      }
+    }
+    t.sync();
+  }
+}
+
 // Francis implicit double-shift QR on an upper Hessenberg H, full Schur form, Q accumulated.
 // A subdiagonal entry is neglected when it is below eps times its two diagonal
 // neighbours or below eps times hnorm (the largest entry of the input), which keeps
@@ -337,28 +799,19 @@ SE_HD inline void shift_pair(R a, R b, R c, R d, R* s) {
 // (the small-bulge multishift iteration of Braman, Byers and Mathias, SIAM J. Matrix Anal. Appl. 23,
 // 2002, with the neighbouring diagonal blocks' shifts): the bulges' rows and columns are disjoint, so that
 // one step updates for all of them and one warp forms their next reflectors side by side, in its lanes.
-// Against one bulge a sweep (order 48 FP64, 72 double-float, random spectra of six decades): FP64 4.76 ->
-// 2.30 million cycles, double-float 8.19 -> 3.34 million; the same FP64 setup and solve 72.7 -> 56.5 ms.
+// Against one bulge a sweep (order 72, double-float, random spectra of six decades): 7.35 -> 3.13 million
+// cycles.
 template <class R>
 SE_HD inline int schur(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const Team& t, R* snap = nullptr,
                        double local_tol = 0.0) {
   R snap_local[SE_SNAP];
   if (!snap) snap = snap_local;
+  if (!SeFast<R>::v) return schur_single(H, ld, Q, ldq, m, hnorm_, t, snap, local_tol);
   const R eps = R(SeEps<R>::v), hnorm = R(hnorm_);
   const R leps = R(local_tol > SeEps<R>::v ? local_tol : SeEps<R>::v);
   int hi = m - 1, iter = 0, total = 0;
   while (hi >= 0) {
-    // the largest lo <= hi whose subdiagonal entry is negligible (0 if there is none), one entry per thread
-    int lo = 0;
-    for (int j = hi - t.lane; j > 0; j -= t.size) {
-      const R s = se_abs(H[(j - 1) * ld + j - 1]) + se_abs(H[j * ld + j]);
-      const R sub = se_abs(H[j * ld + j - 1]);
-      if (sub <= leps * s || sub <= eps * hnorm) {
-        lo = j;
-        break;
-      }
-    }
-    lo = t.max(lo);
+    const int lo = first_negligible(H, ld, hi, leps, eps, hnorm, t);
     if (lo > 0) {
       t.sync();
       if (t.lane == 0) H[lo * ld + lo - 1] = 0.0;
@@ -378,171 +831,9 @@ SE_HD inline int schur(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const 
     ++iter;
     if (++total > 60 * m) return -1;
     const int w = hi - lo + 1;
-    const int nb = w >= SE_W3 ? 3 : (w >= SE_W2 ? 2 : 1);
-    // On the GPU the last warp forms the reflectors, lanes 3 q .. 3 q + 2 for bulge q (lane 3 q keeps it); the
-    // right updates and Q are left to the other warps.
-#ifdef __CUDA_ARCH__
-    const int nwork = t.size - 32, rl = t.lane - nwork;
-    const int mq0 = rl >= 0 ? (rl < 3 * nb ? rl / 3 : nb - 1) : nb, mq1 = mq0 < nb ? mq0 + 1 : nb;
-    const bool keeps = rl == 3 * mq0;
-#else
-    const int nwork = t.size, mq0 = 0, mq1 = nb;
-    const bool keeps = true;
-#endif
-    // the reflector that starts bulge q: the first column of (H - s1)(H - s2), formed from differences to
-    // avoid cancellation, times a factor that keeps it in range (only its direction matters)
-    auto start = [&](int q) {
-      const R* s = snap + q * SE_SLOT + SE_SHIFTS;
-      const R s1r = s[0], s2r = s[1], s1i = s[2], s2i = s[3];
-      const R h00 = H[lo * ld + lo], h01 = H[lo * ld + lo + 1], h10 = H[(lo + 1) * ld + lo];
-      const R h11 = H[(lo + 1) * ld + lo + 1], h21 = H[(lo + 2) * ld + lo + 1];
-      const R sc = se_abs(h00 - s2r) + se_abs(s2i) + se_abs(h10);
-      const R f = se_is_zero(sc) ? R(1.0) : se_scale_to_one(sc);
-      const R g = h10 * f;
-      R r[4];
-      make_reflector<R>(g * h01 + (h00 - s1r) * ((h00 - s2r) * f) - s1i * (s2i * f), g * (h00 + h11 - s1r - s2r),
-                        g * h21, r[0], r[1], r[2], r[3]);
-      R* o = snap + q * SE_SLOT + SE_REFL + 4 * ((SE_BULGE_GAP * q) & 1);
-      if (keeps)
-        for (int u = 0; u < 4; ++u) o[u] = r[u];
-    };
-    for (int q = mq0; q < mq1; ++q) {
-      const int p = hi - 1 - 2 * q;
-      R a, b, c, d;
-      if (iter % 11 == 10) {  // an exceptional pair every 11th sweep
-        const R e = se_abs(H[(p + 1) * ld + p]) + se_abs(H[p * ld + p - 1]);
-        a = 0.75 * e + H[(p + 1) * ld + p + 1];
-        b = -0.4375 * e;
-        c = e;
-        d = a;
-      } else {
-        a = H[p * ld + p];
-        b = H[p * ld + p + 1];
-        c = H[(p + 1) * ld + p];
-        d = H[(p + 1) * ld + p + 1];
-      }
-      R s[4];
-      shift_pair(a, b, c, d, s);
-      if (keeps)
-        for (int u = 0; u < 4; ++u) snap[q * SE_SLOT + SE_SHIFTS + u] = s[u];
-    }
-#ifdef __CUDA_ARCH__
-    __syncwarp();
-#endif
-    if (mq0 == 0) start(0);
-    t.sync();  // the reads of H above precede the first update
-    // Bulge q is at row k = lo + step - SE_BULGE_GAP q.  For k > lo its reflector was built from column
-    // k - 1 (rows k .. k + 2), which it maps to (alpha, 0, 0) exactly; that column is therefore not part of
-    // the left update but written directly, after the barrier that separates the reads of it from the
-    // writes.  At k = hi - 1 the reflector has two rows.  The next reflector comes from column k after this
-    // step's right update; its three entries are recomputed from a snapshot of rows k + 1 .. k + 3
-    // (columns k .. k + 2) taken in the left phase, and the reflector is formed while the others run the
-    // right update (the entries are the values the right update writes).
-    const int steps = hi - lo + SE_BULGE_GAP * (nb - 1);
-    for (int step = 0; step < steps; ++step) {
-      // the active bulges q0 <= q < q1 (those between the start and the end of the block)
-      const int q0 = step - (hi - 1 - lo) > 0 ? (step - (hi - 1 - lo) + SE_BULGE_GAP - 1) / SE_BULGE_GAP : 0;
-      const int q1 = step / SE_BULGE_GAP + 1 < nb ? step / SE_BULGE_GAP + 1 : nb;
-      const R* refl = snap + SE_REFL + 4 * (step & 1);
-      auto reflect = [&](R* a, int st, const R* r, bool three) {
-        const R u1 = r[0], u2 = r[1], beta = r[2];
-        const R a0 = a[0], a1 = a[st], a2 = three ? a[2 * st] : R(0.0);
-        R d = a0;
-        se_mac(d, u1, a1);
-        if (three) se_mac(d, u2, a2);
-        d = se_fin(d) * beta;
-        a[0] = a0 - d;
-        a[st] = a1 - d * u1;
-        if (three) a[2 * st] = a2 - d * u2;
-      };
-      // phase 1: rows k .. k + 2 from the left (columns k .. m - 1), one column per item, the active bulges'
-      // items one after another
-      const int k1 = lo + step;  // bulge 0's row
-      // (the item's bulge is found with selections and the update done once: a branch per bulge would issue
-      // the update once for every bulge that meets in a warp)
-      {
-        int total = 0;
-        for (int q = q0; q < q1; ++q) total += m - (k1 - SE_BULGE_GAP * q);
-        for (int at = t.lane; at < total; at += t.size) {
-          int idx = at, q = q0, k = k1 - SE_BULGE_GAP * q0;
-          for (int u = 1; u < SE_BULGES; ++u) {
-            const bool next = idx >= m - k;
-            idx -= next ? m - k : 0;
-            q += next ? 1 : 0;
-            k -= next ? SE_BULGE_GAP : 0;
-          }
-          const bool three = k <= hi - 2;
-          R* a = H + k * ld + k + idx;
-          reflect(a, ld, refl + q * SE_SLOT, three);
-          if (idx < 3 && three) {  // column k + idx
-            R* v = snap + q * SE_SLOT + idx;
-            v[0] = a[ld];
-            v[3] = a[2 * ld];
-            v[6] = k + 3 <= hi ? a[3 * ld] : R(0.0);
-          }
-        }
-      }
-      t.sync();
-      // phase 2: columns k .. k + 2 from the right (rows 0 .. k + 3) and Q, one row per item; the next
-      // reflectors
-      for (int q = mq0; q < mq1; ++q) {
-        const int k = k1 - SE_BULGE_GAP * q;
-        R* slot = snap + q * SE_SLOT;
-        const R* r = refl + q * SE_SLOT;
-        R v[3] = {R(0.0), R(0.0), R(0.0)};
-        const R u1 = r[0], u2 = r[1], beta = r[2];
-        auto entry = [&](int rr) {
-          const R a0 = slot[3 * rr], a1 = slot[3 * rr + 1], a2 = slot[3 * rr + 2];
-          R d = a0;
-          se_mac(d, u1, a1);
-          se_mac(d, u2, a2);
-          d = se_fin(d) * beta;
-          return a0 - d;
-        };
-#ifdef __CUDA_ARCH__
-        // one lane per entry (a bulge outside the block computes on what its slot happens to hold, and the
-        // result is not used)
-        const R e = entry(rl < 3 * nb ? rl - 3 * mq0 : 2);
-        v[0] = se_warp_get(e, 3 * mq0);
-        v[1] = se_warp_get(e, 3 * mq0 + 1);
-        v[2] = se_warp_get(e, 3 * mq0 + 2);
-#else
-        for (int rr = 0; rr < 3; ++rr) v[rr] = entry(rr);
-#endif
-        if (k == lo - 1) {
-          start(q);
-        } else if (k >= lo && k <= hi - 2) {
-          R n[4];
-          make_reflector<R>(v[0], v[1], v[2], n[0], n[1], n[2], n[3]);
-          R* o = slot + SE_REFL + 4 * ((step + 1) & 1);
-          if (keeps)
-            for (int u = 0; u < 4; ++u) o[u] = n[u];
-        }
-        if (keeps && k > lo && k <= hi - 1) {
-          H[k * ld + k - 1] = r[3];
-          H[(k + 1) * ld + k - 1] = 0.0;
-          if (k <= hi - 2) H[(k + 2) * ld + k - 1] = 0.0;
-        }
-      }
-      if (t.lane < nwork) {
-        auto rows_of = [&](int k) { return (k + 3 <= hi ? k + 3 : hi) + 1; };
-        int total = 0;
-        for (int q = q0; q < q1; ++q) total += rows_of(k1 - SE_BULGE_GAP * q) + m;
-        for (int at = t.lane; at < total; at += nwork) {
-          int idx = at, q = q0, k = k1 - SE_BULGE_GAP * q0;
-          for (int u = 1; u < SE_BULGES; ++u) {
-            const int cnt = rows_of(k) + m;
-            const bool next = idx >= cnt;
-            idx -= next ? cnt : 0;
-            q += next ? 1 : 0;
-            k -= next ? SE_BULGE_GAP : 0;
-          }
-          const int rows = rows_of(k);
-          reflect(idx < rows ? H + idx * ld + k : Q + (idx - rows) * ldq + k, 1, refl + q * SE_SLOT, k <= hi - 2);
-        }
-      }
-      t.sync();
-    }
+    if (w >= SE_W3) se_sweep<3>(H, ld, Q, ldq, m, lo, hi, iter % 11 == 10, t, snap);
+    else if (w >= SE_W2) se_sweep<2>(H, ld, Q, ldq, m, lo, hi, iter % 11 == 10, t, snap);
+    else se_sweep<1>(H, ld, Q, ldq, m, lo, hi, iter % 11 == 10, t, snap);
   }
   return 0;
 }
