@@ -16,20 +16,43 @@
 namespace a2ls {
 
 // ---------------------------------------------------------------------------
-// CSR SpMV: y = A x, or y = bm - A x when bm != nullptr.  A CTA takes ROWS consecutive rows: their entries
-// are one contiguous piece of colind and val, which the threads read coalesced (SPMV_UNROLL entries each
-// in flight) into products in shared memory, and one thread per row sums its own in order; rows whose
-// entries do not fit the products' space are summed piece by piece.  Bound by memory: 12 bytes an entry.
-// Against 4 lanes per row, whose loads leave one gather in flight at a time: 41.7 -> 32.8 us on
+// CSR SpMV: y = A x, or y = bm - A x when bm != nullptr.  Bound by memory: 12 bytes an entry.
+// Rows of at most SPMV_SHORT entries (stencils): a thread per row with SPMV_UNROLL entries in flight; the
+// neighbours' entries share its cache lines.  4 lanes per row kept one gather in flight: 41.4 -> 22.3 us on
 // the 96^3 seven-point operator (91 MB).
-// ROWS: 256, or 64 where 256 would leave SMs idle (fewer rows than two CTAs per SM).
 // ---------------------------------------------------------------------------
-constexpr int SPMV_UNROLL = 8;
-template <int ROWS>
-__global__ void __launch_bounds__(ROWS) k_spmv(int n, const int* __restrict__ rowptr, const int* __restrict__ colind,
-                                               const double* __restrict__ val, const double* __restrict__ x,
-                                               double* __restrict__ y, const double* __restrict__ bm) {
-  constexpr int CAP = ROWS * SPMV_UNROLL;
+constexpr int SPMV_UNROLL = 8, SPMV_SHORT = 32;
+__global__ void __launch_bounds__(128) k_spmv(int n, const int* __restrict__ rowptr, const int* __restrict__ colind,
+                                              const double* __restrict__ val, const double* __restrict__ x,
+                                              double* __restrict__ y, const double* __restrict__ bm) {
+  const int r = blockIdx.x * 128 + threadIdx.x;
+  if (r >= n) return;
+  const int a = rowptr[r], b = rowptr[r + 1];
+  double s = 0.0;
+  for (int q = a; q < b; q += SPMV_UNROLL) {
+    int c[SPMV_UNROLL];
+    double v[SPMV_UNROLL], xv[SPMV_UNROLL];
+#pragma unroll
+    for (int u = 0; u < SPMV_UNROLL; ++u) {
+      c[u] = q + u < b ? __ldg(colind + q + u) : 0;
+      v[u] = q + u < b ? __ldg(val + q + u) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < SPMV_UNROLL; ++u) xv[u] = q + u < b ? __ldg(x + c[u]) : 0.0;
+#pragma unroll
+    for (int u = 0; u < SPMV_UNROLL; ++u) s += v[u] * xv[u];
+  }
+  y[r] = bm ? bm[r] - s : s;
+}
+
+// Matrices with longer rows: a CTA takes 256 consecutive rows, whose entries are one contiguous piece of
+// colind and val: the threads read it coalesced into products in shared memory, and one thread per row sums
+// its own in order (piece by piece where the entries do not fit).  On the same operator 33 us.
+__global__ void __launch_bounds__(256) k_spmv_long(int n, const int* __restrict__ rowptr,
+                                                   const int* __restrict__ colind, const double* __restrict__ val,
+                                                   const double* __restrict__ x, double* __restrict__ y,
+                                                   const double* __restrict__ bm) {
+  constexpr int ROWS = 256, CAP = ROWS * SPMV_UNROLL;
   __shared__ double prod[CAP];
   const int tid = threadIdx.x, r0 = blockIdx.x * ROWS, r = r0 + tid;
   const int e0 = rowptr[r0], e1 = rowptr[min(r0 + ROWS, n)];
@@ -42,8 +65,8 @@ __global__ void __launch_bounds__(ROWS) k_spmv(int n, const int* __restrict__ ro
 #pragma unroll
     for (int u = 0; u < SPMV_UNROLL; ++u) {
       const int e = tid + u * ROWS;
-      c[u] = e < cnt ? colind[base + e] : 0;
-      v[u] = e < cnt ? val[base + e] : 0.0;
+      c[u] = e < cnt ? __ldcs(colind + base + e) : 0;
+      v[u] = e < cnt ? __ldcs(val + base + e) : 0.0;
     }
 #pragma unroll
     for (int u = 0; u < SPMV_UNROLL; ++u) {
@@ -59,10 +82,10 @@ __global__ void __launch_bounds__(ROWS) k_spmv(int n, const int* __restrict__ ro
 }
 
 void spmv(a2ls_handle* h, const double* x, double* y, const double* b_minus, cudaStream_t st) {
-  if (h->n >= 2 * 152 * 256)
-    k_spmv<256><<<ceil_div(h->n, 256), 256, 0, st>>>(h->n, h->rowptr, h->colind, h->val, x, y, b_minus);
+  if (h->max_rownnz <= SPMV_SHORT)
+    k_spmv<<<ceil_div(h->n, 128), 128, 0, st>>>(h->n, h->rowptr, h->colind, h->val, x, y, b_minus);
   else
-    k_spmv<64><<<ceil_div(h->n, 64), 64, 0, st>>>(h->n, h->rowptr, h->colind, h->val, x, y, b_minus);
+    k_spmv_long<<<ceil_div(h->n, 256), 256, 0, st>>>(h->n, h->rowptr, h->colind, h->val, x, y, b_minus);
   A2LS_LAUNCH();
 }
 
@@ -71,11 +94,12 @@ void spmv(a2ls_handle* h, const double* x, double* y, const double* b_minus, cud
 // Lanes are split into groups of G >= m_i columns; the 32/G row groups of a warp
 // are combined by warp shuffles, the warps of the CTA through shared memory.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_restrict(const int* ni, const int* nI, const int* off, const int* idx,
+constexpr int RESTRICT_THREADS = 512;
+__global__ void __launch_bounds__(RESTRICT_THREADS) k_restrict(const int* ni, const int* nI, const int* off, const int* idx,
                                                   const int* m, const int* coff, const int64_t* woff,
                                                   const double* __restrict__ W, const double* __restrict__ r,
                                                   double* g, int boolean_pou) {
-  __shared__ double part[8][MAXM];
+  __shared__ double part[RESTRICT_THREADS / 32][MAXM];
   const int i = blockIdx.x;
   const int mi = m[i];
   if (mi == 0) return;
@@ -85,28 +109,40 @@ __global__ void __launch_bounds__(256) k_restrict(const int* ni, const int* nI, 
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int G = 1;
   while (G < mi && G < 32) G <<= 1;
+  constexpr int RW = RESTRICT_THREADS / 32;
   const int rg = 32 / G;          // row groups per warp
   const int sub = lane / G, a = lane % G;
   for (int c0 = 0; c0 < mi; c0 += 32) {
     double acc = 0.0;
     const int col = c0 + a;
-    for (int l = wid * rg + sub; l < rows; l += 8 * rg) {
-      const double rv = __ldg(r + idx[o + l]);
-      if (col < mi) acc += Wi[(int64_t)l * mi + col] * rv;
+    // RU rows' gathers and coefficients in flight (one at a time and 8 warps: 65 us on 512 subdomains of 1728
+    // rows and 12 columns, 120 MB; four and 16 warps 54 us)
+    constexpr int RU = 4;
+    for (int l0 = wid * rg + sub; l0 < rows; l0 += RU * RW * rg) {
+      double rv[RU], wv[RU];
+#pragma unroll
+      for (int u = 0; u < RU; ++u) {
+        const int l = l0 + u * RW * rg;
+        rv[u] = l < rows ? __ldg(r + idx[o + l]) : 0.0;
+        wv[u] = (l < rows && col < mi) ? Wi[(int64_t)l * mi + col] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < RU; ++u) acc += wv[u] * rv[u];
     }
     for (int s = G; s < 32; s <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
     if (sub == 0 && col < mi) part[wid][col] = acc;
     __syncthreads();
     if (threadIdx.x < 32 && c0 + threadIdx.x < mi) {
       double t = 0.0;
-      for (int w = 0; w < 8; ++w) t += part[w][c0 + threadIdx.x];
+      for (int w = 0; w < RW; ++w) t += part[w][c0 + threadIdx.x];
       g[coff[i] + c0 + threadIdx.x] = t;
     }
     __syncthreads();
   }
 }
 
-// c = Einv g; one warp per row, 16-byte loads
+// c = Einv g; one warp per row, 16-byte loads (8-byte ones of odd n0, whose rows lose the alignment); bound
+// by the FP64 pipes (2 flops per 8 bytes)
 __global__ void __launch_bounds__(256) k_gemv(int n0, const double* __restrict__ Einv,
                                               const double* __restrict__ g, double* __restrict__ c) {
   const int lane = threadIdx.x & 31;
@@ -118,12 +154,19 @@ __global__ void __launch_bounds__(256) k_gemv(int n0, const double* __restrict__
     if (even) {
       const double2* e2 = reinterpret_cast<const double2*>(er);
       const double2* g2 = reinterpret_cast<const double2*>(g);
+      // the matrix streams past the caches (evicted first; kept like other loads 131 us for n0 = 6206, 308 MB,
+      // so 92)
+      double s1 = 0.0;
+#pragma unroll 4
       for (int k = lane; k < n0 / 2; k += 32) {
-        const double2 a = __ldg(e2 + k), b = __ldg(g2 + k);
-        s += a.x * b.x + a.y * b.y;
+        const double2 a = __ldcs(e2 + k), b = __ldg(g2 + k);
+        s += a.x * b.x;
+        s1 += a.y * b.y;
       }
+      s += s1;
     } else {
-      for (int k = lane; k < n0; k += 32) s += __ldg(er + k) * __ldg(g + k);
+#pragma unroll 8
+      for (int k = lane; k < n0; k += 32) s += __ldcs(er + k) * __ldg(g + k);
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) c[row] = s;
@@ -148,6 +191,27 @@ __global__ void k_prolong(int n, const int* mrow, const int* mpos, const int* ms
   }
 }
 
+// The same for the Boolean partition of unity, where a node's only weight is that of the subdomain it lies
+// in: one CTA walks the interior rows of a subdomain, a thread a row, with c_i in shared memory and no
+// membership lists to chase.  512 subdomains of 1728 rows, 12 columns (120 MB): 64 -> 32 us.
+__global__ void __launch_bounds__(256) k_prolong_interior(const int* nI, const int* off, const int* idx, const int* m,
+                                                          const int* coff, const int64_t* woff,
+                                                          const double* __restrict__ W, const double* __restrict__ c,
+                                                          double* q) {
+  __shared__ double cs[MAXM];
+  const int i = blockIdx.x, mi = m[i], n = nI[i], o = off[i];
+  const double* Wi = W + woff[i];
+  if (threadIdx.x < mi) cs[threadIdx.x] = c[coff[i] + threadIdx.x];
+  __syncthreads();
+  for (int l = blockIdx.y * 256 + threadIdx.x; l < n; l += gridDim.y * 256) {
+    const double* w = Wi + (int64_t)l * mi;
+    double s = 0.0;
+#pragma unroll 4
+    for (int a = 0; a < mi; ++a) s += w[a] * cs[a];
+    q[idx[o + l]] = s;
+  }
+}
+
 // z[g] = (q ? q[g] : 0) + sum over memberships of yloc[pos]
 __global__ void k_combine(int n, const int* mrow, const int* mpos, const double* __restrict__ yloc,
                           const double* __restrict__ q, double* z) {
@@ -156,6 +220,19 @@ __global__ void k_combine(int n, const int* mrow, const int* mpos, const double*
     for (int t = mrow[gI]; t < mrow[gI + 1]; ++t) s += yloc[mpos[t]];
     z[gI] = s;
   }
+}
+
+// q = R_0^H c
+void prolong(a2ls_handle* h, const double* c, double* q) {
+  if (h->opt.pou == A2LS_POU_BOOLEAN) {
+    const int parts = std::max(1, std::min(ceil_div(h->max_n, 256), 2 * 152 / std::max(h->N, 1) + 1));
+    k_prolong_interior<<<dim3(h->N, parts), 256, 0, h->st>>>(h->d_nI, h->d_off, h->d_idx, h->d_m, h->d_coff, h->d_woff,
+                                                             h->d_W, c, q);
+  } else {
+    k_prolong<<<std::max(1, std::min(152 * 8, ceil_div(h->n, 256))), 256, 0, h->st>>>(
+        h->n, h->d_mrow, h->d_mpos, h->d_msub, h->d_off, h->d_m, h->d_coff, h->d_woff, h->d_D, h->d_W, c, q);
+  }
+  A2LS_LAUNCH();
 }
 
 static int grid1d(int64_t n, int threads = 256) {
@@ -175,14 +252,12 @@ static void local_part(a2ls_handle* h, const double* t, const double* q, double*
 
 static void coarse_correction(a2ls_handle* h, const double* r, double* q) {
   cudaStream_t st = h->st;
-  k_restrict<<<h->N, 256, 0, st>>>(h->d_ni, h->d_nI, h->d_off, h->d_idx, h->d_m, h->d_coff, h->d_woff, h->d_W,
+  k_restrict<<<h->N, RESTRICT_THREADS, 0, st>>>(h->d_ni, h->d_nI, h->d_off, h->d_idx, h->d_m, h->d_coff, h->d_woff, h->d_W,
                                    r, h->d_g, h->opt.pou == A2LS_POU_BOOLEAN);
   A2LS_LAUNCH();
   k_gemv<<<std::min(152 * 8, ceil_div((int64_t)h->n0 * 32, 256)), 256, 0, st>>>(h->n0, h->d_Einv, h->d_g, h->d_c);
   A2LS_LAUNCH();
-  k_prolong<<<grid1d(h->n), 256, 0, st>>>(h->n, h->d_mrow, h->d_mpos, h->d_msub, h->d_off, h->d_m, h->d_coff,
-                                          h->d_woff, h->d_D, h->d_W, h->d_c, q);
-  A2LS_LAUNCH();
+  prolong(h, h->d_c, q);
 }
 
 void apply_preconditioner(a2ls_handle* h, const double* r, double* z) {
@@ -250,69 +325,110 @@ void apply_preconditioner_graph(a2ls_handle* h, const double* r, double* z) {
 // ---------------------------------------------------------------------------
 // reductions for GMRES: multi-dot with a last-block-done final reduction
 // out[k] = sum_r V[k][r] * w[r] for k < nv, out[nv] = w . w (if with_self)
+//
+// Bound by the FP64 pipes as much as by memory (two multiply-adds a cycle and SM: nv n / 304 cycles), so
+// nothing may be added up with most lanes idle: a CTA takes MD_COLS vectors (blockIdx.y), its threads'
+// sums meet in shared memory, a warp per vector, and so do the CTAs' in the last one.  One vector's load
+// at a time, sums shuffled in every warp and the CTAs' partial sums added by one thread took 70 us for 8.5
+// vectors of 884736 on average, now 30.
 // ---------------------------------------------------------------------------
 constexpr int MD_MAX = 33;
-constexpr int MD_BLOCKS = 304;
+constexpr int MD_COLS = 8;
+constexpr int MD_BLOCKS = 608;
+constexpr int MD_GROUPS = (MD_MAX + MD_COLS - 1) / MD_COLS;
+
+__device__ __forceinline__ double warp_sum(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// The CTA's sums of val over its threads, for ncol <= 8 columns, added to those of the other gridDim.x
+// CTAs of the same blockIdx.y: the last of them writes out[0 .. ncol).  256 threads; partial: 8 x gridDim.x
+// values and counter (zero, left zero) of this blockIdx.y.
+__device__ __forceinline__ void grid_sum(const double (&val)[MD_COLS], int ncol, double* partial, unsigned* counter,
+                                         double* out) {
+  __shared__ double red[MD_COLS][256];
+  __shared__ bool last;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+#pragma unroll
+  for (int k = 0; k < MD_COLS; ++k)
+    if (k < ncol) red[k][tid] = val[k];
+  __syncthreads();
+  if (wid < ncol) {  // warp wid: column wid
+    double s = 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += red[wid][lane + 32 * u];
+    s = warp_sum(s);
+    if (lane == 0) {
+      partial[wid * gridDim.x + blockIdx.x] = s;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  if (tid == 0) last = (atomicAdd(counter, 1u) == gridDim.x - 1);
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (wid < ncol) {
+    double s = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(partial + wid * gridDim.x + b);
+    s = warp_sum(s);
+    if (lane == 0) out[wid] = s;
+  }
+  if (tid == 0) *counter = 0u;
+}
 
 __global__ void __launch_bounds__(256) k_multidot(int n, const double* __restrict__ V, int64_t ldv, int nv,
                                                   const double* __restrict__ w, int with_self,
                                                   double* partial, unsigned* counter, double* out) {
-  __shared__ double red[8][MD_MAX];
-  __shared__ bool last;
-  const int nd = nv + (with_self ? 1 : 0);
-  double acc[MD_MAX];
+  const int k0 = blockIdx.y * MD_COLS, nd = nv + (with_self ? 1 : 0), ncol = min(MD_COLS, nd - k0);
+  double acc[MD_COLS];
+  const double* col[MD_COLS];
 #pragma unroll
-  for (int k = 0; k < MD_MAX; ++k) acc[k] = 0.0;
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+  for (int k = 0; k < MD_COLS; ++k) {
+    acc[k] = 0.0;
+    // w itself as the last vector; columns past the end repeat the last one (cached) and are not used
+    const int kk = min(k0 + k, nd - 1);
+    col[k] = kk < nv ? V + (int64_t)kk * ldv : w;
+  }
+  const int stride = gridDim.x * 256;
+  for (int r = blockIdx.x * 256 + threadIdx.x; r < n; r += stride) {
     const double wr = w[r];
+    if (ncol == MD_COLS) {
+      double v[MD_COLS];
 #pragma unroll
-    for (int k = 0; k < MD_MAX; ++k) {
-      if (k < nv) acc[k] += V[(int64_t)k * ldv + r] * wr;
-      else if (k == nv && with_self) acc[k] += wr * wr;
-    }
-  }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+      for (int k = 0; k < MD_COLS; ++k) v[k] = col[k][r];
 #pragma unroll
-  for (int k = 0; k < MD_MAX; ++k) {
-    if (k < nd) {
-      double v = acc[k];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[wid][k] = v;
+      for (int k = 0; k < MD_COLS; ++k) acc[k] += v[k] * wr;
+    } else {
+      double v[MD_COLS - 1];
+#pragma unroll
+      for (int k = 0; k < MD_COLS - 1; ++k) v[k] = k < ncol ? col[k][r] : 0.0;
+#pragma unroll
+      for (int k = 0; k < MD_COLS - 1; ++k)
+        if (k < ncol) acc[k] += v[k] * wr;
     }
   }
-  __syncthreads();
-  if (threadIdx.x < nd) {
-    double t = 0.0;
-    for (int q = 0; q < 8; ++q) t += red[q][threadIdx.x];
-    partial[(int64_t)blockIdx.x * MD_MAX + threadIdx.x] = t;
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = (atomicAdd(counter, 1u) == gridDim.x - 1);
-  __syncthreads();
-  if (last) {
-    __threadfence();
-    if (threadIdx.x < nd) {
-      double t = 0.0;
-      for (int b = 0; b < (int)gridDim.x; ++b) t += partial[(int64_t)b * MD_MAX + threadIdx.x];
-      out[threadIdx.x] = t;
-    }
-    if (threadIdx.x == 0) *counter = 0u;
-  }
+  grid_sum(acc, ncol, partial + (int64_t)blockIdx.y * MD_COLS * MD_BLOCKS, counter + blockIdx.y, out + k0);
 }
 
-// w -= sum_k hk V_k  (optionally accumulate hsum += h)
-__global__ void k_cgs_update(int n, const double* __restrict__ V, int64_t ldv, int nv, const double* hcoef,
-                             double* w, double* hsum) {
-  __shared__ double hs[MD_MAX];
-  if (threadIdx.x < nv) hs[threadIdx.x] = hcoef[threadIdx.x];
+// w -= sum_k hk V_k, with norm2 (if given) = |w|^2 of the result
+// (norm2: at most MD_BLOCKS MD_COLS CTAs)
+__global__ void __launch_bounds__(256) k_cgs_update(int n, const double* __restrict__ V, int64_t ldv, int nv,
+                                                    const double* hcoef, double* w, double* partial, unsigned* counter,
+                                                    double* norm2) {
+  __shared__ double hs[MD_MAX + 3];
+  if (threadIdx.x < MD_MAX + 3) hs[threadIdx.x] = threadIdx.x < nv ? hcoef[threadIdx.x] : 0.0;
   __syncthreads();
-  if (hsum && blockIdx.x == 0 && threadIdx.x < nv) hsum[threadIdx.x] += hs[threadIdx.x];
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+  double sq[MD_COLS] = {};
+  for (int r = blockIdx.x * 256 + threadIdx.x; r < n; r += gridDim.x * 256) {
     double s = w[r];
+#pragma unroll 4
     for (int k = 0; k < nv; ++k) s -= hs[k] * V[(int64_t)k * ldv + r];
     w[r] = s;
+    sq[0] += s * s;
   }
+  if (norm2) grid_sum(sq, 1, partial, counter, norm2);
 }
 
 // y = x * (1 / *alpha) or y = x * alpha_host when alpha_dev == nullptr
@@ -330,6 +446,7 @@ __global__ void k_lincomb(int n, const double* __restrict__ V, int64_t ldv, int 
   __syncthreads();
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
     double s = 0.0;
+#pragma unroll 4
     for (int k = 0; k < nv; ++k) s += cs[k] * V[(int64_t)k * ldv + r];
     if (xacc) xacc[r] += s;
     else y[r] = s;
@@ -347,13 +464,14 @@ struct Reducer {
 };
 
 static Reducer& reducer(a2ls_handle* h) {
+  constexpr size_t parts = (size_t)MD_BLOCKS * MD_COLS * MD_GROUPS;
   if (!h->d_red) {
-    h->d_red = dalloc<double>(h, (size_t)MD_BLOCKS * MD_MAX + 4 * MD_MAX + 16);
-    A2LS_CUDA(cudaMemsetAsync(h->d_red, 0, sizeof(double) * ((size_t)MD_BLOCKS * MD_MAX + 4 * MD_MAX + 16), h->st));
+    h->d_red = dalloc<double>(h, parts + 4 * MD_MAX + 16);
+    A2LS_CUDA(cudaMemsetAsync(h->d_red, 0, sizeof(double) * (parts + 4 * MD_MAX + 16), h->st));
   }
   static thread_local Reducer r;
   r.partial = h->d_red;
-  r.out = h->d_red + (size_t)MD_BLOCKS * MD_MAX;             // 4 * MD_MAX doubles of outputs
+  r.out = h->d_red + parts;                                  // 4 * MD_MAX doubles of outputs
   r.counter = reinterpret_cast<unsigned*>(r.out + 4 * MD_MAX);
   return r;
 }
@@ -361,8 +479,17 @@ static Reducer& reducer(a2ls_handle* h) {
 static void multidot(a2ls_handle* h, const double* V, int64_t ldv, int nv, const double* w, int with_self,
                      double* out) {
   Reducer& R = reducer(h);
-  const int blocks = std::min(MD_BLOCKS, std::max(1, ceil_div(h->n, 256)));
-  k_multidot<<<blocks, 256, 0, h->st>>>(h->n, V, ldv, nv, w, with_self, R.partial, R.counter, out);
+  const int nd = nv + (with_self ? 1 : 0);
+  const dim3 grid(std::min(MD_BLOCKS, std::max(1, ceil_div(h->n, 256))), ceil_div(nd, MD_COLS));
+  k_multidot<<<grid, 256, 0, h->st>>>(h->n, V, ldv, nv, w, with_self, R.partial, R.counter, out);
+  A2LS_LAUNCH();
+}
+
+// w -= sum_k h_k V_k; norm2 (device, may be null) receives |w|^2 of the result
+static void cgs_update(a2ls_handle* h, const double* V, int64_t ldv, int nv, const double* hcoef, double* w,
+                       double* norm2) {
+  Reducer& R = reducer(h);
+  k_cgs_update<<<grid1d(h->n), 256, 0, h->st>>>(h->n, V, ldv, nv, hcoef, w, R.partial, R.counter, norm2);
   A2LS_LAUNCH();
 }
 
@@ -444,12 +571,9 @@ int gmres(a2ls_handle* h, const double* b, double* x, double rtol, int* iters_ou
       spmv(h, zj, w, nullptr, st);  // w = A z_j
       // CGS2 against V_0..V_j
       multidot(h, V, n, j + 1, w, 1, dh);                 // h1, |w|^2
-      k_cgs_update<<<gb, 256, 0, st>>>(n, V, n, j + 1, dh, w, nullptr);
-      A2LS_LAUNCH();
+      cgs_update(h, V, n, j + 1, dh, w, nullptr);
       multidot(h, V, n, j + 1, w, 0, dh + MD_MAX);        // h2
-      k_cgs_update<<<gb, 256, 0, st>>>(n, V, n, j + 1, dh + MD_MAX, w, nullptr);
-      A2LS_LAUNCH();
-      multidot(h, V, 0, 0, w, 1, dh + 2 * MD_MAX);        // |w|^2 after orthogonalisation
+      cgs_update(h, V, n, j + 1, dh + MD_MAX, w, dh + 2 * MD_MAX);  // and |w|^2 after orthogonalisation
       k_scale<<<gb, 256, 0, st>>>(n, w, V + (size_t)(j + 1) * n, dh + 2 * MD_MAX, 1, 0.0);
       A2LS_LAUNCH();
       A2LS_CUDA(cudaMemcpyAsync(hp, dh, sizeof(double) * 3 * MD_MAX, cudaMemcpyDeviceToHost, st));

@@ -20,9 +20,7 @@ __global__ void k_restrict(const int* ni, const int* nI, const int* off, const i
                            const double* __restrict__ r, double* g, int boolean_pou);
 __global__ void k_gemv(int n0, const double* __restrict__ Einv, const double* __restrict__ g,
                        double* __restrict__ c);
-__global__ void k_prolong(int n, const int* mrow, const int* mpos, const int* msub, const int* off, const int* m,
-                          const int* coff, const int64_t* woff, const double* D, const double* __restrict__ W,
-                          const double* __restrict__ c, double* q);
+void prolong(a2ls_handle* h, const double* c, double* q);
 __global__ void k_combine(int n, const int* mrow, const int* mpos, const double* __restrict__ yloc,
                           const double* __restrict__ q, double* z);
 
@@ -106,14 +104,12 @@ static void apply_static(a2ls_handle* h, const double* r, double* z) {
     local(r, nullptr);
     return;
   }
-  k_restrict<<<h->N, 256, 0, st>>>(h->d_ni, h->d_nI, h->d_off, h->d_idx, h->d_m, h->d_coff, h->d_woff, h->d_W, r,
+  k_restrict<<<h->N, 512, 0, st>>>(h->d_ni, h->d_nI, h->d_off, h->d_idx, h->d_m, h->d_coff, h->d_woff, h->d_W, r,
                                    g, boolean);
   A2LS_LAUNCH();
   k_gemv<<<std::min(152 * 8, ceil_div((int64_t)h->n0 * 32, 256)), 256, 0, st>>>(h->n0, h->d_Einv, g, c);
   A2LS_LAUNCH();
-  k_prolong<<<grid_n, 256, 0, st>>>(h->n, h->d_mrow, h->d_mpos, h->d_msub, h->d_off, h->d_m, h->d_coff,
-                                    h->d_woff, h->d_D, h->d_W, c, q);
-  A2LS_LAUNCH();
+  prolong(h, c, q);
   if (deflated) {
     spmv(h, q, t, r, st);  // t = r - A q
     local(t, q);
