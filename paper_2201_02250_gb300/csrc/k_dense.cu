@@ -24,6 +24,12 @@ template <> struct AccOf<float> { using type = float; };
 template <> struct AccOf<double> { using type = double; };
 template <> struct AccOf<dfloat> { using type = dfloat; };
 
+// |x| <= bound in x's own arithmetic: a pivot is tested on the chain of every elimination step, where a few
+// FP64 instructions of double-float or FP32 factors took as long as the rest of the step
+__device__ __forceinline__ bool abs_at_most(double x, double bound) { return fabs(x) <= bound; }
+__device__ __forceinline__ bool abs_at_most(float x, double bound) { return fabsf(x) <= (float)bound; }
+__device__ __forceinline__ bool abs_at_most(dfloat x, double bound) { return se_abs(x) <= dfloat(bound); }
+
 // depth of the operand chunks staged by the tile products
 constexpr int GK = 32;
 
@@ -72,52 +78,54 @@ __device__ __forceinline__ void cta_gemm_narrow(const T* __restrict__ A, int64_t
 }
 
 // Inverses of the triangles of a factored tb x tb block t (unit lower L strictly below the diagonal,
-// U on and above it) into s, given rp[c] = 1 / U_cc.  256 threads, two per column: each sums every
-// other term of the column's dot products with two accumulators (a quarter of the serial chain);
-// threads 0-127 form inv(L), 128-255 inv(U).  The pair sums are full-warp shuffles, so every thread
-// of the block must call this.
-template <class R>
+// U on and above it) into s, given rp[c] = 1 / U_cc.  128 H threads, H (2 .. 32) per column: each sums every
+// H-th term of the column's dot products with two accumulators (1 / (2 H) of the serial chain); the first
+// 64 H threads form inv(L), the others inv(U).  The H sums meet in full-warp shuffles, so every thread of
+// the block must call this.
+template <class R, int H = 2>
 __device__ void tile_inverses(const R (*t)[TB + 1], R (*s)[TB + 1], const R* rp, int tb) {
   const int tid = threadIdx.x;
-  const int col = (tid & 127) >> 1, h = tid & 1;
+  const int col = (tid & (64 * H - 1)) / H, h = tid & (H - 1);
   const bool active_col = col < tb;
-  if (tid < 128) {
+  if (tid < 64 * H) {
     // inv(L), column col: x_r = -(L[r][col] + sum_{q=col+1}^{r-1} L[r][q] x_q); this thread sums the q
-    // with (q - col - 1) % 2 == h and writes the rows r with (r - col - 1) % 2 == h, so it reads only
+    // with (q - col - 1) % H == h and writes the rows r with (r - col - 1) % H == h, so it reads only
     // entries that it wrote itself
     for (int r = 1; r < TB; ++r) {  // uniform across the warp
       R a0 = R(0.0), a1 = R(0.0);
       const bool act = active_col && r > col && r < tb;
       if (act) {
         int q = col + 1 + h;
-        for (; q + 2 < r; q += 4) {
+        for (; q + H < r; q += 2 * H) {
           mac(a0, t[r][q], s[q][col]);
-          mac(a1, t[r][q + 2], s[q + 2][col]);
+          mac(a1, t[r][q + H], s[q + H][col]);
         }
         if (q < r) mac(a0, t[r][q], s[q][col]);
       }
       R v = finish(a0) + finish(a1);
-      v += warp_xor(v, 1);
-      if (act && ((r - col - 1) & 1) == h) s[r][col] = -(t[r][col] + v);
+#pragma unroll
+      for (int w = 1; w < H; w <<= 1) v += warp_xor(v, w);
+      if (act && ((r - col - 1) & (H - 1)) == h) s[r][col] = -(t[r][col] + v);
     }
   } else {
     // inv(U), column col: x_col = 1 / U_col,col, x_r = -(sum_{q=r+1}^{col} U[r][q] x_q) / U_rr; this
-    // thread sums the q with (col - q) % 2 == h and writes the rows with (col - r) % 2 == h
+    // thread sums the q with (col - q) % H == h and writes the rows with (col - r) % H == h
     if (active_col && h == 0) s[col][col] = rp[col];
     for (int r = TB - 2; r >= 0; --r) {
       R a0 = R(0.0), a1 = R(0.0);
       const bool act = active_col && r < col;
       if (act) {
         int q = col - h;
-        for (; q - 2 > r; q -= 4) {
+        for (; q - H > r; q -= 2 * H) {
           mac(a0, t[r][q], s[q][col]);
-          mac(a1, t[r][q - 2], s[q - 2][col]);
+          mac(a1, t[r][q - H], s[q - H][col]);
         }
         if (q > r) mac(a0, t[r][q], s[q][col]);
       }
       R v = finish(a0) + finish(a1);
-      v += warp_xor(v, 1);
-      if (act && ((col - r) & 1) == h) s[r][col] = -(v * rp[r]);
+#pragma unroll
+      for (int w = 1; w < H; w <<= 1) v += warp_xor(v, w);
+      if (act && ((col - r) & (H - 1)) == h) s[r][col] = -(v * rp[r]);
     }
   }
 }
@@ -252,7 +260,7 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
         // whether A~_ii is singular
         last_pivot[i] = (double)Dm[c * 65 + c];
         Dm[c * 65 + c] = (Acc)scale;
-      } else if (fabs((double)Dm[c * 65 + c]) <= tiny) {
+      } else if (abs_at_most(Dm[c * 65 + c], tiny)) {
         // static pivoting: counted and replaced; otherwise an error (the replacement keeps the
         // remaining steps finite until the host reads the status)
         if (boost)
@@ -1139,17 +1147,22 @@ namespace a2ls {
 // pivoting, spread over many CTAs, then the explicit inverse.
 // ---------------------------------------------------------------------------
 // Factor the 64x64 diagonal block at (k0, k0) and invert its triangles in place, in the arithmetic
-// and storage R (FP64, or double-float in the mixed form).  256 threads.
-// LU: thread (ty, tx) = (tid / 64, tid % 64) owns column tx and the rows ty, ty + 4, ...; step c
+// and storage R (FP64, or double-float in the mixed form).  One CTA, one step of a chain as long as the
+// matrix, so every step counts: double-float takes 1024 threads (a quarter of the rows and of the inverses'
+// terms each: E_DIAG_TIMES), FP64, whose pipe is the limit, 256.
+// LU: thread (ty, tx) = (tid / 64, tid % 64) owns column tx and the rows ty, ty + NG, ...; step c
 // subtracts a21 (a12 / pivot)^T from the trailing block, so that the multipliers of column c are
 // formed only once, after the loop (l_rc = a_rc / pivot_c).  The owner of entry (c+1, c+1) checks the
 // next pivot right after its own update, so each step needs one barrier.
-// Inverses: tile_inverses (two threads per column).
+// Inverses: tile_inverses.
+template <class R> struct EDiagThreads { static constexpr int v = 256; };
+template <> struct EDiagThreads<dfloat> { static constexpr int v = 1024; };
 template <class R>
 __device__ __forceinline__ R e_recip(R x) { return R(1.0) / x; }
 
 template <class R>
-__global__ void __launch_bounds__(256) k_e_diag(R* A, int n, int64_t ld, int k0, double scale, int* st) {
+__global__ void __launch_bounds__(EDiagThreads<R>::v) k_e_diag(R* A, int n, int64_t ld, int k0, double scale, int* st) {
+  constexpr int NT = EDiagThreads<R>::v, NG = NT / TB;
   __shared__ R t[TB][TB + 1], s[TB][TB + 1];
   __shared__ R rp[TB];
   const int tb = min(TB, n - k0);
@@ -1159,7 +1172,7 @@ __global__ void __launch_bounds__(256) k_e_diag(R* A, int n, int64_t ld, int k0,
   __syncthreads();
   auto pivot = [&](int c) {
     R piv = t[c][c];
-    if (fabs((double)piv) <= 1e-14 * scale) {
+    if (abs_at_most(piv, 1e-14 * scale)) {
       raise_status(st, A2LS_ERR_SINGULAR, -1, k0 + c);
       piv = R(scale);
       t[c][c] = piv;
@@ -1172,8 +1185,8 @@ __global__ void __launch_bounds__(256) k_e_diag(R* A, int n, int64_t ld, int k0,
   for (int c = 0; c + 1 < tb; ++c) {
     if (tx > c && tx < tb) {
       const R u = t[c][tx] * rp[c];
-      for (int r = c + 1 + ((ty - c - 1) & 3); r < tb; r += 4) t[r][tx] -= t[r][c] * u;
-      if (tx == c + 1 && ty == ((c + 1) & 3)) pivot(c + 1);
+      for (int r = c + 1 + ((ty - c - 1) & (NG - 1)); r < tb; r += NG) t[r][tx] -= t[r][c] * u;
+      if (tx == c + 1 && ty == ((c + 1) & (NG - 1))) pivot(c + 1);
     }
     __syncthreads();
   }
@@ -1183,7 +1196,7 @@ __global__ void __launch_bounds__(256) k_e_diag(R* A, int n, int64_t ld, int k0,
     if (r > c) t[r][c] *= rp[c];
   }
   __syncthreads();
-  tile_inverses<R>(t, s, rp, tb);
+  tile_inverses<R, NT / 128>(t, s, rp, tb);
   __syncthreads();
   for (int e = tid; e < tb * tb; e += blockDim.x) {
     const int r = e / tb, c = e % tb;
@@ -1347,7 +1360,7 @@ static void dense_inverse_t(a2ls_handle* h, R* E, int n, double scale, R* Einv, 
   {
     KTime kt(h, KT_COARSE_LU, lu_flops);
     for (int k0 = 0; k0 < n; k0 += TB) {
-      k_e_diag<R><<<1, 256, 0, st>>>(E, n, ld, k0, scale, h->d_status);
+      k_e_diag<R><<<1, EDiagThreads<R>::v, 0, st>>>(E, n, ld, k0, scale, h->d_status);
       A2LS_LAUNCH();
       // entries farther than the bandwidth from the diagonal are zero and stay zero
       const int rest = min(n - k0 - min(TB, n - k0), band + TB);

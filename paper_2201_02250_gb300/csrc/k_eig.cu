@@ -266,18 +266,41 @@ __global__ void __launch_bounds__(EIG_THREADS) k_project_k(const int* ni, const 
   if ((active && !active[i]) || !kd[i]) return;
   const int n = ni[i], p = pvec[i], o = off[i];
   T* Xi = X + xoff[i] + col0;
-  for (int c = threadIdx.x; c < p; c += EIG_THREADS) dots[c] = 0;
-  __syncthreads();
-  // one warp per column
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int c = wid; c < p; c += EIG_THREADS / 32) {
-    Acc d = 0;
-    for (int l = lane; l < n; l += 32) mac(d, kvec[o + l], (Acc)Xi[(int64_t)l * ldx + c]);
-    d = finish(d);
-    for (int w = 16; w > 0; w >>= 1) d += warp_xor(d, w);
-    if (lane == 0) dots[c] = d;
+  if constexpr (std::is_same<Acc, double>::value) {
+    // (in the order FP64 results have always had, see se::SeFast)
+    for (int c = threadIdx.x; c < p; c += EIG_THREADS) dots[c] = 0;
+    __syncthreads();
+    // one warp per column
+    for (int c = wid; c < p; c += EIG_THREADS / 32) {
+      Acc d = 0;
+      for (int l = lane; l < n; l += 32) mac(d, kvec[o + l], (Acc)Xi[(int64_t)l * ldx + c]);
+      d = finish(d);
+      for (int w = 16; w > 0; w >>= 1) d += warp_xor(d, w);
+      if (lane == 0) dots[c] = d;
+    }
+    __syncthreads();
+  } else {
+    // a lane per column, the rows spread over the warps: whole rows are read at once (a warp per column read
+    // 32 rows 768 bytes apart for each load: PROJ_TIMES)
+    constexpr int NW = EIG_THREADS / 32;
+    __shared__ Acc part[NW][32];
+    for (int c0 = 0; c0 < p; c0 += 32) {
+      const int c = c0 + lane;
+      Acc d = 0;
+      if (c < p)
+#pragma unroll 4
+        for (int l = wid; l < n; l += NW) mac(d, kvec[o + l], (Acc)Xi[(int64_t)l * ldx + c]);
+      part[wid][lane] = finish(d);
+      __syncthreads();
+      if (wid == 0 && c < p) {
+        Acc t = part[0][lane];
+        for (int w = 1; w < NW; ++w) t += part[w][lane];
+        dots[c] = t;
+      }
+      __syncthreads();
+    }
   }
-  __syncthreads();
   for (int e = threadIdx.x; e < n * p; e += EIG_THREADS) {
     const int l = e / p, c = e % p;
     Xi[(int64_t)l * ldx + c] = (T)((Acc)Xi[(int64_t)l * ldx + c] - dots[c] * kvec[o + l]);
@@ -346,8 +369,11 @@ __global__ void k_mu_fix(const int* ni, const int* off, const int64_t* xoff, int
 // Orthogonalisation (k_orth and its helpers): block CGS2 of W against the basis, then Cholesky QR.
 // ---------------------------------------------------------------------------
 
-constexpr int ORTH_THREADS = 512;
-constexpr int ORC_MAX = 64;              // rows staged per chunk in k_orth (64, or 32 with full-space Gram)
+// Threads of k_orth.  Double-float and FP32: 256, with 32-row chunks, so that two CTAs share an SM and one's
+// barriers and staging overlap the other's arithmetic; FP64, whose chunks fix the order of its sums: 512.
+template <class Acc> struct OrthThreads { static constexpr int v = 256; };
+template <> struct OrthThreads<double> { static constexpr int v = 512; };
+// rows staged per chunk in k_orth: 64 in FP64 (32 with full-space Gram), otherwise 32
 // row stride of the staged chunks: even, so that column pairs are 16-byte aligned for vector loads;
 // 98 x 8 bytes puts consecutive rows 4 banks apart
 constexpr int SROW = EIG_MAXP + 2;
@@ -358,10 +384,10 @@ constexpr int GRAM_NG_MAX = 16;          // row groups (split-K) of a Gram produ
 __device__ __forceinline__ double ld_shared_rows(const double* p) { return __ldcg(p); }
 template <class TM>
 __device__ __forceinline__ TM ld_shared_rows(const TM* p) { return *p; }
-template <class Acc, class TM>
+template <class Acc, class TM, int NT = OrthThreads<Acc>::v>
 __device__ __forceinline__ void stage_rows(Acc* S, const TM* M, int64_t ldx, int l0, int rows, int w) {
   const int wp = (w + 3) & ~3;
-  for (int e = threadIdx.x; e < rows * wp; e += ORTH_THREADS) {
+  for (int e = threadIdx.x; e < rows * wp; e += NT) {
     const int r = e / wp, c = e % wp;
     S[r * SROW + c] = c < w ? (Acc)ld_shared_rows(M + (int64_t)(l0 + r) * ldx + c) : (Acc)0;
   }
@@ -388,7 +414,7 @@ __device__ __forceinline__ void ld2(const float* p, float& a, float& b) {
 // dimension ldx).  Each item is a 4 x 2 output block; with fewer blocks than threads the rows are
 // split into ng groups (split-K) whose partial sums are added at the end.  same (X == Y, nx == ny):
 // only the blocks that reach the upper triangle are formed, the lower triangle is mirrored.
-// Xs, Ys: staging chunks; Ps: scratch of ORTH_THREADS x 8 values for the partial sums (may alias
+// Xs, Ys: staging chunks; Ps: scratch of 8 values a thread for the partial sums (may alias
 // the staging chunks).  Ends with a barrier.
 // share, shares: only the output blocks of this share are formed (their sums are those of a whole
 // product); block_share gives an entry's share.
@@ -408,6 +434,7 @@ __device__ __forceinline__ int block_share(int a, int c, int nx, int ny, bool sa
 template <class Acc, class TX, class TY>
 __device__ void gram_product(const TX* X, const TY* Y, int64_t ldx, int n, int nx, int ny, bool same, Acc* Xs,
                              Acc* Ys, double* G, Acc* Ps, int orc, int share = 0, int shares = 1) {
+  constexpr int NT = OrthThreads<Acc>::v;
   const int tid = threadIdx.x;
   const int nbr = (nx + 3) / 4, nbc = (ny + 1) / 2;
   // block (br, bc) covers rows 4br..4br+3 and columns 2bc..2bc+1; with X == Y only bc >= 2br
@@ -420,12 +447,12 @@ __device__ void gram_product(const TX* X, const TY* Y, int64_t ldx, int n, int n
     a0 = 4 * br;
     c0 = 2 * (nbc - row_blocks(br) + b);
   };
-  const int ng = nb >= ORTH_THREADS ? 1 : min(GRAM_NG_MAX, ORTH_THREADS / nb);
+  const int ng = nb >= NT ? 1 : min(GRAM_NG_MAX, NT / nb);
   // this share's blocks b0 .. b0 + nbs - 1
   const int bps = (nb + shares - 1) / shares, b0 = min(nb, share * bps), nbs = min(bps, nb - b0);
   const int items = nbs * ng;
   // more blocks than threads (full-space Gram of a small subdomain): several passes over the rows
-  for (int w0 = 0; w0 < items; w0 += ORTH_THREADS) {
+  for (int w0 = 0; w0 < items; w0 += NT) {
     const int w = w0 + tid;
     const bool valid = w < items;
     int a0 = 0, c0 = 0, g = 0;
@@ -469,7 +496,7 @@ __device__ void gram_product(const TX* X, const TY* Y, int64_t ldx, int n, int n
           const int a = a0 + (q >> 1), c = c0 + (q & 1);
           if (a < nx && c < ny && (!same || c >= a)) G[a * ny + c] = (double)acc[q];
         }
-    } else {  // items <= ORTH_THREADS: a single pass
+    } else {  // items <= NT: a single pass
       if (valid)
 #pragma unroll
         for (int q = 0; q < 8; ++q) Ps[tid * 8 + q] = acc[q];
@@ -488,7 +515,7 @@ __device__ void gram_product(const TX* X, const TY* Y, int64_t ldx, int n, int n
     __syncthreads();
   }
   if (same && shares == 1) {
-    for (int e = tid; e < nx * nx; e += ORTH_THREADS) {
+    for (int e = tid; e < nx * nx; e += NT) {
       const int a = e / nx, c = e % nx;
       if (c < a) G[a * nx + c] = G[c * nx + a];
     }
@@ -611,27 +638,29 @@ __device__ __forceinline__ double cluster_ld(const double* p, int rank) {
 // the order of the ranks, so that every CTA holds the same values.  tmp: count doubles of scratch in shared
 // memory that no other CTA reads.  All threads of the cluster; G complete in every CTA (the barrier orders
 // it), ends with a CTA barrier.
+template <int NT>
 __device__ __forceinline__ void cluster_sum(double* G, int count, double* tmp) {
   const int C = cluster_size();
   if (C == 1) return;
   cluster_sync();
-  for (int e = threadIdx.x; e < count; e += ORTH_THREADS) {
+  for (int e = threadIdx.x; e < count; e += NT) {
     double s = cluster_ld(G + e, 0);
     for (int r = 1; r < C; ++r) s += cluster_ld(G + e, r);
     tmp[e] = s;
   }
   cluster_sync();  // every CTA has read this one's G
-  for (int e = threadIdx.x; e < count; e += ORTH_THREADS) G[e] = tmp[e];
+  for (int e = threadIdx.x; e < count; e += NT) G[e] = tmp[e];
   __syncthreads();
 }
 
 // G (nx x ny) complete in every CTA of the cluster, each of which formed the blocks of its own share; no CTA's
 // share is changed while another may read it.  Ends with a CTA barrier.
+template <int NT>
 __device__ __forceinline__ void cluster_gather(double* G, int nx, int ny, bool same) {
   const int C = cluster_size(), me = cluster_rank();
   if (C == 1) return;
   cluster_sync();
-  for (int e = threadIdx.x; e < nx * ny; e += ORTH_THREADS) {
+  for (int e = threadIdx.x; e < nx * ny; e += NT) {
     const int a = e / ny, c = e % ny;
     if (same && c < a) continue;
     const int owner = block_share(a, c, nx, ny, same, C);
@@ -639,7 +668,7 @@ __device__ __forceinline__ void cluster_gather(double* G, int nx, int ny, bool s
   }
   cluster_sync();
   if (same)
-    for (int e = threadIdx.x; e < nx * nx; e += ORTH_THREADS) {
+    for (int e = threadIdx.x; e < nx * nx; e += NT) {
       const int a = e / nx, c = e % nx;
       if (c < a) G[e] = G[c * nx + a];
     }
@@ -663,12 +692,13 @@ __device__ __forceinline__ void cluster_gather(double* G, int nx, int ny, bool s
 // double-float 48.2 -> 43.1 ms; 256 subdomains unchanged.  By blocks, a launch over 64 FP64 subdomains of about
 // 1950 rows 2.34 -> 1.14 ms, over 16 of 300 rows 460 -> 265 us (by rows 146).
 template <class T, class TW>
-__global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int64_t* xoff, int ldx,
+__global__ void __launch_bounds__(OrthThreads<typename EAcc<T>::type>::v) k_orth(const int* ni, const int64_t* xoff, int ldx,
                                                         const int* pvec, const int* active, int jb_blocks,
                                                         int bcols, T* V, TW* W, double* H, int hr, int hc,
                                                         int vout, const int* fullv, int* rank_flag, int gcap,
                                                         int orc, int* illcond, int* status) {
   using Acc = typename EAcc<T>::type;
+  constexpr int NT = OrthThreads<Acc>::v;
   extern __shared__ __align__(16) double sm[];
   const int C = cluster_size(), rank = cluster_rank();
   const int i = blockIdx.x / C;
@@ -704,7 +734,7 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
   // 64-row chunks and p = 24 that is exactly one item per thread); coefficients padded to pp columns
   const int ncg = (p + 2) / 3, pp = 3 * ncg;
   const int npass = jb > 0 ? 2 : 0;
-  for (int e = tid + h0; e < jb * p; e += ORTH_THREADS) Hi[(e / p) * EIG_MAXP + hc + e % p] = 0.0;
+  for (int e = tid + h0; e < jb * p; e += NT) Hi[(e / p) * EIG_MAXP + hc + e % p] = 0.0;
   for (int pass = 0; pass < npass; ++pass) {
     if (BY_BLOCKS && C > 1 && pass > 0) {
       __threadfence();
@@ -713,16 +743,16 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
     // G = V[:, 0:jb]^T W[:, 0:p]
     if (BY_BLOCKS) {
       gram_product<Acc>(Va, Wa, (int64_t)ldx, nall, jb, p, false, sv, sw, G, sv, orc, rank, C);
-      cluster_gather(G, jb, p, false);
+      cluster_gather<NT>(G, jb, p, false);
     } else {
       gram_product<Acc>(Vi, Wi, (int64_t)ldx, n, jb, p, false, sv, sw, G, sv, orc);
-      cluster_sum(G, jb * p, ctmp);
+      cluster_sum<NT>(G, jb * p, ctmp);
     }
-    for (int e = tid + h0; e < jb * p; e += ORTH_THREADS) Hi[(e / p) * EIG_MAXP + hc + e % p] += G[e];
+    for (int e = tid + h0; e < jb * p; e += NT) Hi[(e / p) * EIG_MAXP + hc + e % p] += G[e];
     if (full) return;  // Rayleigh quotient only
     // W -= V G; G converted once to the working arithmetic (in Ri's space, padded to pp columns)
     Acc* Ga = reinterpret_cast<Acc*>(Ri);
-    for (int e = tid; e < jb * pp; e += ORTH_THREADS) {
+    for (int e = tid; e < jb * pp; e += NT) {
       const int a = e / pp, c = e % pp;
       Ga[e] = c < p ? (Acc)G[a * p + c] : (Acc)0;
     }
@@ -731,7 +761,7 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
       const int rows = min(orc, n - l0);
       stage_rows(sv, Vi, ldx, l0, rows, jb);
       __syncthreads();
-      for (int e = tid; e < rows * ncg; e += ORTH_THREADS) {
+      for (int e = tid; e < rows * ncg; e += NT) {
         const int r = e / ncg, c = 3 * (e % ncg);
         Acc s0 = 0, s1 = 0, s2 = 0;
         for (int a = 0; a < jb; ++a) {
@@ -766,10 +796,10 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
         cluster_sync();
       }
       gram_product<Acc>(Wa, Wa, (int64_t)ldx, nall, p, p, true, sw, sw, G, sv, orc, rank, C);
-      cluster_gather(G, p, p, true);
+      cluster_gather<NT>(G, p, p, true);
     } else {
       gram_product<Acc>(Wi, Wi, (int64_t)ldx, n, p, p, true, sw, sw, G, sv, orc);
-      cluster_sum(G, p * p, ctmp);
+      cluster_sum<NT>(G, p * p, ctmp);
     }
     if (tid < 32) {
       // shifted pass: Gs + 11 (n p + p (p + 1)) u tr(Gs) I
@@ -796,21 +826,21 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
     if (rank != 0) {
       // (H below is rank 0's)
     } else if (pass == 0) {
-      for (int e = tid; e < p * p; e += ORTH_THREADS) {
+      for (int e = tid; e < p * p; e += NT) {
         const int a = e / p, c = e % p;
         Hi[(hr + a) * EIG_MAXP + hc + c] = (c >= a) ? G[a * p + c] : 0.0;
       }
     } else if ((size_t)p * p * sizeof(double) <= (size_t)orc * SROW * sizeof(Acc)) {
       // H_blk <- R H_blk (R upper triangular), through a temporary in the staging space
       double* tmp = reinterpret_cast<double*>(sw);
-      for (int e = tid; e < p * p; e += ORTH_THREADS) {
+      for (int e = tid; e < p * p; e += NT) {
         const int a = e / p, c = e % p;
         double s = 0.0;
         for (int q = a; q < p; ++q) s += G[a * p + q] * Hi[(hr + q) * EIG_MAXP + hc + c];
         tmp[e] = s;
       }
       __syncthreads();
-      for (int e = tid; e < p * p; e += ORTH_THREADS) Hi[(hr + e / p) * EIG_MAXP + hc + e % p] = tmp[e];
+      for (int e = tid; e < p * p; e += NT) Hi[(hr + e / p) * EIG_MAXP + hc + e % p] = tmp[e];
     } else {
       // a block too wide for the staging space (a full-space subdomain): in place, row by row from
       // the top (row a of the product reads rows a .. p - 1, not yet overwritten)
@@ -826,7 +856,7 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
     __syncthreads();
     // W <- W inv(R); inv(R) converted once to the working arithmetic (in G's space, padded to pp columns)
     Acc* Ra = reinterpret_cast<Acc*>(G);
-    for (int e = tid; e < p * pp; e += ORTH_THREADS) {
+    for (int e = tid; e < p * pp; e += NT) {
       const int a = e / pp, c = e % pp;
       Ra[e] = c < p ? (Acc)Ri[a * p + c] : (Acc)0;
     }
@@ -835,7 +865,7 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
       const int rows = min(orc, n - l0);
       stage_rows(sw, Wi, ldx, l0, rows, p);
       __syncthreads();
-      for (int e = tid; e < rows * ncg; e += ORTH_THREADS) {
+      for (int e = tid; e < rows * ncg; e += NT) {
         const int r = e / ncg, c = 3 * (e % ncg);
         Acc s0 = 0, s1 = 0, s2 = 0;
         for (int a = 0; a <= c + 2 && a < p; ++a) {
@@ -854,7 +884,7 @@ __global__ void __launch_bounds__(ORTH_THREADS) k_orth(const int* ni, const int6
   }
   // V[:, vout:vout+p] = W
   if (vout >= 0)
-    for (int e = tid; e < n * p; e += ORTH_THREADS) {
+    for (int e = tid; e < n * p; e += NT) {
       const int l = e / p, c = e % p;
       Vi[(int64_t)l * ldx + vout + c] = (T)Wi[(int64_t)l * ldx + c];
     }
@@ -1256,12 +1286,14 @@ __global__ void __launch_bounds__(TR_THREADS) k_thick_restart(const int* active,
   extern __shared__ double sm[];
   const int i = blockIdx.x;
   if (active && !active[i]) return;
-  const int tid = threadIdx.x, mb = m + b, ld = 2 * b;
-  R* U = reinterpret_cast<R*>(sm);  // mb x 2b
+  // an odd row stride: a column's entries, which the lanes of a warp hold, fall on different shared-memory
+  // banks (with 2 b every lane met the same one: TR_TIMES)
+  const int tid = threadIdx.x, mb = m + b, b2 = 2 * b, ld = b2 + 1;
+  R* U = reinterpret_cast<R*>(sm);  // mb x 2b, stride ld
   R* Gs = U + mb * ld;              // b x b
   R* R2 = Gs + b * b;               // b x b
   R* coef = R2 + b * b;             // 2b
-  R* dots = coef + ld;              // 2b
+  R* dots = coef + b2;              // 2b
   __shared__ R red[TR_THREADS / 32];
   const double* Yi = Y + (int64_t)i * EIG_MAXP * EIG_MAXP;
   double* Hi = H + (int64_t)i * EIG_MAXP * EIG_MAXP;
@@ -1310,7 +1342,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_thick_restart(const int* active,
   int cand2 = 0;
   for (int c = 0; c < b; ++c) {
     __syncthreads();  // coef of the previous column read
-    if (tid < ld) coef[tid] = R(0.0);
+    if (tid < b2) coef[tid] = R(0.0);
     __syncthreads();
     double n0 = 0.0;
     bool ok = true;
@@ -1334,7 +1366,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_thick_restart(const int* active,
     if (tid < mb) U[tid * ld + b + c] /= nrm;
   }
   __syncthreads();
-  for (int e = tid; e < mb * ld; e += blockDim.x) Ui[(e / ld) * EIG_MAXP + e % ld] = (double)U[e];
+  for (int e = tid; e < mb * b2; e += blockDim.x) Ui[(e / b2) * EIG_MAXP + e % b2] = (double)U[(e / b2) * ld + e % b2];
   for (int e = tid; e < mb * m; e += blockDim.x) {
     const int a = e / m, c = e % m;
     double v = 0.0;
@@ -1513,7 +1545,7 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
   bool any_full = false;
   for (int i = 0; i < N; ++i) any_full = any_full || (full[i] && act[i]);
   const int gcap_k = EIG_MAXP * 32, gcap_f = any_full ? EIG_MAXP * EIG_MAXP : gcap_k;
-  auto orc_for = [&](int gcap) { return gcap > gcap_k ? 32 : ORC_MAX; };
+  auto orc_for = [&](int gcap) { return std::is_same<Acc, double>::value && gcap <= gcap_k ? 64 : 32; };
   auto orth_smem_for = [&](int gcap) {
     return sizeof(double) * (2 * (size_t)gcap + EIG_MAXP) + sizeof(Acc) * 2 * (size_t)orc_for(gcap) * SROW;
   };
@@ -1535,7 +1567,7 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
   A2LS_CUDA(cudaFuncSetAttribute(k_vy<TV, TV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vy_smem));
   // thick restart (needs a block step after the kept block: s >= 2)
   const bool thick = h->opt.eig_thick_restart != 0 && s >= 2;
-  const size_t tr_smem = sizeof(double) * ((size_t)(s + 1) * b * 2 * b + 2 * (size_t)b * b + 4 * (size_t)b);
+  const size_t tr_smem = sizeof(double) * ((size_t)(s + 1) * b * (2 * b + 1) + 2 * (size_t)b * b + 4 * (size_t)b);
   A2LS_CUDA(cudaFuncSetAttribute(k_thick_restart<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tr_smem));
   int* d_illcond = dalloc<int>(h, N);  // per cycle: a block step needed the shifted factorisation
   int* d_thick = dalloc<int>(h, N);    // per cycle: the next restart may be thick
@@ -1617,10 +1649,10 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
     const int gcap = with_full ? gcap_f : gcap_k;
     int C = 1;
     if (gcap == gcap_k)
-      while (C < 8 && 2 * C * std::max(nact, 1) <= sms) C *= 2;
+      while (C < 8 && 2 * C * std::max(nact, 1) <= sms * (512 / OrthThreads<Acc>::v)) C *= 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(N * C);
-    cfg.blockDim = dim3(ORTH_THREADS);
+    cfg.blockDim = dim3(OrthThreads<Acc>::v);
     cfg.dynamicSmemBytes = orth_smem_for(gcap);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
