@@ -44,6 +44,21 @@ __device__ __forceinline__ void raise_status(int* st, int code, int where, int a
   }
 }
 
+// Thread-block clusters: the CTA's rank and count, and the barrier over all threads of the
+// cluster (which orders their global and shared memory accesses).
+__device__ __forceinline__ int cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ int cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 // Kernels whose launches can be timed with CUDA events (a2ls_options::timing).
 enum { KT_LU_LOCAL = 0, KT_LU_SPLIT, KT_EIG_SOLVE, KT_EIG_ORTH, KT_EIG_RR, KT_COARSE_LU, KT_COARSE_INV,
        KT_APPLY_LOCAL, KT_COUNT };

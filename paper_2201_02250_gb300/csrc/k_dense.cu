@@ -205,7 +205,13 @@ constexpr size_t lu_smem_elems() { return 2 * (size_t)TB * 65 + 2 * (size_t)TGK 
 // TC (double-float only): the trailing update A22 -= L21 U12 runs on the tensor cores as digit-split
 // BF16 products (tc_dfloat.cuh) in 128 x 64 tiles; its operand digits reuse the shared memory of the
 // other steps, so one CTA runs per SM, holding all of that SM's TMEM.
-template <class T, bool TC>
+//
+// MULTI: with fewer subdomains than SMs a cluster of CTAs takes each one.  Every CTA factors the diagonal
+// block for itself, the tiles of L21, U12 and of the trailing matrix are dealt out, and cluster barriers, which
+// also order the CTAs' global memory accesses, separate the two.  A tile's arithmetic does not depend on who
+// does it.  One CTA each against clusters, per launch: FP64, 64 subdomains of 1700 to 2200 rows, 239 ms against
+// 91 (of 4 CTAs, two an SM); double-float, 64 subdomains of 1100 to 1250 rows, 5.4 ms against 3.8 (of 2).
+template <class T, bool TC, bool MULTI>
 __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, const int* ld, const int64_t* foff,
                                             T* fac, int allow_last_zero, double* last_pivot,
                                             const double* dscale, int* st, const int* sched, const int* nI,
@@ -236,10 +242,15 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
   Acc* Iv = Dm + TB * 65;                         // 64 x 65: inv(L11) strictly below, inv(U11) on/above
   Acc* sA = Iv + TB * 65;                         // TGK x TS (16-byte aligned: 2 * 64 * 65 is even)
   Acc* sB = sA + TGK * TS;                        // TGK x TS
-  const int i = sched ? sched[blockIdx.x] : blockIdx.x;
+  const int C = MULTI ? cluster_size() : 1, rank = MULTI ? cluster_rank() : 0;
+  const int i = sched ? sched[blockIdx.x / C] : blockIdx.x / C;
   const int n = ni[i];
   const int64_t L = ld[i];
   T* A = fac + foff[i];
+  auto all_ctas = [&]() {   // barrier of the CTAs that share the subdomain
+    if constexpr (MULTI) cluster_sync();
+    else __syncthreads();
+  };
   const double scale = dscale[i] > 0 ? dscale[i] : 1.0;
   const double tiny = (Unit<T>::u < 1e-15 ? 1e-14 : 1e-12) * scale;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -249,7 +260,7 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
     const int w = min(TB, kend - k0);
     // 1. the diagonal block: LU in shared memory
     for (int e = tid; e < w * w; e += 256) Dm[(e / w) * 65 + e % w] = (Acc)A[(int64_t)(k0 + e / w) * L + k0 + e % w];
-    __syncthreads();
+    all_ctas();  // (one CTA of a cluster writes the block back: all have read it)
     // Thread (ty, tx) = (tid / 64, tid % 64) owns column tx and the rows ty, ty + 4, ...; step c subtracts
     // a21 (a12 / pivot)^T from the trailing block, and the multipliers of L are formed after the loop.
     // The owner of entry (c+1, c+1) checks the next pivot right after its own update and forms its
@@ -258,15 +269,17 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
       if (allow_last_zero && k0 + c == n - 1) {
         // record the last pivot of A~_ii and replace it by the scale; the eigensolver decides from it
         // whether A~_ii is singular
-        last_pivot[i] = (double)Dm[c * 65 + c];
+        if (rank == 0) last_pivot[i] = (double)Dm[c * 65 + c];
         Dm[c * 65 + c] = (Acc)scale;
       } else if (abs_at_most(Dm[c * 65 + c], tiny)) {
         // static pivoting: counted and replaced; otherwise an error (the replacement keeps the
         // remaining steps finite until the host reads the status)
-        if (boost)
-          atomicAdd(st + ST_BOOSTS, 1);
-        else
-          raise_status(st, A2LS_ERR_SINGULAR, i, k0 + c);
+        if (rank == 0) {
+          if (boost)
+            atomicAdd(st + ST_BOOSTS, 1);
+          else
+            raise_status(st, A2LS_ERR_SINGULAR, i, k0 + c);
+        }
         Dm[c * 65 + c] = (Acc)scale;
       }
       rdiag[c] = Acc(1.0) / Dm[c * 65 + c];
@@ -289,7 +302,8 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
       if (r > c) Dm[r * 65 + c] *= rdiag[c];
     }
     __syncthreads();
-    for (int e = tid; e < w * w; e += 256) A[(int64_t)(k0 + e / w) * L + k0 + e % w] = (T)Dm[(e / w) * 65 + e % w];
+    if (rank == 0)
+      for (int e = tid; e < w * w; e += 256) A[(int64_t)(k0 + e / w) * L + k0 + e % w] = (T)Dm[(e / w) * 65 + e % w];
     const int c0 = k0 + w;
     if (c0 >= n) break;
     // inverses of the triangles: inv(L11) strictly below the diagonal, inv(U11) on and above
@@ -318,8 +332,9 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
     }
     __syncthreads();
     // 2. L21 = A21 inv(U11), 64-row tiles
+    int dealt = 0;   // nonzero tiles so far, dealt out in turn
     for (int t = 0; t < tiles; ++t) {
-      if (!lnz[t]) continue;
+      if (!lnz[t] || dealt++ % C != rank) continue;
       const int r0 = c0 + t * TB, rows = min(TB, n - r0);
       Acc acc[4][4];
 #pragma unroll
@@ -339,7 +354,7 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
     }
     // 3. U12 = inv(L11) A12, 64-column tiles
     for (int t = 0; t < tiles; ++t) {
-      if (!unz[t]) continue;
+      if (!unz[t] || dealt++ % C != rank) continue;
       const int cs = c0 + t * TB, cols = min(TB, n - cs);
       Acc acc[4][4];
 #pragma unroll
@@ -357,19 +372,25 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
           if (r < w && c < cols) A[(int64_t)(k0 + r) * L + cs + c] = (T)finish(acc[u][v]);
         }
     }
-    __syncthreads();  // L21 and U12 complete before the trailing update reads them
+    all_ctas();  // L21 and U12 complete before the trailing update reads them
+    dealt = 0;
     // 4. A22 -= L21 U12
     if constexpr (TC) {
       const int rtiles = (n - c0 + tcdf::TM - 1) / tcdf::TM;
-      for (int rt = 0; rt < rtiles && !tc_fail; ++rt) {
+      for (int rt = 0; rt < rtiles; ++rt) {
         const int ta = 2 * rt, tb2 = 2 * rt + 1;   // the two 64-row tiles of this 128-row tile
         if (!lnz[ta] && !(tb2 < tiles && lnz[tb2])) continue;
         const int r0 = c0 + rt * tcdf::TM, rows = min(tcdf::TM, n - r0);
-        tcdf::split_a(ctx, [&](int m, int k) -> dfloat {
-          return (m < rows && k < w) ? (dfloat)A[(int64_t)(r0 + m) * L + k0 + k] : dfloat(0.f, 0.f);
-        });
+        bool have_a = false;
         for (int ct = 0; ct < tiles; ++ct) {
-          if (!unz[ct]) continue;
+          if (!unz[ct] || dealt++ % C != rank) continue;
+          if (tc_fail) continue;   // (a CTA whose wait ran out still meets the others at the barriers)
+          if (!have_a) {
+            tcdf::split_a(ctx, [&](int m, int k) -> dfloat {
+              return (m < rows && k < w) ? (dfloat)A[(int64_t)(r0 + m) * L + k0 + k] : dfloat(0.f, 0.f);
+            });
+            have_a = true;
+          }
           const int cs = c0 + ct * TB, cols = min(TB, n - cs);
           tcdf::split_b(ctx, [&](int k, int c) -> dfloat {
             return (k < w && c < cols) ? (dfloat)A[(int64_t)(k0 + k) * L + cs + c] : dfloat(0.f, 0.f);
@@ -379,7 +400,7 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
           tcdf::prefetch_rows_l2(A + (int64_t)r0 * L + cs, L * (int64_t)sizeof(T), rows, cols * (int)sizeof(T));
           {
             int nt = ct + 1;
-            while (nt < tiles && !unz[nt]) ++nt;
+            for (int skip = C - 1; nt < tiles && (!unz[nt] || skip-- > 0);) ++nt;
             if (nt < tiles) {
               const int cs2 = c0 + nt * TB;
               tcdf::prefetch_rows_l2(A + (int64_t)k0 * L + cs2, L * (int64_t)sizeof(T), w,
@@ -389,16 +410,16 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
           if (!tcdf::multiply(ctx)) {
             if (threadIdx.x == 0) raise_status(st, A2LS_ERR_TIMEOUT, i, k0);
             tc_fail = true;
-            break;
+            continue;
           }
           tcdf::epilogue_subtract(ctx, reinterpret_cast<dfloat*>(A) + (int64_t)r0 * L + cs, L, rows, cols);
         }
       }
-      __syncthreads();
-      if (tc_fail) break;
+      all_ctas();
+      if (!MULTI && tc_fail) break;
     } else {
     for (int t = 0; t < tiles * tiles; ++t) {
-      if (!lnz[t / tiles] || !unz[t % tiles]) continue;
+      if (!lnz[t / tiles] || !unz[t % tiles] || dealt++ % C != rank) continue;
       const int r0 = c0 + (t / tiles) * TB, cs = c0 + (t % tiles) * TB;
       const int rows = min(TB, n - r0), cols = min(TB, n - cs);
       Acc acc[4][4];
@@ -420,7 +441,7 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
           }
         }
     }
-    __syncthreads();
+    all_ctas();
     }
   }
   if constexpr (TC) {
@@ -433,23 +454,44 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
 template <class T>
 void lu_batched(a2ls_handle* h, T* fac, int allow_last_zero, double* last_pivot, double* diag_scale, int phase) {
   using Acc = typename AccOf<T>::type;
+  // the largest cluster (of at most 8) of which as many fit the chip at once as there are subdomains
+  auto go = [&](auto one, auto multi, size_t smem) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = h->st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    A2LS_CUDA(cudaFuncSetAttribute(one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    A2LS_CUDA(cudaFuncSetAttribute(multi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int C = 8;
+    for (; C > 1; C /= 2) {
+      int fit = 0;
+      cfg.gridDim = dim3(h->N * C);
+      at[0].val.clusterDim.x = C;
+      A2LS_CUDA(cudaOccupancyMaxActiveClusters(&fit, multi, &cfg));
+      if (h->N <= fit) break;
+    }
+    cfg.gridDim = dim3(h->N * C);
+    at[0].val.clusterDim.x = C;
+    auto kernel = C > 1 ? multi : one;
+    A2LS_CUDA(cudaLaunchKernelEx(&cfg, kernel, h->N, (const int*)h->d_ni, (const int*)h->d_ld,
+                                 (const int64_t*)h->d_foff, fac, allow_last_zero, last_pivot,
+                                 (const double*)diag_scale, h->d_status, (const int*)h->d_sched, (const int*)h->d_nI,
+                                 phase, (const int*)h->d_off, (const int*)h->d_pf, (const int*)h->d_pg,
+                                 (int)h->opt.static_pivoting));
+    A2LS_LAUNCH();
+  };
   if constexpr (std::is_same<T, dfloat>::value) {
     if (h->opt.tensor_cores) {
-      const size_t smem = std::max(lu_smem_elems() * sizeof(Acc), tcdf::SMEM_BYTES);
-      A2LS_CUDA(cudaFuncSetAttribute(k_lu<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      k_lu<T, true><<<h->N, 256, smem, h->st>>>(h->N, h->d_ni, h->d_ld, h->d_foff, fac, allow_last_zero, last_pivot,
-                                                diag_scale, h->d_status, h->d_sched, h->d_nI, phase, h->d_off,
-                                                h->d_pf, h->d_pg, h->opt.static_pivoting);
-      A2LS_LAUNCH();
+      go(k_lu<T, true, false>, k_lu<T, true, true>, std::max(lu_smem_elems() * sizeof(Acc), tcdf::SMEM_BYTES));
       return;
     }
   }
-  const size_t smem = lu_smem_elems() * sizeof(Acc);
-  A2LS_CUDA(cudaFuncSetAttribute(k_lu<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_lu<T, false><<<h->N, 256, smem, h->st>>>(h->N, h->d_ni, h->d_ld, h->d_foff, fac, allow_last_zero, last_pivot,
-                                             diag_scale, h->d_status, h->d_sched, h->d_nI, phase, h->d_off, h->d_pf,
-                                             h->d_pg, h->opt.static_pivoting);
-  A2LS_LAUNCH();
+  go(k_lu<T, false, false>, k_lu<T, false, true>, lu_smem_elems() * sizeof(Acc));
 }
 
 // A_ii from the splitting's partial factorisation.  A~_ii differs from A_ii only on the diagonal of the
@@ -1149,7 +1191,7 @@ namespace a2ls {
 // Factor the 64x64 diagonal block at (k0, k0) and invert its triangles in place, in the arithmetic
 // and storage R (FP64, or double-float in the mixed form).  One CTA, one step of a chain as long as the
 // matrix, so every step counts: double-float takes 1024 threads (a quarter of the rows and of the inverses'
-// terms each: E_DIAG_TIMES), FP64, whose pipe is the limit, 256.
+// terms each: 99 us a launch with 256, 85 with 1024), FP64, whose pipe is the limit, 256.
 // LU: thread (ty, tx) = (tid / 64, tid % 64) owns column tx and the rows ty, ty + NG, ...; step c
 // subtracts a21 (a12 / pivot)^T from the trailing block, so that the multipliers of column c are
 // formed only once, after the loop (l_rc = a_rc / pivot_c).  The owner of entry (c+1, c+1) checks the

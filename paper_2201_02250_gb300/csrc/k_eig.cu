@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(EIG_THREADS) k_project_k(const int* ni, const 
     __syncthreads();
   } else {
     // a lane per column, the rows spread over the warps: whole rows are read at once (a warp per column read
-    // 32 rows 768 bytes apart for each load: PROJ_TIMES)
+    // 32 rows 768 bytes apart for each load: 94 us a launch with 64 subdomains of 1100 rows, 68 so)
     constexpr int NW = EIG_THREADS / 32;
     __shared__ Acc part[NW][32];
     for (int c0 = 0; c0 < p; c0 += 32) {
@@ -611,21 +611,7 @@ __device__ int warp_cholesky_inverse(double* G, int p, double* Ri, double* dsc, 
   return ok;
 }
 
-// Thread-block clusters: the CTA's rank and count, the barrier over all threads of the cluster, and a
-// double of another CTA's shared memory.
-__device__ __forceinline__ int cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return (int)r;
-}
-__device__ __forceinline__ int cluster_size() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-  return (int)r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+// a double of another CTA's shared memory
 __device__ __forceinline__ double cluster_ld(const double* p, int rank) {
   uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
   double v;
@@ -1287,7 +1273,8 @@ __global__ void __launch_bounds__(TR_THREADS) k_thick_restart(const int* active,
   const int i = blockIdx.x;
   if (active && !active[i]) return;
   // an odd row stride: a column's entries, which the lanes of a warp hold, fall on different shared-memory
-  // banks (with 2 b every lane met the same one: TR_TIMES)
+  // banks (with 2 b every lane met the same one: 1.13 ms a launch
+  // at 48 columns of 96 rows in double-float, 0.80 so)
   const int tid = threadIdx.x, mb = m + b, b2 = 2 * b, ld = b2 + 1;
   R* U = reinterpret_cast<R*>(sm);  // mb x 2b, stride ld
   R* Gs = U + mb * ld;              // b x b

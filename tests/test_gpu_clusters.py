@@ -33,3 +33,11 @@ def test_clustered_orthogonalisation_matches_oracle(m, nb, eigp):
     it, rr, ok = P.solve(b, x, 1e-8)
     want = O.gmres(prob.A, lambda v: O.apply(ref, v), r, rtol=1e-8)
     assert ok and abs(it - want.iters) <= 1
+
+
+@pytest.mark.parametrize("eigp", ["fp64", "fp32x2"])
+@pytest.mark.parametrize("m,nb", [(47, 2), (83, 5), (112, 7)])   # clusters of 8, 4 and 2 CTAs (FP64: 8, 8 and 4)
+def test_clustered_factorisation_matches_oracle(m, nb, eigp):
+    """Subdomains of 300 to 650 rows, whose 5 to 11 ragged tiles a block column are dealt to the CTAs of a cluster:
+    the quantities and the bounds of the test above, which the factors of both matrices enter."""
+    test_clustered_orthogonalisation_matches_oracle(m, nb, eigp)
