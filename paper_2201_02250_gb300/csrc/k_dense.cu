@@ -202,28 +202,41 @@ __device__ __forceinline__ void tile_gemm(FA fa, FB fb, int K, Acc (&acc)[4][4],
 // overlap rows is left in place); 1 the remaining columns [n_I, n).
 constexpr size_t lu_smem_elems() { return 2 * (size_t)TB * 65 + 2 * (size_t)TGK * TS; }
 
-// TC (double-float only): the trailing update A22 -= L21 U12 runs on the tensor cores as digit-split
-// BF16 products (tc_dfloat.cuh) in 128 x 64 tiles; its operand digits reuse the shared memory of the
-// other steps, so one CTA runs per SM, holding all of that SM's TMEM.
+// TC (double-float only): L21, U12 and the trailing update A22 -= L21 U12 run on the tensor cores as digit-split
+// BF16 products (tc_dfloat.cuh); their operand digits and the staging of a tile take most of the shared memory, so
+// one CTA of 512 threads runs per SM, holding all of that SM's TMEM.  A tile's cost is the splitting of its
+// operands and the double-float arithmetic on its results, not the MMAs: these run while the old values and the
+// next operand are on their way.  304 matrices of 1728 rows: 43.1 ms with L21 and U12 on the FP32 pipe and 256
+// threads that waited for each tile's MMAs, 32.8 with this order of a tile and digit products throughout, 28.2 with
+// 512 threads (18.4 at the copy bandwidth for what the right-looking order reads and writes); 512 subdomains of
+// 2200 to 2744 rows, interior columns, 146 -> 106 ms.  Against a long double factorisation L and U are as exact as
+// with FP32-pipe L21 and U12 (convection-diffusion L 6.0e-15, before 6.1e-15; lognormal 1.9e-14, 1.9e-14; jumps of
+// 1e6 1.8e-10, 1.7e-10, and 1.4e-10 with nothing on the tensor cores).  Only where rows and columns are both
+// scaled by random factors of 10^-3 to 10^3 does L lose digits (5e-12, before 9e-14; the backward error is 8e-15
+// both): digits are relative to the largest entry of a row of A21 (tc_dfloat.cuh).
 //
 // MULTI: with fewer subdomains than SMs a cluster of CTAs takes each one.  Every CTA factors the diagonal
 // block for itself, the tiles of L21, U12 and of the trailing matrix are dealt out, and cluster barriers, which
 // also order the CTAs' global memory accesses, separate the two.  A tile's arithmetic does not depend on who
 // does it.  One CTA each against clusters, per launch: FP64, 64 subdomains of 1700 to 2200 rows, 239 ms against
-// 91 (of 4 CTAs, two an SM); double-float, 64 subdomains of 1100 to 1250 rows, 5.4 ms against 3.8 (of 2).
+// 91 (of 4 CTAs, two an SM); double-float before the steps above, 64 subdomains of 1100 to 1250 rows, 5.4 ms
+// against 3.8 (of 2).
+template <bool TC> struct LuThreads { static constexpr int value = 256; };
+template <> struct LuThreads<true> { static constexpr int value = tcdf::THREADS; };
 template <class T, bool TC, bool MULTI>
-__global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, const int* ld, const int64_t* foff,
+__global__ void __launch_bounds__(LuThreads<TC>::value, TC ? 1 : 2) k_lu(int N, const int* ni, const int* ld, const int64_t* foff,
                                             T* fac, int allow_last_zero, double* last_pivot,
                                             const double* dscale, int* st, const int* sched, const int* nI,
                                             int phase, const int* off, const int* pf, const int* pg, int boost) {
   using Acc = typename AccOf<T>::type;
+  constexpr int NT = LuThreads<TC>::value, NG = NT / 64;
   static_assert(!TC || std::is_same<T, dfloat>::value, "tensor-core trailing update is for double-float");
   extern __shared__ __align__(16) unsigned char lu_smem_raw[];
   __shared__ unsigned char lnz[MAXN_LOCAL / TB + 1], unz[MAXN_LOCAL / TB + 1];
   __shared__ __align__(8) uint64_t tc_bar;
   __shared__ uint32_t tc_base;
-  __shared__ int tc_eA[TC ? tcdf::TM : 1], tc_eB[TC ? tcdf::TN : 1];
-  __shared__ float tc_red[TC ? 4 * tcdf::TN : 1];
+  __shared__ int tc_eA[TC ? tcdf::TM : 1], tc_eB[TC ? 2 * tcdf::TN : 1];
+  __shared__ float tc_red[TC ? 8 * tcdf::TN : 1];
   tcdf::Ctx ctx{lu_smem_raw, &tc_bar, 0u, 0u, tc_eA, tc_eB};
   bool tc_fail = false;
   if constexpr (TC) {
@@ -239,7 +252,8 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
   }
   __shared__ Acc rdiag[TB];                       // reciprocals of the diagonal block's pivots
   Acc* Dm = reinterpret_cast<Acc*>(lu_smem_raw);  // 64 x 65: the diagonal block, factored in place
-  Acc* Iv = Dm + TB * 65;                         // 64 x 65: inv(L11) strictly below, inv(U11) on/above
+  // 64 x 65: inv(L11) strictly below, inv(U11) on/above (TC: past the digits, which take Dm's place)
+  Acc* Iv = TC ? reinterpret_cast<Acc*>(lu_smem_raw + tcdf::SMEM_BYTES) : Dm + TB * 65;
   Acc* sA = Iv + TB * 65;                         // TGK x TS (16-byte aligned: 2 * 64 * 65 is even)
   Acc* sB = sA + TGK * TS;                        // TGK x TS
   const int C = MULTI ? cluster_size() : 1, rank = MULTI ? cluster_rank() : 0;
@@ -259,9 +273,9 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
   for (int k0 = kbeg; k0 < kend; k0 += TB) {
     const int w = min(TB, kend - k0);
     // 1. the diagonal block: LU in shared memory
-    for (int e = tid; e < w * w; e += 256) Dm[(e / w) * 65 + e % w] = (Acc)A[(int64_t)(k0 + e / w) * L + k0 + e % w];
+    for (int e = tid; e < w * w; e += NT) Dm[(e / w) * 65 + e % w] = (Acc)A[(int64_t)(k0 + e / w) * L + k0 + e % w];
     all_ctas();  // (one CTA of a cluster writes the block back: all have read it)
-    // Thread (ty, tx) = (tid / 64, tid % 64) owns column tx and the rows ty, ty + 4, ...; step c subtracts
+    // Thread (ty, tx) = (tid / 64, tid % 64) owns column tx and the rows ty, ty + NG, ...; step c subtracts
     // a21 (a12 / pivot)^T from the trailing block, and the multipliers of L are formed after the loop.
     // The owner of entry (c+1, c+1) checks the next pivot right after its own update and forms its
     // reciprocal in the working arithmetic, so each step needs one barrier.
@@ -291,29 +305,29 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
       for (int c = 0; c + 1 < w; ++c) {
         if (cx > c && cx < w) {
           const Acc u = Dm[c * 65 + cx] * rdiag[c];
-          for (int r = c + 1 + ((ry - c - 1) & 3); r < w; r += 4) Dm[r * 65 + cx] -= Dm[r * 65 + c] * u;
-          if (cx == c + 1 && ry == ((c + 1) & 3)) pivot(c + 1);
+          for (int r = c + 1 + ((ry - c - 1) & (NG - 1)); r < w; r += NG) Dm[r * 65 + cx] -= Dm[r * 65 + c] * u;
+          if (cx == c + 1 && ry == ((c + 1) & (NG - 1))) pivot(c + 1);
         }
         __syncthreads();
       }
     }
-    for (int e = tid; e < w * w; e += 256) {
+    for (int e = tid; e < w * w; e += NT) {
       const int r = e / w, c = e % w;
       if (r > c) Dm[r * 65 + c] *= rdiag[c];
     }
     __syncthreads();
     if (rank == 0)
-      for (int e = tid; e < w * w; e += 256) A[(int64_t)(k0 + e / w) * L + k0 + e % w] = (T)Dm[(e / w) * 65 + e % w];
+      for (int e = tid; e < w * w; e += NT) A[(int64_t)(k0 + e / w) * L + k0 + e % w] = (T)Dm[(e / w) * 65 + e % w];
     const int c0 = k0 + w;
     if (c0 >= n) break;
     // inverses of the triangles: inv(L11) strictly below the diagonal, inv(U11) on and above
-    tile_inverses<Acc>(reinterpret_cast<const Acc(*)[TB + 1]>(Dm), reinterpret_cast<Acc(*)[TB + 1]>(Iv), rdiag, w);
+    tile_inverses<Acc, NT / 128>(reinterpret_cast<const Acc(*)[TB + 1]>(Dm), reinterpret_cast<Acc(*)[TB + 1]>(Iv), rdiag, w);
     const int tiles = (n - c0 + TB - 1) / TB;
     // envelope: a row tile of L21 is nonzero only if one of its rows starts left of c0, a column tile
     // of U12 only if one of its columns starts above c0
     {
       const int lane = tid & 31, warp = tid >> 5, o = off[i];
-      for (int t = warp; t < tiles; t += 8) {
+      for (int t = warp; t < tiles; t += NT / 32) {
         const int a0 = c0 + t * TB, a1 = min(n, a0 + TB);
         int fm = n, gm = n;
         for (int r = a0 + lane; r < a1; r += 32) {
@@ -331,88 +345,176 @@ __global__ void __launch_bounds__(256, TC ? 1 : 2) k_lu(int N, const int* ni, co
       }
     }
     __syncthreads();
-    // 2. L21 = A21 inv(U11), 64-row tiles
+    // 2. L21 = A21 inv(U11) and 3. U12 = inv(L11) A12
     int dealt = 0;   // nonzero tiles so far, dealt out in turn
-    for (int t = 0; t < tiles; ++t) {
-      if (!lnz[t] || dealt++ % C != rank) continue;
-      const int r0 = c0 + t * TB, rows = min(TB, n - r0);
-      Acc acc[4][4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0;
-      tile_gemm<Acc>([&](int m, int k) -> Acc { return (m < rows && k < w) ? (Acc)A[(int64_t)(r0 + m) * L + k0 + k] : (Acc)0; },
-                     [&](int k, int c) -> Acc { return (k < w && c < w && c >= k) ? Iv[k * 65 + c] : (Acc)0; },
-                     w, acc, sA, sB);
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const int r = ty * 4 + u, c = tx * 4 + v;
-          if (r < rows && c < w) A[(int64_t)(r0 + r) * L + k0 + c] = (T)finish(acc[u][v]);
+    if constexpr (TC) {
+      auto multiply = [&]() {   // the tile product; false (in every thread) once a wait has run out
+        tcdf::issue(ctx);
+        if (!tcdf::wait(ctx)) {
+          if (tid == 0) raise_status(st, A2LS_ERR_TIMEOUT, i, k0);
+          tc_fail = true;
         }
-    }
-    // 3. U12 = inv(L11) A12, 64-column tiles
-    for (int t = 0; t < tiles; ++t) {
-      if (!unz[t] || dealt++ % C != rank) continue;
-      const int cs = c0 + t * TB, cols = min(TB, n - cs);
-      Acc acc[4][4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0;
-      tile_gemm<Acc>([&](int m, int k) -> Acc { return (m < w && k < w) ? (k < m ? Iv[m * 65 + k] : (k == m ? (Acc)1 : (Acc)0)) : (Acc)0; },
-                     [&](int k, int c) -> Acc { return (k < w && c < cols) ? (Acc)A[(int64_t)(k0 + k) * L + cs + c] : (Acc)0; },
-                     w, acc, sA, sB);
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const int r = ty * 4 + u, c = tx * 4 + v;
-          if (r < w && c < cols) A[(int64_t)(k0 + r) * L + cs + c] = (T)finish(acc[u][v]);
+        return !tc_fail;
+      };
+      const int pairs = (tiles + 1) / 2, warp = tid >> 5, lane = tid & 31;
+      dfloat vb[8];
+      ctx.eB = tc_eB;
+      // L21, 128 rows a tile; staged where the A digits were
+      tcdf::load_b([&](int k, int c) -> dfloat { return c >= k && c < w ? Iv[k * 65 + c] : dfloat(0.f, 0.f); }, vb);
+      tcdf::write_b(ctx, vb, tc_red);
+      dfloat* S = reinterpret_cast<dfloat*>(lu_smem_raw);
+      for (int t = 0; t < pairs; ++t) {
+        if (!lnz[2 * t] && !(2 * t + 1 < tiles && lnz[2 * t + 1])) continue;
+        if (dealt++ % C != rank || tc_fail) continue;
+        T* P = A + (int64_t)(c0 + t * tcdf::TM) * L + k0;
+        const int rows = min(tcdf::TM, n - c0 - t * tcdf::TM);
+        tcdf::split_a(ctx, [&](int m, int k) -> dfloat {
+          return m < rows && k < w ? (dfloat)P[(int64_t)m * L + k] : dfloat(0.f, 0.f);
+        });
+        if (!multiply()) continue;
+        for (int half = 0; half < 2; ++half) {
+          tcdf::stage_half(ctx, ctx.eB, half, S);
+          __syncthreads();
+          const int c = half * 32 + lane;
+          for (int r = warp; r < rows; r += NT / 32)
+            if (c < w) P[(int64_t)r * L + c] = (T)finish(S[r * tcdf::SUB_LD + lane]);
+          __syncthreads();
         }
+      }
+      // U12 as its transpose, A12^T inv(L11)^T, 128 columns a tile: a thread holds a column and a warp's
+      // accesses run along the rows of memory
+      tcdf::load_b([&](int k, int c) -> dfloat {
+        return k < c && c < w ? Iv[c * 65 + k] : dfloat(k == c && c < w ? 1.f : 0.f, 0.f);
+      }, vb);
+      tcdf::write_b(ctx, vb, tc_red);
+      for (int t = 0; t < pairs; ++t) {
+        if (!unz[2 * t] && !(2 * t + 1 < tiles && unz[2 * t + 1])) continue;
+        if (dealt++ % C != rank || tc_fail) continue;
+        T* P = A + (int64_t)k0 * L + c0 + t * tcdf::TM;
+        const int cols = min(tcdf::TM, n - c0 - t * tcdf::TM);
+        tcdf::split_a(ctx, [&](int m, int k) -> dfloat {
+          return m < cols && k < w ? (dfloat)P[(int64_t)k * L + m] : dfloat(0.f, 0.f);
+        });
+        if (!multiply()) continue;
+        const int m = (warp & 3) * 32 + lane;
+#pragma unroll 1
+        for (int cb = (warp >> 2) * 16, ce = cb + 16; cb < ce; cb += 8)
+          tcdf::product8(ctx, ctx.eB, cb, [&](int r, dfloat v) {
+            if (m < cols && r < w) P[(int64_t)r * L + m] = (T)finish(v);
+          });
+        __syncthreads();
+      }
+    } else {
+      for (int t = 0; t < tiles; ++t) {
+        if (!lnz[t] || dealt++ % C != rank) continue;
+        const int r0 = c0 + t * TB, rows = min(TB, n - r0);
+        Acc acc[4][4];
+  #pragma unroll
+        for (int u = 0; u < 4; ++u)
+  #pragma unroll
+          for (int v = 0; v < 4; ++v) acc[u][v] = 0;
+        tile_gemm<Acc>([&](int m, int k) -> Acc { return (m < rows && k < w) ? (Acc)A[(int64_t)(r0 + m) * L + k0 + k] : (Acc)0; },
+                       [&](int k, int c) -> Acc { return (k < w && c < w && c >= k) ? Iv[k * 65 + c] : (Acc)0; },
+                       w, acc, sA, sB);
+  #pragma unroll
+        for (int u = 0; u < 4; ++u)
+  #pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const int r = ty * 4 + u, c = tx * 4 + v;
+            if (r < rows && c < w) A[(int64_t)(r0 + r) * L + k0 + c] = (T)finish(acc[u][v]);
+          }
+      }
+      // 64-column tiles of U12
+      for (int t = 0; t < tiles; ++t) {
+        if (!unz[t] || dealt++ % C != rank) continue;
+        const int cs = c0 + t * TB, cols = min(TB, n - cs);
+        Acc acc[4][4];
+  #pragma unroll
+        for (int u = 0; u < 4; ++u)
+  #pragma unroll
+          for (int v = 0; v < 4; ++v) acc[u][v] = 0;
+        tile_gemm<Acc>([&](int m, int k) -> Acc { return (m < w && k < w) ? (k < m ? Iv[m * 65 + k] : (k == m ? (Acc)1 : (Acc)0)) : (Acc)0; },
+                       [&](int k, int c) -> Acc { return (k < w && c < cols) ? (Acc)A[(int64_t)(k0 + k) * L + cs + c] : (Acc)0; },
+                       w, acc, sA, sB);
+  #pragma unroll
+        for (int u = 0; u < 4; ++u)
+  #pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const int r = ty * 4 + u, c = tx * 4 + v;
+            if (r < w && c < cols) A[(int64_t)(k0 + r) * L + cs + c] = (T)finish(acc[u][v]);
+          }
+      }
     }
     all_ctas();  // L21 and U12 complete before the trailing update reads them
     dealt = 0;
     // 4. A22 -= L21 U12
     if constexpr (TC) {
-      const int rtiles = (n - c0 + tcdf::TM - 1) / tcdf::TM;
+      // 128 x 64 tiles.  While a tile's MMAs run its old values and the next tile's U12 block are loaded into
+      // registers; then the next tile's digits are written, the product leaves TMEM by way of the staging buffer
+      // (half of it at a time), and the next MMAs start before its second half goes to memory.
+      const int rtiles = (n - c0 + tcdf::TM - 1) / tcdf::TM, warp = tid >> 5, lane = tid & 31;
+      dfloat* S = reinterpret_cast<dfloat*>(lu_smem_raw + tcdf::SMEM_BYTES);
+      auto next_tile = [&](int t) {   // the next column tile at or after t that is this CTA's
+        while (t < tiles && (!unz[t] || dealt++ % C != rank)) ++t;
+        return t;
+      };
+      auto load_u12 = [&](int ct, dfloat (&v)[8]) {
+        const T* P = A + (int64_t)k0 * L + c0 + ct * TB;
+        const int cols = min(TB, n - c0 - ct * TB);
+        tcdf::load_b([&](int k, int c) -> dfloat {
+          return k < w && c < cols ? (dfloat)P[(int64_t)k * L + c] : dfloat(0.f, 0.f);
+        }, v);
+      };
       for (int rt = 0; rt < rtiles; ++rt) {
         const int ta = 2 * rt, tb2 = 2 * rt + 1;   // the two 64-row tiles of this 128-row tile
         if (!lnz[ta] && !(tb2 < tiles && lnz[tb2])) continue;
+        int ct = next_tile(0);
+        if (ct >= tiles || tc_fail) continue;   // (a CTA whose wait ran out still meets the others at the barriers)
         const int r0 = c0 + rt * tcdf::TM, rows = min(tcdf::TM, n - r0);
-        bool have_a = false;
-        for (int ct = 0; ct < tiles; ++ct) {
-          if (!unz[ct] || dealt++ % C != rank) continue;
-          if (tc_fail) continue;   // (a CTA whose wait ran out still meets the others at the barriers)
-          if (!have_a) {
-            tcdf::split_a(ctx, [&](int m, int k) -> dfloat {
-              return (m < rows && k < w) ? (dfloat)A[(int64_t)(r0 + m) * L + k0 + k] : dfloat(0.f, 0.f);
-            });
-            have_a = true;
-          }
-          const int cs = c0 + ct * TB, cols = min(TB, n - cs);
-          tcdf::split_b(ctx, [&](int k, int c) -> dfloat {
-            return (k < w && c < cols) ? (dfloat)A[(int64_t)(k0 + k) * L + cs + c] : dfloat(0.f, 0.f);
-          }, tc_red);
-          // while the MMAs run: this tile's A22 rows (read by the epilogue) and the next column tile of
-          // U12 (read by the next split) into L2
-          tcdf::prefetch_rows_l2(A + (int64_t)r0 * L + cs, L * (int64_t)sizeof(T), rows, cols * (int)sizeof(T));
-          {
-            int nt = ct + 1;
-            for (int skip = C - 1; nt < tiles && (!unz[nt] || skip-- > 0);) ++nt;
-            if (nt < tiles) {
-              const int cs2 = c0 + nt * TB;
-              tcdf::prefetch_rows_l2(A + (int64_t)k0 * L + cs2, L * (int64_t)sizeof(T), w,
-                                     min(TB, n - cs2) * (int)sizeof(T));
+        dfloat vb[8];
+        load_u12(ct, vb);
+        tcdf::split_a(ctx, [&](int m, int k) -> dfloat {
+          return (m < rows && k < w) ? (dfloat)A[(int64_t)(r0 + m) * L + k0 + k] : dfloat(0.f, 0.f);
+        });
+        tcdf::write_b(ctx, vb, tc_red);
+        tcdf::issue(ctx);
+        while (true) {
+          const int cols = min(TB, n - c0 - ct * TB);
+          T* P = A + (int64_t)r0 * L + c0 + ct * TB;
+          dfloat old[2][8];
+#pragma unroll
+          for (int half = 0; half < 2; ++half)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const int r = warp + 16 * q, c = half * 32 + lane;
+              old[half][q] = r < rows && c < cols ? (dfloat)P[(int64_t)r * L + c] : dfloat(0.f, 0.f);
             }
-          }
-          if (!tcdf::multiply(ctx)) {
-            if (threadIdx.x == 0) raise_status(st, A2LS_ERR_TIMEOUT, i, k0);
+          const int nt = next_tile(ct + 1);
+          if (nt < tiles) load_u12(nt, vb);
+          if (!tcdf::wait(ctx)) {
+            if (tid == 0) raise_status(st, A2LS_ERR_TIMEOUT, i, k0);
             tc_fail = true;
-            continue;
+            break;
           }
-          tcdf::epilogue_subtract(ctx, reinterpret_cast<dfloat*>(A) + (int64_t)r0 * L + cs, L, rows, cols);
+          const int* eB = ctx.eB;
+          if (nt < tiles) {
+            ctx.eB = eB == tc_eB ? tc_eB + tcdf::TN : tc_eB;
+            tcdf::write_b(ctx, vb, tc_red);
+          }
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            tcdf::stage_half(ctx, eB, half, S);
+            if (half == 1 && nt < tiles) tcdf::issue(ctx);
+            else __syncthreads();
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const int r = warp + 16 * q, c = half * 32 + lane;
+              if (r < rows && c < cols) P[(int64_t)r * L + c] = (T)(old[half][q] - S[r * tcdf::SUB_LD + lane]);
+            }
+            if (half == 0) __syncthreads();
+          }
+          if (nt >= tiles) break;
+          ct = nt;
         }
       }
       all_ctas();
@@ -455,10 +557,10 @@ template <class T>
 void lu_batched(a2ls_handle* h, T* fac, int allow_last_zero, double* last_pivot, double* diag_scale, int phase) {
   using Acc = typename AccOf<T>::type;
   // the largest cluster (of at most 8) of which as many fit the chip at once as there are subdomains
-  auto go = [&](auto one, auto multi, size_t smem) {
+  auto go = [&](auto one, auto multi, size_t smem, int threads) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
-    cfg.blockDim = dim3(256);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = h->st;
     cfg.attrs = at;
@@ -487,11 +589,12 @@ void lu_batched(a2ls_handle* h, T* fac, int allow_last_zero, double* last_pivot,
   };
   if constexpr (std::is_same<T, dfloat>::value) {
     if (h->opt.tensor_cores) {
-      go(k_lu<T, true, false>, k_lu<T, true, true>, std::max(lu_smem_elems() * sizeof(Acc), tcdf::SMEM_BYTES));
+      go(k_lu<T, true, false>, k_lu<T, true, true>, tcdf::SMEM_BYTES + tcdf::STAGE_BYTES,
+         LuThreads<true>::value);
       return;
     }
   }
-  go(k_lu<T, false, false>, k_lu<T, false, true>, lu_smem_elems() * sizeof(Acc));
+  go(k_lu<T, false, false>, k_lu<T, false, true>, lu_smem_elems() * sizeof(Acc), LuThreads<false>::value);
 }
 
 // A_ii from the splitting's partial factorisation.  A~_ii differs from A_ii only on the diagonal of the

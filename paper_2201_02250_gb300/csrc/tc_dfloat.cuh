@@ -1,5 +1,5 @@
-// Double-float tile products on the tensor cores: C(128 x 64) -= A(128 x 64) B(64 x 64), where A, B
-// and C hold double-float values, computed with BF16 x BF16 -> FP32 tcgen05 MMAs.
+// Double-float tile products on the tensor cores: A(128 x 64) B(64 x 64) of double-float values, computed with
+// BF16 x BF16 -> FP32 tcgen05 MMAs.
 //
 // Method (an error-free splitting in the manner of Ozaki, Ogita, Oishi and Rump, "Error-free
 // transformations of matrix multiplication by using fast routines of matrix multiplication and its
@@ -36,6 +36,7 @@ constexpr uint32_t A_DIGIT_BYTES = TM * TK * 2;
 constexpr uint32_t B_DIGIT_BYTES = TN * TK * 2;
 constexpr size_t SMEM_BYTES = (size_t)NDIG * (A_DIGIT_BYTES + B_DIGIT_BYTES);   // 172032
 constexpr uint32_t TMEM_COLS = 512;
+constexpr int THREADS = 512;                 // of the CTA that calls the functions of a tile below
 constexpr long WAIT_LIMIT = 1L << 26;        // polls of the completion barrier before giving up
 
 // 2^k as a float for k in [-126, 127]
@@ -102,65 +103,67 @@ struct Ctx {
   uint32_t tmem;         // TMEM base address (TMEM_COLS columns)
   uint32_t phase;        // parity of the next completion
   int* eA;               // shared, TM row exponents
-  int* eB;               // shared, TN column exponents
+  int* eB;               // shared, TN column exponents (of the B written last)
 };
 
-// A digits: rows [0, TM) x k [0, TK) of A(m, k) = fa(m, k) (zero outside), 256 threads: two per row.
+// A digits: rows [0, TM) x k [0, TK) of A(m, k) = fa(m, k) (zero outside): four threads per row.
 template <class FA>
 __device__ __forceinline__ void split_a(Ctx& c, FA fa) {
-  const int tid = threadIdx.x, r = tid >> 1, h = tid & 1;
-  dfloat v[32];
-  float mx = 0.f;
-#pragma unroll
-  for (int q = 0; q < 32; ++q) {
-    v[q] = fa(r, h * 32 + q);
-    mx = fmaxf(mx, fabsf(v[q].hi));
-  }
-  mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-  const int e = scale_exponent(mx);
-  if (h == 0) c.eA[r] = e;
-#pragma unroll
-  for (int q8 = 0; q8 < 4; ++q8) {
-    float dg[8][NDIG];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) df_digits(v[q8 * 8 + q], e, dg[q]);
-    const uint32_t off = tc::operand_offset(r, h * 32 + q8 * 8, TK);
-#pragma unroll
-    for (int s = 0; s < NDIG; ++s) *reinterpret_cast<uint4*>(c.smem + s * A_DIGIT_BYTES + off) = pack_digits(dg, s);
-  }
-}
-
-// B digits: k [0, TK) x columns [0, TN) of B(k, n) = fb(k, n), stored as the K-major operand (n, k);
-// 256 threads: column n = tid % 64, k quarter tid / 64.  red: shared scratch of 4 x TN floats.
-template <class FB>
-__device__ __forceinline__ void split_b(Ctx& c, FB fb, float* red) {
-  const int tid = threadIdx.x, n = tid & (TN - 1), qk = tid >> 6;
+  const int tid = threadIdx.x, r = tid >> 2, h = tid & 3;
   dfloat v[16];
   float mx = 0.f;
 #pragma unroll
   for (int q = 0; q < 16; ++q) {
-    v[q] = fb(qk * 16 + q, n);
+    v[q] = fa(r, h * 16 + q);
     mx = fmaxf(mx, fabsf(v[q].hi));
   }
-  red[qk * TN + n] = mx;
-  __syncthreads();
-  mx = fmaxf(fmaxf(red[n], red[TN + n]), fmaxf(red[2 * TN + n], red[3 * TN + n]));
+  mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+  mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
   const int e = scale_exponent(mx);
-  if (qk == 0) c.eB[n] = e;
+  if (h == 0) c.eA[r] = e;
 #pragma unroll
   for (int q8 = 0; q8 < 2; ++q8) {
     float dg[8][NDIG];
 #pragma unroll
     for (int q = 0; q < 8; ++q) df_digits(v[q8 * 8 + q], e, dg[q]);
-    const uint32_t off = tc::operand_offset(n, qk * 16 + q8 * 8, TK);
+    const uint32_t off = tc::operand_offset(r, h * 16 + q8 * 8, TK);
 #pragma unroll
-    for (int s = 0; s < NDIG; ++s) *reinterpret_cast<uint4*>(c.smem + NDIG * A_DIGIT_BYTES + s * B_DIGIT_BYTES + off) = pack_digits(dg, s);
+    for (int s = 0; s < NDIG; ++s) *reinterpret_cast<uint4*>(c.smem + s * A_DIGIT_BYTES + off) = pack_digits(dg, s);
   }
 }
 
-// After split_a / split_b by all threads: the 40 MMAs of the 28 digit pairs, issued by thread 0, then
-// a bounded wait by every thread.  Returns false (on every thread) if the products did not complete.
-__device__ __forceinline__ bool multiply(Ctx& c) {
+// B digits: k [0, TK) x columns [0, TN) of B(k, n) = fb(k, n), stored as the K-major operand (n, k); column
+// n = tid % 64, k eighth tid / 64.  red: shared scratch of 8 x TN floats.  In two parts, so that the loads can be
+// in flight during the MMAs of another tile: load_b, and write_b once the B region is free.
+template <class FB>
+__device__ __forceinline__ void load_b(FB fb, dfloat (&v)[8]) {
+  const int tid = threadIdx.x, n = tid & (TN - 1), qk = tid >> 6;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v[q] = fb(qk * 8 + q, n);
+}
+__device__ __forceinline__ void write_b(Ctx& c, const dfloat (&v)[8], float* red) {
+  const int tid = threadIdx.x, n = tid & (TN - 1), qk = tid >> 6;
+  float mx = 0.f;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) mx = fmaxf(mx, fabsf(v[q].hi));
+  red[qk * TN + n] = mx;
+  __syncthreads();
+  mx = 0.f;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) mx = fmaxf(mx, red[q * TN + n]);
+  const int e = scale_exponent(mx);
+  if (qk == 0) c.eB[n] = e;
+  float dg[8][NDIG];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) df_digits(v[q], e, dg[q]);
+  const uint32_t off = tc::operand_offset(n, qk * 8, TK);
+#pragma unroll
+  for (int s = 0; s < NDIG; ++s) *reinterpret_cast<uint4*>(c.smem + NDIG * A_DIGIT_BYTES + s * B_DIGIT_BYTES + off) = pack_digits(dg, s);
+}
+
+// After split_a and write_b by all threads (and their last product8 of an earlier tile): the 40 MMAs of the 28
+// digit pairs, issued by thread 0.  Contains a barrier.
+__device__ __forceinline__ void issue(Ctx& c) {
   tc::fence_proxy_async();
   tc::fence_before_sync();
   __syncthreads();
@@ -187,72 +190,50 @@ __device__ __forceinline__ bool multiply(Ctx& c) {
     tc::commit(c.bar);
   }
   __syncwarp();
+}
+
+// A bounded wait by every thread for the MMAs issued last.  Returns false (on every thread) if they did not
+// complete.
+__device__ __forceinline__ bool wait(Ctx& c) {
   const bool ok = tc::mbar_wait_bounded(c.bar, c.phase, WAIT_LIMIT);
   c.phase ^= 1u;
   tc::fence_after_sync();
   return __syncthreads_and(ok) != 0;
 }
 
-// L2 prefetch of rows [0, rows) x bytes [0, row_bytes) starting at base with the given row pitch,
-// spread over the CTA (one 128-byte line per request)
-__device__ __forceinline__ void prefetch_rows_l2(const void* base, int64_t pitch_bytes, int rows, int row_bytes) {
-  // one request per 128-byte line the row's bytes touch, at the line's aligned start (a row may start
-  // anywhere in a line; no request reaches past the row's last byte's line)
-  if (row_bytes <= 0) return;
-  const int lines = (row_bytes + 127) / 128 + 1;
-  for (int e = threadIdx.x; e < rows * lines; e += blockDim.x) {
-    const uintptr_t first = reinterpret_cast<uintptr_t>(base) + (uintptr_t)((e / lines) * pitch_bytes);
-    const uintptr_t line = (first & ~(uintptr_t)127) + (uintptr_t)(e % lines) * 128;
-    if (line <= first + row_bytes - 1) asm volatile("prefetch.global.L2 [%0];" ::"l"(line));
+// Columns [col, col + 8) of the tile product for this thread's row 32 (warp % 4) + lane, handed to put(column,
+// value) unnormalised; eB: the column exponents of the tile's B.  A single multiplication by the power of two
+// where it has one (df_scale's result, in a third of its instructions).
+template <class F>
+__device__ __forceinline__ void product8(const Ctx& c, const int* eB, int col, F put) {
+  const int w4 = (threadIdx.x >> 5) & 3;
+  const int em = c.eA[w4 * 32 + (threadIdx.x & 31)] - 16;
+  const uint32_t addr = c.tmem + ((uint32_t)(w4 * 32) << 16) + col;
+  __syncwarp();   // the loads are warp-wide, and the values' scaling and put may have diverged
+  float acc[NBLK][8];
+#pragma unroll
+  for (int g = 0; g < NBLK; ++g) tc::tmem_ld8(addr + g * TN, acc[g]);
+  tc::tmem_wait_ld();
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const dfloat sum = sum_blocks(acc[0][q], acc[1][q], acc[2][q], acc[3][q], acc[4][q], acc[5][q], acc[6][q]);
+    const int e = em + eB[col + q];
+    if (e >= -126 && e <= 127) {
+      const float f = pow2f(e);
+      put(col + q, dfloat(__fmul_rn(sum.hi, f), __fmul_rn(sum.lo, f)));
+    } else {
+      put(col + q, df_scale(sum, e));
+    }
   }
 }
 
-// C(rows x cols) -= the tile product, for C in global memory (double-float, row pitch ldc elements),
-// coalesced: in two halves of 32 columns, the old values are read row-contiguously into shared memory
-// (the B digits' region, free once the MMAs have completed), each thread subtracts the product for 16
-// outputs of its TMEM lane (warp w: rows 32 (w % 4) .., columns 16 (w / 4) .. of the half), and the
-// half is written back row-contiguously.  Ends with the fences and barrier that let the next tile reuse
-// TMEM and shared memory.
+// A tile product is turned from one row a thread into one row a warp for its memory accesses in a staging
+// buffer of TM rows x 32 columns.
 constexpr int SUB_LD = 33;   // staging row stride in double-float values (odd: spreads the banks)
-__device__ __forceinline__ void epilogue_subtract(Ctx& c, dfloat* C, int64_t ldc, int rows, int cols) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m = (warp & 3) * 32 + lane, nq = (warp >> 2) * 16;
-  const uint32_t lane_addr = c.tmem + ((uint32_t)((warp & 3) * 32) << 16);
-  dfloat* S = reinterpret_cast<dfloat*>(c.smem + NDIG * A_DIGIT_BYTES);   // TM x SUB_LD
-  const int em = c.eA[m];
-#pragma unroll 1
-  for (int half = 0; half < 2; ++half) {
-    const int cbase = half * 32;
-    // old values: one warp per row, one 8-byte value per thread (C's column offset can be odd: the
-    // overlap phase of the factorisation starts at column n_I, so wider accesses could be misaligned)
-    for (int e = tid; e < TM * 32; e += 256) {
-      const int r = e >> 5, cc = e & 31, col = cbase + cc;
-      S[r * SUB_LD + cc] = (r < rows && col < cols) ? C[(int64_t)r * ldc + col] : dfloat(0.f, 0.f);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int cb = 0; cb < 16; cb += 8) {
-      float acc[NBLK][8];
-#pragma unroll
-      for (int g = 0; g < NBLK; ++g) tc::tmem_ld8(lane_addr + g * TN + cbase + nq + cb, acc[g]);
-      tc::tmem_wait_ld();
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const dfloat sum = sum_blocks(acc[0][q], acc[1][q], acc[2][q], acc[3][q], acc[4][q], acc[5][q], acc[6][q]);
-        const int e = em + c.eB[cbase + nq + cb + q] - 16;
-        dfloat& o = S[m * SUB_LD + nq + cb + q];
-        o = o - df_scale(sum, e);
-      }
-    }
-    __syncthreads();
-    for (int e = tid; e < TM * 32; e += 256) {
-      const int r = e >> 5, cc = e & 31, col = cbase + cc;
-      if (r < rows && col < cols) C[(int64_t)r * ldc + col] = S[r * SUB_LD + cc];
-    }
-    __syncthreads();
-  }
-  tc::fence_before_sync();
-  __syncthreads();
+constexpr size_t STAGE_BYTES = (size_t)TM * SUB_LD * sizeof(dfloat);
+__device__ __forceinline__ void stage_half(const Ctx& c, const int* eB, int half, dfloat* S) {
+  const int warp = threadIdx.x >> 5, m = (warp & 3) * 32 + (threadIdx.x & 31);
+  product8(c, eB, half * 32 + (warp >> 2) * 8, [&](int col, dfloat v) { S[m * SUB_LD + col - half * 32] = v; });
 }
 
 }  // namespace tcdf
