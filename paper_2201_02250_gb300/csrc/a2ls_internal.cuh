@@ -59,6 +59,15 @@ __device__ __forceinline__ int cluster_size() {
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// a double of another CTA's shared memory
+__device__ __forceinline__ double cluster_ld(const double* p, int rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
+  return v;
+}
+
 // Kernels whose launches can be timed with CUDA events (a2ls_options::timing).
 enum { KT_LU_LOCAL = 0, KT_LU_SPLIT, KT_EIG_SOLVE, KT_EIG_ORTH, KT_EIG_RR, KT_COARSE_LU, KT_COARSE_INV,
        KT_APPLY_LOCAL, KT_COUNT };

@@ -611,15 +611,6 @@ __device__ int warp_cholesky_inverse(double* G, int p, double* Ri, double* dsc, 
   return ok;
 }
 
-// a double of another CTA's shared memory
-__device__ __forceinline__ double cluster_ld(const double* p, int rank) {
-  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
-  double v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
-  return v;
-}
-
 // G <- the sum of the cluster's G (count doubles of shared memory at the same place in every CTA), added in
 // the order of the ranks, so that every CTA holds the same values.  tmp: count doubles of scratch in shared
 // memory that no other CTA reads.  All threads of the cluster; G complete in every CTA (the barrier orders

@@ -425,76 +425,93 @@ __global__ void __launch_bounds__(PROP_THREADS) k_propagate_smem(const int* off,
 }
 
 // ---------------------------------------------------------------------------
-// loss: one CTA per subdomain
+// loss: a cluster of CTAs per subdomain
 // ---------------------------------------------------------------------------
 // Solves (Y^T Y + eps I) C = Y^T Z, R = Z - Y C, L_i = (||R||^2 + eps ||C||^2) / m,
 // dY = -2 R C^T / m * scale (scale = 1 / number of subdomains with a target).
+// The FP64 pipe bounds it, and a conversion to FP64 costs it as much as a product: the rows are converted once,
+// into shared memory, the symmetric Y^T Y is formed in its lower triangle only, and the rows of a subdomain are
+// spread over the CTAs of its cluster (whose sums meet in the order of their ranks); a warp factors, a lane a
+// row.  64 subdomains of 1250 rows and 10 targets: 720 us a launch with one CTA each and a conversion a product, 217 so
+// (clusters of 2).
 __global__ void __launch_bounds__(256) k_loss(const int* off, const int* zm, const int64_t* zoff,
                                               const float* __restrict__ Z, const float* __restrict__ Y, float scale,
                                               double* loss_i, float* dY) {
-  __shared__ float Ys[TILE][OUT + 1];
-  __shared__ float Zs[TILE][MAXZ + 1];
-  __shared__ double G[OUT * OUT], B[OUT * MAXZ], red[32];
+  constexpr int NG = OUT * (OUT + 1) / 2;   // entries of a lower triangle
+  __shared__ double Ys[TILE][OUT + 1], Zs[TILE][MAXZ + 1];
+  __shared__ double P[NG + OUT * MAXZ], G[OUT * OUT], B[OUT * MAXZ], red[32], rsum;
   __shared__ int okflag;
-  const int i = blockIdx.x, o = off[i], n = off[i + 1] - o, m = zm[i], tid = threadIdx.x;
+  const int C = cluster_size(), rank = cluster_rank();
+  const int i = blockIdx.x / C, o = off[i], n = off[i + 1] - o, m = zm[i], tid = threadIdx.x;
+  const int per = (n + C - 1) / C, l0 = min(n, rank * per), l1 = min(n, l0 + per);   // this CTA's rows
   if (m == 0) {
-    for (int e = tid; e < n * OUT; e += blockDim.x) dY[(int64_t)o * OUT + e] = 0.f;
-    if (tid == 0) loss_i[i] = 0.0;
+    for (int e = l0 * OUT + tid; e < l1 * OUT; e += blockDim.x) dY[(int64_t)o * OUT + e] = 0.f;
+    if (tid == 0 && rank == 0) loss_i[i] = 0.0;
     return;
   }
   const float* Zi = Z + zoff[i];
-  const int nout = OUT * OUT + OUT * m;
+  const int nout = NG + OUT * m;
+  static_assert(NG + OUT * MAXZ <= 3 * 256, "three outputs a thread");
   double acc[3] = {0.0, 0.0, 0.0};
-  for (int r0 = 0; r0 < n; r0 += TILE) {
-    const int rows = min(TILE, n - r0);
-    for (int e = tid; e < TILE * OUT; e += blockDim.x) {
-      const int r = e / OUT, c = e % OUT;
-      Ys[r][c] = r < rows ? Y[(int64_t)(o + r0 + r) * OUT + c] : 0.f;
-    }
-    for (int e = tid; e < TILE * m; e += blockDim.x) {
-      const int r = e / m, c = e % m;
-      Zs[r][c] = r < rows ? Zi[(int64_t)(r0 + r) * m + c] : 0.f;
-    }
+  const double *pa[3], *pb[3];   // the columns of output tid + 256 k
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int q = tid + 256 * k;
+    int j1 = 0;
+    while (j1 + 1 < OUT && (j1 + 1) * (j1 + 2) / 2 <= q) ++j1;
+    const int e = q - NG;
+    pa[k] = q < NG ? &Ys[0][j1] : &Ys[0][min(e / m, OUT - 1)];
+    pb[k] = q < NG ? &Ys[0][q - j1 * (j1 + 1) / 2] : &Zs[0][e % m];
+  }
+  for (int r0 = l0; r0 < l1; r0 += TILE) {
+    const int rows = min(TILE, l1 - r0);
+    for (int e = tid; e < rows * OUT; e += blockDim.x) Ys[e / OUT][e % OUT] = Y[(int64_t)(o + r0) * OUT + e];
+    for (int e = tid; e < rows * m; e += blockDim.x) Zs[e / m][e % m] = Zi[(int64_t)r0 * m + e];
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const int q = tid + 256 * k;
-      if (q >= nout) break;
+      if (tid + 256 * k >= nout) break;
+      const double *x = pa[k], *y = pb[k];
+      const int sy = tid + 256 * k < NG ? OUT + 1 : MAXZ + 1;
       double a = 0.0;
-      if (q < OUT * OUT) {
-        const int j1 = q / OUT, j2 = q % OUT;
-        for (int r = 0; r < rows; ++r) a += (double)Ys[r][j1] * (double)Ys[r][j2];
-      } else {
-        const int j = (q - OUT * OUT) / m, c = (q - OUT * OUT) % m;
-        for (int r = 0; r < rows; ++r) a += (double)Ys[r][j] * (double)Zs[r][c];
-      }
+#pragma unroll 4
+      for (int r = 0; r < rows; ++r) a += x[r * (OUT + 1)] * y[r * sy];
       acc[k] += a;
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const int q = tid + 256 * k;
-    if (q < OUT * OUT) G[q] = acc[k] + ((q / OUT == q % OUT) ? LOSS_EPS : 0.0);
-    else if (q < nout) B[q - OUT * OUT] = acc[k];
+  for (int k = 0; k < 3; ++k)
+    if (tid + 256 * k < nout) P[tid + 256 * k] = acc[k];
+  cluster_sync();
+  for (int q = tid; q < nout; q += blockDim.x) {
+    double v = cluster_ld(P + q, 0);
+    for (int r = 1; r < C; ++r) v += cluster_ld(P + q, r);
+    if (q < NG) {
+      int j1 = 0;
+      while (j1 + 1 < OUT && (j1 + 1) * (j1 + 2) / 2 <= q) ++j1;
+      const int j2 = q - j1 * (j1 + 1) / 2;
+      G[j1 * OUT + j2] = v + (j1 == j2 ? LOSS_EPS : 0.0);
+    } else {
+      B[q - NG] = v;
+    }
   }
   __syncthreads();
-  if (tid == 0) {
-    // Cholesky G = L L^T in place (lower triangle)
-    int ok = 1;
+  if (tid < 32) {
+    // Cholesky G = L L^T in place (lower triangle); every row sums in the order of its columns
+    const int r = min(tid, OUT - 1);
+    bool ok = true;
     for (int j = 0; j < OUT; ++j) {
-      double d = G[j * OUT + j];
-      for (int k = 0; k < j; ++k) d -= G[j * OUT + k] * G[j * OUT + k];
-      if (!(d > 0.0)) { ok = 0; d = 1e-300; }
-      d = sqrt(d);
-      G[j * OUT + j] = d;
-      for (int r = j + 1; r < OUT; ++r) {
-        double v = G[r * OUT + j];
+      double v = G[r * OUT + j];
+      if (r >= j)
         for (int k = 0; k < j; ++k) v -= G[r * OUT + k] * G[j * OUT + k];
-        G[r * OUT + j] = v / d;
-      }
+      double d = __shfl_sync(0xffffffffu, v, j);
+      if (!(d > 0.0)) { ok = false; d = 1e-300; }
+      d = sqrt(d);
+      if (tid < OUT && r >= j) G[r * OUT + j] = r == j ? d : v / d;
+      __syncwarp();
     }
-    okflag = ok;
+    if (tid == 0) okflag = ok;
   }
   __syncthreads();
   if (tid < m) {
@@ -514,9 +531,8 @@ __global__ void __launch_bounds__(256) k_loss(const int* off, const int* zm, con
   __syncthreads();
   double rsq = 0.0;
   const float f = -2.f / (float)m * scale;
-  for (int l = tid; l < n; l += blockDim.x) {
-    float y[OUT];
-    double dy[OUT];
+  for (int l = l0 + tid; l < l1; l += blockDim.x) {
+    double y[OUT], dy[OUT];
 #pragma unroll
     for (int j = 0; j < OUT; ++j) {
       y[j] = Y[(int64_t)(o + l) * OUT + j];
@@ -525,7 +541,7 @@ __global__ void __launch_bounds__(256) k_loss(const int* off, const int* zm, con
     for (int c = 0; c < m; ++c) {
       double r = Zi[(int64_t)l * m + c];
 #pragma unroll
-      for (int j = 0; j < OUT; ++j) r -= (double)y[j] * B[j * m + c];
+      for (int j = 0; j < OUT; ++j) r -= y[j] * B[j * m + c];
       rsq += r * r;
 #pragma unroll
       for (int j = 0; j < OUT; ++j) dy[j] += r * B[j * m + c];
@@ -537,7 +553,33 @@ __global__ void __launch_bounds__(256) k_loss(const int* off, const int* zm, con
   for (int e = tid; e < OUT * m; e += blockDim.x) csq += B[e] * B[e];
   rsq = block_reduce(rsq, red, false);
   csq = block_reduce(csq, red, false);
-  if (tid == 0) loss_i[i] = okflag ? (rsq + LOSS_EPS * csq) / m : NAN;
+  if (tid == 0) rsum = rsq;
+  cluster_sync();
+  if (tid == 0 && rank == 0) {
+    for (int r = 1; r < C; ++r) rsq += cluster_ld(&rsum, r);
+    loss_i[i] = okflag ? (rsq + LOSS_EPS * csq) / m : NAN;
+  }
+  cluster_sync();   // no CTA leaves before its sum has been read
+}
+
+// the largest cluster (of at most 8) with which all subdomains' CTAs have an SM each
+static void launch_loss(cudaStream_t st, int N, const int* off, const int* zm, const int64_t* zoff, const float* Z,
+                 const float* Y, float scale, double* loss_i, float* dY) {
+  int dev = 0, sms = 152, C = 1;
+  A2LS_CUDA(cudaGetDevice(&dev));
+  A2LS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  while (C < 8 && 2 * C * N <= sms) C *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(N * C);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  A2LS_CUDA(cudaLaunchKernelEx(&cfg, k_loss, off, zm, zoff, Z, Y, scale, loss_i, dY));
 }
 
 // ---------------------------------------------------------------------------
@@ -1263,7 +1305,7 @@ int a2ls_gnn_loss_grad(a2ls_gnn* g, a2ls_gnn_sample* s, double* loss) {
       forward(st, &g->launches, gr, g->w16, g->theta, true, a);
       double* d_loss = galloc<double>(tmp, N, st);
       float* dY = galloc<float>(tmp, (size_t)S * OUT, st);
-      k_loss<<<N, 256, 0, st>>>(s->off, s->zm, s->zoff, s->Z, a.Y, 1.f / (float)s->ntarget, d_loss, dY);
+      launch_loss(st, N, s->off, s->zm, s->zoff, s->Z, a.Y, 1.f / (float)s->ntarget, d_loss, dY);
       GNN_LAUNCH(&g->launches);
       // dp_0 into a.p0 (p_0 itself is no longer needed), scratch a.pa / a.pb / a.Y
       propagate<true>(st, &g->launches, gr, dY, a.pa, a.pb, a.Y, a.p0);
