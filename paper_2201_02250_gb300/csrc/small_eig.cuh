@@ -53,9 +53,9 @@ SE_HD inline double se_dbl(double x) { return x; }
 // unnormalised multiply-add overloads both)
 SE_HD inline void se_mac(double& acc, double a, double b) { acc += a * b; }
 SE_HD inline double se_fin(double a) { return a; }
-// Whether schur() chases several bulges with reflectors formed from se_rsqrt(a) = 1 / sqrt(a), se_recip12(b) =
-// 1 / b for b in [1, 2] and se_scale_to_one(a), a factor that brings a to about 1 (double-float), or keeps to
-// the single bulge with the library's roots and quotients.  FP64 keeps to those and with them its results
+// Whether schur() forms its reflectors from se_rsqrt(a) = 1 / sqrt(a), se_recip12(b) = 1 / b for b in [1, 2] and
+// se_scale_to_one(a), a factor that brings a to about 1 (double-float), or keeps to the library's roots and
+// quotients.  FP64 keeps to those and with them its results
 // bit for bit: the block Krylov iteration amplifies a changed rounding until the eigenvectors, kept at a
 // residual of 1e-10, differ at that size, and with them the ninth digit of the preconditioner, which FP64
 // callers compare.
@@ -217,7 +217,7 @@ SE_HD inline int first_negligible(const R* H, int ld, int hi, R leps, R eps, R h
   return t.max(lo);
 }
 
-// ---- the single bulge with the library's square root and division ----
+// ---- with the library's square root and division ----
 // GB300's FP64 pipe takes about 64 cycles for every warp instruction of an SM quarter, however few lanes
 // are active, so the chain of the reflectors' FP64 instructions is the time: the next reflector's three
 // entries and its two quotients go to lanes of one warp (order 48: 7.5 -> 5.2 million cycles, the same
@@ -319,7 +319,7 @@ SE_HD inline void split_2x2_div(R* H, int ld, R* Q, int ldq, int m, int p, const
   t.sync();
 }
 
-// schur() with one bulge a sweep (see there for the arguments)
+// schur() with the library's square root and division (see there for the arguments)
 template <class R>
 SE_HD inline int schur_single(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const Team& t, R* snap,
                               double local_tol) {
@@ -519,7 +519,7 @@ SE_HD inline int schur_single(R* H, int ld, R* Q, int ldq, int m, double hnorm_,
   return 0;
 }
 
-// ---- several bulges ----
+// ---- reflectors without square roots and quotients ----
 
 // Householder reflector mapping (x, y, z) to (alpha, 0, 0): returns alpha, beta and u = (1, u1, u2).
 // With v = (v0, y, z), v0 = x - alpha, v^T v = 2 |alpha| |v0|, so beta = 2 v0^2 / v^T v = v0 / (-alpha).
@@ -593,14 +593,10 @@ SE_HD inline void split_2x2(R* H, int ld, R* Q, int ldq, int m, int p, const Tea
   t.sync();
 }
 
-// Most bulges chased together, their distance in rows, and the scratch schur() wants: per bulge the nine
-// entries of the next reflector's snapshot, the four shift values and two sets of u1, u2, beta, alpha.
-constexpr int SE_BULGES = 3;
-constexpr int SE_BULGE_GAP = 4;
-constexpr int SE_SLOT = 21;
-constexpr int SE_SNAP = SE_BULGES * SE_SLOT;
+// The scratch schur() wants: the nine entries of the next reflector's snapshot, the four shift values and two
+// sets of u1, u2, beta, alpha.
+constexpr int SE_SNAP = 21;
 enum { SE_SHIFTS = 9, SE_REFL = 13 };
-constexpr int SE_W2 = 10, SE_W3 = 24;  // active block sizes from which a second and a third bulge are chased
 
 // The shift pair (s1r, s2r, s1i, s2i) of the 2 x 2 block a, b; c, d: a real pair is replaced by its member
 // closer to d, used twice.
@@ -621,25 +617,38 @@ SE_HD inline void shift_pair(R a, R b, R c, R d, R* s) {
   }
 }
 
-// One sweep of NB bulges over the active block lo .. hi (see schur); exceptional: with shifts of the size of
-// the last subdiagonal entries.  Starts after the team has seen H, ends with a barrier.
-template <int NB, class R>
+// One sweep over the active block lo .. hi (see schur); exceptional: with shifts of the size of the last
+// subdiagonal entries.  Starts after the team has seen H, ends with a barrier.
+template <class R>
 SE_HD inline void se_sweep(R* H, int ld, R* Q, int ldq, int m, int lo, int hi, bool exceptional, const Team& t,
                            R* snap) {
-  // On the GPU the last warp forms the reflectors, lanes 3 q .. 3 q + 2 for bulge q (lane 3 q keeps it); the
-  // right updates and Q are left to the other warps.
+  // On the GPU the last warp forms the reflectors (its lane 0 keeps them); the right updates and Q are left to
+  // the other warps.
 #ifdef __CUDA_ARCH__
   const int nwork = t.size - 32, rl = t.lane - nwork;
-  const int mq0 = rl >= 0 ? (rl < 3 * NB ? rl / 3 : NB - 1) : NB, mq1 = mq0 < NB ? mq0 + 1 : NB;
-  const bool keeps = rl == 3 * mq0;
+  const bool maker = rl >= 0, keeps = rl == 0;
 #else
-  const int nwork = t.size, mq0 = 0, mq1 = NB;
-  const bool keeps = true;
+  const int nwork = t.size;
+  const bool maker = true, keeps = true;
 #endif
-  // the reflector that starts bulge q: the first column of (H - s1)(H - s2), formed from differences to
-  // avoid cancellation, times a factor that keeps it in range (only its direction matters)
-  auto start = [&](int q) {
-    const R* s = snap + q * SE_SLOT + SE_SHIFTS;
+  if (maker) {
+    R a, b, c, d;
+    if (exceptional) {
+      const R e = se_abs(H[hi * ld + hi - 1]) + se_abs(H[(hi - 1) * ld + hi - 2]);
+      a = 0.75 * e + H[hi * ld + hi];
+      b = -0.4375 * e;
+      c = e;
+      d = a;
+    } else {
+      a = H[(hi - 1) * ld + hi - 1];
+      b = H[(hi - 1) * ld + hi];
+      c = H[hi * ld + hi - 1];
+      d = H[hi * ld + hi];
+    }
+    R s[4];
+    shift_pair(a, b, c, d, s);
+    // the first column of (H - s1)(H - s2), formed from differences to avoid cancellation, times a factor
+    // that keeps it in range (only its direction matters)
     const R s1r = s[0], s2r = s[1], s1i = s[2], s2i = s[3];
     const R h00 = H[lo * ld + lo], h01 = H[lo * ld + lo + 1], h10 = H[(lo + 1) * ld + lo];
     const R h11 = H[(lo + 1) * ld + lo + 1], h21 = H[(lo + 2) * ld + lo + 1];
@@ -649,45 +658,17 @@ SE_HD inline void se_sweep(R* H, int ld, R* Q, int ldq, int m, int lo, int hi, b
     R r[4];
     make_reflector<R>(g * h01 + (h00 - s1r) * ((h00 - s2r) * f) - s1i * (s2i * f), g * (h00 + h11 - s1r - s2r),
                       g * h21, r[0], r[1], r[2], r[3]);
-    R* o = snap + q * SE_SLOT + SE_REFL + 4 * ((SE_BULGE_GAP * q) & 1);
     if (keeps)
-      for (int u = 0; u < 4; ++u) o[u] = r[u];
-  };
-  for (int q = mq0; q < mq1; ++q) {
-    const int p = hi - 1 - 2 * q;
-    R a, b, c, d;
-    if (exceptional) {
-      const R e = se_abs(H[(p + 1) * ld + p]) + se_abs(H[p * ld + p - 1]);
-      a = 0.75 * e + H[(p + 1) * ld + p + 1];
-      b = -0.4375 * e;
-      c = e;
-      d = a;
-    } else {
-      a = H[p * ld + p];
-      b = H[p * ld + p + 1];
-      c = H[(p + 1) * ld + p];
-      d = H[(p + 1) * ld + p + 1];
-    }
-    R s[4];
-    shift_pair(a, b, c, d, s);
-    if (keeps)
-      for (int u = 0; u < 4; ++u) snap[q * SE_SLOT + SE_SHIFTS + u] = s[u];
+      for (int u = 0; u < 4; ++u) snap[SE_REFL + u] = r[u];
   }
-#ifdef __CUDA_ARCH__
-  __syncwarp();
-#endif
-  if (mq0 == 0) start(0);
   t.sync();  // the reads of H above precede the first update
-  // Bulge q is at row k = lo + step - SE_BULGE_GAP q.  For k > lo its reflector was built from column
-  // k - 1 (rows k .. k + 2), which it maps to (alpha, 0, 0) exactly; that column is therefore not part of
-  // the left update but written directly, after the barrier that separates the reads of it from the
-  // writes.  At k = hi - 1 the reflector has two rows.  The next reflector comes from column k after this
-  // step's right update; its three entries are recomputed from a snapshot of rows k + 1 .. k + 3
-  // (columns k .. k + 2) taken in the left phase, and the reflector is formed while the others run the
-  // right update (the entries are the values the right update writes).
-  // An item of a phase is a bulge and a column or row of the whole matrix, of which those outside the
-  // update are passed over: the position costs a few instructions where a list of just the active ones
-  // took a hundred, as long as the update itself.
+  // The bulge is at row k.  For k > lo its reflector was built from column k - 1 (rows k .. k + 2), which it
+  // maps to (alpha, 0, 0) exactly; that column is therefore not part of the left update but written directly,
+  // after the barrier that separates the reads of it from the writes.  At k = hi - 1 the reflector has two
+  // rows.  The next reflector comes from column k after this step's right update; its three entries are
+  // recomputed from a snapshot of rows k + 1 .. k + 3 (columns k .. k + 2) taken in the left phase, and the
+  // reflector is formed while the others run the right update (the entries are the values the right update
+  // writes).
   auto reflect = [&](R* a, int st, const R* r, bool three) {
     const R u1 = r[0], u2 = r[1], beta = r[2];
     const R a0 = a[0], a1 = a[st], a2 = three ? a[2 * st] : R(0.0);
@@ -699,85 +680,54 @@ SE_HD inline void se_sweep(R* H, int ld, R* Q, int ldq, int m, int lo, int hi, b
     a[st] = a1 - d * u1;
     if (three) a[2 * st] = a2 - d * u2;
   };
-  const int steps = hi - lo + SE_BULGE_GAP * (NB - 1);
-  for (int step = 0; step < steps; ++step) {
-    const R* refl = snap + SE_REFL + 4 * (step & 1);
-    const int k1 = lo + step;  // bulge 0's row
+  for (int k = lo; k < hi; ++k) {
+    const R* r = snap + SE_REFL + 4 * ((k - lo) & 1);
+    const bool three = k <= hi - 2;
     // phase 1: rows k .. k + 2 from the left (columns k .. m - 1), one column per item
-    for (int at = t.lane; at < NB * m; at += t.size) {
-      int q = 0, c = at;
-      for (int u = 1; u < NB; ++u) {
-        const bool next = c >= m;
-        q += next ? 1 : 0;
-        c -= next ? m : 0;
-      }
-      const int k = k1 - SE_BULGE_GAP * q;
-      const bool three = k <= hi - 2;
-      if (c < k || (NB > 1 && (k < lo || k > hi - 1))) continue;
+    for (int c = k + t.lane; c < m; c += t.size) {
       R* a = H + k * ld + c;
-      reflect(a, ld, refl + q * SE_SLOT, three);
+      reflect(a, ld, r, three);
       if (c < k + 3 && three) {
-        R* v = snap + q * SE_SLOT + (c - k);
+        R* v = snap + (c - k);
         v[0] = a[ld];
         v[3] = a[2 * ld];
         v[6] = k + 3 <= hi ? a[3 * ld] : R(0.0);
       }
     }
     t.sync();
-    // phase 2: columns k .. k + 2 from the right (rows 0 .. k + 3) and Q, one row per item; the next
-    // reflectors
-    for (int q = mq0; q < mq1; ++q) {
-      const int k = k1 - SE_BULGE_GAP * q;
-      R* slot = snap + q * SE_SLOT;
-      const R* r = refl + q * SE_SLOT;
-      R v[3] = {R(0.0), R(0.0), R(0.0)};
+    // phase 2: columns k .. k + 2 from the right (rows 0 .. k + 3) and Q, one row per item; the next reflector
+    if (maker) {
       const R u1 = r[0], u2 = r[1], beta = r[2];
       auto entry = [&](int rr) {
-        const R a0 = slot[3 * rr], a1 = slot[3 * rr + 1], a2 = slot[3 * rr + 2];
+        const R a0 = snap[3 * rr], a1 = snap[3 * rr + 1], a2 = snap[3 * rr + 2];
         R d = a0;
         se_mac(d, u1, a1);
         se_mac(d, u2, a2);
         d = se_fin(d) * beta;
         return a0 - d;
       };
+      if (three) {
+        R v[3], n[4];
 #ifdef __CUDA_ARCH__
-      // one lane per entry (a bulge outside the block computes on what its slot happens to hold, and the
-      // result is not used)
-      const R e = entry(rl < 3 * NB ? rl - 3 * mq0 : 2);
-      v[0] = se_warp_get(e, 3 * mq0);
-      v[1] = se_warp_get(e, 3 * mq0 + 1);
-      v[2] = se_warp_get(e, 3 * mq0 + 2);
+        const R e = entry(rl < 3 ? rl : 2);   // one lane per entry
+        for (int rr = 0; rr < 3; ++rr) v[rr] = se_warp_get(e, rr);
 #else
-      for (int rr = 0; rr < 3; ++rr) v[rr] = entry(rr);
+        for (int rr = 0; rr < 3; ++rr) v[rr] = entry(rr);
 #endif
-      if (NB > 1 && k == lo - 1) {
-        start(q);
-      } else if (k >= lo && k <= hi - 2) {
-        R n[4];
         make_reflector<R>(v[0], v[1], v[2], n[0], n[1], n[2], n[3]);
-        R* o = slot + SE_REFL + 4 * ((step + 1) & 1);
         if (keeps)
-          for (int u = 0; u < 4; ++u) o[u] = n[u];
+          for (int u = 0; u < 4; ++u) snap[SE_REFL + 4 * ((k + 1 - lo) & 1) + u] = n[u];
       }
-      if (keeps && k > lo && k <= hi - 1) {
+      if (keeps && k > lo) {
         H[k * ld + k - 1] = r[3];
         H[(k + 1) * ld + k - 1] = 0.0;
-        if (k <= hi - 2) H[(k + 2) * ld + k - 1] = 0.0;
+        if (three) H[(k + 2) * ld + k - 1] = 0.0;
       }
     }
     if (t.lane < nwork) {
-      for (int at = t.lane; at < 2 * NB * m; at += nwork) {
-        const bool isq = at >= NB * m;
-        int q = 0, e = isq ? at - NB * m : at;
-        for (int u = 1; u < NB; ++u) {
-          const bool next = e >= m;
-          q += next ? 1 : 0;
-          e -= next ? m : 0;
-        }
-        const int k = k1 - SE_BULGE_GAP * q;
-        if ((!isq && e > (k + 3 <= hi ? k + 3 : hi)) || (NB > 1 && (k < lo || k > hi - 1))) continue;
-        reflect((isq ? Q + e * ldq : H + e * ld) + k, 1, refl + q * SE_SLOT, k <= hi - 2);
-      }
+      const int rows = (k + 3 <= hi ? k + 3 : hi) + 1;
+      for (int e = t.lane; e < rows + m; e += nwork)
+        reflect((e < rows ? H + e * ld : Q + (e - rows) * ldq) + k, 1, r, three);
     }
     t.sync();
   }
@@ -794,13 +744,11 @@ SE_HD inline void se_sweep(R* H, int ld, R* Q, int ldq, int m, int lo, int hi, b
 // hnorm always uses the machine epsilon.
 //
 // A sweep's time is the chain of its reflectors, each formed from what the one before it leaves, and not
-// the updates.  A sweep therefore chases up to SE_BULGES bulges, each with the shifts of its own 2 x 2
-// block (the trailing one, the one before it, ...), SE_BULGE_GAP rows apart and in step with one another
-// (the small-bulge multishift iteration of Braman, Byers and Mathias, SIAM J. Matrix Anal. Appl. 23,
-// 2002, with the neighbouring diagonal blocks' shifts): the bulges' rows and columns are disjoint, so that
-// one step updates for all of them and one warp forms their next reflectors side by side, in its lanes.
-// Against one bulge a sweep (order 72, double-float, random spectra of six decades): 7.35 -> 3.13 million
-// cycles.
+// the updates.  Three bulges chased in step with one another (the small-bulge multishift iteration of Braman, Byers
+// and Mathias, SIAM J. Matrix Anal. Appl. 23, 2002) shorten it by a further third, but neglect other entries: with
+// a loose local_tol the Ritz vectors then differ by up to 6e-5 from one bulge's, as far as these are from the
+// exact Schur form's.  Set-up and solve with 256 subdomains of order 72: 120.5 ms with roots and quotients, 116.2
+// without; later, with the other kernels faster, 95.8 against 93.4 with three bulges.
 template <class R>
 SE_HD inline int schur(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const Team& t, R* snap = nullptr,
                        double local_tol = 0.0) {
@@ -830,10 +778,7 @@ SE_HD inline int schur(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const 
     }
     ++iter;
     if (++total > 60 * m) return -1;
-    const int w = hi - lo + 1;
-    if (w >= SE_W3) se_sweep<3>(H, ld, Q, ldq, m, lo, hi, iter % 11 == 10, t, snap);
-    else if (w >= SE_W2) se_sweep<2>(H, ld, Q, ldq, m, lo, hi, iter % 11 == 10, t, snap);
-    else se_sweep<1>(H, ld, Q, ldq, m, lo, hi, iter % 11 == 10, t, snap);
+    se_sweep(H, ld, Q, ldq, m, lo, hi, iter % 11 == 10, t, snap);
   }
   return 0;
 }
