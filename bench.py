@@ -56,7 +56,7 @@ BF16_PEAK_KEY = "bf16_tflops"
 # tensor-pipe activity (sm__pipe_tensor_cycles_active, % of the active SMs' cycles) of the tensor-core
 # kernels in one ncu capture on the 48^3 case (profiles/); DRAM traffic per launch is not scaled to
 # the 96^3 launches, whose active subdomains change from cycle to cycle (traffic null)
-NCU_TENSOR_ACTIVE = {"lu_splitting": 0.074, "eig_triangular_solves": 0.156}
+NCU_TENSOR_ACTIVE = {"lu_splitting": 0.107, "eig_triangular_solves": 0.258}
 
 def parse_args():
     p = argparse.ArgumentParser()
@@ -535,7 +535,7 @@ def report(args, res, world) -> dict:
                   "frac_of_measured_hbm": apply_local_gbs / res["hbm_peak"] if res["hbm_peak"] else None,
                   "bytes": res["ab_mixed"]["apply"], "local_solve_config": res["tuning"]},
         "roofline": roof,
-        "dtype": ("f32 local factors and solves; f32x2 (double-float) splitting LU (trailing update as BF16 digit "
+        "dtype": ("f32 local factors and solves; f32x2 (double-float) splitting LU (tile products as BF16 digit "
                   "products on tcgen05), eigensolves and coarse factorisation; f64 GMRES, SpMV, coarse apply"),
         "data": f"synthetic (seeded generator, workloads.pde, {prob.name})",
         "config": {"workload": workload, "n": prob.n, "nnz": int(prob.A.nnz), "subdomains": int(prob.nparts),
