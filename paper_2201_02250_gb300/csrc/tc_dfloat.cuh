@@ -55,11 +55,13 @@ __device__ __forceinline__ dfloat df_scale(dfloat x, int k) {
 // plus 128 as its bytes, the first signed above them; a byte becomes a float by way of 2^23's mantissa.
 // About 40 instructions where rounding digit by digit in double-float takes 90, and the split of an
 // operand is on the critical chain of every block of the triangular solves (k_tcsolve.cu).
+// A NaN or an infinity makes the first digit NaN, and with it every product of its row or column, so that the
+// Rayleigh-Ritz step's test of its matrix sees it.
 __device__ __forceinline__ void df_digits(dfloat x, int e, float (&d)[NDIG]) {
   const dfloat y = df_scale(x, 56 - e);
   const long long v = __float2ll_rn(y.hi) + __float2ll_rn(y.lo) + 0x0000808080808080ll;
   const uint32_t lo = (uint32_t)v, mid = (uint32_t)((unsigned long long)v >> 32);
-  d[0] = (float)(int)(v >> 48);
+  d[0] = __fmaf_rn(x.hi, 0.f, (float)(int)(v >> 48));   // NaN where x is not finite, which no integer can show
 #pragma unroll
   for (int s = 1; s < NDIG; ++s) {
     const uint32_t byte = s < 3 ? (mid >> (8 * (2 - s))) & 0xffu : (lo >> (8 * (6 - s))) & 0xffu;
