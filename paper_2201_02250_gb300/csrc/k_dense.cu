@@ -24,11 +24,14 @@ template <> struct AccOf<float> { using type = float; };
 template <> struct AccOf<double> { using type = double; };
 template <> struct AccOf<dfloat> { using type = dfloat; };
 
-// |x| <= bound in x's own arithmetic: a pivot is tested on the chain of every elimination step, where a few
-// FP64 instructions of double-float or FP32 factors took as long as the rest of the step
+// |x| <= bound (false for a NaN) in x's own arithmetic: a pivot is tested on the chain of every elimination step,
+// where a few FP64 instructions of double-float or FP32 factors took as long as the rest of the step
 __device__ __forceinline__ bool abs_at_most(double x, double bound) { return fabs(x) <= bound; }
 __device__ __forceinline__ bool abs_at_most(float x, double bound) { return fabsf(x) <= (float)bound; }
-__device__ __forceinline__ bool abs_at_most(dfloat x, double bound) { return se_abs(x) <= dfloat(bound); }
+__device__ __forceinline__ bool abs_at_most(dfloat x, double bound) {
+  const dfloat a = se_abs(x), b(bound);
+  return a.hi < b.hi || (a.hi == b.hi && a.lo <= b.lo);   // (a dfloat's <= holds for a NaN)
+}
 
 // depth of the operand chunks staged by the tile products
 constexpr int GK = 32;

@@ -27,3 +27,11 @@ def test_tensor_core_digits_keep_what_is_not_finite(entry, value):
     digits (1e39 is infinite in double-float)."""
     from paper_2201_02250_gb300 import a2ls
     assert _setup_error(value, entry, precision="fp32", tensor_cores=1, static_pivoting=1) == a2ls.A2LS_ERR_EIGEN
+
+
+@pytest.mark.parametrize("tensor_cores", [0, 1])
+@pytest.mark.parametrize("entry", ["diagonal", "off"])
+def test_nan_pivot_is_not_a_tiny_one(entry, tensor_cores):
+    """A NaN is no small pivot, which would be reported as singular (or replaced): the eigensolve reports it."""
+    from paper_2201_02250_gb300 import a2ls
+    assert _setup_error(np.nan, entry, precision="fp32", tensor_cores=tensor_cores) == a2ls.A2LS_ERR_EIGEN
