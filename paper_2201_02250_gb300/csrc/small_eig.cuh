@@ -96,7 +96,15 @@ template <class R> struct SeEps {
 
 template <class R>
 SE_HD inline R sgn(R a, R b) { return b >= R(0.0) ? se_abs(a) : -se_abs(a); }
-SE_HD inline double sgn(double a, double b) { return copysign(a, b); }
+SE_HD inline double sgn(double a, double b) {
+#ifdef __CUDA_ARCH__
+  // the same rule (-0 counts as positive) on the integer pipe
+  const long long u = __double_as_longlong(b);
+  return u < 0 && (u << 1) != 0 ? -fabs(a) : fabs(a);
+#else
+  return b >= 0.0 ? fabs(a) : -fabs(a);
+#endif
+}
 
 // x_r -= d v_r for r = 0 .. n-1 (x with stride st), four elements loaded ahead of their stores: x and v may
 // be the same kind of memory, so the compiler may not move a load over a store by itself
@@ -914,22 +922,45 @@ SE_HD inline void schur_vector(const R* S, int ld, int m, int p, double lr_, dou
   }
 }
 
-// Order of eigenvalues by decreasing modulus; within a pair the +imag member first, otherwise equal
-// moduli in the order of their positions.  perm: m ints; mod: m doubles of scratch (the moduli).  One
-// eigenvalue per thread finds its rank; ends with a barrier.
+// Order of eigenvalues by decreasing modulus; within a pair the +imag member first.  Moduli that differ by
+// 1e-14 or less count as equal and are taken as the selection below meets them, so that which of them comes
+// first, and which one the cut at nev keeps, does not hang on their last bits.  perm: m ints; mod: m doubles of
+// scratch (the moduli).  Where no moduli but those of a pair are that close, every rule gives the same order and each
+// thread finds the rank of its eigenvalue; otherwise one thread selects.  Ends with a barrier.
 SE_HD inline void order_by_modulus(const double* wr, const double* wi, int m, int* perm, double* mod,
                                    const Team& t = Team{0, 1}) {
-  for (int j = t.lane; j < m; j += t.size) {
-    const double a = hypot(wr[j], wi[j]);
-    mod[j] = a >= 0.0 ? a : -1.0;  // a NaN ranks last: the ranks stay a permutation
-  }
+  for (int j = t.lane; j < m; j += t.size) mod[j] = hypot(wr[j], wi[j]);
   t.sync();
+  int close = 0;
   for (int j = t.lane; j < m; j += t.size) {
     int rank = 0;
     const double mj = mod[j], ij = wi[j];
-    for (int k = 0; k < m; ++k)
-      rank += (mod[k] > mj || (mod[k] == mj && (wi[k] > ij || (!(wi[k] < ij) && k < j)))) ? 1 : 0;
+    for (int k = 0; k < m; ++k) {
+      rank += (mod[k] > mj || (mod[k] == mj && wi[k] > ij)) ? 1 : 0;
+      const bool partner = wr[k] == wr[j] && wi[k] == -ij && ij != 0.0;
+      // (a NaN is close to everything)
+      if (k != j && !partner && !(fabs(mod[k] - mj) > 2e-14 * mj)) close = 1;
+    }
     perm[rank] = j;
+  }
+  if (t.max(close)) {
+    if (t.lane == 0) {
+      for (int j = 0; j < m; ++j) perm[j] = j;
+      for (int a = 0; a < m; ++a) {
+        int best = a;
+        double bm = mod[perm[a]];
+        for (int b = a + 1; b < m; ++b) {
+          const double mb = mod[perm[b]];
+          if (mb > bm * (1 + 1e-14) || (fabs(mb - bm) <= 1e-14 * bm && wi[perm[b]] > wi[perm[best]])) {
+            best = b;
+            bm = mb;
+          }
+        }
+        const int tmp = perm[a];
+        perm[a] = perm[best];
+        perm[best] = tmp;
+      }
+    }
   }
   t.sync();
 }

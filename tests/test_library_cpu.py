@@ -171,3 +171,40 @@ def test_small_eigensolver_on_krylov_matrices_of_a_nonnormal_operator(small_eig_
     for l, k in zip(lam, kappa):
         assert np.min(np.abs(ev - l)) <= 1e-13 * k * sn
     assert max(res) <= 1e-12 * sn
+
+
+def _selection_order(ev):
+    """Selection by decreasing modulus in which moduli within 1e-14 count as equal, the +imag member first."""
+    mod, perm = np.hypot(ev.real, ev.imag), list(range(len(ev)))
+    for a in range(len(ev)):
+        best, bm = a, mod[perm[a]]
+        for b in range(a + 1, len(ev)):
+            mb = mod[perm[b]]
+            if mb > bm * (1 + 1e-14) or (abs(mb - bm) <= 1e-14 * bm and ev[perm[b]].imag > ev[perm[best]].imag):
+                best, bm = b, mb
+        perm[a], perm[best] = perm[best], perm[a]
+    return ev[perm]
+
+
+@pytest.mark.parametrize("seed", range(8))
+def test_order_of_nearly_equal_moduli(small_eig_exe, seed):
+    """Diagonal matrices (their own Schur form): moduli apart, equal, of opposite signs, and a few ulp apart."""
+    rng = np.random.Generator(np.random.PCG64(seed))
+    base = rng.choice([1.0, 2.0, 3.0, 5.0, 7.5], 30) * rng.choice([-1.0, 1.0], 30)
+    d = base * (1 + 2.0**-52 * rng.integers(-60, 61, 30)) if seed else rng.permutation(np.arange(1.0, 31.0))
+    rc, ev, _ = _run_small_eig(small_eig_exe, np.diag(d))
+    assert rc == 0
+    np.testing.assert_array_equal(ev, _selection_order(d + 0j))
+
+
+def test_sign_of_negative_zero(tmp_path):
+    """sgn(a, b) is +|a| for every b >= 0, and -0 >= 0."""
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("g++ not available")
+    src = tmp_path / "sgn.cpp"
+    src.write_text('#include "%s"\nint main() { using a2ls::se::sgn; return !(sgn(2.0, -0.0) == 2.0 && sgn(2.0, 0.0) == 2.0 '
+                   '&& sgn(2.0, -1.0) == -2.0 && sgn(-2.0, 1.0) == 2.0); }\n'
+                   % os.path.join(os.path.dirname(HERE), "paper_2201_02250_gb300", "csrc", "small_eig.cuh"))
+    subprocess.run([gxx, str(src), "-o", str(tmp_path / "sgn")], check=True)
+    assert subprocess.run([str(tmp_path / "sgn")]).returncode == 0
