@@ -273,7 +273,8 @@ void tc_solve_prepare(a2ls_handle* h, const dfloat* fac, TcSolve& ts);   // digi
 void tc_solve_release(a2ls_handle* h, TcSolve& ts);
 // one sweep over the subdomains with 1 <= p <= 32 columns (forward: inv(L), else inv(U))
 void tc_block_solve(a2ls_handle* h, const TcSolve& ts, dfloat* X, const int64_t* xoff, int col0, int ldx,
-                    const int* pvec, const int* active, int forward, unsigned char* xdig = nullptr);
+                    const int* pvec, const int* active, int forward, unsigned char* xdig = nullptr,
+                    long wait_limit = 1L << 26);   // polls of a barrier before the sweep gives up
 constexpr int TC_SOLVE_MAX_P = 32;
 
 // k_stream.cu: pack the factors (after the diagonal tiles are inverted) into the stream of the

@@ -212,10 +212,14 @@ __device__ __forceinline__ void fold(uint32_t tmem, int buf, bool upper, int h, 
 // items: the sweep's products of every subdomain in order, ioff[i] .. ioff[i + 1]: {factor digit tile, block c
 // of X} for a panel product, {tile, -1} for the product with a block's inverted diagonal triangle, which
 // ends the block.  The panel product with the block finished last comes first in its block.
+// A wait that runs out (wait_limit polls) sets abort_flag, after which no wait waits: the folding warps pass
+// through their remaining products without reading TMEM, and the control lane waits (up to WAIT_LIMIT polls
+// each) for the MMAs, stores and loads that it has begun, so that nothing of the CTA is in flight when it gives
+// its TMEM back.
 __global__ void __launch_bounds__(ALL_THREADS, 1) k_block_solve_tc(
     const int* ni, const int* sched, const int* active, const int* pvec, dfloat* X, const int64_t* xoff, int col0,
     int ldx, const int64_t* ioff, const int2* __restrict__ items, const unsigned char* __restrict__ fdig,
-    unsigned char* xdig, const int64_t* xdoff, int forward, int* st) {
+    unsigned char* xdig, const int64_t* xdoff, int forward, long wait_limit, int* st) {
   extern __shared__ __align__(128) unsigned char sm[];
   // full: operands of a stage loaded; done: MMAs of a TMEM buffer completed; folded: a TMEM buffer read;
   // sdig, xdig_rdy: the digits of X_b - panel, of X_b, split; stored: those of X_b in the scratch array
@@ -262,7 +266,8 @@ __global__ void __launch_bounds__(ALL_THREADS, 1) k_block_solve_tc(
   unsigned char* xd = xdig + xdoff[i];
   const int dir = forward ? 1 : -1, b0 = forward ? 0 : nb - 1;
   auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
-    if (!abort_flag && tc::mbar_wait_bounded(bar, parity, tcdf::WAIT_LIMIT)) return true;
+    for (long it2 = 0; it2 < wait_limit && !abort_flag; ++it2)
+      if (tc::mbar_try_wait(bar, parity)) return true;
     abort_flag = 1;
     return false;
   };
@@ -272,7 +277,8 @@ __global__ void __launch_bounds__(ALL_THREADS, 1) k_block_solve_tc(
     if (lane == 0) {
       const uint64_t pol_stream = policy_evict_first(), pol_keep = policy_evict_last();
       bool ok = true, storing = false, late_b = false;
-      int b = b0, loads = 0;   // the current product's block; full-barrier phases begun
+      int2 late = {0, 0};      // the product whose B part is held back
+      int b = b0, loads = 0, issued = 0;   // the current product's block; full- and done-barrier phases begun
       // operands of product m: A, and B unless it is a diagonal product or taken in place (direct)
       auto load_a = [&](int m, int2 x, bool direct) {
         uint64_t* bar = &full[m & 1];
@@ -299,7 +305,7 @@ __global__ void __launch_bounds__(ALL_THREADS, 1) k_block_solve_tc(
           storing = false;
         }
         if (late_b) {                  // product m's B part, held back while its stage held X digits
-          load_b(m, cur);
+          load_b(m, late);
           late_b = false;
         }
         if (m + 1 < nitems) {
@@ -310,8 +316,12 @@ __global__ void __launch_bounds__(ALL_THREADS, 1) k_block_solve_tc(
           if (nxt.y >= 0 && !ndirect) {
             // the B slot of its stage holds X digits if product m - 1 was a diagonal one: product m multiplies
             // them, or they are still to be stored
-            if (prev_diag) late_b = true;
-            else load_b(m + 1, nxt);
+            if (prev_diag) {
+              late_b = true;
+              late = nxt;
+            } else {
+              load_b(m + 1, nxt);
+            }
           }
         }
         const int blk = (b - b0) * dir;                       // blocks finished before this one
@@ -323,6 +333,7 @@ __global__ void __launch_bounds__(ALL_THREADS, 1) k_block_solve_tc(
         tc::fence_after_sync();
         const unsigned char* A = sm + (m & 1) * STAGE;
         issue_mmas(tmem, m & 1, A, sm + ((direct ? m - 1 : m) & 1) * STAGE + STAGE_A, &done[m & 1]);
+        issued = m + 1;
         if (prev_diag) {
           // the digits of the block just finished, from the stage of its diagonal product
           bulk_store(xd + (size_t)last * B_TILE, sm + ((m - 1) & 1) * STAGE + STAGE_A, B_BYTES);
@@ -336,10 +347,12 @@ __global__ void __launch_bounds__(ALL_THREADS, 1) k_block_solve_tc(
         }
         cur = nxt;
       }
-      // nothing of this CTA may be in flight when it leaves: the loads begun, the stores
-      if (!ok)
-        for (int m = max(0, loads - 2); m < loads; ++m) tc::mbar_wait_bounded(&full[m & 1], (m >> 1) & 1, tcdf::WAIT_LIMIT);
+      // nothing of this CTA may be in flight when it leaves: the MMAs, the stores, the loads begun (of which the
+      // last may still want its B part)
+      for (int m = max(0, issued - 2); m < issued; ++m) tc::mbar_wait_bounded(&done[m & 1], (m >> 1) & 1, tcdf::WAIT_LIMIT);
       bulk_stores_done();
+      if (late_b) load_b(loads - 1, late);
+      for (int m = max(0, loads - 2); m < loads; ++m) tc::mbar_wait_bounded(&full[m & 1], (m >> 1) & 1, tcdf::WAIT_LIMIT);
     }
     __syncwarp();
   } else {
@@ -402,6 +415,7 @@ __global__ void __launch_bounds__(ALL_THREADS, 1) k_block_solve_tc(
         clear();
       }
       if (!wait(&done[m & 1], (m >> 1) & 1)) ok = false;
+      ok = __all_sync(0xffffffffu, ok) != 0;   // the loads from TMEM are the whole warp's
       tc::fence_after_sync();
       if (ok) fold(tmem, m & 1, upper, h, fr, diag ? facS : facX + cur.y * NC, acc);
       tc::fence_before_sync();
@@ -430,10 +444,10 @@ __global__ void __launch_bounds__(ALL_THREADS, 1) k_block_solve_tc(
       cur = nxt;
       fr = nfr;
     }
-    if (!ok && tid == 0) raise_status(st, A2LS_ERR_TIMEOUT, i, forward);
   }
   tc::fence_before_sync();
   __syncthreads();
+  if (tid == 0 && abort_flag) raise_status(st, A2LS_ERR_TIMEOUT, i, forward);   // whichever wait ran out
   if (warp == 0) tc::tmem_dealloc(tmem, TMEM_COLS);
 }
 
@@ -518,11 +532,12 @@ void tc_solve_release(a2ls_handle* h, TcSolve& ts) {
 }
 
 void tc_block_solve(a2ls_handle* h, const TcSolve& ts, dfloat* X, const int64_t* xoff, int col0, int ldx,
-                    const int* pvec, const int* active, int forward, unsigned char* xdig) {
+                    const int* pvec, const int* active, int forward, unsigned char* xdig, long wait_limit) {
   using namespace tcs;
   tcs::k_block_solve_tc<<<h->N, ALL_THREADS, smem_bytes(ceil_div(h->max_n, M)), h->st>>>(h->d_ni, h->d_sched, active, pvec, X, xoff, col0, ldx,
                                                             ts.d_ioff[forward != 0], ts.d_items[forward != 0], ts.d_fdig,
-                                                            xdig ? xdig : ts.d_xdig, ts.d_xdoff, forward, h->d_status);
+                                                            xdig ? xdig : ts.d_xdig, ts.d_xdoff, forward,
+                                                            wait_limit, h->d_status);
   A2LS_LAUNCH();
 }
 
