@@ -12,6 +12,7 @@
 #pragma once
 
 #include <math.h>
+#include <string.h>
 
 #ifdef __CUDACC__
 #define SE_HD __host__ __device__
@@ -98,9 +99,9 @@ template <class R>
 SE_HD inline R sgn(R a, R b) { return b >= R(0.0) ? se_abs(a) : -se_abs(a); }
 SE_HD inline double sgn(double a, double b) {
 #ifdef __CUDA_ARCH__
-  // the same rule (-0 counts as positive) on the integer pipe
-  const long long u = __double_as_longlong(b);
-  return u < 0 && (u << 1) != 0 ? -fabs(a) : fabs(a);
+  // the same rule (-0 counts as positive) in bits, b's before a's: a is the end of a chain of FP64 instructions
+  const int hi = __double2hiint(b), sign = ((hi << 1) | __double2loint(b)) != 0 ? hi & (int)0x80000000 : 0;
+  return __hiloint2double((__double2hiint(a) & 0x7fffffff) | sign, __double2loint(a));
 #else
   return b >= 0.0 ? fabs(a) : -fabs(a);
 #endif
@@ -922,11 +923,29 @@ SE_HD inline void schur_vector(const R* S, int ld, int m, int p, double lr_, dou
   }
 }
 
+// the bits of x: those of non-negative values are ordered like the values
+SE_HD inline long long se_bits(double x) {
+#ifdef __CUDA_ARCH__
+  return __double_as_longlong(x);
+#else
+  long long u;
+  memcpy(&u, &x, sizeof(u));
+  return u;
+#endif
+}
+// whether the non-negative values with these bits may be within 1e-14 of each other (96 ulp are 1.06e-14 at least)
+// or are not ordered by their bits (a NaN)
+SE_HD inline bool may_be_close(long long a, long long b) {
+  const long long inf = 0x7ff0000000000000ll;
+  return (a - b <= 96 && b - a <= 96) || a > inf || b > inf;
+}
+
 // Order of eigenvalues by decreasing modulus; within a pair the +imag member first.  Moduli that differ by
 // 1e-14 or less count as equal and are taken as the selection below meets them, so that which of them comes
 // first, and which one the cut at nev keeps, does not hang on their last bits.  perm: m ints; mod: m doubles of
 // scratch (the moduli).  Where no moduli but those of a pair are that close, every rule gives the same order and each
-// thread finds the rank of its eigenvalue; otherwise one thread selects.  Ends with a barrier.
+// thread finds the rank of its eigenvalue; otherwise one thread selects.  The comparisons are of integers:
+// an FP64 one holds GB300's FP64 pipe as long as a multiply-add of a whole warp.  Ends with a barrier.
 SE_HD inline void order_by_modulus(const double* wr, const double* wi, int m, int* perm, double* mod,
                                    const Team& t = Team{0, 1}) {
   for (int j = t.lane; j < m; j += t.size) mod[j] = hypot(wr[j], wi[j]);
@@ -934,12 +953,17 @@ SE_HD inline void order_by_modulus(const double* wr, const double* wi, int m, in
   int close = 0;
   for (int j = t.lane; j < m; j += t.size) {
     int rank = 0;
-    const double mj = mod[j], ij = wi[j];
+    const long long mj = se_bits(mod[j]), rj = se_bits(wr[j]), ij = se_bits(wi[j]);
     for (int k = 0; k < m; ++k) {
-      rank += (mod[k] > mj || (mod[k] == mj && wi[k] > ij)) ? 1 : 0;
-      const bool partner = wr[k] == wr[j] && wi[k] == -ij && ij != 0.0;
-      // (a NaN is close to everything)
-      if (k != j && !partner && !(fabs(mod[k] - mj) > 2e-14 * mj)) close = 1;
+      const long long mk = se_bits(mod[k]);
+      rank += mk > mj ? 1 : 0;
+      if (k != j && may_be_close(mk, mj)) {
+        const long long ik = se_bits(wi[k]);
+        if (se_bits(wr[k]) == rj && (ik ^ ij) < 0 && (ik << 1) == (ij << 1) && (ij << 1) != 0)
+          rank += ij < 0 ? 1 : 0;   // the partner of its pair
+        else
+          close = 1;
+      }
     }
     perm[rank] = j;
   }
@@ -951,7 +975,9 @@ SE_HD inline void order_by_modulus(const double* wr, const double* wi, int m, in
         double bm = mod[perm[a]];
         for (int b = a + 1; b < m; ++b) {
           const double mb = mod[perm[b]];
-          if (mb > bm * (1 + 1e-14) || (fabs(mb - bm) <= 1e-14 * bm && wi[perm[b]] > wi[perm[best]])) {
+          if (may_be_close(se_bits(mb), se_bits(bm))
+                  ? mb > bm * (1 + 1e-14) || (fabs(mb - bm) <= 1e-14 * bm && wi[perm[b]] > wi[perm[best]])
+                  : se_bits(mb) > se_bits(bm)) {
             best = b;
             bm = mb;
           }
