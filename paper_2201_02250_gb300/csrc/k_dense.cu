@@ -195,6 +195,56 @@ __device__ __forceinline__ void tile_gemm(FA fa, FB fb, int K, Acc (&acc)[4][4],
   }
 }
 
+// The same for the panels of a CTA of 512 threads: each half of it multiplies a lower triangle ft(m, k) (zero for
+// k > m) by an operand fb(k, c) of its own, with its own staging buffers; along_k: consecutive threads fetch fb
+// along k.  A warp skips the slabs that hold only zeros of its eight rows (a sum's terms keep their order).
+template <class Acc, class FT, class FB>
+__device__ __forceinline__ void tile_trmm(FT ft, FB fb, bool along_k, int K, Acc (&acc)[4][4], Acc* sA, Acc* sB) {
+  const int tid = threadIdx.x & 255, tx = tid & 15, ty = tid >> 4;
+  Acc ra[4], rb[4];
+  auto b_index = [&](int e, int& k, int& c) {
+    k = along_k ? e % TGK : e / 64;
+    c = along_k ? e / TGK : e % 64;
+  };
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = tid + u * 256;
+      int k, c;
+      b_index(e, k, c);
+      ra[u] = ft(e / TGK, k0 + e % TGK);
+      rb[u] = fb(k0 + k, c);
+    }
+  };
+  fetch(0);
+  for (int k0 = 0; k0 < K; k0 += TGK) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = tid + u * 256;
+      int k, c;
+      b_index(e, k, c);
+      sA[(e % TGK) * TS + e / TGK] = ra[u];
+      sB[k * TS + c] = rb[u];
+    }
+    __syncthreads();
+    if (k0 + TGK < K) fetch(k0 + TGK);
+    if (((tid >> 5) + 1) * 8 > k0) {
+      const int kk = min(TGK, K - k0);
+#pragma unroll 8
+      for (int k = 0; k < kk; ++k) {
+        Acc a[4], b[4];
+        load4(sA + k * TS + ty * 4, a);
+        load4(sB + k * TS + tx * 4, b);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int v = 0; v < 4; ++v) mac(acc[u][v], a[u], b[v]);
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // Blocked right-looking LU without pivoting, one CTA per subdomain (largest first).  Each step
 // factors a diagonal block of up to 64 columns in shared memory and inverts its triangles there;
 // the block column below it (L21 = A21 inv(U11)), the block row to its right (U12 = inv(L11) A12)
@@ -205,18 +255,16 @@ __device__ __forceinline__ void tile_gemm(FA fa, FB fb, int K, Acc (&acc)[4][4],
 // overlap rows is left in place); 1 the remaining columns [n_I, n).
 constexpr size_t lu_smem_elems() { return 2 * (size_t)TB * 65 + 2 * (size_t)TGK * TS; }
 
-// TC (double-float only): L21, U12 and the trailing update A22 -= L21 U12 run on the tensor cores as digit-split
-// BF16 products (tc_dfloat.cuh); their operand digits and the staging of a tile take most of the shared memory, so
-// one CTA of 512 threads runs per SM, holding all of that SM's TMEM.  A tile's cost is the splitting of its
-// operands and the double-float arithmetic on its results, not the MMAs: these run while the old values and the
-// next operand are on their way.  304 matrices of 1728 rows: 43.1 ms with L21 and U12 on the FP32 pipe and 256
-// threads that waited for each tile's MMAs, 32.8 with this order of a tile and digit products throughout, 28.2 with
-// 512 threads (18.4 at the copy bandwidth for what the right-looking order reads and writes); 512 subdomains of
-// 2200 to 2744 rows, interior columns, 146 -> 106 ms.  Against a long double factorisation L and U are as exact as
-// with FP32-pipe L21 and U12 (convection-diffusion L 6.0e-15, before 6.1e-15; lognormal 1.9e-14, 1.9e-14; jumps of
-// 1e6 1.8e-10, 1.7e-10, and 1.4e-10 with nothing on the tensor cores).  Only where rows and columns are both
-// scaled by random factors of 10^-3 to 10^3 does L lose digits (5e-12, before 9e-14; the backward error is 8e-15
-// both): digits are relative to the largest entry of a row of A21 (tc_dfloat.cuh).
+// TC (double-float only): the trailing update A22 -= L21 U12 runs on the tensor cores as digit-split BF16 products
+// (tc_dfloat.cuh); their operand digits and the staging of a tile take most of the shared memory, so one CTA of 512
+// threads runs per SM, holding all of that SM's TMEM.  A tile's cost is the splitting of its operands and the
+// double-float arithmetic on its results, not the MMAs: these run while the old values and the next operand are
+// on their way.  L21 and U12 stay on the FP32 pipe.  As digit products they are faster, but digits are
+// relative to the largest entry of a row of A21, and where rows and columns are both scaled by random factors
+// of 10^-3 to 10^3 the error of L against a long double factorisation grew from 9e-14 to 5e-12 (now 1e-13; without
+// tensor cores 7e-15).  304 matrices of 1728 rows: 43.1 ms with 256 threads that waited for each tile's MMAs, 33.0
+// with 512 and the tiles overlapped (28.2 with digits throughout); the splittings of 512 subdomains of about 2400
+// rows 215.7 -> 148.2 ms (132.6).
 //
 // MULTI: with fewer subdomains than SMs a cluster of CTAs takes each one.  Every CTA factors the diagonal
 // block for itself, the tiles of L21, U12 and of the trailing matrix are dealt out, and cluster barriers, which
@@ -351,77 +399,68 @@ __global__ void __launch_bounds__(LuThreads<TC>::value, TC ? 1 : 2) k_lu(int N, 
     // 2. L21 = A21 inv(U11) and 3. U12 = inv(L11) A12
     int dealt = 0;   // nonzero tiles so far, dealt out in turn
     if constexpr (TC) {
-      auto multiply = [&]() {   // the tile product; false (in every thread) once a wait has run out
-        tcdf::issue(ctx);
-        if (!tcdf::wait(ctx)) {
-          if (tid == 0) raise_status(st, A2LS_ERR_TIMEOUT, i, k0);
-          tc_fail = true;
-        }
-        return !tc_fail;
+      // on the FP32 pipe, in double-float as with no tensor cores: a row of A21 may mix magnitudes far apart (badly
+      // scaled unknowns), which digits relative to its largest entry do not hold.  A half of the CTA takes a tile
+      // of 64 columns of U12, or of 64 rows of L21 as the columns of L21^T = inv(U11)^T A21^T.
+      const int half = tid >> 8;
+      Acc* hA = reinterpret_cast<Acc*>(lu_smem_raw) + half * 2 * TGK * TS;   // (the diagonal block is written back)
+      auto panel = [&](int q) {   // tile q of L21, or q - tiles of U12; q < 0: no tile, the barriers only
+        const bool u12 = q >= tiles;
+        const int s0 = c0 + (u12 ? q - tiles : q) * TB, cols = q < 0 ? 0 : min(TB, n - s0);
+        T* P = u12 ? A + (int64_t)k0 * L + s0 : A + (int64_t)s0 * L + k0;   // entry (k, c) of the operand
+        const int64_t lk = u12 ? L : 1, lc = u12 ? 1 : L;
+        Acc acc[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int v = 0; v < 4; ++v) acc[u][v] = 0;
+        tile_trmm<Acc>(
+            [&](int m, int k) -> Acc {
+              if (m >= w || k > m) return Acc(0.f);
+              return u12 ? (k < m ? Iv[m * 65 + k] : Acc(1.f)) : Iv[k * 65 + m];
+            },
+            [&](int k, int c) -> Acc { return k < w && c < cols ? (Acc)P[k * lk + c * lc] : Acc(0.f); },
+            !u12, w, acc, hA, hA + TGK * TS);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const int k = (tid & 255) / 16 * 4 + u, c = tx * 4 + v;
+            if (k < w && c < cols) P[k * lk + c * lc] = (T)finish(acc[u][v]);
+          }
       };
-      const int pairs = (tiles + 1) / 2, warp = tid >> 5, lane = tid & 31;
-      dfloat vb[8];
-      ctx.eB = tc_eB;
-      // L21, 128 rows a tile; staged where the A digits were
-      tcdf::load_b([&](int k, int c) -> dfloat { return c >= k && c < w ? Iv[k * 65 + c] : dfloat(0.f, 0.f); }, vb);
-      tcdf::write_b(ctx, vb, tc_red);
-      dfloat* S = reinterpret_cast<dfloat*>(lu_smem_raw);
-      for (int t = 0; t < pairs; ++t) {
-        if (!lnz[2 * t] && !(2 * t + 1 < tiles && lnz[2 * t + 1])) continue;
-        if (dealt++ % C != rank || tc_fail) continue;
-        T* P = A + (int64_t)(c0 + t * tcdf::TM) * L + k0;
-        const int rows = min(tcdf::TM, n - c0 - t * tcdf::TM);
-        tcdf::split_a(ctx, [&](int m, int k) -> dfloat {
-          return m < rows && k < w ? (dfloat)P[(int64_t)m * L + k] : dfloat(0.f, 0.f);
-        });
-        if (!multiply()) continue;
-        for (int half = 0; half < 2; ++half) {
-          tcdf::stage_half(ctx, ctx.eB, half, S);
-          __syncthreads();
-          const int c = half * 32 + lane;
-          for (int r = warp; r < rows; r += NT / 32)
-            if (c < w) P[(int64_t)r * L + c] = (T)finish(S[r * tcdf::SUB_LD + lane]);
-          __syncthreads();
+      int first = -1;
+      for (int q = 0; q <= 2 * tiles; ++q) {   // pairs of nonzero tiles are dealt out; the last may lack its second
+        const bool end = q == 2 * tiles;
+        if (!end) {
+          if (!(q < tiles ? lnz[q] : unz[q - tiles])) continue;
+          const int d = dealt++;
+          if ((d >> 1) % C != rank) continue;
+          if (!(d & 1)) {
+            first = q;
+            continue;
+          }
+        } else if (first < 0) {
+          break;
         }
-      }
-      // U12 as its transpose, A12^T inv(L11)^T, 128 columns a tile: a thread holds a column and a warp's
-      // accesses run along the rows of memory
-      tcdf::load_b([&](int k, int c) -> dfloat {
-        return k < c && c < w ? Iv[c * 65 + k] : dfloat(k == c && c < w ? 1.f : 0.f, 0.f);
-      }, vb);
-      tcdf::write_b(ctx, vb, tc_red);
-      for (int t = 0; t < pairs; ++t) {
-        if (!unz[2 * t] && !(2 * t + 1 < tiles && unz[2 * t + 1])) continue;
-        if (dealt++ % C != rank || tc_fail) continue;
-        T* P = A + (int64_t)k0 * L + c0 + t * tcdf::TM;
-        const int cols = min(tcdf::TM, n - c0 - t * tcdf::TM);
-        tcdf::split_a(ctx, [&](int m, int k) -> dfloat {
-          return m < cols && k < w ? (dfloat)P[(int64_t)k * L + m] : dfloat(0.f, 0.f);
-        });
-        if (!multiply()) continue;
-        const int m = (warp & 3) * 32 + lane;
-#pragma unroll 1
-        for (int cb = (warp >> 2) * 16, ce = cb + 16; cb < ce; cb += 8)
-          tcdf::product8(ctx, ctx.eB, cb, [&](int r, dfloat v) {
-            if (m < cols && r < w) P[(int64_t)r * L + m] = (T)finish(v);
-          });
-        __syncthreads();
+        panel(half ? (end ? -1 : q) : first);
+        first = -1;
       }
     } else {
       for (int t = 0; t < tiles; ++t) {
         if (!lnz[t] || dealt++ % C != rank) continue;
         const int r0 = c0 + t * TB, rows = min(TB, n - r0);
         Acc acc[4][4];
-  #pragma unroll
+#pragma unroll
         for (int u = 0; u < 4; ++u)
-  #pragma unroll
+#pragma unroll
           for (int v = 0; v < 4; ++v) acc[u][v] = 0;
         tile_gemm<Acc>([&](int m, int k) -> Acc { return (m < rows && k < w) ? (Acc)A[(int64_t)(r0 + m) * L + k0 + k] : (Acc)0; },
                        [&](int k, int c) -> Acc { return (k < w && c < w && c >= k) ? Iv[k * 65 + c] : (Acc)0; },
                        w, acc, sA, sB);
-  #pragma unroll
+#pragma unroll
         for (int u = 0; u < 4; ++u)
-  #pragma unroll
+#pragma unroll
           for (int v = 0; v < 4; ++v) {
             const int r = ty * 4 + u, c = tx * 4 + v;
             if (r < rows && c < w) A[(int64_t)(r0 + r) * L + k0 + c] = (T)finish(acc[u][v]);
@@ -432,16 +471,16 @@ __global__ void __launch_bounds__(LuThreads<TC>::value, TC ? 1 : 2) k_lu(int N, 
         if (!unz[t] || dealt++ % C != rank) continue;
         const int cs = c0 + t * TB, cols = min(TB, n - cs);
         Acc acc[4][4];
-  #pragma unroll
+#pragma unroll
         for (int u = 0; u < 4; ++u)
-  #pragma unroll
+#pragma unroll
           for (int v = 0; v < 4; ++v) acc[u][v] = 0;
         tile_gemm<Acc>([&](int m, int k) -> Acc { return (m < w && k < w) ? (k < m ? Iv[m * 65 + k] : (k == m ? (Acc)1 : (Acc)0)) : (Acc)0; },
                        [&](int k, int c) -> Acc { return (k < w && c < cols) ? (Acc)A[(int64_t)(k0 + k) * L + cs + c] : (Acc)0; },
                        w, acc, sA, sB);
-  #pragma unroll
+#pragma unroll
         for (int u = 0; u < 4; ++u)
-  #pragma unroll
+#pragma unroll
           for (int v = 0; v < 4; ++v) {
             const int r = ty * 4 + u, c = tx * 4 + v;
             if (r < w && c < cols) A[(int64_t)(k0 + r) * L + cs + c] = (T)finish(acc[u][v]);
