@@ -145,7 +145,8 @@ typedef struct {
                                (pipelined kernel), 3000 / 3004 / 3008 (streaming kernel on the
                                repacked factors: one CTA of 8 consumer warps, two of 4, two of 8 per
                                SM; FP32 and BF16 factors only: for
-                               FP64 factors they are the autotuner's to choose) */
+                               FP64 factors they are the autotuner's to choose, where the repacked
+                               copy leaves as much memory free as it takes) */
   int32_t eig_block_size;   /* columns of the local eigensolves' blocks: 0 (default) = the larger of
                                nev + max(4, nev / 2) and min(2 nev, 24), at most 32; otherwise that many
                                (at least nev + 1, at most 32) */

@@ -90,7 +90,7 @@ struct Phase { enum { SETUP_GRAPH, SETUP_EXTRACT, SETUP_LU, SETUP_EIG, SETUP_COA
 
 // the apply's local factors repacked as one stream in solve order (k_stream.cu)
 struct StreamSolve {
-  bool ready = false;
+  bool ready = false, withheld = false;      // withheld: no copy for want of memory
   int elem_bytes = 0, nchunks = 0, xcap = 0;
   int64_t stream_elems = 0;
   void* d_stream = nullptr;
@@ -253,6 +253,7 @@ template <class T> void local_solves(a2ls_handle* h, const T* fac, const double*
 template <class T> void autotune_local_solves(a2ls_handle* h, const T* fac, const double* t, double* scratch,
                                               int mode);
 int autotune_lookup(const char* key);            // 0 if unknown
+template <class T> int tuned_local_solves(a2ls_handle* h, int mode);   // the cached choice, 0 if unknown
 void autotune_store(const char* key, int value);
 void dense_inverse(a2ls_handle* h, double* E, int n, double scale, double* Einv, int band);
 // skip_p_le > 0: subdomains with at most that many columns are left to another kernel
@@ -280,6 +281,8 @@ constexpr int TC_SOLVE_MAX_P = 32;
 // k_stream.cu: pack the factors (after the diagonal tiles are inverted) into the stream of the
 // streaming local solves, and those solves (FP32 or BF16 factors)
 template <class T> void stream_prepare(a2ls_handle* h, const T* fac);
+void stream_release(a2ls_handle* h);
+size_t available_memory(a2ls_handle* h);   // of the device: free, or kept unused by the library's pool
 template <class T> void launch_local_solve_stream(a2ls_handle* h, int config, const double* t, const double* q,
                                                   double* z, int mode);
 

@@ -121,6 +121,18 @@ void* dalloc_bytes(a2ls_handle* h, size_t bytes) {
   return p;
 }
 
+size_t available_memory(a2ls_handle* h) {
+  size_t free = 0, total = 0;
+  A2LS_CUDA(cudaMemGetInfo(&free, &total));
+  if (h->pool) {
+    uint64_t reserved = 0, used = 0;
+    A2LS_CUDA(cudaMemPoolGetAttribute(h->pool, cudaMemPoolAttrReservedMemCurrent, &reserved));
+    A2LS_CUDA(cudaMemPoolGetAttribute(h->pool, cudaMemPoolAttrUsedMemCurrent, &used));
+    free += (size_t)(reserved - std::min(reserved, used));
+  }
+  return free;
+}
+
 void dfree(a2ls_handle* h, void* p) {
   if (!p) return;
   auto it = std::find(h->allocs.begin(), h->allocs.end(), p);
@@ -522,18 +534,23 @@ int a2ls_setup(const a2ls_csr* A, const int32_t* partition, int32_t overlap, int
       dfree(h, h->d_fac);
       h->d_fac = fb;
     }
-    // the factors repacked for the streaming local solves
-    if (o.precision == A2LS_BF16) stream_prepare<__nv_bfloat16>(h, static_cast<const __nv_bfloat16*>(h->d_fac));
-    else if (o.precision == A2LS_FP32) stream_prepare<float>(h, static_cast<const float*>(h->d_fac));
-    else if (o.local_solve_kernel == 0) stream_prepare<double>(h, static_cast<const double*>(h->d_fac));
     // apply workspace
     h->d_q = dalloc<double>(h, h->n);
     h->d_t = dalloc<double>(h, h->n);
     h->d_yloc = dalloc<double>(h, h->sum_n);
+    const bool ras = v == A2LS_DEFLATED_RAS || v == A2LS_ADDITIVE_RAS || v == A2LS_ONE_LEVEL_RAS;
+    const int mode = ras ? (o.pou == A2LS_POU_BOOLEAN ? 0 : 1) : 2;
+    // the factors repacked for the streaming local solves (FP64: unless another kernel is known to be faster)
+    if (o.precision == A2LS_BF16) {
+      stream_prepare<__nv_bfloat16>(h, static_cast<const __nv_bfloat16*>(h->d_fac));
+    } else if (o.precision == A2LS_FP32) {
+      stream_prepare<float>(h, static_cast<const float*>(h->d_fac));
+    } else if (o.local_solve_kernel == 0) {
+      const int known = tuned_local_solves<double>(h, mode);
+      if (known <= 0 || known >= LS_STREAM) stream_prepare<double>(h, static_cast<const double*>(h->d_fac));
+    }
     // pick the CTA width of the local solves for this problem (timed on its own factors)
     {
-      const bool ras = v == A2LS_DEFLATED_RAS || v == A2LS_ADDITIVE_RAS || v == A2LS_ONE_LEVEL_RAS;
-      const int mode = ras ? (o.pou == A2LS_POU_BOOLEAN ? 0 : 1) : 2;
       A2LS_CUDA(cudaMemsetAsync(h->d_t, 0, sizeof(double) * h->n, st));
       double* scratch = mode == 0 ? h->d_q : h->d_yloc;
       const int timing = h->opt.timing;
@@ -549,6 +566,7 @@ int a2ls_setup(const a2ls_csr* A, const int32_t* partition, int32_t overlap, int
         autotune_local_solves<__nv_bfloat16>(h, static_cast<__nv_bfloat16*>(h->d_fac), h->d_t, scratch, mode);
       else autotune_local_solves<float>(h, static_cast<float*>(h->d_fac), h->d_t, scratch, mode);
       h->opt.timing = timing;
+      if (o.precision == A2LS_FP64 && h->ls_width < LS_STREAM) stream_release(h);
     }
     // load the module holding a2ls_apply_static's scratch array now, while allocation is allowed
     prime_static_scratch();

@@ -1169,11 +1169,19 @@ void local_solves(a2ls_handle* h, const T* fac, const double* t, const double* q
 // keep the fastest; results are cached per (precision, subdomain count, largest subdomain, mode)
 // in the process and, when A2LS_AUTOTUNE_CACHE names a file, in that JSON file.
 template <class T>
-void autotune_local_solves(a2ls_handle* h, const T* fac, const double* t, double* scratch, int mode) {
+static std::string tune_key(const a2ls_handle* h, int mode) {
   char key[128];
   snprintf(key, sizeof(key), "local_solve4_%s_N%d_max%d_mode%d",
            sizeof(T) == 8 ? "fp64" : (sizeof(T) == 4 ? "fp32" : "bf16"), h->N, h->max_n, mode);
-  int cached = autotune_lookup(key);
+  return key;
+}
+template <class T>
+int tuned_local_solves(a2ls_handle* h, int mode) { return autotune_lookup(tune_key<T>(h, mode).c_str()); }
+
+template <class T>
+void autotune_local_solves(a2ls_handle* h, const T* fac, const double* t, double* scratch, int mode) {
+  const std::string key = tune_key<T>(h, mode);
+  const int cached = autotune_lookup(key.c_str());
   if (cached > 0 && (cached != LS_STREAM || h->ss.shape[0].ready) && (cached != LS_STREAM2 || h->ss.shape[1].ready) &&
       (cached != LS_STREAM3 || h->ss.shape[2].ready)) {
     h->ls_width = cached;
@@ -1204,7 +1212,7 @@ void autotune_local_solves(a2ls_handle* h, const T* fac, const double* t, double
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   h->ls_width = best;
-  autotune_store(key, best);
+  if (!h->ss.withheld) autotune_store(key.c_str(), best);
 }
 
 // ---------------------------------------------------------------------------
@@ -1314,6 +1322,7 @@ template void local_solves<__nv_bfloat16>(a2ls_handle*, const __nv_bfloat16*, co
                                           int);
 template void autotune_local_solves<__nv_bfloat16>(a2ls_handle*, const __nv_bfloat16*, const double*, double*, int);
 template void local_solves<double>(a2ls_handle*, const double*, const double*, const double*, double*, int);
+template int tuned_local_solves<double>(a2ls_handle*, int);
 template void autotune_local_solves<float>(a2ls_handle*, const float*, const double*, double*, int);
 template void autotune_local_solves<double>(a2ls_handle*, const double*, const double*, double*, int);
 template void block_solve<float>(a2ls_handle*, const float*, float*, const int64_t*, int, int, const int*, int,

@@ -613,11 +613,21 @@ void stream_prepare(a2ls_handle* h, const T* fac) {
   S.elem_bytes = (int)sizeof(T);
   S.nchunks = (int)meta.size();
   S.stream_elems = soff[N];
+  if (sizeof(T) == 8) {
+    // FP64 handles hold the largest factors and do without the copy where memory is short: it has to leave
+    // the vectors of GMRES and as much again as it takes itself, for the caller and for other handles
+    const double copy = sizeof(T) * ((double)soff[N] + W) + sizeof(int4) * (double)meta.size();
+    const double basis = sizeof(double) * (2.0 * std::max(30, h->opt.restart) + 3) * h->n;
+    if (2 * copy + basis > (double)available_memory(h)) {
+      S.withheld = true;
+      return;
+    }
+  }
   try {
     S.d_stream = dalloc<T>(h, (size_t)soff[N] + W);
   } catch (const Error& e) {
-    // FP64 handles hold the largest factors: without room for the second copy they keep to the other kernels
     if (sizeof(T) != 8 || e.code != A2LS_ERR_OOM) throw;
+    S.withheld = true;
     return;
   }
   S.d_meta = dalloc<int4>(h, meta.size());
@@ -676,6 +686,16 @@ void stream_prepare(a2ls_handle* h, const T* fac) {
   S.d_order = dalloc<int>(h, N);
   A2LS_CUDA(cudaMemcpyAsync(S.d_order, order.data(), sizeof(int) * N, cudaMemcpyHostToDevice, st));
   A2LS_CUDA(cudaStreamSynchronize(st));
+}
+
+void stream_release(a2ls_handle* h) {
+  StreamSolve& S = h->ss;
+  dfree(h, S.d_stream);
+  dfree(h, S.d_meta);
+  dfree(h, S.d_choff);
+  dfree(h, S.d_soff);
+  dfree(h, S.d_order);
+  S = StreamSolve{};
 }
 
 // config: LS_STREAM (8 consumer warps, one CTA per SM), LS_STREAM2 (4 consumer warps, two CTAs per SM) or

@@ -80,3 +80,39 @@ def test_handles_of_different_sizes_side_by_side(kernel, first, second):
         P.apply(r, z)
         torch.cuda.synchronize()
         assert np.array_equal(z.cpu().numpy(), want.cpu().numpy())
+
+
+FOOTPRINT_SCRIPT = """
+import sys
+import torch
+from paper_2201_02250_gb300 import a2ls
+from workloads import pde
+prob = pde.tiny_conv_diff(m=300, nb=5, overlap=1, nev=0)
+P, keep = a2ls.from_scipy(prob.A, prob.part, prob.overlap, 0, variant="ras", local_solve_kernel=int(sys.argv[1]))
+P.solve(torch.as_tensor(prob.b, device="cuda"), torch.zeros(prob.n, dtype=torch.float64, device="cuda"), 1e-1,
+        allow_not_converged=True)
+a2ls.trim_memory()
+free, total = torch.cuda.mem_get_info()
+print(P.tuning()["local_solve_threads"], total - free, max(len(a) + len(b) for a, b in P.subdomains()))
+"""
+
+
+def test_fp64_factors_are_held_once_unless_streamed(tmp_path):
+    """What the device holds for a handle of 25 subdomains of 3600 rows (band 60, so that a second copy of the factors
+    is 2 x 90000 x 60 doubles and more): a kernel known to be faster than the streaming one leaves none behind."""
+    copy = 2 * 90000 * 60 * 8
+
+    def footprint(option, cached=None):
+        cache = tmp_path / f"tune{option}_{cached}.json"
+        cache.write_text("{}" if cached is None else json.dumps({f"local_solve4_fp64_N25_max{rows}_mode0": cached}))
+        r = subprocess.run([sys.executable, "-c", FOOTPRINT_SCRIPT, str(option)], cwd=ROOT, capture_output=True, text=True,
+                           env=dict(os.environ, A2LS_AUTOTUNE_CACHE=str(cache)), timeout=300)
+        assert r.returncode == 0, r.stdout + r.stderr
+        return [int(v) for v in r.stdout.split()]
+
+    kernel, base, rows = footprint(512)
+    assert kernel == 512
+    kernel, held, _ = footprint(0, 512)
+    assert kernel == 512 and held - base < copy // 2
+    kernel, held, _ = footprint(0, 3000)
+    assert kernel == 3000 and held - base > copy // 2
