@@ -17,19 +17,21 @@ namespace a2ls {
 
 // ---------------------------------------------------------------------------
 // CSR SpMV: y = A x, or y = bm - A x when bm != nullptr.  Bound by memory: 12 bytes an entry.
-// Rows of at most SPMV_SHORT entries (stencils): a thread per row with SPMV_UNROLL entries in flight; the
-// neighbours' entries share its cache lines.  4 lanes per row kept one gather in flight: 41.4 -> 22.3 us on
-// the 96^3 seven-point operator (91 MB).
+// Stencils (SPMV_SHORT entries a row on average, or fewer): a thread per row with SPMV_UNROLL entries in flight;
+// the neighbours' entries share its cache lines.  4 lanes per row kept one gather in flight: 41.4 -> 22.3 us on
+// the 96^3 seven-point operator (91 MB); 150,000 rows of 5, 9, 15 entries 15.0, 15.0, 19.1 -> 10.9, 13.0, 15.0.
+// A row of more than SPMV_LONG entries is the whole warp's (that operator with one row of 2000: 140 us with four
+// lanes, 42 so).
 // ---------------------------------------------------------------------------
-constexpr int SPMV_UNROLL = 8, SPMV_SHORT = 32;
+constexpr int SPMV_UNROLL = 8, SPMV_SHORT = 16, SPMV_LONG = 64;
 __global__ void __launch_bounds__(128) k_spmv(int n, const int* __restrict__ rowptr, const int* __restrict__ colind,
                                               const double* __restrict__ val, const double* __restrict__ x,
                                               double* __restrict__ y, const double* __restrict__ bm) {
-  const int r = blockIdx.x * 128 + threadIdx.x;
-  if (r >= n) return;
-  const int a = rowptr[r], b = rowptr[r + 1];
+  const int r = blockIdx.x * 128 + threadIdx.x, lane = threadIdx.x & 31;
+  const int a = r < n ? rowptr[r] : 0, b = r < n ? rowptr[r + 1] : 0;
+  const bool is_long = b - a > SPMV_LONG;
   double s = 0.0;
-  for (int q = a; q < b; q += SPMV_UNROLL) {
+  for (int q = a; q < b && !is_long; q += SPMV_UNROLL) {
     int c[SPMV_UNROLL];
     double v[SPMV_UNROLL], xv[SPMV_UNROLL];
 #pragma unroll
@@ -42,50 +44,43 @@ __global__ void __launch_bounds__(128) k_spmv(int n, const int* __restrict__ row
 #pragma unroll
     for (int u = 0; u < SPMV_UNROLL; ++u) s += v[u] * xv[u];
   }
-  y[r] = bm ? bm[r] - s : s;
-}
-
-// Matrices with longer rows: a CTA takes 256 consecutive rows, whose entries are one contiguous piece of
-// colind and val: the threads read it coalesced into products in shared memory, and one thread per row sums
-// its own in order (piece by piece where the entries do not fit).  On the same operator 33 us.
-__global__ void __launch_bounds__(256) k_spmv_long(int n, const int* __restrict__ rowptr,
-                                                   const int* __restrict__ colind, const double* __restrict__ val,
-                                                   const double* __restrict__ x, double* __restrict__ y,
-                                                   const double* __restrict__ bm) {
-  constexpr int ROWS = 256, CAP = ROWS * SPMV_UNROLL;
-  __shared__ double prod[CAP];
-  const int tid = threadIdx.x, r0 = blockIdx.x * ROWS, r = r0 + tid;
-  const int e0 = rowptr[r0], e1 = rowptr[min(r0 + ROWS, n)];
-  const int a = r < n ? rowptr[r] : e1, b = r < n ? rowptr[r + 1] : e1;
-  double s = 0.0;
-  for (int base = e0; base < e1; base += CAP) {
-    const int cnt = min(CAP, e1 - base);
-    int c[SPMV_UNROLL];
-    double v[SPMV_UNROLL];
-#pragma unroll
-    for (int u = 0; u < SPMV_UNROLL; ++u) {
-      const int e = tid + u * ROWS;
-      c[u] = e < cnt ? __ldcs(colind + base + e) : 0;
-      v[u] = e < cnt ? __ldcs(val + base + e) : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < SPMV_UNROLL; ++u) {
-      const int e = tid + u * ROWS;
-      if (e < cnt) prod[e] = v[u] * __ldg(x + c[u]);
-    }
-    __syncthreads();
-    const int q1 = min(b - base, cnt);
-    for (int q = max(a - base, 0); q < q1; ++q) s += prod[q];
-    __syncthreads();
+  for (unsigned todo = __ballot_sync(0xffffffffu, is_long); todo; todo &= todo - 1) {
+    const int owner = __ffs(todo) - 1;
+    const int a2 = __shfl_sync(0xffffffffu, a, owner), b2 = __shfl_sync(0xffffffffu, b, owner);
+    double t = 0.0;
+#pragma unroll 4
+    for (int q = a2 + lane; q < b2; q += 32) t += __ldg(val + q) * __ldg(x + __ldg(colind + q));
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == owner) s = t;
   }
   if (r < n) y[r] = bm ? bm[r] - s : s;
 }
 
+// Other matrices: 4 lanes per row.  150,000 rows of 17, 33, 65, 301 entries: 19, 25, 38, 122 us, with a thread each 19,
+// 29, 50, 193.
+__global__ void k_spmv_wide(int n, const int* __restrict__ rowptr, const int* __restrict__ colind,
+                            const double* __restrict__ val, const double* __restrict__ x, double* __restrict__ y,
+                            const double* __restrict__ bm) {
+  const int sub = threadIdx.x & 3;
+  const unsigned row_lanes = 0xfu << (threadIdx.x & 28);
+  for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 2; r < n; r += (gridDim.x * blockDim.x) >> 2) {
+    double s = 0.0;
+    const int a = rowptr[r], b = rowptr[r + 1];
+    for (int q = a + sub; q < b; q += 4) s += val[q] * __ldg(x + colind[q]);
+    s += __shfl_xor_sync(row_lanes, s, 1);
+    s += __shfl_xor_sync(row_lanes, s, 2);
+    if (sub == 0) y[r] = bm ? bm[r] - s : s;
+  }
+}
+
 void spmv(a2ls_handle* h, const double* x, double* y, const double* b_minus, cudaStream_t st) {
-  if (h->max_rownnz <= SPMV_SHORT)
+  if (h->nnz <= (int64_t)SPMV_SHORT * h->n) {
     k_spmv<<<ceil_div(h->n, 128), 128, 0, st>>>(h->n, h->rowptr, h->colind, h->val, x, y, b_minus);
-  else
-    k_spmv_long<<<ceil_div(h->n, 256), 256, 0, st>>>(h->n, h->rowptr, h->colind, h->val, x, y, b_minus);
+  } else {
+    const int threads = 256;
+    const int blocks = std::min(152 * 8, ceil_div((int64_t)h->n * 4, threads));
+    k_spmv_wide<<<blocks, threads, 0, st>>>(h->n, h->rowptr, h->colind, h->val, x, y, b_minus);
+  }
   A2LS_LAUNCH();
 }
 

@@ -71,3 +71,23 @@ def test_network_by_subdomain_size_and_count(m, nb):
     net.close()
     S.close()
     P.close()
+
+
+@pytest.mark.parametrize("lengths", [(3, 65, 64, 200), (16, 16, 16, 17), (1, 700, 33, 1000)])
+def test_spmv_of_rows_far_apart_in_length(lengths):
+    """Rows of the given lengths, one long one in 40: a thread's or a whole warp's where the rows are short on
+    average, else four lanes'; the bound of the test above."""
+    from paper_2201_02250_gb300 import a2ls
+    n, r = 1003, np.random.default_rng(sum(lengths))
+    A = sp.lil_matrix((n, n))
+    for i in range(n):
+        k = lengths[i % 4] if lengths[0] == 16 or i % 40 < 4 else lengths[0]
+        cols = r.choice(n, min(k, n), replace=False)
+        A[i, cols] = r.uniform(-1, 1, len(cols)) / n
+    A = (A + sp.diags(np.full(n, 4.0))).tocsr()
+    P, _keep = a2ls.from_scipy(A, (np.arange(n) * 4 // n).astype(np.int32), 0, 0, variant="ras")
+    x = r.uniform(-1, 1, n)
+    y = torch.empty(n, dtype=torch.float64, device="cuda")
+    P.spmv(torch.as_tensor(x, device="cuda"), y)
+    bound = 2 * (max(lengths) + 1) * 2.0**-53 * (abs(A) @ abs(x))
+    assert np.all(np.abs(y.cpu().numpy() - A @ x) <= bound)
