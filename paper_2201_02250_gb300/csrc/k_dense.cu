@@ -59,8 +59,9 @@ __device__ __forceinline__ void cta_gemm_narrow(const T* __restrict__ A, int64_t
       }
       sA[k * 65 + m] = v;
     }
-    for (int e = tid; e < GK * NCW; e += THREADS) {
-      const int k = e / NCW, c = e % NCW;
+    static_assert(GK * NCW <= THREADS, "one entry a thread");   // (a loop took 8 more registers, a CTA an SM less)
+    if (GK * NCW == THREADS || tid < GK * NCW) {
+      const int k = tid / NCW, c = tid % NCW;
       const int kk = k0 + k;
       sB[k * (NCW + 1) + c] = (c < Nc && kk < K) ? (Acc)B[kk * ldb + c] : (Acc)0;
     }
@@ -72,8 +73,8 @@ __device__ __forceinline__ void cta_gemm_narrow(const T* __restrict__ A, int64_t
 #pragma unroll 8
       for (int k = 0; k < GK; ++k) {
         const Acc a = sA[k * 65 + ty];
-#pragma unroll
-        for (int v = 0; v < CPT; ++v) mac(acc[v], a, sB[k * (NCW + 1) + tx * CPT + v]);
+        mac(acc[0], a, sB[k * (NCW + 1) + tx * CPT]);   // (written out: an inner loop cost k_e_inverse 3 %)
+        if constexpr (CPT > 1) mac(acc[1], a, sB[k * (NCW + 1) + tx * CPT + 1]);
       }
     }
     __syncthreads();
@@ -1298,19 +1299,25 @@ void block_solve(a2ls_handle* h, const T* fac, T* X, const int64_t* xoff, int co
   if (pmax <= skip_p_le) return;
   const int p = std::max(pmax, 1);
   if (nact <= 0) nact = h->N;
-  // at least three CTAs per SM where narrower chunks give them: 64 FP64 subdomains of 1950 rows, p = 16, 4.58 ->
-  // 3.13 ms a sweep; 16 of 300 rows 151 -> 117 us (8 columns against 2)
+  // FP64, bound by its pipe: at least three CTAs per SM where narrower chunks give them (64 subdomains of 1950 rows,
+  // p = 16, 4.58 -> 3.13 ms a sweep; 16 of 300 rows 151 -> 117 us, 8 columns against 2).  Double-float: one (9
+  // subdomains of 1300 rows, p = 16, 7.4 -> 6.4 ms a set-up; with three, 64 subdomains lose 6 %).  FP32 is bound by
+  // the staging of the factors, which every chunk repeats: always 8 columns (27 subdomains of 1900 rows 69 ms,
+  // narrower ones 95 to 123)
+  constexpr int ctas = std::is_same<T, double>::value ? 3 * 152 : (std::is_same<T, dfloat>::value ? 152 : 0);
   int w = 8;
-  while (w > 2 && (int64_t)nact * ceil_div(p, w) < 3 * 152) w /= 2;
+  while (w > 2 && (int64_t)nact * ceil_div(p, w) < ctas) w /= 2;
   const dim3 grid(h->N, ceil_div(p, w));
   auto go = [&](auto kernel, int threads) {
     kernel<<<grid, threads, 0, h->st>>>(h->d_ni, h->d_ld, h->d_foff, fac, X, xoff, col0, ldx, pvec, active, forward,
                                         backward, h->d_sched, h->d_toff, h->d_tf, h->d_tg, skip_p_le);
     A2LS_LAUNCH();
   };
-  if (w == 8) go(k_block_solve<T, 8>, narrow_threads<8>());
-  else if (w == 4) go(k_block_solve<T, 4>, narrow_threads<4>());
-  else go(k_block_solve<T, 2>, narrow_threads<2>());
+  if constexpr (ctas > 0) {
+    if (w == 4) return go(k_block_solve<T, 4>, narrow_threads<4>());
+    if (w == 2) return go(k_block_solve<T, 2>, narrow_threads<2>());
+  }
+  go(k_block_solve<T, 8>, narrow_threads<8>());
 }
 
 template void lu_batched<float>(a2ls_handle*, float*, int, double*, double*, int);

@@ -41,3 +41,19 @@ def test_clustered_factorisation_matches_oracle(m, nb, eigp):
     """Subdomains of 300 to 650 rows, whose 5 to 11 ragged tiles a block column are dealt to the CTAs of a cluster:
     the quantities and the bounds of the test above, which the factors of both matrices enter."""
     test_clustered_orthogonalisation_matches_oracle(m, nb, eigp)
+
+
+@pytest.mark.parametrize("m,nb", [(21, 2), (40, 9), (70, 13)])   # 4, 81 and 169 subdomains of 8 columns: chunks of 2, 4 and 8
+def test_double_float_chunk_widths_match_oracle(m, nb):
+    """The triangular solves without tensor cores at each width of their column chunks: eigenvalues as above."""
+    from paper_2201_02250_gb300 import a2ls
+    prob = pde.tiny_conv_diff(m=m, nb=nb, overlap=1, nev=4)
+    P, _keep = a2ls.from_scipy(prob.A, prob.part, prob.overlap, prob.nev, eig_precision="fp32x2", eig_tol=1e-9,
+                               tensor_cores=0)
+    ref = O.setup(prob.A, prob.part, prob.overlap, prob.nev)
+    ev, res = P.eigenvalues(), P.eig_residuals()
+    assert np.sum(res <= 1e-9) >= 0.9 * len(res)
+    for i, e in enumerate(ref.eig):
+        mine = ev[i][np.isfinite(ev[i].real)]
+        if res[i] <= 1e-9:
+            assert abs(np.abs(mine).max() - np.abs(e.selected).max()) <= 1e-7 * np.abs(e.selected).max()
