@@ -369,11 +369,12 @@ __global__ void k_mu_fix(const int* ni, const int* off, const int64_t* xoff, int
 // Orthogonalisation (k_orth and its helpers): block CGS2 of W against the basis, then Cholesky QR.
 // ---------------------------------------------------------------------------
 
-// Threads of k_orth.  Double-float and FP32: 256, with 32-row chunks, so that two CTAs share an SM and one's
-// barriers and staging overlap the other's arithmetic; FP64, whose chunks fix the order of its sums: 512.
-template <class Acc> struct OrthThreads { static constexpr int v = 256; };
-template <> struct OrthThreads<double> { static constexpr int v = 512; };
-// rows staged per chunk in k_orth: 64 in FP64 (32 with full-space Gram), otherwise 32
+// Threads of k_orth.  Double-float: 256, with 32-row chunks, so that two CTAs share an SM and one's barriers and
+// staging overlap the other's arithmetic; FP64, whose chunks fix the order of its sums, and FP32: 512 (256 subdomains
+// of about 1200 rows in FP32 11.0 ms a set-up, with 256 threads and 32 rows, which spill, 14.4).
+template <class Acc> struct OrthThreads { static constexpr int v = 512; };
+template <> struct OrthThreads<dfloat> { static constexpr int v = 256; };
+// rows staged per chunk in k_orth: 64 (32 with full-space Gram), in double-float 32
 // row stride of the staged chunks: even, so that column pairs are 16-byte aligned for vector loads;
 // 98 x 8 bytes puts consecutive rows 4 banks apart
 constexpr int SROW = EIG_MAXP + 2;
@@ -1523,7 +1524,7 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
   bool any_full = false;
   for (int i = 0; i < N; ++i) any_full = any_full || (full[i] && act[i]);
   const int gcap_k = EIG_MAXP * 32, gcap_f = any_full ? EIG_MAXP * EIG_MAXP : gcap_k;
-  auto orc_for = [&](int gcap) { return std::is_same<Acc, double>::value && gcap <= gcap_k ? 64 : 32; };
+  auto orc_for = [&](int gcap) { return !std::is_same<Acc, dfloat>::value && gcap <= gcap_k ? 64 : 32; };
   auto orth_smem_for = [&](int gcap) {
     return sizeof(double) * (2 * (size_t)gcap + EIG_MAXP) + sizeof(Acc) * 2 * (size_t)orc_for(gcap) * SROW;
   };
