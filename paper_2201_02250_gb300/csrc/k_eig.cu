@@ -287,11 +287,16 @@ __global__ void __launch_bounds__(EIG_THREADS) k_project_k(const int* ni, const 
     __shared__ Acc part[NW][32];
     for (int c0 = 0; c0 < p; c0 += 32) {
       const int c = c0 + lane;
-      Acc d = 0;
-      if (c < p)
-#pragma unroll 4
-        for (int l = wid; l < n; l += NW) mac(d, kvec[o + l], (Acc)Xi[(int64_t)l * ldx + c]);
-      part[wid][lane] = finish(d);
+      // four sums a lane: chains of n / 32 terms, as many as with a warp per column
+      Acc d[4] = {0, 0, 0, 0};
+      if (c < p) {
+        int l = wid;
+        for (; l + 3 * NW < n; l += 4 * NW)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) mac(d[u], kvec[o + l + u * NW], (Acc)Xi[(int64_t)(l + u * NW) * ldx + c]);
+        for (; l < n; l += NW) mac(d[0], kvec[o + l], (Acc)Xi[(int64_t)l * ldx + c]);
+      }
+      part[wid][lane] = (finish(d[0]) + finish(d[1])) + (finish(d[2]) + finish(d[3]));
       __syncthreads();
       if (wid == 0 && c < p) {
         Acc t = part[0][lane];
