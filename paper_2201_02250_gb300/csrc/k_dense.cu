@@ -622,6 +622,9 @@ void lu_batched(a2ls_handle* h, T* fac, int allow_last_zero, double* last_pivot,
     }
     cfg.gridDim = dim3(h->N * C);
     at[0].val.clusterDim.x = C;
+    // no attribute for CTAs on their own: clusters of one are placed otherwise, and 512 FP64 subdomains of 1500 to
+    // 4000 rows took 674 ms with it, 615 without
+    cfg.numAttrs = C > 1 ? 1 : 0;
     auto kernel = C > 1 ? multi : one;
     A2LS_CUDA(cudaLaunchKernelEx(&cfg, kernel, h->N, (const int*)h->d_ni, (const int*)h->d_ld,
                                  (const int64_t*)h->d_foff, fac, allow_last_zero, last_pivot,

@@ -1644,7 +1644,7 @@ static void eigensolve_t(a2ls_handle* h, T* fac, const double* last_pivot, const
     at[0].val.clusterDim.x = C;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = C > 1 ? 1 : 0;
     A2LS_CUDA(cudaLaunchKernelEx(&cfg, k_orth<TV, T>, (const int*)h->d_ni, (const int64_t*)d_vo, P, (const int*)d_pv,
                                  actv, jb_blocks, b, V, W, Hout, hr, hc, vout, fullv, d_rank, gcap, orc_for(gcap),
                                  illc, h->d_status));

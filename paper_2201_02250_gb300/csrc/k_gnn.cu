@@ -578,7 +578,7 @@ static void launch_loss(cudaStream_t st, int N, const int* off, const int* zm, c
   at[0].val.clusterDim.x = C;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = C > 1 ? 1 : 0;
   A2LS_CUDA(cudaLaunchKernelEx(&cfg, k_loss, off, zm, zoff, Z, Y, scale, loss_i, dY));
 }
 
