@@ -271,7 +271,7 @@ constexpr size_t lu_smem_elems() { return 2 * (size_t)TB * 65 + 2 * (size_t)TGK 
 // block for itself, the tiles of L21, U12 and of the trailing matrix are dealt out, and cluster barriers, which
 // also order the CTAs' global memory accesses, separate the two.  A tile's arithmetic does not depend on who
 // does it.  One CTA each against clusters, per launch: FP64, 64 subdomains of 1700 to 2200 rows, 239 ms against
-// 91 (of 4 CTAs, two an SM); double-float before the steps above, 64 subdomains of 1100 to 1250 rows, 5.4 ms
+// 91 (of 4, two an SM); double-float before the steps above, 64 subdomains of 1100 to 1250 rows, 5.4 ms
 // against 3.8 (of 2).
 template <bool TC> struct LuThreads { static constexpr int value = 256; };
 template <> struct LuThreads<true> { static constexpr int value = tcdf::THREADS; };
@@ -599,7 +599,19 @@ __global__ void __launch_bounds__(LuThreads<TC>::value, TC ? 1 : 2) k_lu(int N, 
 template <class T>
 void lu_batched(a2ls_handle* h, T* fac, int allow_last_zero, double* last_pivot, double* diag_scale, int phase) {
   using Acc = typename AccOf<T>::type;
-  // the largest cluster (of at most 8) of which as many fit the chip at once as there are subdomains
+  // The largest cluster (of at most 8) of which as many fit the chip at once as there are subdomains.  In FP64 two
+  // CTAs share an SM's pipe, which pays where the largest subdomain takes longer than most (its CTAs are soon on
+  // their own: 125 uneven 3D subdomains of 250 to 2600 rows 5.3, 9.9, 48, 199 -> 4.2, 8.1, 36, 130 ms with clusters of
+  // 2) and where a step has tile products enough for all (144 even 2D ones, 9.8 a step, 245 -> 236 ms; 64, clusters
+  // of 4 for 2, 144 -> 139).  Even subdomains with fewer (2.0 a step: 121 of 1152 rows 16.2 -> 17.4 ms, 64 9.9 -> 11.7)
+  // have an SM for every CTA.
+  double flops = 0.0, most = 0.0, steps = 0.0;
+  for (int i = 0; i < h->N; ++i) {
+    flops += h->h_env[4 * i];
+    most = std::max(most, h->h_env[4 * i]);
+    steps += ceil_div(h->h_n[i], TB);
+  }
+  const bool alone = std::is_same<T, double>::value && most * h->N < 1.4 * flops && flops < 8.0 * 2.0 * TB * TB * TB * steps;
   auto go = [&](auto one, auto multi, size_t smem, int threads) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
@@ -611,19 +623,22 @@ void lu_batched(a2ls_handle* h, T* fac, int allow_last_zero, double* last_pivot,
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     A2LS_CUDA(cudaFuncSetAttribute(one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    A2LS_CUDA(cudaFuncSetAttribute(multi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    A2LS_CUDA(cudaFuncSetAttribute(multi, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)std::max(smem, (size_t)128 << 10)));
     int C = 8;
     for (; C > 1; C /= 2) {
       int fit = 0;
       cfg.gridDim = dim3(h->N * C);
       at[0].val.clusterDim.x = C;
+      cfg.dynamicSmemBytes = alone ? std::max(smem, (size_t)128 << 10) : smem;   // (more than half of an SM's)
       A2LS_CUDA(cudaOccupancyMaxActiveClusters(&fit, multi, &cfg));
       if (h->N <= fit) break;
     }
+    cfg.dynamicSmemBytes = smem;
     cfg.gridDim = dim3(h->N * C);
     at[0].val.clusterDim.x = C;
-    // no attribute for CTAs on their own: clusters of one are placed otherwise, and 512 FP64 subdomains of 1500 to
-    // 4000 rows took 674 ms with it, 615 without
+    // no attribute for CTAs on their own: clusters of one are placed otherwise, and 512 FP64 subdomains (727 to 2983
+    // nodes and their overlap) took 674 ms with it, 615 without
     cfg.numAttrs = C > 1 ? 1 : 0;
     auto kernel = C > 1 ? multi : one;
     A2LS_CUDA(cudaLaunchKernelEx(&cfg, kernel, h->N, (const int*)h->d_ni, (const int*)h->d_ld,
