@@ -54,33 +54,20 @@ SE_HD inline double se_dbl(double x) { return x; }
 // unnormalised multiply-add overloads both)
 SE_HD inline void se_mac(double& acc, double a, double b) { acc += a * b; }
 SE_HD inline double se_fin(double a) { return a; }
-// Whether schur() forms its reflectors from se_rsqrt(a) = 1 / sqrt(a), se_recip12(b) = 1 / b for b in [1, 2] and
-// se_scale_to_one(a), a factor that brings a to about 1 (double-float), or keeps to the library's roots and
-// quotients.  FP64 keeps to those and with them its results
+// Whether hessenberg() and schur() form their reflectors from se_rsqrt(a) = 1 / sqrt(a), se_recip12(b) = 1 / b for b in
+// [1, 2], se_scale_to_one(a), a factor that brings a to about 1, se_pow2(a) and se_pow2_inv(p), a's power of two
+// and its inverse, and the warp sums and maxima se_warp_sum and se_warp_maxabs (double-float brings them), or keep
+// to the library's roots and quotients.  FP64 keeps to those and with them its results
 // bit for bit: the block Krylov iteration amplifies a changed rounding until the eigenvectors, kept at a
 // residual of 1e-10, differ at that size, and with them the ninth digit of the preconditioner, which FP64
 // callers compare.
 template <class R> struct SeFast { static constexpr bool v = false; };
-SE_HD inline double se_rsqrt(double a) { return 1.0 / sqrt(a); }
-SE_HD inline double se_recip12(double b) { return 1.0 / b; }
-SE_HD inline double se_scale_to_one(double a) { return 1.0 / a; }
-// (of fast arithmetics: a magnitude's power of two and its inverse, the largest magnitude of a warp)
-SE_HD inline double se_pow2(double) { return 1.0; }
-SE_HD inline double se_pow2_inv(double p) { return p; }
-SE_HD inline double se_warp_maxabs(double) { return 1.0; }
 SE_HD inline bool se_is_zero(double a) {
 #ifdef __CUDA_ARCH__
   return (__double_as_longlong(a) << 1) == 0;
 #else
   return a == 0.0;
 #endif
-}
-// the sum of v over a warp (every lane receives it); a one-thread team has v itself
-SE_HD inline double se_warp_sum(double v) {
-#ifdef __CUDA_ARCH__
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-#endif
-  return v;
 }
 SE_HD inline double se_warp_get(double v, int lane) {
 #ifdef __CUDA_ARCH__
@@ -142,8 +129,9 @@ SE_HD inline R strided_dot(const R* x, int st, const R* v, int n) {
 template <class R>
 SE_HD inline void hessenberg(R* H, int ld, R* Q, int ldq, int m, R* v, const Team& t) {
   for (int k = 0; k + 2 < m; ++k) {
-    R up = 1.0, x0, alpha, beta;
-    if (SeFast<R>::v) {
+    [[maybe_unused]] R up = 1.0;
+    R x0, alpha, beta;
+    if constexpr (SeFast<R>::v) {
       // Householder vector for x = H[k+1.., k], scaled; every warp sums |x|^2 for itself, in the same order
 #ifdef __CUDA_ARCH__
       const int l0 = t.lane & 31, ls = 32;
@@ -232,34 +220,20 @@ SE_HD inline int first_negligible(const R* H, int ld, int hi, R leps, R eps, R h
 // entries and its two quotients go to lanes of one warp (order 48: 7.5 -> 5.2 million cycles, the same
 // bits).
 
-// Apply a 3-element (or 2-element when nv == 2) reflector I - beta u u^T with u = (1, u1, u2)
-// to rows k..k+nv-1 of H from the left (columns c0..m-1) and to columns k..k+nv-1 from the
-// right (rows 0..r1) and to Q's columns.
+// Apply a 2-element reflector I - beta u u^T with u = (1, u1) to rows k, k+1 of H from the left (columns c0..m-1) and to
+// columns k, k+1 from the right (rows 0..r1) and to Q's columns.
 template <class R>
-SE_HD inline void apply_reflector(R* H, int ld, R* Q, int ldq, int m, int k, int nv, R u1, R u2, R beta,
-                                  int c0, int r1, const Team& t) {
-  for (int c = c0 + t.lane; c < m; c += t.size) {
-    R d = H[k * ld + c] + u1 * H[(k + 1) * ld + c] + (nv == 3 ? u2 * H[(k + 2) * ld + c] : 0.0);
+SE_HD inline void apply_reflector2(R* H, int ld, R* Q, int ldq, int m, int k, R u1, R beta, int c0, int r1, const Team& t) {
+  auto reflect = [&](R* a, int st) {
+    R d = a[0] + u1 * a[st];
     d *= beta;
-    H[k * ld + c] -= d;
-    H[(k + 1) * ld + c] -= d * u1;
-    if (nv == 3) H[(k + 2) * ld + c] -= d * u2;
-  }
+    a[0] -= d;
+    a[st] -= d * u1;
+  };
+  for (int c = c0 + t.lane; c < m; c += t.size) reflect(H + k * ld + c, ld);
   t.sync();
-  for (int r = t.lane; r <= r1; r += t.size) {
-    R d = H[r * ld + k] + u1 * H[r * ld + k + 1] + (nv == 3 ? u2 * H[r * ld + k + 2] : 0.0);
-    d *= beta;
-    H[r * ld + k] -= d;
-    H[r * ld + k + 1] -= d * u1;
-    if (nv == 3) H[r * ld + k + 2] -= d * u2;
-  }
-  for (int r = t.lane; r < m; r += t.size) {
-    R d = Q[r * ldq + k] + u1 * Q[r * ldq + k + 1] + (nv == 3 ? u2 * Q[r * ldq + k + 2] : 0.0);
-    d *= beta;
-    Q[r * ldq + k] -= d;
-    Q[r * ldq + k + 1] -= d * u1;
-    if (nv == 3) Q[r * ldq + k + 2] -= d * u2;
-  }
+  for (int r = t.lane; r <= r1; r += t.size) reflect(H + r * ld + k, 1);
+  for (int r = t.lane; r < m; r += t.size) reflect(Q + r * ldq + k, 1);
   t.sync();
 }
 
@@ -407,7 +381,6 @@ SE_HD inline int schur_single(R* H, int ld, R* Q, int ldq, int m, double hnorm_,
     // the right update, instead of every thread forming it after that update (the entries are the
     // values the right update writes).
     t.sync();  // the shift and deflation reads above precede the first update
-    const bool early = true;
     R u1, u2, beta, alpha;
     bool have = make_reflector_div(x, y, z, u1, u2, beta, alpha);
     for (int k = lo; k <= hi - 2; ++k) {
@@ -439,7 +412,7 @@ SE_HD inline int schur_single(R* H, int ld, R* Q, int ldq, int m, double hnorm_,
           a[0] -= d;
           a[st] -= d * u1;
           a[2 * st] -= d * u2;
-          if (early && more && idx < 3) {  // column c0 + idx = k + idx
+          if (more && idx < 3) {  // column c0 + idx = k + idx
             snap[idx] = a[st];
             snap[3 + idx] = a[2 * st];
             snap[6 + idx] = H[(k + 3) * ld + k + idx];
@@ -457,7 +430,7 @@ SE_HD inline int schur_single(R* H, int ld, R* Q, int ldq, int m, double hnorm_,
 #else
         const bool forms = true;
 #endif
-        if (early && more && forms) {
+        if (more && forms) {
           auto entry = [&](int rr) {
             const R a0 = snap[3 * rr], a1 = snap[3 * rr + 1], a2 = snap[3 * rr + 2];
             R d = a0;
@@ -492,15 +465,12 @@ SE_HD inline int schur_single(R* H, int ld, R* Q, int ldq, int m, double hnorm_,
           a[2] -= d * u2;
         }
         t.sync();
-        if (more && early) {
+        if (more) {
           nu1 = snap[9];
           nu2 = snap[10];
           nbeta = snap[11];
           nalpha = snap[12];
           nhave = !se_is_zero(snap[13]);
-        } else if (more) {
-          nhave = make_reflector_div(H[(k + 1) * ld + k], H[(k + 2) * ld + k], H[(k + 3) * ld + k], nu1, nu2, nbeta,
-                                 nalpha);
         }
       } else if (more) {
         nhave = make_reflector_div(H[(k + 1) * ld + k], H[(k + 2) * ld + k], H[(k + 3) * ld + k], nu1, nu2, nbeta,
@@ -519,7 +489,7 @@ SE_HD inline int schur_single(R* H, int ld, R* Q, int ldq, int m, double hnorm_,
       R u1, u2, beta, alpha;
       if (make_reflector_div<R>(x, y, R(0.0), u1, u2, beta, alpha)) {
         t.sync();
-        apply_reflector<R>(H, ld, Q, ldq, m, hi - 1, 2, u1, R(0.0), beta, hi - 2, hi, t);
+        apply_reflector2<R>(H, ld, Q, ldq, m, hi - 1, u1, beta, hi - 2, hi, t);
         if (t.lane == 0) H[hi * ld + hi - 2] = 0.0;
         t.sync();
       }
@@ -602,10 +572,10 @@ SE_HD inline void split_2x2(R* H, int ld, R* Q, int ldq, int m, int p, const Tea
   t.sync();
 }
 
-// The scratch schur() wants: the nine entries of the next reflector's snapshot, the four shift values and two
-// sets of u1, u2, beta, alpha.
-constexpr int SE_SNAP = 21;
-enum { SE_SHIFTS = 9, SE_REFL = 13 };
+// The scratch schur() wants: the nine entries of the next reflector's snapshot and, from SE_REFL, two sets of u1, u2,
+// beta, alpha.
+constexpr int SE_REFL = 9;
+constexpr int SE_SNAP = SE_REFL + 8;
 
 // The shift pair (s1r, s2r, s1i, s2i) of the 2 x 2 block a, b; c, d: a real pair is replaced by its member
 // closer to d, used twice.
@@ -742,28 +712,10 @@ SE_HD inline void se_sweep(R* H, int ld, R* Q, int ldq, int m, int lo, int hi, b
   }
 }
 
-// Francis implicit double-shift QR on an upper Hessenberg H, full Schur form, Q accumulated.
-// A subdiagonal entry is neglected when it is below eps times its two diagonal
-// neighbours or below eps times hnorm (the largest entry of the input), which keeps
-// clusters of eigenvalues near zero from stalling the iteration; the result is
-// backward stable relative to hnorm.  Returns 0 on success, -1 on no convergence.
-// snap: SE_SNAP values of scratch shared by the team (may be null for a one-thread team).
-// local_tol (>= the machine epsilon of R; 0 selects it): the neighbour-relative test may use a looser
-// threshold when the caller needs the Schur form only to that relative accuracy; the test against
-// hnorm always uses the machine epsilon.
-//
-// A sweep's time is the chain of its reflectors, each formed from what the one before it leaves, and not
-// the updates.  Three bulges chased in step with one another (the small-bulge multishift iteration of Braman, Byers
-// and Mathias, SIAM J. Matrix Anal. Appl. 23, 2002) shorten it by a further third, but neglect other entries: with
-// a loose local_tol the Ritz vectors then differ by up to 6e-5 from one bulge's, as far as these are from the
-// exact Schur form's.  Set-up and solve with 256 subdomains of order 72: 120.5 ms with roots and quotients, 116.2
-// without; later, with the other kernels faster, 95.8 against 93.4 with three bulges.
+// schur() without square roots and quotients (see there for the arguments)
 template <class R>
-SE_HD inline int schur(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const Team& t, R* snap = nullptr,
-                       double local_tol = 0.0) {
-  R snap_local[SE_SNAP];
-  if (!snap) snap = snap_local;
-  if (!SeFast<R>::v) return schur_single(H, ld, Q, ldq, m, hnorm_, t, snap, local_tol);
+SE_HD inline int schur_fast(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const Team& t, R* snap,
+                            double local_tol) {
   const R eps = R(SeEps<R>::v), hnorm = R(hnorm_);
   const R leps = R(local_tol > SeEps<R>::v ? local_tol : SeEps<R>::v);
   int hi = m - 1, iter = 0, total = 0;
@@ -790,6 +742,31 @@ SE_HD inline int schur(R* H, int ld, R* Q, int ldq, int m, double hnorm_, const 
     se_sweep(H, ld, Q, ldq, m, lo, hi, iter % 11 == 10, t, snap);
   }
   return 0;
+}
+
+// Francis implicit double-shift QR on an upper Hessenberg H, full Schur form, Q accumulated.
+// A subdiagonal entry is neglected when it is below eps times its two diagonal
+// neighbours or below eps times hnorm (the largest entry of the input), which keeps
+// clusters of eigenvalues near zero from stalling the iteration; the result is
+// backward stable relative to hnorm.  Returns 0 on success, -1 on no convergence.
+// snap: SE_SNAP values of scratch shared by the team (may be null for a one-thread team).
+// local_tol (>= the machine epsilon of R; 0 selects it): the neighbour-relative test may use a looser
+// threshold when the caller needs the Schur form only to that relative accuracy; the test against
+// hnorm always uses the machine epsilon.
+//
+// A sweep's time is the chain of its reflectors, each formed from what the one before it leaves, and not
+// the updates.  Three bulges chased in step with one another (the small-bulge multishift iteration of Braman, Byers
+// and Mathias, SIAM J. Matrix Anal. Appl. 23, 2002) shorten it by a further third, but neglect other entries: with
+// a loose local_tol the Ritz vectors then differ by up to 6e-5 from one bulge's, as far as these are from the
+// exact Schur form's.  Set-up and solve with 256 subdomains of order 72: 120.5 ms with roots and quotients, 116.2
+// without; later, with the other kernels faster, 95.8 against 93.4 with three bulges.
+template <class R>
+SE_HD inline int schur(R* H, int ld, R* Q, int ldq, int m, double hnorm, const Team& t, R* snap = nullptr,
+                       double local_tol = 0.0) {
+  R snap_local[SE_SNAP];
+  if (!snap) snap = snap_local;
+  if constexpr (SeFast<R>::v) return schur_fast(H, ld, Q, ldq, m, hnorm, t, snap, local_tol);
+  else return schur_single(H, ld, Q, ldq, m, hnorm, t, snap, local_tol);
 }
 
 // Eigenvalues of the quasi-triangular S: wr[j], wi[j] (a complex pair occupies j, j+1 with wi[j] > 0).
