@@ -1151,7 +1151,7 @@ static void launch_local_solve(a2ls_handle* h, const T* fac, const double* t, co
 // configurations of the local solves the autotuner chooses from: 256 / 512 / 1024 = the one-pass kernel
 // with that CTA width; 1256 / 1512 / 2256 = the pipelined kernel with 256 or 512 threads and two
 // (1xxx) or four (2xxx) vector loads per row in flight; 3000 / 3004 / 3008 = the streaming kernel on
-// the packed factors (FP32 and BF16 factors) with 8 consumer warps and one CTA per SM / 4 consumer
+// the packed factors with 8 consumer warps and one CTA per SM / 4 consumer
 // warps and two CTAs per SM / 8 consumer warps and two CTAs per SM
 template <class T>
 static void launch_local_solve_width(a2ls_handle* h, int width, const T* fac, const double* t, const double* q,

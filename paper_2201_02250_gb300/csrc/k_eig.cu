@@ -281,20 +281,31 @@ __global__ void __launch_bounds__(EIG_THREADS) k_project_k(const int* ni, const 
     }
     __syncthreads();
   } else {
-    // a lane per column, the rows spread over the warps: whole rows are read at once (a warp per column read
-    // 32 rows 768 bytes apart for each load: 94 us a launch with 64 subdomains of 1100 rows, 68 so)
+    // a lane per column, the rows spread over the warps: whole rows are read at once, eight in flight (a warp per column
+    // read 32 rows 768 bytes apart for each load: 64 subdomains of 1100 rows 94 us a launch, 55 so).  Four sums a lane: 32
+    // chains a column, as many as with a warp per column.
     constexpr int NW = EIG_THREADS / 32;
     __shared__ Acc part[NW][32];
     for (int c0 = 0; c0 < p; c0 += 32) {
       const int c = c0 + lane;
-      // four sums a lane: chains of n / 32 terms, as many as with a warp per column
       Acc d[4] = {0, 0, 0, 0};
       if (c < p) {
+        constexpr int RU = 8;
+        const int64_t step = (int64_t)NW * ldx;
+        const T* x = Xi + (int64_t)wid * ldx + c;
+        const Acc* k = kvec + o + wid;
         int l = wid;
-        for (; l + 3 * NW < n; l += 4 * NW)
+        for (; l + (RU - 1) * NW < n; l += RU * NW, x += RU * step, k += RU * NW) {
+          Acc xv[RU], kv[RU];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) mac(d[u], kvec[o + l + u * NW], (Acc)Xi[(int64_t)(l + u * NW) * ldx + c]);
-        for (; l < n; l += NW) mac(d[0], kvec[o + l], (Acc)Xi[(int64_t)l * ldx + c]);
+          for (int u = 0; u < RU; ++u) {
+            xv[u] = (Acc)x[u * step];
+            kv[u] = k[u * NW];
+          }
+#pragma unroll
+          for (int u = 0; u < RU; ++u) mac(d[u & 3], kv[u], xv[u]);
+        }
+        for (; l < n; l += NW, x += step, k += NW) mac(d[0], *k, (Acc)*x);
       }
       part[wid][lane] = (finish(d[0]) + finish(d[1])) + (finish(d[2]) + finish(d[3]));
       __syncthreads();
