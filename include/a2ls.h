@@ -132,9 +132,11 @@ typedef struct {
                                largest relative residual of the wanted Ritz pairs has not halved over
                                this many cycles stops with the Ritz vectors it has (counted as
                                unconverged, and as stagnated by A2LS_Q_EIG_UNCONVERGED); 0 = off */
-  int32_t tensor_cores;     /* 1 (default): the trailing updates of the double-float LU run on the tensor
-                               cores (BF16 digit products accumulated exactly in FP32, to double-float
-                               accuracy); 0: on the FP32 pipe */
+  int32_t tensor_cores;     /* 1 (default): the trailing updates of the double-float LU and the eigensolves'
+                               triangular solves run on the tensor cores (BF16 digit products accumulated
+                               exactly in FP32, to double-float accuracy of the largest entry of a row and
+                               of a column); 0: on the FP32 pipe, exact entry by entry, for matrices whose
+                               rows and columns are scaled by very different factors */
   int32_t eig_thick_restart; /* 1 (default): a restart of the local eigensolves keeps the block of Ritz
                                vectors together with its image under the operator, so that a restarted
                                cycle spans the same block Krylov space with one block application fewer;
