@@ -135,7 +135,7 @@ typedef struct {
   int32_t tensor_cores;     /* 1 (default): the trailing updates of the double-float LU and the eigensolves'
                                triangular solves run on the tensor cores (BF16 digit products accumulated
                                exactly in FP32, to double-float accuracy of the largest entry of a row and
-                               of a column); 0: on the FP32 pipe, exact entry by entry, for matrices whose
+                               of a column); 0: on the FP32 pipe, accurate entry by entry, for matrices whose
                                rows and columns are scaled by very different factors */
   int32_t eig_thick_restart; /* 1 (default): a restart of the local eigensolves keeps the block of Ritz
                                vectors together with its image under the operator, so that a restarted
