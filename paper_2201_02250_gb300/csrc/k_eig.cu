@@ -397,16 +397,14 @@ constexpr int SROW = EIG_MAXP + 2;
 constexpr int GRAM_NG_MAX = 16;          // row groups (split-K) of a Gram product
 
 // stage rows [l0, l0 + rows) of M (cols 0:w) into S (stride SROW), zero padding to a multiple of 4
-// (FP64 rows past L1: a cluster's CTAs read what the others have written)
-__device__ __forceinline__ double ld_shared_rows(const double* p) { return __ldcg(p); }
-template <class TM>
-__device__ __forceinline__ TM ld_shared_rows(const TM* p) { return *p; }
+// (In FP64 a cluster's CTAs read rows that the others have written, by plain loads: the cluster barrier between
+// acquires them.  Loads past L1 cost launches of single CTAs 1 %.)
 template <class Acc, class TM, int NT = OrthThreads<Acc>::v>
 __device__ __forceinline__ void stage_rows(Acc* S, const TM* M, int64_t ldx, int l0, int rows, int w) {
   const int wp = (w + 3) & ~3;
   for (int e = threadIdx.x; e < rows * wp; e += NT) {
     const int r = e / wp, c = e % wp;
-    S[r * SROW + c] = c < w ? (Acc)ld_shared_rows(M + (int64_t)(l0 + r) * ldx + c) : (Acc)0;
+    S[r * SROW + c] = c < w ? (Acc)M[(int64_t)(l0 + r) * ldx + c] : (Acc)0;
   }
 }
 
