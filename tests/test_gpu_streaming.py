@@ -116,3 +116,13 @@ def test_fp64_factors_are_held_once_unless_streamed(tmp_path):
     assert kernel == 512 and held - base < copy // 2
     kernel, held, _ = footprint(0, 3000)
     assert kernel == 3000 and held - base > copy // 2
+
+
+def test_fp64_copy_is_withheld_and_given_back(tmp_path):
+    from paper_2201_02250_gb300 import _build
+    exe, libdir = str(tmp_path / "stream_memory"), os.path.dirname(_build.LIB)
+    subprocess.run([_build.nvcc(), *_build.ARCH, "-O2", "-std=c++17", "--expt-relaxed-constexpr",
+                    os.path.join(ROOT, "tests", "cpp", "stream_memory.cu"), "-L", libdir, "-lA2LS", "-Xlinker", "-rpath=" + libdir,
+                    "-o", exe], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and r.stdout == "ok\n", r.stdout + r.stderr
